@@ -1,4 +1,4 @@
-// Backward pass of the prefill attention on the tcgen05 tensor cores (head dimension 128), Sec. 3.2.2.
+// Backward pass of the prefill attention on the tcgen05 tensor cores, Sec. 3.2.2.
 //
 // One block owns a tile of 128 keys of one (sequence, kv head) and walks the 64-row query tiles that can
 // see it, for every query head of the GQA group.  All five products of a step run as tcgen05.mma with the
@@ -8,19 +8,23 @@
 //   dP^T = V  dO^T   [128 keys x 64 rows]   A = V tile, B = dO tile
 //   dV  += P^T  dO   [128 keys x D]         A = P^T in tensor memory (bf16), B = dO tile read MN-major
 //   dK  += dS^T Q    [128 keys x D]         A = dS^T in tensor memory,        B = Q tile read MN-major
-//   dQ^T = K^T dS^T  [D x 64 rows]          A = K tile read MN-major, B = dS^T in shared memory (MN-major)
+//   D = 128:  dQ^T = K^T dS^T [D x 64 rows]   A = K tile read MN-major, B = dS^T in shared memory (MN-major)
+//   D =  64:  dQ   = dS  K    [64 rows x D]   A = dS^T in shared memory read MN-major, B = K tile read MN-major
 //
 // with P^T = exp2(S^T * scale * log2e - lse2[row]) and dS^T = P^T * (scale * dP^T - scale * delta[row]) computed by
 // the thread that owns the key (one tensor-memory lane per key).  dV and dK stay in tensor memory for the
-// whole block; dQ^T goes through shared memory (transposed to [rows][D], in the ring stage of the step's Q and dO
-// tiles, which are dead by then) and is added to an fp32 accumulator in global memory by one bulk reduce-add copy (per-lane atomics saturate the L2 atomic units and stall the block's
+// whole block; dQ goes through shared memory (as [rows][D], in the ring stage of the step's Q and dO
+// tiles, which are dead by then) and is added to an fp32 accumulator in global memory by bulk reduce-add copies
+// (per-lane atomics saturate the L2 atomic units and stall the block's
 // other shared-memory traffic behind them).  Two groups of four warps take alternate steps, each with its own S^T/dP^T columns, so the
 // element-wise work of one step overlaps the products of the other.
 //
-// Tensor memory (512 columns): dV [0,128) | dK [128,256) | X_0 [256,384) | X_1 [384,512); X_g holds
-// S^T [0,64) and dP^T [64,128) of the group's step, then P^T (bf16 pairs, [0,32)) and dS^T ([64,96)),
+// Tensor memory (512 columns).  D = 128: dV [0,128) | dK [128,256) | X_0 [256,384) | X_1 [384,512).
+// D = 64: dV [0,64) | dK [64,128) | X_0 [128,256) | X_1 [256,384) | dQ_0 [384,448) | dQ_1 [448,512).  X_g holds
+// S^T [0,64) and dP^T [64,128) of the group's step, then P^T (bf16 pairs, [0,32)) and dS^T ([64,96)); at D = 128
 // then dQ^T [0,64).  The tensor core runs the products of one issuing thread in order, which is what
-// makes these overlays safe.
+// makes these overlays safe.  At D = 64 dQ has columns of its own (64 rows = 16 lanes of every quadrant), so the products
+// that feed a group's next step are issued before it and never wait for its read-out.
 //
 // Warps 0-7: the two element-wise groups; warp 8: TMA producer (K, V once; Q, dO and the row terms per
 // step through a ring of four stages); warp 9: MMA issuer.  Every wait is bounded.
@@ -38,13 +42,14 @@ constexpr int kBwdTcRows = 64;     // query rows per step
 constexpr int kBwdTcThreads = 320;
 constexpr int kBwdTcStages = 4;    // ring of (Q, dO, row terms); a stage also stages the step's dQ on its way out
 
+template <int D>
 struct BackwardTcSmem {
-    static constexpr int D = 128;
-    static constexpr int kKVTileBytes = kBwdTcKeys * D * 2;    // 32 KiB: two panels of [128][64 ch]
+    static constexpr int kPanels = D / 64;
+    static constexpr int kKVTileBytes = kBwdTcKeys * D * 2;    // panels of [128][64 ch]
     static constexpr int kKVPanelBytes = kBwdTcKeys * 128;
-    static constexpr int kQTileBytes = kBwdTcRows * D * 2;     // 16 KiB: two panels of [64][64 ch]
+    static constexpr int kQTileBytes = kBwdTcRows * D * 2;     // panels of [64][64 ch]
     static constexpr int kQPanelBytes = kBwdTcRows * 128;
-    static constexpr int kStageBytes = 2 * kQTileBytes;        // Q then dO
+    static constexpr int kStageBytes = 2 * kQTileBytes;        // Q then dO; later dQ [64][D] fp32
     static constexpr int kDSBytes = kBwdTcKeys * 128;          // dS^T [128 keys][64 rows] bf16
     static constexpr int kOffK = 0, kOffV = kKVTileBytes;
     static constexpr int kOffRing = 2 * kKVTileBytes;
@@ -74,15 +79,17 @@ __device__ __forceinline__ bool group_all(bool pred, int id) {
     return r != 0;
 }
 
+template <int D>
 __global__ void __launch_bounds__(kBwdTcThreads, 1)
 backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
                    const __grid_constant__ CUtensorMap tm_dq, const BackwardParams p) {
-    using L = BackwardTcSmem;
-    constexpr int D = 128, BK = kBwdTcKeys, BR = kBwdTcRows, NQ = kBwdTcStages;
+    using L = BackwardTcSmem<D>;
+    constexpr int BK = kBwdTcKeys, BR = kBwdTcRows, NQ = kBwdTcStages;
     constexpr uint32_t kIdS = make_idesc(BK, BR, 0);      // S^T, dP^T
     constexpr uint32_t kIdKV = make_idesc(BK, D, 1);      // dV, dK (A from tensor memory)
-    constexpr uint32_t kIdDQ = make_idesc_mn_mn(D, BR);   // dQ^T
+    constexpr bool kWide = D == 128;
+    constexpr uint32_t kIdDQ = kWide ? make_idesc_mn_mn(D, BR) : make_idesc_mn_mn(BR, D);  // dQ^T / dQ
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t smem_base = smem_u32(smem_raw);
@@ -102,9 +109,10 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int hk = blockIdx.y, b = blockIdx.z;
-    // blockIdx.x -> (key tile, chunk of its query range); see backward_kernel
+    // blockIdx.x -> (key tile, chunk of its query range): the tiles that hold sink keys meet every later query
+    // tile, so their range is cut into chunks of kBwdChunkTiles query tiles handled by separate blocks
     int n_tile, chunk = -1;
     if ((int)blockIdx.x < p.sink_tiles * p.chunks) {
         n_tile = (int)blockIdx.x / p.chunks;
@@ -152,8 +160,10 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    const uint32_t tDV = tmem_base, tDK = tmem_base + 128u;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const uint32_t tDV = tmem_base, tDK = tmem_base + (uint32_t)D;
+    constexpr uint32_t kX = 2u * (uint32_t)D;          // first column of X_0
+    constexpr uint32_t kDQ = kX + 256u;                // first column of dQ_0 (D = 64)
     const float sl2 = p.scale * 1.4426950408889634f;
 
     if (warp == 8) {
@@ -162,7 +172,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         if (lane == 0) {
             mbar_arrive_expect_tx(bar(BAR_KV), 2u * (uint32_t)L::kKVTileBytes);
 #pragma unroll
-            for (int pn = 0; pn < 2; ++pn) {
+            for (int pn = 0; pn < L::kPanels; ++pn) {
                 tma_load_3d(sK + pn * L::kKVPanelBytes, &tm_k, pn * 64, hk, seq_start + j0, bar(BAR_KV));
                 tma_load_3d(sV + pn * L::kKVPanelBytes, &tm_v, pn * 64, hk, seq_start + j0, bar(BAR_KV));
             }
@@ -177,7 +187,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 const uint32_t dst = sRing + (uint32_t)st * L::kStageBytes;
                 mbar_arrive_expect_tx(bar(BAR_QF + st), (uint32_t)L::kStageBytes);
 #pragma unroll
-                for (int pn = 0; pn < 2; ++pn) {
+                for (int pn = 0; pn < L::kPanels; ++pn) {
                     tma_load_3d(dst + pn * L::kQPanelBytes, &tm_q, pn * 64, h, seq_start + i0, bar(BAR_QF + st));
                     tma_load_3d(dst + L::kQTileBytes + pn * L::kQPanelBytes, &tm_do, pn * 64, h, seq_start + i0,
                                 bar(BAR_QF + st));
@@ -205,90 +215,116 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         __syncwarp();
     } else if (warp == 9) {
         // =================================================================================== issuer
-        if (lane == 0) {
-            const uint32_t hi = (uint32_t)(smem_desc_sw128(0, 0, 1024) >> 32);
-            const uint32_t k_a = (uint32_t)smem_desc_sw128(sK, 16, 1024);                    // K tile, K-major (A)
-            const uint32_t v_a = (uint32_t)smem_desc_sw128(sV, 16, 1024);                    // V tile, K-major (A)
-            const uint32_t k_t = (uint32_t)smem_desc_sw128(sK, L::kKVPanelBytes, 1024);      // K tile, MN-major (A)
-            const uint32_t q_b0 = (uint32_t)smem_desc_sw128(sRing, 16, 1024);                // Q tile of stage 0, K-major (B)
-            const uint32_t q_t0 = (uint32_t)smem_desc_sw128(sRing, L::kQPanelBytes, 1024);   // Q tile of stage 0, MN-major (B)
-            const uint32_t ds_t0 = (uint32_t)smem_desc_sw128(sDS, 16, 1024);                 // dS^T of group 0, MN-major (B)
-            constexpr uint32_t kStageStep = (uint32_t)L::kStageBytes >> 4, kDoStep = (uint32_t)L::kQTileBytes >> 4;
-            constexpr uint32_t kDsStep = (uint32_t)L::kDSBytes >> 4;
-            // S^T = K Q^T (columns [0,64) of X_{s & 1}) and dP^T = V dO^T (columns [64,128)) of step s
-            auto issue_st = [&](int s) {
-                const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + 256u + 128u * (uint32_t)(s & 1);
+        // The warp runs the loop as a whole, one elected lane issues: see elect_one.
+        const bool el = elect_one();
+        const uint32_t hi = (uint32_t)(smem_desc_sw128(0, 0, 1024) >> 32);
+        const uint32_t k_a = (uint32_t)smem_desc_sw128(sK, 16, 1024);                    // K tile, K-major (A)
+        const uint32_t v_a = (uint32_t)smem_desc_sw128(sV, 16, 1024);                    // V tile, K-major (A)
+        const uint32_t k_t = (uint32_t)smem_desc_sw128(sK, L::kKVPanelBytes, 1024);      // K tile, MN-major (A, or B at D = 64)
+        const uint32_t q_b0 = (uint32_t)smem_desc_sw128(sRing, 16, 1024);                // Q tile of stage 0, K-major (B)
+        const uint32_t q_t0 = (uint32_t)smem_desc_sw128(sRing, L::kQPanelBytes, 1024);   // Q tile of stage 0, MN-major (B)
+        const uint32_t ds_t0 = (uint32_t)smem_desc_sw128(sDS, 16, 1024);                 // dS^T of group 0, MN-major (B, or A at D = 64)
+        constexpr uint32_t kStageStep = (uint32_t)L::kStageBytes >> 4, kDoStep = (uint32_t)L::kQTileBytes >> 4;
+        constexpr uint32_t kDsStep = (uint32_t)L::kDSBytes >> 4;
+        // S^T = K Q^T (columns [0,64) of X_{s & 1}) and dP^T = V dO^T (columns [64,128)) of step s
+        auto issue_st = [&](int s) {
+            const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
-                    const uint32_t ob = ((uint32_t)(kk >> 2) * L::kQPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
-                    mma_ss_lh(tX, k_a + oa, qb + ob, hi, kIdS, kk > 0 ? 1u : 0u);
-                }
-            };
-            auto issue_dp = [&](int s) {
-                const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + 256u + 128u * (uint32_t)(s & 1);
+            for (int kk = 0; kk < D / 16; ++kk) {
+                const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
+                const uint32_t ob = ((uint32_t)(kk >> 2) * L::kQPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
+                mma_ss_lh(tX, k_a + oa, qb + ob, hi, kIdS, kk > 0 ? 1u : 0u);
+            }
+        };
+        auto issue_dp = [&](int s) {
+            const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
-                    const uint32_t ob = ((uint32_t)(kk >> 2) * L::kQPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
-                    mma_ss_lh(tX + 64u, v_a + oa, qb + kDoStep + ob, hi, kIdS, kk > 0 ? 1u : 0u);
-                }
-            };
-            // dV += P^T dO, dK += dS^T Q, dQ^T = K^T dS^T of step s
-            auto issue_g = [&](int s) {
-                const uint32_t qt = q_t0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + 256u + 128u * (uint32_t)(s & 1);
-                const uint32_t ds = ds_t0 + (uint32_t)(s & 1) * kDsStep;
+            for (int kk = 0; kk < D / 16; ++kk) {
+                const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
+                const uint32_t ob = ((uint32_t)(kk >> 2) * L::kQPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
+                mma_ss_lh(tX + 64u, v_a + oa, qb + kDoStep + ob, hi, kIdS, kk > 0 ? 1u : 0u);
+            }
+        };
+        // dV += P^T dO, dK += dS^T Q of step s
+        auto issue_dkv = [&](int s) {
+            const uint32_t qt = q_t0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
 #pragma unroll
-                for (int kk = 0; kk < BR / 16; ++kk) {  // 16 rows: 8 columns of bf16 pairs, 16 rows of 128 bytes
-                    const uint32_t ob = ((uint32_t)kk * 2048u) >> 4;
-                    mma_ts_lh(tDV, tX + (uint32_t)kk * 8u, qt + kDoStep + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
-                    mma_ts_lh(tDK, tX + 64u + (uint32_t)kk * 8u, qt + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
-                }
+            for (int kk = 0; kk < BR / 16; ++kk) {  // 16 rows: 8 columns of bf16 pairs, 16 rows of 128 bytes
+                const uint32_t ob = ((uint32_t)kk * 2048u) >> 4;
+                mma_ts_lh(tDV, tX + (uint32_t)kk * 8u, qt + kDoStep + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
+                mma_ts_lh(tDK, tX + 64u + (uint32_t)kk * 8u, qt + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
+            }
+        };
+        // dQ^T = K^T dS^T (D = 128, over S^T) or dQ = dS K (D = 64) of step s
+        auto issue_dq = [&](int s) {
+            const uint32_t g = (uint32_t)(s & 1), ds = ds_t0 + g * kDsStep;
+            const uint32_t d = tmem_base + (kWide ? kX + 128u * g : kDQ + 64u * g);
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk) {  // 16 keys: 16 rows of 128 bytes in both operands
-                    const uint32_t o = ((uint32_t)kk * 2048u) >> 4;
-                    mma_ss_lh(tX, k_t + o, ds + o, hi, kIdDQ, kk > 0 ? 1u : 0u);
-                }
-            };
-            bool ok = mbar_wait(bar(BAR_KV), 0u, abort_flag);
-            for (int s = 0; s < 2 && s < n_steps && ok; ++s) {
-                ok = mbar_wait(bar(BAR_QF + s % NQ), 0u, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
+            for (int kk = 0; kk < BK / 16; ++kk) {  // 16 keys: 16 rows of 128 bytes in both operands
+                const uint32_t o = ((uint32_t)kk * 2048u) >> 4;
+                mma_ss_lh(d, (kWide ? k_t : ds) + o, (kWide ? ds : k_t) + o, hi, kIdDQ, kk > 0 ? 1u : 0u);
+            }
+        };
+        bool ok = warp_wait(bar(BAR_KV), 0u, abort_flag);
+        for (int s = 0; s < 2 && s < n_steps && ok; ++s) {
+            ok = warp_wait(bar(BAR_QF + s % NQ), 0u, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            if (el) {
                 issue_dp(s);
                 issue_st(s);
                 tc_commit(bar(BAR_SF + s));
             }
-            // Steady state: G(s) as soon as the group has written P^T, dS^T of step s; then the products that feed
-            // the same group's step s + 2.  dP^T(s+2) only needs columns [64,128), free once G(s) has run (products
-            // run in issue order), and fills the time until the group has taken dQ^T(s) out of the columns that
-            // S^T(s+2) overwrites.  (Every look at a barrier costs this thread about 80 cycles during which no
-            // product is issued; folding the tile barrier into the group's arrival was slower all the same, because
-            // dP^T then waits for the read-out too.)
-            for (int s = 0; s < n_steps && ok; ++s) {
-                const int g = s & 1;
-                const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-                ok = mbar_wait(bar(BAR_PR + g), ph, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                issue_g(s);
-                tc_commit(bar(BAR_DQ + g));
-                if (s + 2 < n_steps) {
-                    // (this look falls under the tail of G(s); ahead of the wait for the group it was slower)
-                    ok = mbar_wait(bar(BAR_QF + (s + 2) % NQ), (uint32_t)((s + 2) / NQ) & 1u, abort_flag);
+        }
+        // Steady state: the gradients of step s as soon as the group has written P^T, dS^T; then (D = 64: before dQ) the
+        // products that feed the same group's step s + 2.  dP^T(s+2) only needs columns [64,128), free once dK(s) has run
+        // (products run in issue order); at D = 128 it fills the time until the group has taken dQ^T(s) out of the
+        // columns that S^T(s+2) overwrites.  (At D = 64 the columns of dQ(s - 2) were read out before the group's arrival
+        // with P^T of step s.)
+        for (int s = 0; s < n_steps && ok; ++s) {
+            const int g = s & 1;
+            const uint32_t ph = (uint32_t)(s >> 1) & 1u;
+            const bool more = s + 2 < n_steps;
+            ok = warp_wait(bar(BAR_PR + g), ph, abort_flag);
+            if (!ok) break;
+            tc_fence_after();
+            if (el) issue_dkv(s);
+            if (kWide) {
+                if (el) {
+                    issue_dq(s);
+                    tc_commit(bar(BAR_DQ + g));
+                }
+                if (more) {
+                    ok = warp_wait(bar(BAR_QF + (s + 2) % NQ), (uint32_t)((s + 2) / NQ) & 1u, abort_flag);
                     if (!ok) break;
-                    issue_dp(s + 2);
-                    ok = mbar_wait(bar(BAR_DR + g), ph, abort_flag);
+                    if (el) issue_dp(s + 2);
+                    ok = warp_wait(bar(BAR_DR + g), ph, abort_flag);
                     if (!ok) break;
                     tc_fence_after();
-                    issue_st(s + 2);
-                    tc_commit(bar(BAR_SF + g));
+                    if (el) {
+                        issue_st(s + 2);
+                        tc_commit(bar(BAR_SF + g));
+                    }
+                }
+            } else {
+                if (more) {
+                    ok = warp_wait(bar(BAR_QF + (s + 2) % NQ), (uint32_t)((s + 2) / NQ) & 1u, abort_flag);
+                    if (!ok) break;
+                    if (el) {
+                        issue_st(s + 2);
+                        issue_dp(s + 2);
+                        tc_commit(bar(BAR_SF + g));
+                    }
+                }
+                if (el) {
+                    issue_dq(s);
+                    tc_commit(bar(BAR_DQ + g));
                 }
             }
-            // all products issued by this thread must have retired before the tensor memory is read or freed
-            tc_commit(bar(BAR_FIN));
-            mbar_wait(bar(BAR_FIN), 0u, abort_flag);
         }
+        // all products issued by this warp must have retired before the tensor memory is read or freed
+        if (el) tc_commit(bar(BAR_FIN));
+        warp_wait(bar(BAR_FIN), 0u, abort_flag);
         __syncwarp();
     } else {
         // ===================================================================== element-wise groups
@@ -296,7 +332,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int kl = 32 * quad + lane;  // tensor-memory lane: the key (S^T, dP^T, dV, dK) or the channel (dQ^T)
         const int j = j0 + kl;
         const uint32_t lane_bits = (uint32_t)(32 * quad) << 16;
-        const uint32_t tX = tmem_base + lane_bits + 256u + 128u * (uint32_t)grp;
+        const uint32_t tX = tmem_base + lane_bits + kX + 128u * (uint32_t)grp;
         const uint32_t sDSg = sDS + (uint32_t)grp * L::kDSBytes + (uint32_t)kl * 128u;
         // rows of the step that this key sees: i in [max(j, .), hi) with hi = end of the window (or of the sequence)
         const int vis_hi = (full || j < p.n_sink) ? Lseq : (int)min((long long)Lseq, (long long)j + p.window);
@@ -386,15 +422,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             tc_fence_before();
             mbar_arrive(bar(BAR_PR + grp));
 
-            // ---- dQ^T of this step (lane = channel, column = row) -> [64 rows][128 channels] fp32 in the step's
-            // ring stage (Q and dO are no longer needed once dQ^T is complete) -> one bulk reduce-add of the box
-            // into the fp32 accumulator.  Rows of the box past the end of the sequence receive exact zeros (their
+            // ---- dQ of this step -> [64 rows][D] fp32 in the step's
+            // ring stage (Q and dO are no longer needed once dQ is complete) -> bulk reduce-add
+            // into the fp32 accumulator.  Rows past the end of the sequence receive exact zeros (their
             // dS^T columns are zero); rows past T are clipped by the copy.
             ok = group_all(mbar_wait(bar(BAR_DQ + grp), ph, abort_flag), 1 + grp);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t stg = sRing + (uint32_t)st * L::kStageBytes + (uint32_t)kl * 4u;
-            {
+            const uint32_t stage = sRing + (uint32_t)st * L::kStageBytes;
+            if (kWide) {  // dQ^T: lane = channel, column = row
+                const uint32_t stg = stage + (uint32_t)kl * 4u;
                 uint32_t v0[32], v1[32];
                 tmem_ld32(tX, v0);
                 tmem_ld32(tX + 32u, v1);
@@ -407,11 +444,27 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + (uint32_t)(e * 512)), "r"(v0[e]) : "memory");
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + (uint32_t)((32 + e) * 512)), "r"(v1[e]) : "memory");
                 }
+            } else {  // dQ: row 16 * quad + lane in lanes 0..15 of the quadrant, column = channel; panels of 32 channels, swizzled
+                const uint32_t tQ = tmem_base + lane_bits + kDQ + 64u * (uint32_t)grp;
+                const int r = 16 * quad + (lane & 15);
+#pragma unroll
+                for (int pn = 0; pn < 2; ++pn) {
+                    uint32_t v[32];
+                    tmem_ld32(tQ + 32u * (uint32_t)pn, v);
+                    tc_wait_ld();
+                    if (lane < 16)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            st_shared_v4(stage + (uint32_t)(pn * 8192 + r * 128 + ((j ^ (r & 7)) << 4)), v[4 * j], v[4 * j + 1],
+                                         v[4 * j + 2], v[4 * j + 3]);
+                }
+                tc_fence_before();
             }
             fence_proxy_async_smem();
             asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
             if (kl == 0) {
-                tma_reduce_add_3d(&tm_dq, sRing + (uint32_t)st * L::kStageBytes, 0, h, seq_start + i0);
+                tma_reduce_add_3d(&tm_dq, stage, 0, h, seq_start + i0);
+                if (!kWide) tma_reduce_add_3d(&tm_dq, stage + 8192u, 32, h, seq_start + i0);
                 tma_store_commit();
                 pending_stage = st;
             }
@@ -421,14 +474,14 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         if (ok) ok = mbar_wait(bar(BAR_FIN), 0u, abort_flag);
         if (ok) {
             tc_fence_after();
-            const uint32_t tAcc = tmem_base + lane_bits + 128u * (uint32_t)grp;
+            const uint32_t tAcc = tmem_base + lane_bits + (uint32_t)(D * grp);
             if (split) {
                 const int sink_rows = p.sink_tiles * BK;
                 const size_t plane = (size_t)p.B * sink_rows * p.Hkv * D;
                 float* dst = p.dkv_accum + (size_t)(1 - grp) * plane +  // plane 0: dk, plane 1: dv
                              (((size_t)b * sink_rows + j) * p.Hkv + hk) * D;
 #pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
+                for (int c4 = 0; c4 < D / 32; ++c4) {
                     uint32_t v[32];
                     tmem_ld32(tAcc + 32u * (uint32_t)c4, v);
                     tc_wait_ld();
@@ -442,7 +495,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             } else {
                 __nv_bfloat16* dst = (grp == 0 ? p.dv : p.dk) + ((size_t)(seq_start + j) * p.Hkv + hk) * D;
 #pragma unroll
-                for (int c4 = 0; c4 < 4; ++c4) {
+                for (int c4 = 0; c4 < D / 32; ++c4) {
                     uint32_t v[32];
                     tmem_ld32(tAcc + 32u * (uint32_t)c4, v);
                     tc_wait_ld();

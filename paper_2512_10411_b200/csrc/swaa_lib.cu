@@ -419,16 +419,18 @@ static int make_token_major_map_uncached(CUtensorMap* map, const void* base, int
     return r == CUDA_SUCCESS ? SWAA_OK : SWAA_ERR_CUDA;
 }
 
-// fp32 [T][H][D] accumulator, boxes of [rows][1 head][D] without swizzle (target of bulk reduce-add copies).
+// fp32 [T][H][D] accumulator (target of bulk reduce-add copies): boxes of [rows][1 head][D] without swizzle at D = 128,
+// of [rows][1 head][32 channels] with the 128-byte swizzle at D = 64.
 static int make_accum_map(CUtensorMap* map, const float* base, int T, int H, int D, int box_rows) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return SWAA_ERR_CUDA;
     const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T};
     const cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)H * D * 4};
-    const cuuint32_t box[3] = {(cuuint32_t)D, 1, (cuuint32_t)box_rows};
+    const cuuint32_t box[3] = {(cuuint32_t)(D == 128 ? 128 : 32), 1, (cuuint32_t)box_rows};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr,
-                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE,
+                           D == 128 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? SWAA_OK : SWAA_ERR_CUDA;
 }
@@ -672,7 +674,7 @@ struct BackwardWorkspace {
 
 static BackwardWorkspace backward_workspace(int B, int T, int Hq, int Hkv, int D, int n_sink) {
     BackwardWorkspace w;
-    // rows of the key tiles that hold sink keys, in whole tiles of the wider of the two kernels
+    // rows of the key tiles that hold sink keys, in whole tiles
     const long long t_rows = ((long long)T + kBwdTcKeys - 1) / kBwdTcKeys * kBwdTcKeys;
     const long long s_rows = ((long long)n_sink + kBwdTcKeys - 1) / kBwdTcKeys * kBwdTcKeys;
     w.sink_rows = (int)(s_rows < t_rows ? s_rows : t_rows);
@@ -684,42 +686,30 @@ static BackwardWorkspace backward_workspace(int B, int T, int Hq, int Hkv, int D
     return w;
 }
 
-// D = 128 runs on the tcgen05 kernel (128-key tiles), D = 64 on the warp-level kernel (64-key tiles).
 template <int D>
 static int launch_backward(const void* q, const void* k, const void* v, const void* out, const void* dout,
                            const BackwardParams& p, void* dq, int max_seqlen, size_t dkv_zero_bytes, cudaStream_t st) {
-    constexpr bool kTc = D == 128;
-    constexpr int kKeyTile = kTc ? kBwdTcKeys : kBwdTile;
-    constexpr int kRowTile = kTc ? kBwdTcRows : kBwdTile;
-    CUtensorMap tq, tk, tv, tdo;
+    constexpr int kKeyTile = kBwdTcKeys;
+    CUtensorMap tq, tk, tv, tdo, tacc;
     int rc;
-    if ((rc = make_token_major_map(&tq, q, p.T, p.Hq, D, kRowTile)) != SWAA_OK) return rc;
+    if ((rc = make_token_major_map(&tq, q, p.T, p.Hq, D, kBwdTcRows)) != SWAA_OK) return rc;
     if ((rc = make_token_major_map(&tk, k, p.T, p.Hkv, D, kKeyTile)) != SWAA_OK) return rc;
     if ((rc = make_token_major_map(&tv, v, p.T, p.Hkv, D, kKeyTile)) != SWAA_OK) return rc;
-    if ((rc = make_token_major_map(&tdo, dout, p.T, p.Hq, D, kRowTile)) != SWAA_OK) return rc;
+    if ((rc = make_token_major_map(&tdo, dout, p.T, p.Hq, D, kBwdTcRows)) != SWAA_OK) return rc;
+    if ((rc = make_accum_map(&tacc, p.dq_accum, p.T, p.Hq, D, kBwdTcRows)) != SWAA_OK) return rc;
     const size_t n_acc = (size_t)p.T * p.Hq * D;
     // the dq accumulator is cleared by the kernel that computes the row terms; the (small) dk, dv accumulators here
     if (dkv_zero_bytes > 0 && cudaMemsetAsync(p.dkv_accum, 0, dkv_zero_bytes, st) != cudaSuccess) return SWAA_ERR_CUDA;
-    const int rows = p.T * p.Hq;
-    backward_delta_kernel<D><<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(
+    const long long delta_threads = (long long)p.T * p.Hq * (D / 8);
+    backward_delta_kernel<D><<<(unsigned)((delta_threads + 255) / 256), 256, 0, st>>>(
         static_cast<const __nv_bfloat16*>(out), static_cast<const __nv_bfloat16*>(dout), p.lse,
         const_cast<float*>(p.delta), const_cast<float*>(p.lse2), p.dq_accum, p.T, p.Hq);
     const int ntiles = (max_seqlen + kKeyTile - 1) / kKeyTile;
     const dim3 grid((unsigned)(p.sink_tiles * p.chunks + (ntiles - p.sink_tiles)), (unsigned)p.Hkv, (unsigned)p.B);
-    if constexpr (kTc) {
-        if (cudaFuncSetAttribute(backward_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 BackwardTcSmem::kDynamicBytes) != cudaSuccess)
-            return SWAA_ERR_CUDA;
-        CUtensorMap tacc;
-        if ((rc = make_accum_map(&tacc, p.dq_accum, p.T, p.Hq, D, kBwdTcRows)) != SWAA_OK) return rc;
-        backward_tc_kernel<<<grid, kBwdTcThreads, BackwardTcSmem::kDynamicBytes, st>>>(tq, tk, tv, tdo, tacc, p);
-    } else {
-        using L = BackwardSmem<D>;
-        if (cudaFuncSetAttribute(backward_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kDynamicBytes) !=
-            cudaSuccess)
-            return SWAA_ERR_CUDA;
-        backward_kernel<D><<<grid, kBwdThreads, L::kDynamicBytes, st>>>(tq, tk, tv, tdo, p);
-    }
+    using L = BackwardTcSmem<D>;
+    static std::atomic<bool> attr_done[64];
+    if (ensure_dynamic_smem(backward_tc_kernel<D>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
+    backward_tc_kernel<D><<<grid, kBwdTcThreads, L::kDynamicBytes, st>>>(tq, tk, tv, tdo, tacc, p);
     backward_convert_dq_kernel<<<(unsigned)((n_acc / 4 + 255) / 256 + 1), 256, 0, st>>>(
         p.dq_accum, static_cast<__nv_bfloat16*>(dq), n_acc);
     int launches = 3;
@@ -783,7 +773,7 @@ extern "C" int swaa_prefill_backward(const void* q, const void* k, const void* v
     p.scale = scale > 0.f ? scale : 1.0f / sqrtf((float)D);
     // Key tiles that hold sink keys meet every later query tile: with long sequences their query range is cut
     // into chunks handled by separate blocks, which add dk, dv into the fp32 accumulators.
-    const int key_tile = D == 128 ? kBwdTcKeys : kBwdTile;  // the two kernels' key tiles; both step over 64 query rows
+    const int key_tile = kBwdTcKeys;  // steps go over 64 query rows
     const int ntiles = (max_seqlen + key_tile - 1) / key_tile;
     p.chunks = ((max_seqlen + 63) / 64 + kBwdChunkTiles - 1) / kBwdChunkTiles;
     p.sink_tiles = 0;
