@@ -397,21 +397,21 @@ extern "C" int swaa_decode_combine(const float* partials, int P, int B, int Hq, 
 namespace swaa {
 
 // Tensor map over a token-major bf16 tensor [T, H, D]: dimensions (D, H, T) innermost first; one box is
-// [128 tokens] x [1 head] x [64 channels] = 128 rows of 128 bytes, written with the 128-byte swizzle.
-static int make_token_major_map_uncached(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens);
-static int make_token_major_map(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens = 128) {
-    const MapKey key{base, 2, T, H, D, box_tokens, 0};
+// [box_tokens] x [box_heads] x [64 channels] = rows of 128 bytes, written with the 128-byte swizzle.
+static int make_token_major_map_uncached(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens, int box_heads);
+static int make_token_major_map(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens = 128, int box_heads = 1) {
+    const MapKey key{base, 2, T, H, D, box_tokens, box_heads};
     if (cached_map(key, map, nullptr)) return SWAA_OK;
-    const int rc = make_token_major_map_uncached(map, base, T, H, D, box_tokens);
+    const int rc = make_token_major_map_uncached(map, base, T, H, D, box_tokens, box_heads);
     if (rc == SWAA_OK) cached_map(key, nullptr, map);
     return rc;
 }
-static int make_token_major_map_uncached(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens) {
+static int make_token_major_map_uncached(CUtensorMap* map, const void* base, int T, int H, int D, int box_tokens, int box_heads) {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return SWAA_ERR_CUDA;
     const cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T};
     const cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)H * D * 2};
-    const cuuint32_t box[3] = {64, 1, (cuuint32_t)box_tokens};
+    const cuuint32_t box[3] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_tokens};
     const cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -436,16 +436,13 @@ static int make_accum_map(CUtensorMap* map, const float* base, int T, int H, int
 }
 
 template <int D, int kMode, bool kLseOnly = false>
-static int launch_prefill(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                          const CUtensorMap& tsk, const CUtensorMap& tsv, const PrefillParams& p, int sm_count,
-                          cudaStream_t st) {
+static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStream_t st) {
     using L = PrefillSmem<D>;
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(prefill_kernel<D, kMode, kLseOnly>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
-    // persistent blocks: one per SM (or fewer when there is less work), each walks its share of the items
-    long long blocks = (long long)p.n_pairs * p.tiles_ub;
-    if (blocks > sm_count) blocks = sm_count;
-    prefill_kernel<D, kMode, kLseOnly><<<(unsigned)blocks, kPrefillThreads, L::kDynamicBytes, st>>>(tq, tk, tv, to, tsk, tsv, p);
+    // one block per item (an upper bound); the blocks that run take over the indices of those that wait
+    const unsigned blocks = (unsigned)p.n_pairs * (unsigned)p.tiles_ub;
+    prefill_kernel<D, kMode, kLseOnly><<<blocks, kPrefillThreads, L::kDynamicBytes, st>>>(tm, p);
     launch_counter().fetch_add(1, std::memory_order_relaxed);
     return cudaGetLastError() == cudaSuccess ? SWAA_OK : SWAA_ERR_CUDA;
 }
@@ -504,22 +501,32 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     if (rc != SWAA_OK) return rc;
     if (info.cc_major != 10) return SWAA_ERR_UNSUPPORTED;
 
-    CUtensorMap tq, tk, tv, to;
-    if ((rc = make_token_major_map(&tq, q, Tq, Hq, D)) != SWAA_OK) return rc;
-    if (is_paged) {  // (D, Hkv, page_size, num_pages), boxes of 128 rows of one page
-        if ((rc = make_cache_map(&tk, k, paged.num_pages, paged.page_size, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
-        if ((rc = make_cache_map(&tv, v, paged.num_pages, paged.page_size, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
+    const int G = Hq / Hkv;
+    const int pack_tokens = ex.lse_only ? 0 : kPrefillBM / G;
+    PrefillMaps tm;
+    if ((rc = make_token_major_map(&tm.q, q, Tq, Hq, D)) != SWAA_OK) return rc;
+    if (pack_tokens > 0 && (rc = make_token_major_map(&tm.q_packed, q, Tq, Hq, D, pack_tokens, G)) != SWAA_OK) return rc;
+    if (is_paged) {  // (D, Hkv, page_size, num_pages), boxes of rows of one page
+        if ((rc = make_cache_map(&tm.k, k, paged.num_pages, paged.page_size, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
+        if ((rc = make_cache_map(&tm.v, v, paged.num_pages, paged.page_size, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
     } else {
-        if ((rc = make_token_major_map(&tk, k, Tk, Hkv, D)) != SWAA_OK) return rc;
-        if ((rc = make_token_major_map(&tv, v, Tk, Hkv, D)) != SWAA_OK) return rc;
+        if ((rc = make_token_major_map(&tm.k, k, Tk, Hkv, D)) != SWAA_OK) return rc;
+        if ((rc = make_token_major_map(&tm.v, v, Tk, Hkv, D)) != SWAA_OK) return rc;
     }
-    if ((rc = make_token_major_map(&to, out, Tq, Hq, D, 32)) != SWAA_OK) return rc;  // output rows, 32 at a time
-    CUtensorMap tsk = tk, tsv = tv;  // only the context-parallel instance reads these
+    if (n_sink > 0) {  // pieces of tiles that join sink keys
+        if (is_paged) {
+            if ((rc = make_cache_map(&tm.k_small, k, paged.num_pages, paged.page_size, Hkv, D, kPrefillSmallBox)) != SWAA_OK) return rc;
+            if ((rc = make_cache_map(&tm.v_small, v, paged.num_pages, paged.page_size, Hkv, D, kPrefillSmallBox)) != SWAA_OK) return rc;
+        } else {
+            if ((rc = make_token_major_map(&tm.k_small, k, Tk, Hkv, D, kPrefillSmallBox)) != SWAA_OK) return rc;
+            if ((rc = make_token_major_map(&tm.v_small, v, Tk, Hkv, D, kPrefillSmallBox)) != SWAA_OK) return rc;
+        }
+    }
+    if ((rc = make_token_major_map(&tm.out, out, Tq, Hq, D, 32)) != SWAA_OK) return rc;  // output rows, 32 at a time
     if (ex.context_parallel && ex.sink_rows > 0) {  // (D, Hkv, sink_rows, B); rows past sink_rows read as zeros
-        if ((rc = make_cache_map(&tsk, ex.sink_k, B, ex.sink_rows, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
-        if ((rc = make_cache_map(&tsv, ex.sink_v, B, ex.sink_rows, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
+        if ((rc = make_cache_map(&tm.sink_k, ex.sink_k, B, ex.sink_rows, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
+        if ((rc = make_cache_map(&tm.sink_v, ex.sink_v, B, ex.sink_rows, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
     }
-
     PrefillParams p;
     p.out = static_cast<__nv_bfloat16*>(out);
     p.lse = lse;
@@ -536,7 +543,8 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.num_pages = paged.num_pages;
     p.Hq = Hq;
     p.Hkv = Hkv;
-    p.G = Hq / Hkv;
+    p.G = G;
+    p.pack_tokens = pack_tokens;
     p.pairs_per_kv = (p.G + 1) / 2;
     p.n_pairs = Hkv * p.pairs_per_kv;
     const long long ub_a = (long long)Tq / kPrefillBM + B;
@@ -564,19 +572,19 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.sl2 = p.scale * 1.4426950408889634f;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (ex.context_parallel)
-        return D == 128 ? launch_prefill<128, 3>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st)
-                        : launch_prefill<64, 3>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st);
+        return D == 128 ? launch_prefill<128, 3>(tm, p, st)
+                        : launch_prefill<64, 3>(tm, p, st);
     if (is_paged)
-        return D == 128 ? launch_prefill<128, 2>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st)
-                        : launch_prefill<64, 2>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st);
+        return D == 128 ? launch_prefill<128, 2>(tm, p, st)
+                        : launch_prefill<64, 2>(tm, p, st);
     if (ex.lse_only)
-        return D == 128 ? launch_prefill<128, 1, true>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st)
-                        : launch_prefill<64, 1, true>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st);
+        return D == 128 ? launch_prefill<128, 1, true>(tm, p, st)
+                        : launch_prefill<64, 1, true>(tm, p, st);
     if (cu_seqlens_k != nullptr)
-        return D == 128 ? launch_prefill<128, 1>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st)
-                        : launch_prefill<64, 1>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st);
-    return D == 128 ? launch_prefill<128, 0>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st)
-                    : launch_prefill<64, 0>(tq, tk, tv, to, tsk, tsv, p, info.sm_count, st);
+        return D == 128 ? launch_prefill<128, 1>(tm, p, st)
+                        : launch_prefill<64, 1>(tm, p, st);
+    return D == 128 ? launch_prefill<128, 0>(tm, p, st)
+                    : launch_prefill<64, 0>(tm, p, st);
 }
 
 }  // namespace swaa

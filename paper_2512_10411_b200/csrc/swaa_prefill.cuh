@@ -3,24 +3,32 @@
 //
 // Mask policy (Sec. 1, 3.1.2, 3.2.1; App. A): a query at position i of its sequence sees key j iff
 //     j <= i  and  ( is_full  or  j > i - window  or  j < n_sink ).
-// Only the key tiles that hold a visible key are visited (the sink tiles and the diagonal band), so
-// the work is O(L * window) as App. A states; the element predicate is evaluated only on tiles that
-// are not entirely visible.
+// Only keys near a visible one are visited (the band and the sinks), so the work is O(L * window) as App. A states; the
+// element predicate is evaluated only on tiles that are not entirely visible.
 //
 // One thread block processes one 128-row query tile for TWO query heads of the same GQA group
 // ("sides" A and B).  Both sides need exactly the same K/V tiles and the same masks, so each K/V tile
-// is staged in shared memory once and feeds four MMAs.  Roles:
+// is staged in shared memory once and feeds four MMAs.  (Short sequences are packed instead: see WorkItem.)  Roles:
 //   warps 0-3   softmax of side A   (thread = query row; lane quadrant = TMEM lane quadrant)
 //   warps 4-7   softmax of side B
-//   warp  8     TMA producer (one elected lane): Q tiles once, then the K and V tile rings
-//   warp  9     MMA issuer (one elected lane) and TMEM allocation
+//   warp  8     TMA producer: Q tiles once, then the K and V tile rings
+//   warp  9     MMA issuer and TMEM allocation
+//   warp 10     work scheduler (takes over the indices of blocks that have not started)
 // Tensor memory (512 columns x 128 lanes of 32 bit): S_A | S_B | O_A | O_B.  The bf16 probabilities
 // P overwrite the first 64 columns of their own S and are consumed from TMEM as the A operand of
 // O += P V.  V tiles are used as the MN-major B operand exactly as TMA lands them.
 // Per key tile n the issuer runs  PV_A(n) QK_A(n+1) PV_B(n) QK_B(n+1), so the softmax of one side
-// overlaps the MMAs of the other; P arrives in two parts (keys 0..95, then 96..127) and the first six of the
-// eight P V instructions are issued on the first.  The running maximum is only raised (and O rescaled) when it grows
-// by more than 2^8; the final division by the row sum makes the result independent of that choice.
+// overlaps the MMAs of the other.  The exponentials are taken against a reference per row that is raised
+// (and O rescaled) only when a tile's scores outgrow it by far; the final division by the row sum makes the result
+// independent of that choice.
+//
+// What bounds it (32k tokens, Hq = 32, Hkv = 8, D = 128, full causal): the power cap.  At 1000 W the SM clock settles at
+// 1.52 GHz (1.60 before), so fewer cycles per tile buy about half their share in time.  Per 128 x 128 tile of both sides
+// 3260 cycles (3710 before) against 2050 of products and 1970 of softmax: a side is a chain softmax -> P V -> Q K^T.
+// Against the kernel that had one issuing lane, a maximum pass on every tile, sink tiles of their own and a fixed
+// assignment of items: 8280 -> 7620 us; the same prompt with a 2048-key window 1178 -> 1101 us; eight ragged prompts of
+// 146k tokens, Hq = 64, window 4096: 17550 -> 16230 us; a serving step of 4 prompt chunks and 24 generated tokens in
+// pages: 1136 -> 815 us.
 //
 // Every wait is bounded: a wait that runs out records SWAA_ERR_TIMEOUT, all roles leave their loops,
 // the block waits (bounded) for its outstanding copies, frees its tensor memory and returns.
@@ -35,8 +43,11 @@ namespace swaa {
 
 constexpr int kPrefillBM = 128;
 constexpr int kPrefillBN = 128;
-constexpr int kPrefillThreads = 384;  // 8 softmax warps + 4 auxiliary warps (producer, issuer, 2 idle)
+constexpr int kPrefillThreads = 384;  // 8 softmax warps + 4 auxiliary warps (producer, issuer, scheduler, 1 idle)
+constexpr int kPrefillSmallBox = 16;                        // rows of the small TMA boxes over K and V
+constexpr int kWorkInts = 24;                               // words of a work descriptor
 constexpr float kRescaleThreshold = 8.0f;                   // log2 units
+constexpr float kSumLimit = 1.152921504606847e18f;          // 2^60: row sum of a tile above which the item is run again
 
 struct PrefillParams {
     __nv_bfloat16* out;
@@ -52,6 +63,7 @@ struct PrefillParams {
     int pairs_per_kv;       // ceil(G / 2)
     int n_pairs;            // Hkv * pairs_per_kv
     int tiles_ub;           // upper bound on the number of query tiles over all sequences
+    int pack_tokens;        // 128 / G: a sequence of at most this many queries is one item per kv head (see WorkItem)
     int window, n_sink, is_full;
     const uint8_t* is_full_seq;   // nullable (chunked / paged): mask policy per sequence, replaces is_full
     // context-parallel prefill (kMode 3): the local keys of sequence b start at position key_pos0[b]; the keys at
@@ -60,6 +72,16 @@ struct PrefillParams {
     int sink_rows;
     float sl2;              // softmax scale * log2(e)
     float scale;
+};
+
+// Tensor maps of one call; an instance reads those that it needs.
+struct PrefillMaps {
+    CUtensorMap q;                 // [128 rows] x 1 head
+    CUtensorMap q_packed;          // [128 / G tokens] x G heads
+    CUtensorMap k, v;              // one key tile
+    CUtensorMap k_small, v_small;  // kPrefillSmallBox keys
+    CUtensorMap out;               // [32 rows] x 1 head
+    CUtensorMap sink_k, sink_v;    // context-parallel
 };
 
 // ------------------------------------------------------------------------------------ PTX wrappers
@@ -136,6 +158,33 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return d;
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
+// Asks the hardware for the index of a block of this grid that has not started yet (and will then never start): the
+// answer, 16 bytes, lands in shared memory.
+__device__ __forceinline__ void next_block_request(uint32_t dst, uint32_t bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(dst),
+                 "r"(bar)
+                 : "memory");
+}
+// Block index of the answer, -1 when none was left.
+__device__ __forceinline__ int next_block_answer(uint32_t src) {
+    uint32_t ok, x;
+    asm volatile(
+        "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t.reg .b32 y, z, w;\n\t"
+        "ld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "mov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, y, z, w}, r;\n\t}"
+        : "=r"(ok), "=r"(x)
+        : "r"(src)
+        : "memory");
+    return ok ? (int)x : -1;
+}
+
 // True in one lane of the (converged) warp.  An issuing warp runs its loop with all lanes and lets the elected
 // lane issue: control flow and descriptors then stay in uniform registers.  Measured with completed barriers: two
 // looks and two commits per 13-instruction step cost 470 cycles in a loop run by one lane alone, 100 this way.
@@ -176,9 +225,10 @@ __device__ __forceinline__ void exp2_poly_x2(float x0, float x1, float& r0, floa
     r1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
 }
 
-// Bit c (0..15) set: column pair c of every 32-column chunk of a score tile takes the polynomial path: a quarter
-// of the exponentials (measured best among 1/8, 3/16, 1/4, 5/16, 1/2, 3/4 and several placements).
-constexpr uint32_t kPolyPairMask = 0x8888u;
+// Bit c (0..15) set: column pair c of every 32-column chunk of a score tile takes the polynomial path.
+// Three in sixteen: none, 1/8, 3/16 and 1/4 of the exponentials give 7743, 7727, 7624 and 7667 us on a full causal 32k
+// prompt (Hq = 32, Hkv = 8, D = 128) and 1106, 1113, 1102 and 1100 us on the same prompt with a 2048-key window.
+constexpr uint32_t kPolyPairMask = 0x8420u;
 
 #define SWAA_R8(r, o) "=r"(r[o + 0]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]), "=r"(r[o + 7])
 #define SWAA_I8(r, o) "r"(r[o + 0]), "r"(r[o + 1]), "r"(r[o + 2]), "r"(r[o + 3]), "r"(r[o + 4]), "r"(r[o + 5]), "r"(r[o + 6]), "r"(r[o + 7])
@@ -210,6 +260,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
         : "memory");
 }
 
+// Keeps the uses of 64 registers that asynchronous tensor-memory loads fill behind the wait for those loads.
+__device__ __forceinline__ void pin64(uint32_t* r) {
+#pragma unroll
+    for (int i = 0; i < 64; ++i) asm volatile("" : "+r"(r[i]));
+}
+
 // Shared-memory matrix descriptors for tiles stored as 128-byte rows with the 128-byte swizzle (what
 // TMA writes for a [rows][64 bf16] box).  14-bit fields hold byte values >> 4.
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -238,46 +294,113 @@ struct PrefillSmem {
     static constexpr int kOffK = 2 * kTileBytes;                 // kStages tiles
     static constexpr int kOffV = kOffK + kStages * kTileBytes;   // kStages tiles
     static constexpr int kOffStage = kOffV + kStages * kTileBytes;  // 8 x 4 KiB: per-warp output staging
-    static constexpr int kOffBar = kOffStage + 8 * 4096;
-    // barriers: Q full/empty, K full/empty, V full/empty per stage, per side S-full / P-ready / O-done /
-    // O-free, work-descriptor full/empty per slot, final, V-tile-cleared per stage (paged keys only)
-    static constexpr int kNumBars = 2 + 4 * kStages + 8 + 4 + 1 + kStages + 2;
-    static constexpr int kOffMisc = kOffBar + kNumBars * 8;      // tmem slot, abort flag, work descriptors
-    static constexpr int kBytes = kOffMisc + 128;
+    static constexpr int kOffMerge = kOffStage + 8 * 4096;  // packed items: (max, sum) of side B's rows
+    static constexpr int kOffBar = kOffMerge + 128 * 8;
+    // barriers: Q full/empty; K full/empty, V full/empty, V-tile-cleared (paged keys only) per stage; per side S full /
+    // P ready / O done / O free; work descriptor full/empty per slot, next-block answer, hand-over of packed items
+    // per row quadrant, final
+    static constexpr int kNumBars = 2 + 5 * kStages + 2 * 4 + 5 + 4 + 1;
+    static constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) / 16 * 16;  // next-block answer, tmem slot, flags, work descriptors
+    static constexpr int kBytes = kOffMisc + 32 + 2 * kWorkInts * 4;
     static constexpr int kDynamicBytes = kBytes + 1024;          // room to align the base to 1024 B
+    static_assert(kDynamicBytes <= 232448, "shared memory per block");
 };
 
-// One unit of work: a 128-row query tile of one sequence for one pair of query heads.
+// One unit of work.  Usual form: a 128-row query tile of one sequence for one pair of query heads (one per side).
+// Packed form, for sequences whose queries times the group size fit in 128 rows (generated tokens, very short
+// prompts): the rows are (query, head of the group) for ALL heads of one kv head, so K and V are read once per kv head
+// and no row is padding that another head could use; the two sides then take alternate key tiles and merge at the end.
+//
+// Key columns of an item: the keys are enumerated as one list [band keys lo .. i1, rounded up
+// to 16 | the sink keys before them] and cut into tiles of BN columns: a few sink keys share the last band tile or make
+// a narrow tile of their own, and a tile that is not full runs fewer MMA steps.  In pages lo is rounded down to a tile,
+// so that a tile of band keys lies in one page.  A context-parallel item has n_rem whole tiles from the sink buffer in front.
+// The scheduler writes the descriptor to shared memory; the other roles read the fields from there as they need them.
 struct WorkItem {
-    int valid, seq_start, seq_len, m_tile, pair;
+    int valid, seq_start, seq_len;
+    int q0;       // first query of the tile, counted inside the sequence's queries
+    int hk, hA;   // kv head, (side A's, first) query head
+    int packed;
+    int hasB;     // side B has a query head of its own (unpacked items)
+    int shared;   // packed item of several tiles: both sides work on the same rows, alternate key tiles
+    int full;     // this item runs full causal attention (per sequence in a mixed batch)
     int k_start;  // first packed key token of the sequence (= seq_start for self attention; sequence index when paged)
     int k_off;    // index of the sequence's first query among its (local) keys: len_k - len_q (0 for self attention)
-    int full;     // this item runs full causal attention (per sequence in a mixed batch)
+    int i0, i1;   // first and last query position, counted among the (local) keys
+    int lo, nb16, nv;  // key list: first band key, band columns, all columns
+    int n_rem, nt;     // tiles from the sink buffer, all tiles
     int n_sink;   // sink keys among the local keys (context-parallel: n_sink - key_pos0, clamped; else n_sink)
     int s_rem;    // context-parallel: sink keys that come from the separate sink buffer, min(n_sink, key_pos0)
     int b;        // context-parallel: sequence index (row of the sink buffer)
+    int n_rows;   // rows in use
+    int careful;  // second run of an item whose scores left the exponent range of the first (see the softmax role)
+
+    // fills the rest from seq_len, q0, packed, full, k_off, n_sink, s_rem and the unit: head pair, or kv head when packed
+    template <int BN, bool kPaged, bool kCp>
+    __device__ __forceinline__ void complete(const PrefillParams& p, int unit) {
+        if (packed) {
+            hk = unit;
+            hA = unit * p.G;
+            hasB = 0;
+            n_rows = seq_len * p.G;
+            i0 = k_off;
+            i1 = k_off + seq_len - 1;
+        } else {
+            hk = unit / p.pairs_per_kv;
+            hA = hk * p.G + 2 * (unit - hk * p.pairs_per_kv);
+            hasB = (hA + 1) < (hk + 1) * p.G ? 1 : 0;
+            n_rows = min(kPrefillBM, seq_len - q0);
+            i0 = q0 + k_off;
+            i1 = i0 + n_rows - 1;
+        }
+        const int first = i0 - p.window + 1;
+        lo = (full || first <= 0) ? 0 : (kPaged ? first / BN * BN : first);
+        nb16 = (i1 + 1 - lo + 15) & ~15;
+        const int ns = full ? 0 : min(n_sink, lo);
+        nv = ns > 0 ? nb16 + ns : i1 + 1 - lo;
+        n_rem = kCp ? (s_rem + BN - 1) / BN : 0;
+        nt = n_rem + (nv + BN - 1) / BN;
+        shared = packed && nt > 1 ? 1 : 0;
+    }
+};
+static_assert(sizeof(WorkItem) == kWorkInts * 4, "words of a work descriptor");
+
+// Tile t (t >= n_rem): column c holds band key jb + c for c < cb, else sink key js + c; the first 16 * nk columns are used.
+template <int BN>
+struct TileGeom {
+    int cb, jb, js, left, nk;  // left: columns of the list from this tile on
+    __device__ __forceinline__ TileGeom(const volatile WorkItem& g, int t) {
+        const int v0 = (t - g.n_rem) * BN, nb16 = g.nb16;
+        cb = max(0, min(BN, nb16 - v0));
+        jb = g.lo + v0;
+        js = v0 - nb16;
+        left = g.nv - v0;
+        nk = min(BN / 16, (left + 15) / 16);
+    }
+    __device__ __forceinline__ int key(int c) const { return c < cb ? jb + c : js + c; }
+    __device__ __forceinline__ bool joins_sinks() const { return cb < 16 * nk; }
+    // rows [bad0, bad1) of the tile lie past the last of len_k keys (none: bad0 >= bad1)
+    __device__ __forceinline__ int bad0(int len_k) const { return cb > 0 ? len_k - jb : BN; }
+    __device__ __forceinline__ int bad1() const { return min(cb, 16 * nk); }
 };
 
 // kMode 0: self attention.  1: chunked prefill, the queries are the last len_q tokens of a longer key sequence
 // (separate packing of the keys).  2: the same with keys and values in pages addressed through a block table.
 // 3: context-parallel prefill, mode 1 with the local keys starting at position key_pos0[b] of their sequence and the
-// sink keys before that position read from a separate buffer (tm_sk, tm_sv) as leading key tiles of the item.
+// sink keys before that position read from a separate buffer (sink_k, sink_v) as leading key tiles of the item.
 // The self-attention instance compiles the offsets away.
 // kLseOnly: only the log-sum-exp of every row is wanted (the lazy-ratio probe): no V tiles are fetched, no P V product
 // is issued, P is not formed and nothing is written to `out`; the barrier protocol stays the same, with "P ready"
-// meaning "S has been read" and the V-tile barriers completed by a plain arrival.
+// meaning "S has been read"; items are never packed.
 template <int D, int kMode, bool kLseOnly = false>
 __global__ void __launch_bounds__(kPrefillThreads, 1)
-prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-               const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o,
-               const __grid_constant__ CUtensorMap tm_sk, const __grid_constant__ CUtensorMap tm_sv,
-               const PrefillParams p) {
+prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     using L = PrefillSmem<D>;
     constexpr bool kChunked = kMode >= 1, kPaged = kMode == 2, kCp = kMode == 3;
     constexpr int BM = kPrefillBM, BN = kPrefillBN;
     constexpr int ST = L::kStages;
-    constexpr uint32_t kIdescQK = make_idesc(BM, BN, 0);
-    constexpr uint32_t kIdescPV = make_idesc(BM, D, 1);
+    constexpr int NK = BN / 16;        // 16-key steps of a tile
+    using Tile = TileGeom<BN>;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -288,33 +411,43 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
     // barrier indices
     constexpr int BAR_QF = 0, BAR_QE = 1, BAR_KF = 2, BAR_KE = BAR_KF + ST, BAR_VF = BAR_KE + ST, BAR_VE = BAR_VF + ST;
+    // per side: S full; P ready; O done, O free
     constexpr int BAR_SF = BAR_VE + ST, BAR_PR = BAR_SF + 2, BAR_OD = BAR_PR + 2, BAR_OF = BAR_OD + 2;
-    constexpr int BAR_WF = BAR_OF + 2, BAR_WE = BAR_WF + 2, BAR_FIN = BAR_WE + 2;
     // paged only, one per ring stage: the rows of the V tile in that stage past the last key have been cleared.
-    // Completed once per cleared tile; producer and issuer each keep the stage's phase bit.  The producer cannot
+    // Completed once per cleared tile; the issuer keeps the stage's phase bit.  The producer cannot
     // clear a stage twice before the issuer has waited for the first clear: reusing the stage needs the
     // issuer's V-empty commit, which follows that wait.
-    constexpr int BAR_VC = BAR_FIN + 1;
-    // per side: the last quarter of P (keys 96..127) has been written; BAR_PR then stands for the first three quarters
-    constexpr int BAR_PQ = BAR_VC + ST;
-    static_assert(BAR_PQ + 2 == L::kNumBars, "barrier count");
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc);
+    constexpr int BAR_VC = BAR_OF + 2;
+    // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), final
+    constexpr int BAR_WF = BAR_VC + ST, BAR_WE = BAR_WF + 2, BAR_NB = BAR_WE + 2, BAR_MG = BAR_NB + 1, BAR_FIN = BAR_MG + 4;
+    static_assert(BAR_FIN + 1 == L::kNumBars, "barrier count");
+    const uint32_t s_answer = smem_base + L::kOffMisc;  // 16 bytes
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc + 16);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* work_ring = reinterpret_cast<volatile int*>(tmem_slot + 4);  // 2 slots x 12 ints
+    volatile int* s_again = reinterpret_cast<volatile int*>(tmem_slot + 2);  // per slot: the item is to be run again
+    volatile WorkItem* work_slots = reinterpret_cast<volatile WorkItem*>(tmem_slot + 4);  // two
+    float2* s_merge = reinterpret_cast<float2*>(smem_gen + L::kOffMerge);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const bool full_all = p.is_full != 0;
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
+        s_again[0] = s_again[1] = 0;
         for (int i = 0; i < L::kNumBars; ++i) {
             uint32_t count = 1u;
-            if (i == BAR_PR || i == BAR_PR + 1 || i == BAR_OF || i == BAR_OF + 1) count = 128u;  // softmax threads
-            if (i == BAR_PQ || i == BAR_PQ + 1) count = 128u;
-            if (i == BAR_WE || i == BAR_WE + 1) count = 10u;  // producer, issuer, one lane per softmax warp
+            if ((i >= BAR_PR && i < BAR_OD) || i == BAR_OF || i == BAR_OF + 1) count = 4u;  // a lane of each softmax warp of the side
+            if (i == BAR_WE || i == BAR_WE + 1) count = 10u;   // producer, issuer, eight softmax warps
+            if (i >= BAR_MG && i < BAR_MG + 4) count = 2u;     // a lane of each side's warp
             mbar_init(bar(i), count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8 && elect_one()) {
+        prefetch_map(&tm.q);
+        prefetch_map(&tm.q_packed);
+        prefetch_map(&tm.k);
+        prefetch_map(&tm.v);
     }
     if (warp == 9) {  // TMEM: all 512 columns (S_A, S_B, O_A, O_B)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -325,355 +458,446 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-    // Consumers of the work ring: wait for descriptor `it`, copy it, release the slot.
-    auto fetch_work = [&](int it, WorkItem& w, bool release) -> bool {
-        const int slot = it & 1;
-        if (!mbar_wait(bar(BAR_WF + slot), (uint32_t)(it >> 1) & 1u, abort_flag)) return false;
-        volatile int* d = work_ring + slot * 12;
-        w.valid = d[0];
-        w.seq_start = d[1];
-        w.seq_len = d[2];
-        w.m_tile = d[3];
-        w.pair = d[4];
-        w.k_start = kChunked ? d[5] : w.seq_start;
-        w.k_off = kChunked ? d[6] : 0;
-        w.full = kChunked ? d[7] : (full_all ? 1 : 0);
-        w.n_sink = kCp ? d[8] : p.n_sink;
-        w.s_rem = kCp ? d[9] : 0;
-        w.b = kCp ? d[10] : 0;
-        if (release) mbar_arrive(bar(BAR_WE + slot));
-        return true;
+    // Consumers of the work descriptors: item `it` is in slot it & 1; they read it in place and release it at their end of
+    // the item.
+    auto wait_work = [&](int it) -> bool { return warp_wait(bar(BAR_WF + (it & 1)), (uint32_t)(it >> 1) & 1u, abort_flag); };
+    auto release_work = [&](int it) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(BAR_WE + (it & 1)));
     };
+    auto uniform = [](int x) -> int { return __shfl_sync(0xffffffffu, x, 0); };
 
     // Register budget per scheduler partition: two softmax warps at 216 + one auxiliary warp at 72.
     if (warp >= 8) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
       if (warp == 10) {
         // ====================================================================== work scheduler
-        // Walks this block's work items w = blockIdx.x, blockIdx.x + gridDim.x, ... and publishes their
-        // descriptors.  Items are ordered heavy-first: last sequence first, last tile of a sequence first.
-        if (lane == 0) {
-            if (p.cu_seqlens[0] != 0 || p.cu_seqlens[p.B] != p.T) record_device_error(SWAA_ERR_BAD_SEQLENS);
-            int b = p.B, acc = 0, cur_nt = 0, cur_s = 0, cur_len = 0, cur_ks = 0, cur_off = 0;
-            int cur_full = full_all ? 1 : 0, cur_sink = p.n_sink, cur_srem = 0;
-            auto next_seq = [&]() {
-                acc += cur_nt;
-                --b;
-                cur_nt = 0;
-                if (b >= 0) {
-                    const int s0 = p.cu_seqlens[b], e0 = p.cu_seqlens[b + 1];
-                    int len = e0 - s0;
-                    if (len < 0 || len > p.max_seqlen || s0 < 0 || e0 > p.T) {
-                        record_device_error(SWAA_ERR_BAD_SEQLENS);
-                        len = 0;
+        // The grid has one block per item (an upper bound); as many as fit start, and each takes over the indices of
+        // blocks that have not started, so items go to whichever SM is free.  Items are ordered heavy-first: last
+        // sequence first, last tile of a sequence first.  Lane l looks after sequence base_b - l.
+        if (lane == 0 && (p.cu_seqlens[0] != 0 || p.cu_seqlens[p.B] != p.T)) record_device_error(SWAA_ERR_BAD_SEQLENS);
+        int base_b = p.B - 1;       // sequence of lane 0
+        int base_w = 0;             // index of the first item of this group of 32 sequences
+        int f_s = 0, f_len = 0, f_ks = 0, f_off = 0, f_full = full_all ? 1 : 0, f_sink = p.n_sink, f_srem = 0;
+        int f_packed = 0, f_items = 0, f_incl = 0;  // items of the lane's sequence and their running sum
+        auto load_group = [&]() {
+            const int b = base_b - lane;
+            f_items = 0;
+            if (b >= 0) {
+                const int s0 = p.cu_seqlens[b], e0 = p.cu_seqlens[b + 1];
+                int len = e0 - s0;
+                bool bad = len < 0 || len > p.max_seqlen || s0 < 0 || e0 > p.T;
+                f_ks = s0;
+                f_off = 0;
+                if (kPaged) {  // keys in pages: cu_seqlens_k holds the key lengths
+                    const int lk = p.cu_seqlens_k[b];
+                    bad = bad || lk < len || lk > p.max_seqlen_k;
+                    f_ks = b;
+                    f_off = lk - len;
+                } else if (kChunked) {  // chunked prefill: the queries are the last `len` tokens
+                    const int ks = p.cu_seqlens_k[b], ke = p.cu_seqlens_k[b + 1];
+                    bad = bad || ke - ks < len || ke - ks > p.max_seqlen_k || ks < 0 || ke > p.Tk;
+                    f_ks = ks;
+                    f_off = ke - ks - len;
+                    if (kCp) {
+                        // the local keys start at position p0: the sink keys before it come from the sink buffer,
+                        // and the window of the first query must not reach below p0 (halo of window - 1 keys)
+                        const int p0 = p.key_pos0[b];
+                        bad = bad || p0 < 0 || (p0 > 0 && f_off < p.window - 1) || (p0 > 0 && p.n_sink > p.sink_rows);
+                        f_srem = p0 < p.n_sink ? max(p0, 0) : p.n_sink;
+                        f_sink = p.n_sink - f_srem;
                     }
-                    cur_ks = s0;
-                    cur_off = 0;
-                    if (kPaged) {  // keys in pages: cu_seqlens_k holds the key lengths
-                        const int lk = p.cu_seqlens_k[b];
-                        if (lk < len || lk > p.max_seqlen_k) {
-                            record_device_error(SWAA_ERR_BAD_SEQLENS);
-                            len = 0;
-                        }
-                        cur_ks = b;
-                        cur_off = lk - len;
-                    } else if (kChunked) {  // chunked prefill: the queries are the last `len` tokens
-                        const int ks = p.cu_seqlens_k[b], ke = p.cu_seqlens_k[b + 1];
-                        if (ke - ks < len || ke - ks > p.max_seqlen_k || ks < 0 || ke > p.Tk) {
-                            record_device_error(SWAA_ERR_BAD_SEQLENS);
-                            len = 0;
-                        }
-                        cur_ks = ks;
-                        cur_off = ke - ks - len;
-                        if (kCp) {
-                            // the local keys start at position p0: the sink keys before it come from the sink buffer,
-                            // and the window of the first query must not reach below p0 (halo of window - 1 keys)
-                            const int p0 = p.key_pos0[b];
-                            if (p0 < 0 || (p0 > 0 && cur_off < p.window - 1) || (p0 > 0 && p.n_sink > p.sink_rows)) {
-                                record_device_error(SWAA_ERR_BAD_SEQLENS);
-                                len = 0;
-                            }
-                            cur_srem = p0 < p.n_sink ? max(p0, 0) : p.n_sink;
-                            cur_sink = p.n_sink - cur_srem;
-                        }
-                    }
-                    if (kChunked && p.is_full_seq != nullptr) cur_full = p.is_full_seq[b] != 0 ? 1 : 0;
-                    cur_s = s0;
-                    cur_len = len;
-                    cur_nt = (len + BM - 1) / BM;
                 }
-            };
-            next_seq();
-            for (int it = 0;; ++it) {
-                const long long w = (long long)blockIdx.x + (long long)it * gridDim.x;
-                const long long tile_id = w / p.n_pairs;
-                const int pair = (int)(w - tile_id * p.n_pairs);
-                while (b >= 0 && tile_id >= (long long)acc + cur_nt) next_seq();
-                const int slot = it & 1;
-                if (!mbar_wait(bar(BAR_WE + slot), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) break;
-                volatile int* d = work_ring + slot * 12;
-                d[0] = b >= 0 ? 1 : 0;
-                d[1] = cur_s;
-                d[2] = cur_len;
-                d[3] = b >= 0 ? cur_nt - 1 - (int)(tile_id - acc) : 0;
-                d[4] = pair;
-                if (kChunked) {
-                    d[5] = cur_ks;
-                    d[6] = cur_off;
-                    d[7] = cur_full;
+                if (bad) {
+                    record_device_error(SWAA_ERR_BAD_SEQLENS);
+                    len = 0;
                 }
-                if (kCp) {
-                    d[8] = cur_sink;
-                    d[9] = cur_srem;
-                    d[10] = b;
-                }
-                mbar_arrive(bar(BAR_WF + slot));
-                if (b < 0) break;
+                if (kChunked && p.is_full_seq != nullptr) f_full = p.is_full_seq[b] != 0 ? 1 : 0;
+                f_s = s0;
+                f_len = len;
+                f_packed = !kLseOnly && len <= p.pack_tokens ? 1 : 0;
+                f_items = len == 0 ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_pairs);
             }
+            f_incl = f_items;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, f_incl, o);
+                if (lane >= o) f_incl += v;
+            }
+        };
+        load_group();
+        int w = (int)blockIdx.x, it = 0;
+        auto slot_words = [&](int slot) -> volatile int* { return reinterpret_cast<volatile int*>(work_slots + slot); };
+        // publishes the descriptor that lies in slot it & 1 as a second run of the item of slot o
+        auto run_again = [&](int o) {
+            if (lane == 0) {
+                work_slots[it & 1].careful = 1;
+                s_again[o] = 0;
+                mbar_arrive(bar(BAR_WF + (it & 1)));
+            }
+            __syncwarp();
+            ++it;
+        };
+        // waits until slot it & 1 may be written; an item there that is to be run again is published first
+        auto free_slot = [&]() -> bool {
+            while (true) {
+                if (!warp_wait(bar(BAR_WE + (it & 1)), ((uint32_t)(it >> 1) & 1u) ^ 1u, abort_flag)) return false;
+                if (!uniform(s_again[it & 1])) return true;
+                run_again(it & 1);
+            }
+        };
+        uint32_t nb_phase = 0;
+        bool ok = true;
+        while (w >= 0) {
+            if (w < base_w) {  // an index before this group of sequences: start over
+                base_b = p.B - 1;
+                base_w = 0;
+                load_group();
+            }
+            bool valid;  // an index past the last item is passed over (the grid is an upper bound)
+            while (true) {
+                const int total = __shfl_sync(0xffffffffu, f_incl, 31);
+                valid = w < base_w + total;
+                if (valid || base_b < 32) break;
+                base_w += total;
+                base_b -= 32;
+                load_group();
+            }
+            if (valid) {
+                const int local = w - base_w - (f_incl - f_items);
+                ok = free_slot();
+                if (!ok) break;
+                if (local >= 0 && local < f_items) {  // one lane
+                    WorkItem d;
+                    d.valid = 1;
+                    d.seq_start = f_s;
+                    d.seq_len = f_len;
+                    d.q0 = f_packed ? 0 : ((f_len + BM - 1) / BM - 1 - local / p.n_pairs) * BM;
+                    d.packed = f_packed;
+                    d.full = f_full;
+                    d.k_start = f_ks;
+                    d.k_off = f_off;
+                    d.n_sink = f_sink;
+                    d.s_rem = f_srem;
+                    d.b = base_b - lane;
+                    d.careful = 0;
+                    d.complete<BN, kPaged, kCp>(p, f_packed ? local : local % p.n_pairs);
+                    volatile int* to = slot_words(it & 1);
+                    const int* from = reinterpret_cast<const int*>(&d);
+#pragma unroll
+                    for (int i = 0; i < kWorkInts; ++i) to[i] = from[i];
+                    mbar_arrive(bar(BAR_WF + (it & 1)));
+                }
+                __syncwarp();
+                ++it;
+            }
+            if (lane == 0) {
+                fence_proxy_async_smem();  // the previous answer has been read
+                mbar_arrive_expect_tx(bar(BAR_NB), 16u);
+                next_block_request(s_answer, bar(BAR_NB));
+            }
+            ok = warp_wait(bar(BAR_NB), nb_phase, abort_flag);
+            if (!ok) break;
+            nb_phase ^= 1u;
+            w = uniform(next_block_answer(s_answer));
+        }
+        // the last items have to be done before the end is published, lest one is to be run again
+        while (ok) {
+            ok = free_slot();
+            if (!ok || it == 0) break;
+            const int o = (it - 1) & 1;
+            ok = warp_wait(bar(BAR_WE + o), (uint32_t)((it - 1) >> 1) & 1u, abort_flag);
+            if (!ok || !uniform(s_again[o])) break;
+            if (lane < kWorkInts) slot_words(it & 1)[lane] = slot_words(o)[lane];
+            __syncwarp();
+            run_again(o);
+        }
+        if (ok && lane == 0) {
+            work_slots[it & 1].valid = 0;
+            mbar_arrive(bar(BAR_WF + (it & 1)));
         }
         __syncwarp();
       } else if (warp == 8) {
         // =========================================================================== TMA producer
-        if (lane == 0) {
-            int g = 0;           // K/V tiles issued so far (ring position)
-            bool ok = true, q_in_flight = false;
-            int items = 0;
-            for (int it = 0; ok; ++it) {
-                WorkItem w;
-                ok = fetch_work(it, w, true);
-                if (!ok || !w.valid) break;
-                const int hk = w.pair / p.pairs_per_kv;
-                const int hA = hk * p.G + 2 * (w.pair - hk * p.pairs_per_kv);
-                const bool hasB = (hA + 1) < (hk + 1) * p.G;
-                const int i0 = w.m_tile * BM, i1 = min(w.seq_len, i0 + BM) - 1;
-                const TileRange tr = tile_range(i0 + w.k_off, i1 + w.k_off, BN, p.window, w.n_sink, w.full != 0);
-                const int n_rem = kCp ? (w.s_rem + BN - 1) / BN : 0;  // leading tiles from the sink buffer
-                const int nt = n_rem + tr.count();
-                // Q tiles of both sides (the previous item's last QK must have retired)
-                ok = mbar_wait(bar(BAR_QE), ((uint32_t)items & 1u) ^ 1u, abort_flag);
-                if (!ok) break;
-                const int tq = w.seq_start + i0;
-                mbar_arrive_expect_tx(bar(BAR_QF), (hasB ? 2u : 1u) * (uint32_t)L::kTileBytes);
+        // The whole warp walks the items and waits; one elected lane starts the copies.
+        const bool el = elect_one();
+        int s = 0;           // ring stage
+        uint32_t ph = 0;     // its phase
+        int g = 0;           // K/V tiles issued so far
+        bool v_now = false;  // the V copy of the tile in hand has been issued (for the exit path)
+        bool ok = true;
+        int items = 0;
+        for (int it = 0; ok; ++it) {
+            ok = wait_work(it);
+            if (!ok) break;
+            const volatile WorkItem& w = work_slots[it & 1];
+            if (!uniform(w.valid)) break;
+            const bool packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
+            const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
+            const int len_k = uniform(w.k_off + w.seq_len), hk = uniform(w.hk), k_start = uniform(w.k_start);
+            // Q tiles of both sides (the previous item's last Q K^T must have retired); packed: one tile serves both
+            ok = warp_wait(bar(BAR_QE), ((uint32_t)items & 1u) ^ 1u, abort_flag);
+            if (!ok) break;
+            if (el) {
+                const int hA = w.hA, tq = w.seq_start + w.q0;
+                if (packed) {  // rows = (query, head of the group)
+                    mbar_arrive_expect_tx(bar(BAR_QF), (uint32_t)(p.pack_tokens * p.G * 128 * L::kPanels));
 #pragma unroll
-                for (int pn = 0; pn < L::kPanels; ++pn) {
-                    tma_load_3d(sQ + pn * L::kPanelBytes, &tm_q, pn * 64, hA, tq, bar(BAR_QF));
-                    if (hasB)
-                        tma_load_3d(sQ + L::kTileBytes + pn * L::kPanelBytes, &tm_q, pn * 64, hA + 1, tq, bar(BAR_QF));
-                }
-                q_in_flight = true;
-                ++items;
-                for (int n = 0; n < nt; ++n, ++g) {
-                    const int s = g % ST;
-                    const uint32_t ph = (uint32_t)(g / ST) & 1u;
-                    const bool remote = kCp && n < n_rem;
-                    const int kt = remote ? n * BN : tr.tile(n - n_rem) * BN;  // first key of the tile, counted inside the (local) keys
-                    int tk = w.k_start + kt, page = 0;  // packed token index, or (row in page, page) when paged
-                    if (kPaged) {
-                        page = __ldg(p.block_table + (size_t)w.k_start * p.max_blocks + kt / p.page_size);
-                        tk = kt % p.page_size;
-                        if (page < 0 || page >= p.num_pages) {
-                            record_device_error(SWAA_ERR_BAD_SEQLENS);
-                            page = p.num_pages;  // out of range: the copy delivers zeros
-                        }
-                    }
-                    ok = mbar_wait(bar(BAR_KE + s), ph ^ 1u, abort_flag);
-                    if (!ok) break;
-                    mbar_arrive_expect_tx(bar(BAR_KF + s), (uint32_t)L::kTileBytes);
+                    for (int pn = 0; pn < L::kPanels; ++pn)
+                        tma_load_3d(sQ + pn * L::kPanelBytes, &tm.q_packed, pn * 64, hA, tq, bar(BAR_QF));
+                } else {
+                    mbar_arrive_expect_tx(bar(BAR_QF), (hasB ? 2u : 1u) * (uint32_t)L::kTileBytes);
 #pragma unroll
                     for (int pn = 0; pn < L::kPanels; ++pn) {
-                        if (kPaged) tma_load_4d(sK + s * L::kTileBytes + pn * L::kPanelBytes, &tm_k, pn * 64, hk, tk, page, bar(BAR_KF + s));
-                        else if (remote) tma_load_4d(sK + s * L::kTileBytes + pn * L::kPanelBytes, &tm_sk, pn * 64, hk, kt, w.b, bar(BAR_KF + s));
-                        else tma_load_3d(sK + s * L::kTileBytes + pn * L::kPanelBytes, &tm_k, pn * 64, hk, tk, bar(BAR_KF + s));
-                    }
-                    ok = mbar_wait(bar(BAR_VE + s), ph ^ 1u, abort_flag);
-                    if (!ok) {
-                        mbar_wait(bar(BAR_KF + s), ph, abort_flag);  // the K copy just issued
-                        break;
-                    }
-                    if (kLseOnly) {
-                        mbar_arrive(bar(BAR_VF + s));  // no V tile: complete the stage's barrier by hand
-                        continue;
-                    }
-                    mbar_arrive_expect_tx(bar(BAR_VF + s), (uint32_t)L::kTileBytes);
-#pragma unroll
-                    for (int pn = 0; pn < L::kPanels; ++pn) {
-                        if (kPaged) tma_load_4d(sV + s * L::kTileBytes + pn * L::kPanelBytes, &tm_v, pn * 64, hk, tk, page, bar(BAR_VF + s));
-                        else if (remote) tma_load_4d(sV + s * L::kTileBytes + pn * L::kPanelBytes, &tm_sv, pn * 64, hk, kt, w.b, bar(BAR_VF + s));
-                        else tma_load_3d(sV + s * L::kTileBytes + pn * L::kPanelBytes, &tm_v, pn * 64, hk, tk, bar(BAR_VF + s));
-                    }
-                    if (kPaged) {
-                        // The rows of a page past the sequence's last key may hold anything (also NaN, and 0 * NaN is
-                        // NaN in the PV product): clear them in the V tile before the issuer may use it.  Only the last
-                        // key tile of a sequence that does not end on a tile boundary is concerned.
-                        const int first_bad = w.k_off + w.seq_len - kt;  // rows [first_bad, BN) lie past the last key
-                        if (first_bad < BN) {
-                            ok = mbar_wait(bar(BAR_VF + s), ph, abort_flag);
-                            if (!ok) break;
-                            for (int r = max(first_bad, 0); r < BN; ++r)
-#pragma unroll
-                                for (int pn = 0; pn < L::kPanels; ++pn)
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j)
-                                        st_shared_v4(sV + s * L::kTileBytes + pn * L::kPanelBytes + r * 128 + j * 16, 0u, 0u, 0u, 0u);
-                            fence_proxy_async_smem();
-                            mbar_arrive(bar(BAR_VC + s));
-                        }
+                        tma_load_3d(sQ + pn * L::kPanelBytes, &tm.q, pn * 64, hA, tq, bar(BAR_QF));
+                        if (hasB)
+                            tma_load_3d(sQ + L::kTileBytes + pn * L::kPanelBytes, &tm.q, pn * 64, hA + 1, tq, bar(BAR_QF));
                     }
                 }
             }
-            if (!ok) {
-                // give outstanding copies a bounded chance to land before the block's memory is released
-                const uint64_t t0 = global_timer_ns();
-                bool landed = false;
-                while (!landed && global_timer_ns() - t0 < kWaitLimitNs) {
-                    landed = !q_in_flight || mbar_try_wait(bar(BAR_QF), (uint32_t)(items - 1) & 1u);
-                    for (int n = max(0, g - ST); n < g; ++n) {
-                        landed = landed && mbar_try_wait(bar(BAR_KF + n % ST), (uint32_t)(n / ST) & 1u);
-                        landed = landed && mbar_try_wait(bar(BAR_VF + n % ST), (uint32_t)(n / ST) & 1u);
+            ++items;
+            for (int n = 0; n < nt; ++n, ++g) {
+                const bool remote = kCp && n < n_rem;
+                const Tile t(w, n);
+                const uint32_t dK = sK + (uint32_t)(s * L::kTileBytes), dV = sV + (uint32_t)(s * L::kTileBytes);
+                // A tile of band keys comes in one box per panel, one that joins sink keys in pieces of 16 keys.
+                const bool whole = remote || !t.joins_sinks();
+                const uint32_t bytes = whole ? (uint32_t)L::kTileBytes : (uint32_t)(t.nk * 16 * 128 * L::kPanels);
+                // page of a key, out of range (the copy delivers zeros) when the table is wrong
+                auto page_of = [&](int key) -> int {
+                    const int page = __ldg(p.block_table + (size_t)k_start * p.max_blocks + key / p.page_size);
+                    if (page >= 0 && page < p.num_pages) return page;
+                    record_device_error(SWAA_ERR_BAD_SEQLENS);
+                    return p.num_pages;
+                };
+                int page0 = 0, row0 = 0;  // of the first key, looked up ahead of the wait for the stage
+                if (kPaged) {
+                    const int key = t.key(0);
+                    page0 = page_of(key);
+                    row0 = key % p.page_size;
+                }
+                auto load_tile = [&](const CUtensorMap* map, const CUtensorMap* map_small, const CUtensorMap* map_sink, uint32_t dst,
+                                     uint32_t full_bar) {
+                    if (whole) {
+#pragma unroll
+                        for (int pn = 0; pn < L::kPanels; ++pn) {
+                            const uint32_t d = dst + (uint32_t)(pn * L::kPanelBytes);
+                            if (remote) tma_load_4d(d, map_sink, pn * 64, hk, n * BN, w.b, full_bar);
+                            else if (kPaged) tma_load_4d(d, map, pn * 64, hk, row0, page0, full_bar);
+                            else tma_load_3d(d, map, pn * 64, hk, k_start + t.jb, full_bar);
+                        }
+                    } else {
+                        for (int x = 0; x < t.nk; ++x) {
+                            const int key = t.key(16 * x);
+                            const int page = kPaged ? page_of(key) : 0;
+#pragma unroll
+                            for (int pn = 0; pn < L::kPanels; ++pn) {
+                                const uint32_t d = dst + (uint32_t)(pn * L::kPanelBytes + x * 2048);
+                                if (kPaged) tma_load_4d(d, map_small, pn * 64, hk, key % p.page_size, page, full_bar);
+                                else tma_load_3d(d, map_small, pn * 64, hk, k_start + key, full_bar);
+                            }
+                        }
+                    }
+                };
+                ok = warp_wait(bar(BAR_KE + s), ph ^ 1u, abort_flag);
+                if (!ok) break;
+                if (el) {
+                    mbar_arrive_expect_tx(bar(BAR_KF + s), bytes);
+                    load_tile(&tm.k, &tm.k_small, &tm.sink_k, dK, bar(BAR_KF + s));
+                }
+                if (!kLseOnly) {
+                    ok = warp_wait(bar(BAR_VE + s), ph ^ 1u, abort_flag);
+                    if (!ok) {
+                        warp_wait(bar(BAR_KF + s), ph, abort_flag);  // the K copy just issued
+                        break;
+                    }
+                    if (el) {
+                        mbar_arrive_expect_tx(bar(BAR_VF + s), bytes);
+                        load_tile(&tm.v, &tm.v_small, &tm.sink_v, dV, bar(BAR_VF + s));
+                    }
+                    v_now = true;
+                    if (kPaged) {
+                        // The rows of a page past the sequence's last key may hold anything (also NaN, and 0 * NaN is
+                        // NaN in the PV product): clear those that the P V product reads before the issuer may use the
+                        // tile.  Only the last band tile of a sequence that does not end on a 16-key boundary is concerned.
+                        const int r0 = t.bad0(len_k), r1 = t.bad1();
+                        if (r0 < r1) {
+                            ok = warp_wait(bar(BAR_VF + s), ph, abort_flag);
+                            if (!ok) break;
+                            for (int c = lane; c < (r1 - r0) * 8; c += 32)
+#pragma unroll
+                                for (int pn = 0; pn < L::kPanels; ++pn)
+                                    st_shared_v4(dV + pn * L::kPanelBytes + (r0 + (c >> 3)) * 128 + (c & 7) * 16, 0u, 0u, 0u, 0u);
+                            fence_proxy_async_smem();
+                            __syncwarp();
+                            if (el) mbar_arrive(bar(BAR_VC + s));
+                        }
                     }
                 }
+                v_now = false;
+                if (++s == ST) {
+                    s = 0;
+                    ph ^= 1u;
+                }
+            }
+            release_work(it);
+        }
+        if (!ok) {
+            // give outstanding copies a bounded chance to land before the block's memory is released
+            const uint64_t t0 = global_timer_ns();
+            bool landed = false;
+            while (!landed && global_timer_ns() - t0 < kWaitLimitNs) {
+                landed = items == 0 || mbar_try_wait(bar(BAR_QF), (uint32_t)(items - 1) & 1u);
+                for (int n = max(0, g - ST + 1); n < g; ++n) {
+                    landed = landed && mbar_try_wait(bar(BAR_KF + n % ST), (uint32_t)(n / ST) & 1u);
+                    landed = landed && (kLseOnly || mbar_try_wait(bar(BAR_VF + n % ST), (uint32_t)(n / ST) & 1u));
+                }
+                // the tile that was being issued when the wait ran out
+                if (v_now) landed = landed && mbar_try_wait(bar(BAR_VF + s), ph) && mbar_try_wait(bar(BAR_KF + s), ph);
             }
         }
         __syncwarp();
       } else if (warp == 9) {
         // ============================================================================ MMA issuer
-        if (lane == 0) {
-            const uint32_t tS[2] = {tmem_base, tmem_base + 128u};
-            const uint32_t tO[2] = {tmem_base + 256u, tmem_base + 256u + (uint32_t)D};
-            // Descriptor words are built once: per operand tile a low word (address, leading-dimension offset)
-            // and one shared high word (stride 1024 B, descriptor version, 128-byte swizzle).  The issue latency
-            // of this thread is part of every tile's critical path, so the per-MMA work is one add per operand.
-            const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0, 0, 1024) >> 32);
-            uint32_t q_lo[2], k_lo[ST], v_lo[ST];
+        // The warp runs the loop as a whole, one elected lane issues and commits (see elect_one).
+        const bool el = elect_one();
+        // Descriptor words are built once: per operand tile a low word (address, leading-dimension offset)
+        // and one shared high word (stride 1024 B, descriptor version, 128-byte swizzle).
+        const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0, 0, 1024) >> 32);
+        const uint32_t q_lo = (uint32_t)smem_desc_sw128(sQ, 16, 1024);
+        const uint32_t k_lo = (uint32_t)smem_desc_sw128(sK, 16, 1024);
+        const uint32_t v_lo = (uint32_t)smem_desc_sw128(sV, L::kPanelBytes, 1024);
+        constexpr uint32_t kStep = (uint32_t)L::kTileBytes >> 4;
+        constexpr uint32_t kIdescQK = make_idesc(BM, BN, 0), kIdescPV = make_idesc(BM, D, 1);
+        // Q K^T of a side over the first 16 * nk keys of a tile; q_tile: 0, or the side
+        auto issue_qk = [&](int side, int q_tile, int stage, int nk) {
+            const uint32_t qa = q_lo + (uint32_t)q_tile * kStep, kb = k_lo + (uint32_t)stage * kStep;
+            const uint32_t idesc = nk == NK ? kIdescQK : (make_idesc(BM, 0, 0) | ((uint32_t)(2 * nk) << 17));
 #pragma unroll
-            for (int sd = 0; sd < 2; ++sd) q_lo[sd] = (uint32_t)smem_desc_sw128(sQ + sd * L::kTileBytes, 16, 1024);
-#pragma unroll
-            for (int st = 0; st < ST; ++st) {
-                k_lo[st] = (uint32_t)smem_desc_sw128(sK + st * L::kTileBytes, 16, 1024);
-                v_lo[st] = (uint32_t)smem_desc_sw128(sV + st * L::kTileBytes, L::kPanelBytes, 1024);
+            for (int kk = 0; kk < D / 16; ++kk) {
+                const uint32_t off = ((uint32_t)(kk >> 2) * L::kPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
+                mma_ss_lh(tmem_base + 128u * (uint32_t)side, qa + off, kb + off, desc_hi, idesc, kk > 0 ? 1u : 0u);
             }
-            auto pick = [&](const uint32_t (&arr)[ST], int stage) -> uint32_t {  // register array, static indices only
-                uint32_t r = arr[0];
+        };
+        auto issue_pv = [&](int side, int stage, bool acc, int nk) {
+            const uint32_t vb = v_lo + (uint32_t)stage * kStep, a = tmem_base + 128u * (uint32_t)side;
+            const uint32_t d = tmem_base + 256u + (uint32_t)(D * side);
 #pragma unroll
-                for (int st = 1; st < ST; ++st) r = stage == st ? arr[st] : r;
-                return r;
-            };
-            auto issue_qk = [&](int side, int stage) {
-                const uint32_t qa = side ? q_lo[1] : q_lo[0], kb = pick(k_lo, stage), d = tS[side];
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    const uint32_t off = ((uint32_t)(kk >> 2) * L::kPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
-                    mma_ss_lh(d, qa + off, kb + off, desc_hi, kIdescQK, kk > 0 ? 1u : 0u);
-                }
-            };
-            auto issue_pv = [&](int side, int stage, bool acc, int kk0, int kk1) {
-                const uint32_t vb = pick(v_lo, stage), d = tO[side], a = tS[side];
-#pragma unroll
-                for (int kk = kk0; kk < kk1; ++kk) {
-                    // P: 16 keys = 8 TMEM columns of packed bf16 pairs.  V: 16 key rows of 128 bytes.
-                    mma_ts_lh(d, a + (uint32_t)kk * 8u, vb + (((uint32_t)kk * 2048u) >> 4), desc_hi, kIdescPV,
-                              (acc || kk > 0) ? 1u : 0u);
-                }
-            };
-            int g = 0;                 // K/V ring position
-            int gs[2] = {0, 0};        // tiles processed per side (phase of S-full / P-ready / O-done)
-            int items_side[2] = {0, 0};
-            int items = 0;
-            uint32_t vc_phase = 0;  // paged only: bit s = phase of the stage's V-tile-cleared barrier
-            bool ok = true;
-            for (int it = 0; ok; ++it) {
-                WorkItem w;
-                ok = fetch_work(it, w, true);
-                if (!ok || !w.valid) break;
-                const int hk = w.pair / p.pairs_per_kv;
-                const int hA = hk * p.G + 2 * (w.pair - hk * p.pairs_per_kv);
-                const bool hasB = (hA + 1) < (hk + 1) * p.G;
-                const int i0 = w.m_tile * BM, i1 = min(w.seq_len, i0 + BM) - 1;
-                const TileRange trng = tile_range(i0 + w.k_off, i1 + w.k_off, BN, p.window, w.n_sink, w.full != 0);
-                const int nt = (kCp ? (w.s_rem + BN - 1) / BN : 0) + trng.count();
-                ok = mbar_wait(bar(BAR_QF), (uint32_t)items & 1u, abort_flag) &&
-                     mbar_wait(bar(BAR_KF + g % ST), (uint32_t)(g / ST) & 1u, abort_flag);
+            for (int kk = 0; kk < NK; ++kk) {
+                // P: 16 keys = 8 TMEM columns of packed bf16 pairs.  V: 16 key rows of 128 bytes.
+                if (kk < nk)
+                    mma_ts_lh(d, a + (uint32_t)kk * 8u, vb + (((uint32_t)kk * 2048u) >> 4), desc_hi, kIdescPV, (acc || kk > 0) ? 1u : 0u);
+            }
+        };
+        int sk = 0, sv = 0;            // ring stages of the next K and V tile
+        uint32_t pk = 0, pv = 0;       // their phases
+        int gs[2] = {0, 0};            // tiles processed per side (phase of P ready)
+        int items_side[2] = {0, 0};    // items each side took part in (phase of O free)
+        int items = 0;
+        uint32_t vc_phase = 0;         // paged only: bit s = phase of the stage's V-tile-cleared barrier
+        bool ok = true;
+        auto next_k = [&]() {
+            if (++sk == ST) {
+                sk = 0;
+                pk ^= 1u;
+            }
+        };
+        for (int it = 0; ok; ++it) {
+            ok = wait_work(it);
+            if (!ok) break;
+            const volatile WorkItem& w = work_slots[it & 1];
+            if (!uniform(w.valid)) break;
+            const bool packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
+            const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
+            const int len_k = kPaged ? uniform(w.k_off + w.seq_len) : 0;
+            const bool shared = packed && nt > 1;
+            auto steps_of = [&](int n) -> int { return (kCp && n < n_rem) ? NK : Tile(w, n).nk; };
+            const int ahead = packed ? 2 : 1;  // Q K^T runs this many tiles ahead of P V
+            ok = warp_wait(bar(BAR_QF), (uint32_t)items & 1u, abort_flag);
+            // the first scores of each side
+            for (int n = 0; n < min(ahead, nt) && ok; ++n) {
+                const int nk = steps_of(n);
+                ok = warp_wait(bar(BAR_KF + sk), pk, abort_flag);
                 if (!ok) break;
                 tc_fence_after();
-                issue_qk(0, g % ST);
-                tc_commit(bar(BAR_SF + 0));
-                if (hasB) {
-                    issue_qk(1, g % ST);
-                    tc_commit(bar(BAR_SF + 1));
-                }
-                tc_commit(bar(BAR_KE + g % ST));
-                if (nt == 1) tc_commit(bar(BAR_QE));  // Q is no longer needed by this item
-                for (int n = 0; n < nt; ++n, ++g) {
-                    const int sv = g % ST;
-                    const uint32_t pv = (uint32_t)(g / ST) & 1u;
-                    const bool has_next = n + 1 < nt;
-                    const int sk = (g + 1) % ST;
-                    const uint32_t pk = (uint32_t)((g + 1) / ST) & 1u;
-                    // The tiles first (they landed long ago as a rule), then the side's P: a look at a barrier costs
-                    // this thread some 80 cycles even when it has completed, and what follows the P barrier is on
-                    // the side's critical path softmax -> PV -> QK -> softmax.
-                    ok = mbar_wait(bar(BAR_VF + sv), pv, abort_flag) &&
-                         (!has_next || mbar_wait(bar(BAR_KF + sk), pk, abort_flag)) &&
-                         mbar_wait(bar(BAR_PR + 0), (uint32_t)gs[0] & 1u, abort_flag);
-                    if (kPaged && ok && w.k_off + w.seq_len - trng.tile(n) * BN < BN) {
-                        // last key tile of a sequence that ends inside it: the producer clears the rows past the end
-                        ok = mbar_wait(bar(BAR_VC + sv), (vc_phase >> sv) & 1u, abort_flag);
-                        vc_phase ^= 1u << sv;
-                    }
-                    // the first PV of an item overwrites O: the previous item's epilogue must have read it
-                    if (ok && n == 0) ok = mbar_wait(bar(BAR_OF + 0), ((uint32_t)items_side[0] & 1u) ^ 1u, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    // the first three quarters of P are there: their products run while the softmax warps finish
-                    // the last quarter
-                    if (!kLseOnly) issue_pv(0, sv, n > 0, 0, 6);
-                    ok = mbar_wait(bar(BAR_PQ + 0), (uint32_t)gs[0] & 1u, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (!kLseOnly) issue_pv(0, sv, n > 0, 6, 8);
-                    // O-done is only waited for by the item's epilogue: between tiles the S-full barrier of tile n + 1
-                    // already implies PV(n) (a commit covers every product issued before it), and every commit costs
-                    // this thread some 40 cycles
-                    if (!has_next) tc_commit(bar(BAR_OD + 0));
-                    ++gs[0];
-                    if (has_next) {
-                        issue_qk(0, sk);
-                        tc_commit(bar(BAR_SF + 0));
-                    }
+                if (el) {
+                    issue_qk(n, 0, sk, nk);
+                    tc_commit(bar(BAR_SF + n));
                     if (hasB) {
-                        ok = mbar_wait(bar(BAR_PR + 1), (uint32_t)gs[1] & 1u, abort_flag);
-                        if (ok && n == 0)
-                            ok = mbar_wait(bar(BAR_OF + 1), ((uint32_t)items_side[1] & 1u) ^ 1u, abort_flag);
+                        issue_qk(1, 1, sk, nk);
+                        tc_commit(bar(BAR_SF + 1));
+                    }
+                    tc_commit(bar(BAR_KE + sk));
+                    if (n == nt - 1) tc_commit(bar(BAR_QE));  // Q is no longer needed by this item
+                }
+                next_k();
+            }
+            for (int n = 0; n < nt && ok; ++n) {
+                const Tile t(w, n);
+                const int nk = (kCp && n < n_rem) ? NK : t.nk;
+                const bool has_next = n + ahead < nt;
+                const int nk_next = has_next ? steps_of(n + ahead) : 0;
+                // The tiles first (they landed long ago as a rule), then the side's P: what follows the P barrier is on
+                // the side's critical path softmax -> P V -> Q K^T -> softmax.
+                if (!kLseOnly) ok = warp_wait(bar(BAR_VF + sv), pv, abort_flag);
+                if (kPaged && ok && t.bad0(len_k) < t.bad1()) {  // rows past the last key, cleared by the producer
+                    ok = warp_wait(bar(BAR_VC + sv), (vc_phase >> sv) & 1u, abort_flag);
+                    vc_phase ^= 1u << sv;
+                }
+                if (has_next && !packed) ok = ok && warp_wait(bar(BAR_KF + sk), pk, abort_flag);
+                if (!ok) break;
+#pragma unroll
+                for (int side = 0; side < 2; ++side) {
+                    if (packed ? (n & 1) != side : (side == 1 && !hasB)) continue;
+                    const bool first = n < ahead;  // the side's first tile of this item
+                    ok = ok && warp_wait(bar(BAR_PR + side), (uint32_t)gs[side] & 1u, abort_flag);
+                    // the first P V of an item overwrites O: the previous item's epilogue must have read it
+                    if (!kLseOnly && first) ok = ok && warp_wait(bar(BAR_OF + side), ((uint32_t)items_side[side] & 1u) ^ 1u, abort_flag);
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (!kLseOnly && el) issue_pv(side, sv, !first, nk);
+                    if (has_next && packed) {  // packed items run at the pace of memory: ask for their K tile late
+                        ok = warp_wait(bar(BAR_KF + sk), pk, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
-                        if (!kLseOnly) issue_pv(1, sv, n > 0, 0, 6);
-                        ok = mbar_wait(bar(BAR_PQ + 1), (uint32_t)gs[1] & 1u, abort_flag);
-                        if (!ok) break;
-                        tc_fence_after();
-                        if (!kLseOnly) issue_pv(1, sv, n > 0, 6, 8);
-                        if (!has_next) tc_commit(bar(BAR_OD + 1));
-                        ++gs[1];
+                    }
+                    if (el) {
+                        // O done is only waited for by the item's epilogue: between tiles S full of the side's next tile
+                        // already implies the P V before it (a commit covers every product issued before it)
+                        if (!kLseOnly && !has_next) tc_commit(bar(BAR_OD + side));
                         if (has_next) {
-                            issue_qk(1, sk);
-                            tc_commit(bar(BAR_SF + 1));
+                            issue_qk(side, packed ? 0 : side, sk, nk_next);
+                            tc_commit(bar(BAR_SF + side));
                         }
                     }
-                    tc_commit(bar(BAR_VE + sv));
-                    if (has_next) {
-                        tc_commit(bar(BAR_KE + sk));
-                        if (n + 2 == nt) tc_commit(bar(BAR_QE));  // that was the item's last QK
+                    ++gs[side];
+                }
+                if (!ok) break;
+                if (!kLseOnly) {
+                    if (el) tc_commit(bar(BAR_VE + sv));
+                    if (++sv == ST) {
+                        sv = 0;
+                        pv ^= 1u;
                     }
                 }
-                ++items;
-                ++items_side[0];
-                if (hasB) ++items_side[1];
+                if (has_next) {
+                    if (el) {
+                        tc_commit(bar(BAR_KE + sk));
+                        if (n + ahead == nt - 1) tc_commit(bar(BAR_QE));
+                    }
+                    next_k();
+                }
             }
-            // all MMAs issued by this thread must have retired before the tensor memory is freed
-            tc_commit(bar(BAR_FIN));
-            mbar_wait(bar(BAR_FIN), 0, abort_flag);
+            ++items;
+            ++items_side[0];
+            if (hasB || shared) ++items_side[1];
+            release_work(it);
         }
+        // all MMAs issued by this warp must have retired before the tensor memory is freed
+        if (el) tc_commit(bar(BAR_FIN));
+        warp_wait(bar(BAR_FIN), 0, abort_flag);
         __syncwarp();
       }
     } else {
@@ -685,123 +909,133 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const uint32_t tS = tmem_base + lane_base + (uint32_t)side * 128u;
         const uint32_t tO = tmem_base + lane_base + 256u + (uint32_t)side * (uint32_t)D;
-        int gs = 0;          // tiles processed by this side so far
-        int items_done = 0;  // items finished by this side (phase of O-done)
+        // phases (bits) of: S full, O done, hand-over of packed items
+        uint32_t phases = 0;
+        constexpr uint32_t kPhS = 1u, kPhO = 2u, kPhM = 4u;
         bool ok = true;
+        auto arrive_warp = [&](int b) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(b));
+        };
         for (int it = 0; ok; ++it) {
-            WorkItem w;
             // every decision taken after a bounded wait is made for the whole warp: the warp-wide tensor-memory
             // instructions and votes below need all 32 lanes
-            ok = __all_sync(0xffffffffu, fetch_work(it, w, false));
+            ok = wait_work(it);
             if (!ok) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BAR_WE + (it & 1)));
-            if (!w.valid) break;
-            const int hk = w.pair / p.pairs_per_kv;
-            const int hA = hk * p.G + 2 * (w.pair - hk * p.pairs_per_kv);
-            const bool hasB = (hA + 1) < (hk + 1) * p.G;
-            if (side == 1 && !hasB) continue;
-            const int seq_start = w.seq_start, seq_len = w.seq_len;
-            const int q0 = w.m_tile * BM;    // first query of the tile, counted inside the sequence's queries
-            const int iq = q0 + row;         // this thread's query, same counting
-            const int i0 = q0 + w.k_off, i1 = min(seq_len, q0 + BM) - 1 + w.k_off;  // positions inside the sequence
-            const bool full = w.full != 0;
-            const TileRange tr = tile_range(i0, i1, BN, p.window, w.n_sink, full);
-            const int n_rem = kCp ? (w.s_rem + BN - 1) / BN : 0;  // leading tiles from the sink buffer
-            const int nt = n_rem + tr.count();
-            const int i = iq + w.k_off;      // index of this thread's query among the (local) keys of its sequence
-            const int h = hA + side;
+            const volatile WorkItem& w = work_slots[it & 1];
+            if (!uniform(w.valid)) break;
+            const bool packed = !kLseOnly && uniform(w.packed) != 0;
+            const bool shared = packed && uniform(w.shared) != 0;
+            if (side == 1 && !shared && !uniform(w.hasB)) {
+                release_work(it);
+                continue;
+            }
+            const int n_rows = uniform(w.n_rows), nt = uniform(w.nt);
+            const bool row_ok = row < n_rows;
+            const bool idle = wq * 32 >= n_rows;  // none of this warp's rows exists: it only keeps the barriers going
             float m_used = -INFINITY, l_sum = 0.f;
-            for (int n = 0; n < nt; ++n, ++gs) {
+            const bool careful = uniform(w.careful) != 0;
+            bool fresh = true;   // some row of this warp has no reference yet, or one that is far behind
+            for (int n = shared ? side : 0; n < nt; n += shared ? 2 : 1) {
                 // a tile from the sink buffer holds positions before every local key: all rows see exactly its keys
                 // below s_rem; no window or causal edge runs through it
-                const bool remote = kCp && n < n_rem;
-                const int j0 = remote ? n * BN : tr.tile(n - n_rem) * BN;
-                const bool need_mask = remote ? (w.s_rem - j0 < BN)
-                                              : tile_needs_mask(i0, i1, j0, j0 + BN - 1, p.window, w.n_sink, full);
-                ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_SF + side), (uint32_t)gs & 1u, abort_flag));
+                const bool remote = kCp && n < w.n_rem;
+                const Tile t(w, n);
+                const bool need_mask = remote ? w.s_rem - n * BN < BN
+                                              : (t.cb < BN ? (t.cb > 0 || t.left < BN)
+                                                           : (t.jb + BN - 1 > w.i0 || (!w.full && t.jb <= w.i1 - p.window)));
+                ok = warp_wait(bar(BAR_SF + side), (phases & kPhS) != 0 ? 1u : 0u, abort_flag);
                 if (!ok) break;
+                phases ^= kPhS;
                 tc_fence_after();
-                uint32_t sr[128];
-                tmem_ld32(tS + 0, sr + 0);
-                tmem_ld32(tS + 32, sr + 32);
-                tmem_ld32(tS + 64, sr + 64);
-                tmem_ld32(tS + 96, sr + 96);
+                if (idle) {
+                    arrive_warp(BAR_PR + side);
+                    continue;
+                }
+                uint32_t sr[BN];
+                tmem_ld32(tS, sr);
+                tmem_ld32(tS + 32u, sr + 32);
                 tc_wait_ld();
-                if (kLseOnly) {  // S is in registers: the next Q K^T of this side may overwrite it
-                    tc_fence_before();
-                    mbar_arrive(bar(BAR_PR + side));
-                    mbar_arrive(bar(BAR_PQ + side));
-                }
-                uint32_t vis[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-                if (need_mask) {
-                    // Bit b of vis[cc] <=> column c = 32*cc + b of this tile is visible to this row:
-                    //   c <= dc  and  ( c > wl  or  c < sk ).
-                    const int dc = remote ? (1 << 20) : i - j0;
-                    const int wl = remote ? (1 << 20) : (full ? -1 : dc - p.window);
-                    const int sk = remote ? w.s_rem - j0 : (full ? 0 : w.n_sink - j0);
+                // the second half is fetched under the first half's exponentials (P goes to columns 0..63)
+                tmem_ld32(tS + 64u, sr + 64);
+                tmem_ld32(tS + 96u, sr + 96);
+                // Usual tile: the exponentials are taken against the reference as it stands, without forming the tile's maximum
+                // first (64 of some 600 instructions per row and tile; 3.5 % of the kernel's time at 32k tokens).  That loses
+                // no precision as long as nothing leaves the exponent range: bf16 P and the fp32 sums do not mind a common
+                // factor.  Masked tiles, and the tile after one whose scores outgrew the reference by 2^16, do form the
+                // maximum, and raise the reference where it is more than 2^8 behind.
+                const bool exact = need_mask || fresh || careful;
+                if (exact) {
+                    tc_wait_ld();
+                    pin64(sr + 64);
+                    if (need_mask) {
+                        // Bit b of vis <=> column c = 32*cc + b of this tile is visible to this row: a band key (c < cb)
+                        // not after the row (c <= dc) that lies in its window (c >= wl) or among the sinks (c < sk), or one
+                        // of the sink keys that follow the band (cb <= c < left), which every row sees.
+                        const bool full = w.full != 0;
+                        // index of this thread's query among the (local) keys; rows past the end take the last one's
+                        const int i = min(w.i0 + (packed ? row / p.G : row), w.i1);
+                        const int dc = remote ? -1 : min(i - t.jb, t.cb - 1);
+                        const int wl = full ? 0 : i - t.jb - p.window + 1;
+                        const int sk = full ? 0 : w.n_sink - t.jb;
+                        const int s0 = remote ? 0 : t.cb, s1 = remote ? w.s_rem - n * BN : t.left;
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        const int d = dc - 32 * cc, wd = wl - 32 * cc, sn = sk - 32 * cc;
-                        const uint32_t causal = d >= 31 ? 0xffffffffu : (d < 0 ? 0u : ((2u << d) - 1u));
-                        const uint32_t win = wd < 0 ? 0xffffffffu : (wd >= 31 ? 0u : ~((2u << wd) - 1u));
-                        const uint32_t snk = sn <= 0 ? 0u : (sn >= 32 ? 0xffffffffu : ((1u << sn) - 1u));
-                        vis[cc] = causal & (win | snk);
+                        for (int cc = 0; cc < 4; ++cc) {
+                            auto below = [&](int x) -> uint32_t {  // bits below x of this 32-column chunk
+                                const int d = x - 32 * cc;
+                                return d <= 0 ? 0u : (d >= 32 ? 0xffffffffu : (1u << d) - 1u);
+                            };
+                            const uint32_t vis = (below(dc + 1) & (~below(wl) | below(sk))) | (below(s1) & ~below(s0));
 #pragma unroll
-                        for (int b = 0; b < 32; ++b)
-                            sr[cc * 32 + b] = ((vis[cc] >> b) & 1u) ? sr[cc * 32 + b] : 0xff800000u;  // -inf
+                            for (int b = 0; b < 32; ++b)
+                                sr[cc * 32 + b] = ((vis >> b) & 1u) ? sr[cc * 32 + b] : 0xff800000u;  // -inf
+                        }
                     }
-                }
-                float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+                    float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
-                for (int c = 0; c < 128; c += 8) {
-                    mx0 = fmax3(mx0, __uint_as_float(sr[c + 0]), __uint_as_float(sr[c + 1]));
-                    mx1 = fmax3(mx1, __uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3]));
-                    mx2 = fmax3(mx2, __uint_as_float(sr[c + 4]), __uint_as_float(sr[c + 5]));
-                    mx3 = fmax3(mx3, __uint_as_float(sr[c + 6]), __uint_as_float(sr[c + 7]));
-                }
-                const float rmax = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
-                const float m_new = fmaxf(m_used, rmax);
-                const bool need = (m_used != -INFINITY) && ((m_new - m_used) * p.sl2 > kRescaleThreshold);
-                if (__any_sync(0xffffffffu, need)) {
-                    // raise the reference maximum of every row of this warp and rescale O accordingly; PV of the
-                    // previous tile has completed: it was issued before the QK whose S-full barrier this warp passed
-                    const float alpha = (m_used == -INFINITY) ? 1.f : ex2f((m_used - m_new) * p.sl2);
-#pragma unroll
-                    for (int cc = 0; cc < (kLseOnly ? 0 : D / 32); ++cc) {
-                        uint32_t orr[32];
-                        tmem_ld32(tO + cc * 32, orr);
-                        tc_wait_ld();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * alpha);
-                        tmem_st32(tO + cc * 32, orr);
+                    for (int c = 0; c < BN; c += 8) {
+                        mx0 = fmax3(mx0, __uint_as_float(sr[c + 0]), __uint_as_float(sr[c + 1]));
+                        mx1 = fmax3(mx1, __uint_as_float(sr[c + 2]), __uint_as_float(sr[c + 3]));
+                        mx2 = fmax3(mx2, __uint_as_float(sr[c + 4]), __uint_as_float(sr[c + 5]));
+                        mx3 = fmax3(mx3, __uint_as_float(sr[c + 6]), __uint_as_float(sr[c + 7]));
                     }
-                    if (!kLseOnly) tc_wait_st();
-                    l_sum *= alpha;
-                    m_used = m_new;
-                } else if (m_used == -INFINITY) {
-                    m_used = m_new;  // nothing accumulated yet for this row
+                    const float rmax = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3));
+                    const float m_new = fmaxf(m_used, rmax);
+                    const bool need = (m_used != -INFINITY) && ((m_new - m_used) * p.sl2 > kRescaleThreshold);
+                    if (__any_sync(0xffffffffu, row_ok && need)) {
+                        // raise the reference maximum of every row of this warp and rescale O accordingly; PV of the
+                        // side's previous tile has completed: it was issued before the QK whose S-full barrier this warp
+                        // passed
+                        const float alpha = (m_used == -INFINITY) ? 1.f : ex2f((m_used - m_new) * p.sl2);
+#pragma unroll
+                        for (int cc = 0; cc < (kLseOnly ? 0 : D / 32); ++cc) {
+                            uint32_t orr[32];
+                            tmem_ld32(tO + cc * 32, orr);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * alpha);
+                            tmem_st32(tO + cc * 32, orr);
+                        }
+                        if (!kLseOnly) tc_wait_st();
+                        l_sum *= alpha;
+                        m_used = m_new;
+                    } else if (m_used == -INFINITY) {
+                        m_used = m_new;  // nothing accumulated yet for this row
+                    }
+                    fresh = __any_sync(0xffffffffu, row_ok && m_used == -INFINITY);
                 }
-                const float off = (m_used == -INFINITY) ? 0.f : m_used * p.sl2;
+                // P = 2^(s * sl2 - off) into tensor memory as bf16 pairs, and into the row sum
+                const float off = m_used == -INFINITY ? 0.f : m_used * p.sl2;
                 const uint64_t sl2x2 = pack_f32x2(p.sl2, p.sl2), noffx2 = pack_f32x2(-off, -off);
                 uint64_t psum_a = pack_f32x2(0.f, 0.f), psum_b = pack_f32x2(0.f, 0.f);
+                float hi = -INFINITY;  // largest argument of the polynomial path
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) {
-                    uint32_t pk[16];
-                    if (need_mask && __all_sync(0xffffffffu, vis[cc] == 0u)) {
-                        // no row of this warp sees any of these 32 keys: P = 0 without touching the MUFU
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) pk[c] = 0u;
-                        if (!kLseOnly) {
-                            tmem_st16(tS + cc * 16, pk);
-                            if (cc == 2) {  // three quarters of P written: hand them to the issuer
-                                tc_wait_st();
-                                tc_fence_before();
-                                mbar_arrive(bar(BAR_PR + side));
-                            }
-                        }
-                        continue;
+                    if (cc == 2) {
+                        tc_wait_ld();
+                        pin64(sr + 64);
                     }
+                    uint32_t pk[16];
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         const uint64_t x = fma_f32x2(
@@ -811,6 +1045,7 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                         unpack_f32x2(x, x0, x1);
                         float p0, p1;
                         if ((kPolyPairMask >> c) & 1u) {
+                            hi = fmax3(hi, x0, x1);
                             exp2_poly_x2(x0, x1, p0, p1);  // FMA pipe: takes load off the special-function unit
                         } else {
                             p0 = ex2f(x0);
@@ -820,86 +1055,154 @@ prefill_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                         else psum_a = add_f32x2(psum_a, pack_f32x2(p0, p1));
                         if (!kLseOnly) pk[c] = pack_bf16x2(p0, p1);
                     }
-                    if (!kLseOnly) {
-                        tmem_st16(tS + cc * 16, pk);
-                        if (cc == 2) {  // three quarters of P written: hand them to the issuer
-                            tc_wait_st();
-                            tc_fence_before();
-                            mbar_arrive(bar(BAR_PR + side));
-                        }
-                    }
+                    if (!kLseOnly) tmem_st16(tS + (uint32_t)cc * 16u, pk);
                 }
+                float sum;
                 {
                     float a0, a1;
                     unpack_f32x2(add_f32x2(psum_a, psum_b), a0, a1);
-                    l_sum += a0 + a1;
+                    sum = a0 + a1;
                 }
-                if (!kLseOnly) {
-                    tc_wait_st();
-                    tc_fence_before();
-                    mbar_arrive(bar(BAR_PQ + side));
+                l_sum += sum;
+                if (!exact && __any_sync(0xffffffffu, row_ok && !(sum <= 65536.f && hi <= 16.f))) {
+                    // Growth shows in the row sum, except in the columns of the polynomial path: those are bounded by their
+                    // largest argument.  Far out of range (also: not a number) the whole item is run again, forming every
+                    // tile's maximum.
+                    fresh = true;
+                    if (__any_sync(0xffffffffu, row_ok && !(sum <= kSumLimit && hi <= 60.f)) && lane == 0) s_again[it & 1] = 1;
                 }
+                if (!kLseOnly) tc_wait_st();
+                tc_fence_before();
+                arrive_warp(BAR_PR + side);
             }
             if (!ok) break;
             // ---- epilogue of this item: O / l -> bf16 -> global
-            ok = __all_sync(0xffffffffu, mbar_wait(bar(BAR_OD + side), (uint32_t)items_done & 1u, abort_flag));
-            if (!ok) break;
-            ++items_done;
-            tc_fence_after();
-            uint32_t orr[D];
             if (!kLseOnly) {
+                ok = warp_wait(bar(BAR_OD + side), (phases & kPhO) != 0 ? 1u : 0u, abort_flag);
+                if (!ok) break;
+                phases ^= kPhO;
+                tc_fence_after();
+            }
+            const int q_row = packed ? row / p.G : w.q0 + row;  // this thread's query, counted inside the sequence
+            const int token = w.seq_start + q_row, tok0 = w.seq_start + w.q0;
+            const int h = packed ? w.hA + row - q_row * p.G : w.hA + side;
+            release_work(it);
+            __nv_bfloat16* orow = p.out + ((size_t)token * p.Hq + h) * D;
+            // eight channels of this thread's row
+            auto pack8 = [](const uint32_t* o, float inv) {
+                return make_uint4(pack_bf16x2(__uint_as_float(o[0]) * inv, __uint_as_float(o[1]) * inv),
+                                  pack_bf16x2(__uint_as_float(o[2]) * inv, __uint_as_float(o[3]) * inv),
+                                  pack_bf16x2(__uint_as_float(o[4]) * inv, __uint_as_float(o[5]) * inv),
+                                  pack_bf16x2(__uint_as_float(o[6]) * inv, __uint_as_float(o[7]) * inv));
+            };
+            auto o_free = [&]() {  // O may be overwritten by the next item's first P V
+                tc_fence_before();
+                arrive_warp(BAR_OF + side);
+            };
+            if (idle) {
+                if (!kLseOnly) o_free();
+                continue;
+            }
+            if (shared) {
+                // Side B hands its rows' (max, sum, O) to the warp of side A with the same rows, through the staging areas
+                // of the two warps: 32 rows x 64 channels of fp32 at a time, 16-byte chunks swizzled by row.
+                const uint32_t mine = sStage + (uint32_t)wq * 4096u +
+                                      (lane < 16 ? (uint32_t)lane * 256u : 16384u + (uint32_t)(lane - 16) * 256u);
+                if (lane == 0) tma_store_wait_read();  // earlier output stores have read the staging areas
+                if (side == 1) s_merge[row] = make_float2(m_used, l_sum);
+                float wa = 1.f, wb = 0.f, inv = 0.f;
+                auto pair_sync = [&]() -> bool {  // the two warps of these rows
+                    arrive_warp(BAR_MG + wq);
+                    phases ^= kPhM;
+                    return warp_wait(bar(BAR_MG + wq), (phases & kPhM) != 0 ? 0u : 1u, abort_flag);
+                };
+#pragma unroll
+                for (int half = 0; half < D / 64 && ok; ++half) {
+                    uint32_t o[64];
+                    tmem_ld32(tO + (uint32_t)(half * 64), o);
+                    tmem_ld32(tO + (uint32_t)(half * 64 + 32), o + 32);
+                    tc_wait_ld();
+                    if (half == D / 64 - 1) o_free();
+                    ok = pair_sync();  // the area is free
+                    if (ok && side == 1) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            st_shared_v4(mine + (uint32_t)((j ^ (lane & 15)) * 16), o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+                    }
+                    ok = ok && pair_sync();  // the area is filled
+                    if (ok && side == 0) {
+                        if (half == 0) {
+                            const float2 other = s_merge[row];
+                            const float M = fmaxf(m_used, other.x);
+                            wa = m_used == -INFINITY ? 0.f : ex2f((m_used - M) * p.sl2);
+                            wb = other.x == -INFINITY ? 0.f : ex2f((other.x - M) * p.sl2);
+                            l_sum = wa * l_sum + wb * other.y;
+                            m_used = M;
+                            inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
+                        }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            uint32_t b4[4];
+                            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                         : "=r"(b4[0]), "=r"(b4[1]), "=r"(b4[2]), "=r"(b4[3])
+                                         : "r"(mine + (uint32_t)((j ^ (lane & 15)) * 16))
+                                         : "memory");
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                // a side without any visible key of the row has no usable O
+                                const float x = wa > 0.f ? __uint_as_float(o[4 * j + e]) * wa : 0.f;
+                                const float y = wb > 0.f ? __uint_as_float(b4[e]) * wb : 0.f;
+                                o[4 * j + e] = __float_as_uint(x + y);
+                            }
+                        }
+                        if (row_ok)
+#pragma unroll
+                            for (int v = 0; v < 8; ++v) *reinterpret_cast<uint4*>(orow + half * 64 + v * 8) = pack8(o + v * 8, inv);
+                    }
+                }
+                // side A has read the last half before side B's next output uses the area
+                ok = ok && pair_sync();
+                if (!ok) break;
+                if (side == 1) continue;
+            } else if (!kLseOnly) {
+                uint32_t orr[D];
 #pragma unroll
                 for (int cc = 0; cc < D / 32; ++cc) tmem_ld32(tO + cc * 32, orr + cc * 32);
                 tc_wait_ld();
-            }
-            tc_fence_before();
-            mbar_arrive(bar(BAR_OF + side));  // O may be overwritten by the next item's first PV
-            const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
-            if (kLseOnly) {
-                // nothing to store but the log-sum-exp below
-            } else if (q0 + wq * 32 + 31 < seq_len) {
-                // all 32 rows of this warp are valid: stage [32 rows][64 ch] panels in shared memory in the
-                // 128-byte-swizzled layout and let TMA write them (fully coalesced, off the LSU path)
-                const uint32_t stage = sStage + (uint32_t)warp * 4096u;
+                o_free();
+                const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
+                if (!packed && wq * 32 + 31 < n_rows) {
+                    // all 32 rows of this warp are valid: stage [32 rows][64 ch] panels in shared memory in the
+                    // 128-byte-swizzled layout and let TMA write them (fully coalesced, off the LSU path)
+                    const uint32_t stage = sStage + (uint32_t)warp * 4096u;
 #pragma unroll
-                for (int pn = 0; pn < D / 64; ++pn) {
-                    if (lane == 0) tma_store_wait_read();  // the previous store has finished reading the stage
-                    __syncwarp();
+                    for (int pn = 0; pn < D / 64; ++pn) {
+                        if (lane == 0) tma_store_wait_read();  // the previous store has finished reading the stage
+                        __syncwarp();
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t* o8 = orr + pn * 64 + j * 8;
-                        st_shared_v4(stage + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) * 16),
-                                     pack_bf16x2(__uint_as_float(o8[0]) * inv, __uint_as_float(o8[1]) * inv),
-                                     pack_bf16x2(__uint_as_float(o8[2]) * inv, __uint_as_float(o8[3]) * inv),
-                                     pack_bf16x2(__uint_as_float(o8[4]) * inv, __uint_as_float(o8[5]) * inv),
-                                     pack_bf16x2(__uint_as_float(o8[6]) * inv, __uint_as_float(o8[7]) * inv));
+                        for (int j = 0; j < 8; ++j) {
+                            const uint4 v = pack8(orr + pn * 64 + j * 8, inv);
+                            st_shared_v4(stage + (uint32_t)lane * 128u + (uint32_t)((j ^ (lane & 7)) * 16), v.x, v.y, v.z, v.w);
+                        }
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_3d(&tm.out, stage, pn * 64, h, tok0 + wq * 32);
+                            tma_store_commit();
+                        }
                     }
-                    fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_3d(&tm_o, stage, pn * 64, h, seq_start + q0 + wq * 32);
-                        tma_store_commit();
-                    }
-                }
-            } else if (iq < seq_len) {
-                // ragged tail of a sequence: plain predicated row stores
-                __nv_bfloat16* orow = p.out + ((size_t)(seq_start + iq) * p.Hq + h) * D;
+                } else if (row_ok) {
+                    // packed rows, or the ragged tail of a sequence: plain predicated row stores
 #pragma unroll
-                for (int v = 0; v < D / 8; ++v) {
-                    uint4 o4;
-                    o4.x = pack_bf16x2(__uint_as_float(orr[v * 8 + 0]) * inv, __uint_as_float(orr[v * 8 + 1]) * inv);
-                    o4.y = pack_bf16x2(__uint_as_float(orr[v * 8 + 2]) * inv, __uint_as_float(orr[v * 8 + 3]) * inv);
-                    o4.z = pack_bf16x2(__uint_as_float(orr[v * 8 + 4]) * inv, __uint_as_float(orr[v * 8 + 5]) * inv);
-                    o4.w = pack_bf16x2(__uint_as_float(orr[v * 8 + 6]) * inv, __uint_as_float(orr[v * 8 + 7]) * inv);
-                    *reinterpret_cast<uint4*>(orow + v * 8) = o4;
+                    for (int v = 0; v < D / 8; ++v) *reinterpret_cast<uint4*>(orow + v * 8) = pack8(orr + v * 8, inv);
                 }
             }
-            if (iq < seq_len && p.lse != nullptr) {
+            if (row_ok && p.lse != nullptr) {
                 const float lse2 = (m_used == -INFINITY) ? -INFINITY : m_used * p.sl2 + log2f(l_sum);
-                p.lse[(size_t)h * p.T + seq_start + iq] = lse2 * 0.6931471805599453f;
+                p.lse[(size_t)h * p.T + token] = lse2 * 0.6931471805599453f;
             }
         }
-        if (lane == 0) tma_store_wait_all();  // outstanding output stores of this warp
+        if (lane == 0) tma_store_wait_read();  // outstanding output stores of this warp have read their staging
     }
 
     // ---- teardown: every thread arrives here (also after a failed wait); free the tensor memory

@@ -1,0 +1,48 @@
+"""GPU parity of the prefill kernel's work items where they can go wrong: sequences around the size that is packed into
+one item per kv head, batches of more sequences than one look of the scheduler covers, tiles that join band and sink
+keys, and scores that outgrow the exponent range of the reference within one tile (the item is then run again)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2512_10411_b200 import inputs
+from helpers import check_against_oracle
+from test_prefill_chunked_gpu import make, run_chunked
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(lq, lk, Hq, Hkv, D, W, S, full, seed, scale=0.0):
+    q, k, v = make(lq, lk, Hq, Hkv, D, seed)
+    out, lse, status = run_chunked(q, k, v, lq, lk, W, S, full, scale)
+    assert status == 0
+    ref = oracle.prefill_chunked(*(inputs.to_f32_numpy(t) for t in (q, k, v)), np.concatenate([[0], np.cumsum(lq)]),
+                                 np.concatenate([[0], np.cumsum(lk)]), W, S, full, scale=scale if scale > 0 else None)
+    check_against_oracle(out, ref["out"], f"{lq[:4]} {lk[:4]} Hq={Hq} Hkv={Hkv} D={D} W={W} S={S} full={full}")
+    np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(2, 2, 128), (4, 2, 64), (7, 1, 128), (16, 2, 128), (128, 1, 64), (130, 1, 128)])
+def test_sequences_around_the_packed_size(Hq, Hkv, D):
+    n = 128 // (Hq // Hkv)  # tokens that fill an item's rows (0: never packed)
+    lq = (max(n - 1, 1), max(n, 1), n + 1, 1, 1)
+    lk = (max(n - 1, 1), max(n, 1) + 300, n + 1 + 77, 1, 513)
+    for W, S, full in ((1, 0, True), (128, 4, False), (100, 20, False), (33, 140, False), (1, 1, False)):
+        _check(lq, lk, Hq, Hkv, D, W, S, full, seed=40 + n)
+
+
+def test_more_sequences_than_one_look_of_the_scheduler():
+    rng = np.random.default_rng(3)
+    lq = tuple(int(x) for x in rng.integers(1, 200, 70))
+    lk = tuple(a + int(x) for a, x in zip(lq, rng.integers(0, 200, 70)))
+    _check(lq, lk, 4, 2, 128, 100, 4, False, seed=60)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("scale", [4.0, 30.0])
+def test_scores_that_leave_the_exponent_range_of_the_reference(D, scale):
+    # |scaled scores| reach 4 * 45 = 180 and 30 * 45 = 1350: from one key tile to the next the largest one of a row grows
+    # by far more than 60 in log2 units.  Tolerances as everywhere: the products are exact in fp32 to 2^-23 * 1350 = 2e-4.
+    for lq, lk in (((700,), (700,)), ((1, 30, 129), (900, 430, 1000))):
+        for W, S, full in ((1, 0, True), (300, 4, False)):
+            _check(lq, lk, 4, 1, D, W, S, full, seed=80 + D, scale=scale)
