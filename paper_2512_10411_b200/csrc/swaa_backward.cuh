@@ -44,6 +44,7 @@ template <int D>
 __global__ void backward_delta_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout,
                                       const float* __restrict__ lse, float* __restrict__ delta,
                                       float* __restrict__ lse2, float* __restrict__ dq_accum, int T, int Hq) {
+    grid_wait();
     constexpr int kLanes = D / 8;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long row = idx / kLanes;
@@ -75,6 +76,7 @@ __global__ void backward_delta_kernel(const __nv_bfloat16* __restrict__ out, con
 
 // dq = bf16(dq_accum)
 __global__ void backward_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, size_t n) {
+    grid_wait();
     const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i + 3 < n) {
         const float4 v = *reinterpret_cast<const float4*>(acc + i);
@@ -88,6 +90,7 @@ __global__ void backward_convert_dq_kernel(const float* __restrict__ acc, __nv_b
 __global__ void backward_convert_dkv_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dk,
                                             __nv_bfloat16* __restrict__ dv, const int32_t* __restrict__ cu_seqlens, int B,
                                             int T, int max_seqlen, int sink_rows, int Hkv, int D) {
+    grid_wait();
     const size_t plane = (size_t)B * sink_rows * Hkv * D;
     const size_t e = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (e >= plane) return;

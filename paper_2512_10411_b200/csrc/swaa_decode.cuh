@@ -242,6 +242,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_v16)) : "memory");
     }
 
+    grid_wait();  // nothing above touches global memory
+
     // ---- where does this block's run of the global tile list start?  (scan of tiles per sequence)
     auto tiles_of = [&](int b) -> long long { return (long long)DecodeWalker<kPaged, kShard>::geom(p, b).nt * p.IPB; };
     // A sequence without tiles.  Dense / paged cache: its length is out of range; report it and zero its output
@@ -710,6 +712,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
 // row without any non-empty partial gives zeros.
 template <int D>
 __global__ void decode_combine_kernel(const float* __restrict__ part, int P, int rows, __nv_bfloat16* __restrict__ out) {
+    grid_wait();
     const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (row >= rows) return;
     float M = -INFINITY;

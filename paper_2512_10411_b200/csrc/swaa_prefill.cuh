@@ -459,6 +459,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    grid_wait();  // nothing above touches global memory
 
     // Consumers of the work descriptors: item `it` is in slot it & 1; they read it in place and release it at their end of
     // the item.

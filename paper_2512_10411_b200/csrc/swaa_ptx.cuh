@@ -9,6 +9,10 @@ namespace swaa {
 
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 
+// Waits until the kernel before this one on the stream has ended and its writes are visible.  Every thread of every kernel
+// calls it before it touches global memory (see launch_overlapped), so the order of the stream's work is unchanged.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
