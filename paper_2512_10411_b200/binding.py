@@ -139,21 +139,25 @@ def status_str(status: int) -> str:
 
 
 def _dev_ptr(t: torch.Tensor | None, dtype, name: str):
+    """Device address of a tensor, for a pointer argument (None stays None)."""
     if t is None:
         return None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream_ptr(stream):
     if stream is None:
+        # the address of the current device's current stream, without building a Stream object (0.3 against 3.1 us)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink: int, is_full: bool,
@@ -162,10 +166,10 @@ def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink:
     lib = load_library()
     T, Hq, D = q.shape
     Hkv = k.shape[1]
-    if tuple(k.shape) != (T, Hkv, D) or tuple(v.shape) != (T, Hkv, D) or tuple(out.shape) != (T, Hq, D):
+    if k.shape != (T, Hkv, D) or v.shape != (T, Hkv, D) or out.shape != (T, Hq, D):
         raise ValueError("swaa_prefill: inconsistent tensor shapes")
     B = cu_seqlens.numel() - 1
-    if lse is not None and tuple(lse.shape) != (Hq, T):
+    if lse is not None and lse.shape != (Hq, T):
         raise ValueError("swaa_prefill: lse must be [Hq, T]")
     bf = torch.bfloat16
     rc = lib.swaa_prefill(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"), _dev_ptr(out, bf, "out"),
@@ -184,12 +188,12 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
     lib = load_library()
     Tq, Hq, D = q.shape
     Tk, Hkv = k.shape[0], k.shape[1]
-    if tuple(k.shape) != (Tk, Hkv, D) or tuple(v.shape) != (Tk, Hkv, D) or tuple(out.shape) != (Tq, Hq, D):
+    if k.shape != (Tk, Hkv, D) or v.shape != (Tk, Hkv, D) or out.shape != (Tq, Hq, D):
         raise ValueError("swaa_prefill_chunked: inconsistent tensor shapes")
     B = cu_seqlens_q.numel() - 1
     if cu_seqlens_k.numel() != B + 1:
         raise ValueError("swaa_prefill_chunked: cu_seqlens_q and cu_seqlens_k must have the same length")
-    if lse is not None and tuple(lse.shape) != (Hq, Tq):
+    if lse is not None and lse.shape != (Hq, Tq):
         raise ValueError("swaa_prefill_chunked: lse must be [Hq, Tq]")
     bf = torch.bfloat16
     if is_full_seq is not None:
@@ -227,7 +231,7 @@ def swaa_prefill_backward(q, k, v, out, dout, lse, cu_seqlens, max_seqlen: int, 
     Hkv = k.shape[1]
     for name, t, shp in (("k", k, (T, Hkv, D)), ("v", v, (T, Hkv, D)), ("out", out, (T, Hq, D)), ("dout", dout, (T, Hq, D)),
                          ("dq", dq, (T, Hq, D)), ("dk", dk, (T, Hkv, D)), ("dv", dv, (T, Hkv, D)), ("lse", lse, (Hq, T))):
-        if tuple(t.shape) != shp:
+        if t.shape != shp:
             raise ValueError(f"swaa_prefill_backward: {name} must be {shp}")
     B = cu_seqlens.numel() - 1
     bf = torch.bfloat16
@@ -248,12 +252,12 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
     lib = load_library()
     Tq, Hq, D = q.shape
     num_pages, page_size, Hkv, _ = kpages.shape
-    if tuple(vpages.shape) != tuple(kpages.shape) or kpages.shape[3] != D or tuple(out.shape) != (Tq, Hq, D):
+    if vpages.shape != kpages.shape or kpages.shape[3] != D or out.shape != (Tq, Hq, D):
         raise ValueError("swaa_prefill_paged: inconsistent tensor shapes")
     B = cu_seqlens_q.numel() - 1
     if block_table.dim() != 2 or block_table.shape[0] != B or seqlens_k.numel() != B:
         raise ValueError("swaa_prefill_paged: block_table must be [B, max_blocks] and seqlens_k [B]")
-    if lse is not None and tuple(lse.shape) != (Hq, Tq):
+    if lse is not None and lse.shape != (Hq, Tq):
         raise ValueError("swaa_prefill_paged: lse must be [Hq, Tq]")
     bf = torch.bfloat16
     if is_full_seq is not None:
@@ -290,7 +294,7 @@ def swaa_prefill_context_parallel(q, k_local, v_local, sink_k, sink_v, out, cu_s
     lib = load_library()
     Tq, Hq, D = q.shape
     Tk, Hkv = k_local.shape[0], k_local.shape[1]
-    if tuple(k_local.shape) != (Tk, Hkv, D) or tuple(v_local.shape) != (Tk, Hkv, D) or tuple(out.shape) != (Tq, Hq, D):
+    if k_local.shape != (Tk, Hkv, D) or v_local.shape != (Tk, Hkv, D) or out.shape != (Tq, Hq, D):
         raise ValueError("swaa_prefill_context_parallel: inconsistent tensor shapes")
     B = cu_seqlens_q.numel() - 1
     if cu_seqlens_k.numel() != B + 1 or key_pos0.numel() != B:
@@ -298,9 +302,9 @@ def swaa_prefill_context_parallel(q, k_local, v_local, sink_k, sink_v, out, cu_s
     sink_rows = 0
     if sink_k is not None:
         sink_rows = sink_k.shape[1]
-        if tuple(sink_k.shape) != (B, sink_rows, Hkv, D) or tuple(sink_v.shape) != tuple(sink_k.shape):
+        if sink_k.shape != (B, sink_rows, Hkv, D) or sink_v.shape != sink_k.shape:
             raise ValueError("swaa_prefill_context_parallel: sink_k, sink_v must be [B, sink_rows, Hkv, D]")
-    if lse is not None and tuple(lse.shape) != (Hq, Tq):
+    if lse is not None and lse.shape != (Hq, Tq):
         raise ValueError("swaa_prefill_context_parallel: lse must be [Hq, Tq]")
     bf = torch.bfloat16
     rc = lib.swaa_prefill_context_parallel(_dev_ptr(q, bf, "q"), _dev_ptr(k_local, bf, "k_local"),
@@ -322,7 +326,7 @@ def swaa_lazy_ratio(q, k, v, cu_seqlens_q, cu_seqlens_k, max_seqlen_q: int, max_
     lib = load_library()
     Tq, Hq, D = q.shape
     Tk, Hkv = k.shape[0], k.shape[1]
-    if tuple(scratch_lse.shape) != (2, Hq, Tq) or tuple(ratio.shape) != (Hq,):
+    if scratch_lse.shape != (2, Hq, Tq) or ratio.shape != (Hq,):
         raise ValueError("swaa_lazy_ratio: inconsistent output / scratch shapes")
     B = cu_seqlens_q.numel() - 1
     bf = torch.bfloat16
@@ -354,8 +358,8 @@ def swaa_decode(q, kcache, vcache, out, seqlens, window: int, n_sink: int, is_fu
     lib = load_library()
     B, Hq, D = q.shape
     _, Lmax, Hkv, _ = kcache.shape
-    if tuple(kcache.shape) != (B, Lmax, Hkv, D) or tuple(vcache.shape) != (B, Lmax, Hkv, D) \
-            or tuple(out.shape) != (B, Hq, D) or seqlens.numel() != B:
+    if kcache.shape != (B, Lmax, Hkv, D) or vcache.shape != (B, Lmax, Hkv, D) \
+            or out.shape != (B, Hq, D) or seqlens.numel() != B:
         raise ValueError("swaa_decode: inconsistent tensor shapes")
     bf = torch.bfloat16
     rc = lib.swaa_decode(_dev_ptr(q, bf, "q"), _dev_ptr(kcache, bf, "kcache"), _dev_ptr(vcache, bf, "vcache"),
@@ -379,7 +383,7 @@ def swaa_decode_paged(q, kpages, vpages, out, block_table, seqlens, window: int,
     lib = load_library()
     B, Hq, D = q.shape
     num_pages, page_size, Hkv, _ = kpages.shape
-    if tuple(vpages.shape) != tuple(kpages.shape) or kpages.shape[3] != D or tuple(out.shape) != (B, Hq, D):
+    if vpages.shape != kpages.shape or kpages.shape[3] != D or out.shape != (B, Hq, D):
         raise ValueError("swaa_decode_paged: inconsistent tensor shapes")
     if block_table.dim() != 2 or block_table.shape[0] != B or seqlens.numel() != B:
         raise ValueError("swaa_decode_paged: block_table must be [B, max_blocks] and seqlens [B]")
@@ -406,8 +410,8 @@ def swaa_decode_partial(q, kshard, vshard, partial_out, seqlens, key_pos0: int, 
     lib = load_library()
     B, Hq, D = q.shape
     _, Lshard, Hkv, _ = kshard.shape
-    if tuple(kshard.shape) != (B, Lshard, Hkv, D) or tuple(vshard.shape) != (B, Lshard, Hkv, D) \
-            or tuple(partial_out.shape) != (B, Hq, D + 2) or seqlens.numel() != B:
+    if kshard.shape != (B, Lshard, Hkv, D) or vshard.shape != (B, Lshard, Hkv, D) \
+            or partial_out.shape != (B, Hq, D + 2) or seqlens.numel() != B:
         raise ValueError("swaa_decode_partial: inconsistent tensor shapes")
     bf = torch.bfloat16
     rc = lib.swaa_decode_partial(_dev_ptr(q, bf, "q"), _dev_ptr(kshard, bf, "kshard"), _dev_ptr(vshard, bf, "vshard"),
@@ -423,7 +427,7 @@ def swaa_decode_combine(partials, out, stream=None) -> None:
     """Forwards to C swaa_decode_combine.  partials f32 [P,B,Hq,D+2]; out bf16 [B,Hq,D]."""
     lib = load_library()
     P, B, Hq, D2 = partials.shape
-    if tuple(out.shape) != (B, Hq, D2 - 2):
+    if out.shape != (B, Hq, D2 - 2):
         raise ValueError("swaa_decode_combine: out must be [B, Hq, D]")
     rc = lib.swaa_decode_combine(_dev_ptr(partials, torch.float32, "partials"), P, B, Hq, D2 - 2,
                                  _dev_ptr(out, torch.bfloat16, "out"), _stream_ptr(stream))
@@ -452,8 +456,8 @@ def swaa_decode_static(q, kcache, vcache, out, seqlens, window: int, n_sink: int
     lib = load_library()
     B, Hq, D = q.shape
     _, Lmax, Hkv, _ = kcache.shape
-    if tuple(kcache.shape) != (B, Lmax, Hkv, D) or tuple(vcache.shape) != (B, Lmax, Hkv, D) \
-            or tuple(out.shape) != (B, Hq, D) or seqlens.numel() != B:
+    if kcache.shape != (B, Lmax, Hkv, D) or vcache.shape != (B, Lmax, Hkv, D) \
+            or out.shape != (B, Hq, D) or seqlens.numel() != B:
         raise ValueError("swaa_decode_static: inconsistent tensor shapes")
     bf = torch.bfloat16
     rc = lib.swaa_decode_static(_dev_ptr(q, bf, "q"), _dev_ptr(kcache, bf, "kcache"), _dev_ptr(vcache, bf, "vcache"),
