@@ -26,9 +26,9 @@
 // 1.52 GHz (1.60 before), so fewer cycles per tile buy about half their share in time.  Per 128 x 128 tile of both sides
 // 3260 cycles (3710 before) against 2050 of products and 1970 of softmax: a side is a chain softmax -> P V -> Q K^T.
 // Against the kernel that had one issuing lane, a maximum pass on every tile, sink tiles of their own and a fixed
-// assignment of items: 8280 -> 7620 us; the same prompt with a 2048-key window 1178 -> 1101 us; eight ragged prompts of
+// assignment of items: 8280 -> 7640 us; the same prompt with a 2048-key window 1178 -> 1101 us; eight ragged prompts of
 // 146k tokens, Hq = 64, window 4096: 17550 -> 16230 us; a serving step of 4 prompt chunks and 24 generated tokens in
-// pages: 1136 -> 815 us.
+// pages: 1136 -> 595 us.
 //
 // Every wait is bounded: a wait that runs out records SWAA_ERR_TIMEOUT, all roles leave their loops,
 // the block waits (bounded) for its outstanding copies, frees its tensor memory and returns.
@@ -290,16 +290,21 @@ struct PrefillSmem {
     static constexpr int kPanelBytes = 128 * 128;   // one [128 rows][64 ch] panel
     static constexpr int kPanels = D / 64;
     static constexpr int kStages = D == 128 ? 2 : 4;
-    static constexpr int kOffQ = 0;                              // two tiles (sides A, B)
-    static constexpr int kOffK = 2 * kTileBytes;                 // kStages tiles
-    static constexpr int kOffV = kOffK + kStages * kTileBytes;   // kStages tiles
-    static constexpr int kOffStage = kOffV + kStages * kTileBytes;  // 8 x 4 KiB: per-warp output staging
-    static constexpr int kOffMerge = kOffStage + 8 * 4096;  // packed items: (max, sum) of side B's rows
+    // Q of side A, then tile-sized slots one after another: Q of side B, kStages of K, kStages of V, the output staging
+    // (8 x 4 KiB, one per softmax warp).  A packed item has one Q tile and no staged output, so all of the slots are
+    // its ring of K and V tiles.
+    static constexpr int kOffQ = 0;
+    static constexpr int kOffSlots = kTileBytes;
+    static constexpr int kSlotK = 1, kSlotV = 1 + kStages, kSlotStage = 1 + 2 * kStages;
+    static constexpr int kStageBytes = 8 * 4096;
+    static constexpr int kSlots = kSlotStage + kStageBytes / kTileBytes;
+    static constexpr int kOffStage = kOffSlots + kSlotStage * kTileBytes;
+    static constexpr int kOffMerge = kOffStage + kStageBytes;  // packed items: (max, sum) of side B's rows
     static constexpr int kOffBar = kOffMerge + 128 * 8;
-    // barriers: Q full/empty; K full/empty, V full/empty, V-tile-cleared (paged keys only) per stage; per side S full /
-    // P ready / O done / O free; work descriptor full/empty per slot, next-block answer, hand-over of packed items
-    // per row quadrant, final
-    static constexpr int kNumBars = 2 + 5 * kStages + 2 * 4 + 5 + 4 + 1;
+    // barriers: Q full/empty; full/empty/V-tile-cleared (paged keys only) per slot; per side S full / P ready / O done /
+    // O free; work descriptor full/empty per slot, next-block answer, hand-over of packed items per row quadrant,
+    // staging free, final
+    static constexpr int kNumBars = 2 + 3 * kSlots + 2 * 4 + 5 + 4 + 2;
     static constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) / 16 * 16;  // next-block answer, tmem slot, flags, work descriptors
     static constexpr int kBytes = kOffMisc + 32 + 2 * kWorkInts * 4;
     static constexpr int kDynamicBytes = kBytes + 1024;          // room to align the base to 1024 B
@@ -384,6 +389,15 @@ struct TileGeom {
     __device__ __forceinline__ int bad1() const { return min(cb, 16 * nk); }
 };
 
+// A flag of a piece of code: known when it is compiled, or read when it runs.
+template <bool kValue>
+struct ConstFlag {
+    static constexpr bool known = true, value = kValue;
+};
+struct RuntimeFlag {
+    static constexpr bool known = false, value = false;
+};
+
 // kMode 0: self attention.  1: chunked prefill, the queries are the last len_q tokens of a longer key sequence
 // (separate packing of the keys).  2: the same with keys and values in pages addressed through a block table.
 // 3: context-parallel prefill, mode 1 with the local keys starting at position key_pos0[b] of their sequence and the
@@ -400,26 +414,32 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     constexpr int BM = kPrefillBM, BN = kPrefillBN;
     constexpr int ST = L::kStages;
     constexpr int NK = BN / 16;        // 16-key steps of a tile
+    // A packed item's ring spans all slots where the keys of a short sequence can be many (generated tokens).  In the
+    // self-attention instance they cannot, and the loops are shorter without the second order of slots.
+    constexpr bool kDeepRing = kChunked && !kLseOnly;
     using Tile = TileGeom<BN>;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-    const uint32_t sQ = smem_base + L::kOffQ, sK = smem_base + L::kOffK, sV = smem_base + L::kOffV;
+    const uint32_t sQ = smem_base + L::kOffQ, sSlots = smem_base + L::kOffSlots;
     const uint32_t sStage = smem_base + L::kOffStage;
     const uint32_t bars = smem_base + L::kOffBar;
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
     // barrier indices
-    constexpr int BAR_QF = 0, BAR_QE = 1, BAR_KF = 2, BAR_KE = BAR_KF + ST, BAR_VF = BAR_KE + ST, BAR_VE = BAR_VF + ST;
+    constexpr int NS = L::kSlots;
+    constexpr int BAR_QF = 0, BAR_QE = 1, BAR_F = 2, BAR_E = BAR_F + NS;  // slot full, slot empty
+    // paged only, one per slot: the rows of the V tile in that slot past the last key have been cleared.
+    // Completed once per cleared tile; the issuer keeps the slot's phase bit.  The producer cannot
+    // clear a slot twice before the issuer has waited for the first clear: reusing the slot needs the
+    // issuer's empty commit, which follows that wait.
+    constexpr int BAR_VC = BAR_E + NS;
     // per side: S full; P ready; O done, O free
-    constexpr int BAR_SF = BAR_VE + ST, BAR_PR = BAR_SF + 2, BAR_OD = BAR_PR + 2, BAR_OF = BAR_OD + 2;
-    // paged only, one per ring stage: the rows of the V tile in that stage past the last key have been cleared.
-    // Completed once per cleared tile; the issuer keeps the stage's phase bit.  The producer cannot
-    // clear a stage twice before the issuer has waited for the first clear: reusing the stage needs the
-    // issuer's V-empty commit, which follows that wait.
-    constexpr int BAR_VC = BAR_OF + 2;
-    // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), final
-    constexpr int BAR_WF = BAR_VC + ST, BAR_WE = BAR_WF + 2, BAR_NB = BAR_WE + 2, BAR_MG = BAR_NB + 1, BAR_FIN = BAR_MG + 4;
+    constexpr int BAR_SF = BAR_VC + NS, BAR_PR = BAR_SF + 2, BAR_OD = BAR_PR + 2, BAR_OF = BAR_OD + 2;
+    // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), staging free
+    // for the ring of a packed item, final
+    constexpr int BAR_WF = BAR_OF + 2, BAR_WE = BAR_WF + 2, BAR_NB = BAR_WE + 2, BAR_MG = BAR_NB + 1, BAR_SG = BAR_MG + 4;
+    constexpr int BAR_FIN = BAR_SG + 1;
     static_assert(BAR_FIN + 1 == L::kNumBars, "barrier count");
     const uint32_t s_answer = smem_base + L::kOffMisc;  // 16 bytes
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc + 16);
@@ -438,7 +458,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             uint32_t count = 1u;
             if ((i >= BAR_PR && i < BAR_OD) || i == BAR_OF || i == BAR_OF + 1) count = 4u;  // a lane of each softmax warp of the side
             if (i == BAR_WE || i == BAR_WE + 1) count = 10u;   // producer, issuer, eight softmax warps
-            if (i >= BAR_MG && i < BAR_MG + 4) count = 2u;     // a lane of each side's warp
+            if (i == BAR_SG) count = 8u;                       // a lane of each softmax warp
             mbar_init(bar(i), count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -624,10 +644,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         // =========================================================================== TMA producer
         // The whole warp walks the items and waits; one elected lane starts the copies.
         const bool el = elect_one();
-        int s = 0;           // ring stage
-        uint32_t ph = 0;     // its phase
-        int g = 0;           // K/V tiles issued so far
-        bool v_now = false;  // the V copy of the tile in hand has been issued (for the exit path)
+        uint32_t phases = 0;             // bit: parity of the slot's next use
+        int sk = 0, sv = 0, sx = 0;      // next stage of the K and V rings, next slot of a packed item's ring
+        uint32_t packed_items = 0;
         bool ok = true;
         int items = 0;
         for (int it = 0; ok; ++it) {
@@ -639,7 +658,8 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
             const int len_k = uniform(w.k_off + w.seq_len), hk = uniform(w.hk), k_start = uniform(w.k_start);
             // Q tiles of both sides (the previous item's last Q K^T must have retired); packed: one tile serves both
-            ok = warp_wait(bar(BAR_QE), ((uint32_t)items & 1u) ^ 1u, abort_flag);
+            auto slot_free = [&](int slot) -> bool { return warp_wait(bar(BAR_E + slot), ((phases >> slot) & 1u) ^ 1u, abort_flag); };
+            ok = warp_wait(bar(BAR_QE), ((uint32_t)items & 1u) ^ 1u, abort_flag) && (!kDeepRing || packed || slot_free(0));
             if (!ok) break;
             if (el) {
                 const int hA = w.hA, tq = w.seq_start + w.q0;
@@ -659,28 +679,30 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 }
             }
             ++items;
-            for (int n = 0; n < nt; ++n, ++g) {
+            // page of a key, out of range (the copy delivers zeros) when the table is wrong
+            auto page_of = [&](int key) -> int {
+                const int page = __ldg(p.block_table + (size_t)k_start * p.max_blocks + key / p.page_size);
+                if (page >= 0 && page < p.num_pages) return page;
+                record_device_error(SWAA_ERR_BAD_SEQLENS);
+                return p.num_pages;
+            };
+            // K or V tile n into a slot.  A tile of band keys comes in one box per panel, one that joins sink keys in pieces of
+            // 16 keys.
+            auto load_tile = [&](int n, int slot, const CUtensorMap* map, const CUtensorMap* map_small,
+                                 const CUtensorMap* map_sink) -> bool {
                 const bool remote = kCp && n < n_rem;
                 const Tile t(w, n);
-                const uint32_t dK = sK + (uint32_t)(s * L::kTileBytes), dV = sV + (uint32_t)(s * L::kTileBytes);
-                // A tile of band keys comes in one box per panel, one that joins sink keys in pieces of 16 keys.
                 const bool whole = remote || !t.joins_sinks();
-                const uint32_t bytes = whole ? (uint32_t)L::kTileBytes : (uint32_t)(t.nk * 16 * 128 * L::kPanels);
-                // page of a key, out of range (the copy delivers zeros) when the table is wrong
-                auto page_of = [&](int key) -> int {
-                    const int page = __ldg(p.block_table + (size_t)k_start * p.max_blocks + key / p.page_size);
-                    if (page >= 0 && page < p.num_pages) return page;
-                    record_device_error(SWAA_ERR_BAD_SEQLENS);
-                    return p.num_pages;
-                };
-                int page0 = 0, row0 = 0;  // of the first key, looked up ahead of the wait for the stage
+                const uint32_t dst = sSlots + (uint32_t)(slot * L::kTileBytes), full_bar = bar(BAR_F + slot);
+                int page0 = 0, row0 = 0;  // of the first key, looked up ahead of the wait for the slot
                 if (kPaged) {
                     const int key = t.key(0);
                     page0 = page_of(key);
                     row0 = key % p.page_size;
                 }
-                auto load_tile = [&](const CUtensorMap* map, const CUtensorMap* map_small, const CUtensorMap* map_sink, uint32_t dst,
-                                     uint32_t full_bar) {
+                if (!slot_free(slot)) return false;
+                if (el) {
+                    mbar_arrive_expect_tx(full_bar, whole ? (uint32_t)L::kTileBytes : (uint32_t)(t.nk * 16 * 128 * L::kPanels));
                     if (whole) {
 #pragma unroll
                         for (int pn = 0; pn < L::kPanels; ++pn) {
@@ -701,48 +723,71 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                             }
                         }
                     }
-                };
-                ok = warp_wait(bar(BAR_KE + s), ph ^ 1u, abort_flag);
-                if (!ok) break;
-                if (el) {
-                    mbar_arrive_expect_tx(bar(BAR_KF + s), bytes);
-                    load_tile(&tm.k, &tm.k_small, &tm.sink_k, dK, bar(BAR_KF + s));
                 }
-                if (!kLseOnly) {
-                    ok = warp_wait(bar(BAR_VE + s), ph ^ 1u, abort_flag);
-                    if (!ok) {
-                        warp_wait(bar(BAR_KF + s), ph, abort_flag);  // the K copy just issued
-                        break;
-                    }
-                    if (el) {
-                        mbar_arrive_expect_tx(bar(BAR_VF + s), bytes);
-                        load_tile(&tm.v, &tm.v_small, &tm.sink_v, dV, bar(BAR_VF + s));
-                    }
-                    v_now = true;
-                    if (kPaged) {
-                        // The rows of a page past the sequence's last key may hold anything (also NaN, and 0 * NaN is
-                        // NaN in the PV product): clear those that the P V product reads before the issuer may use the
-                        // tile.  Only the last band tile of a sequence that does not end on a 16-key boundary is concerned.
-                        const int r0 = t.bad0(len_k), r1 = t.bad1();
-                        if (r0 < r1) {
-                            ok = warp_wait(bar(BAR_VF + s), ph, abort_flag);
-                            if (!ok) break;
-                            for (int c = lane; c < (r1 - r0) * 8; c += 32)
+                phases ^= 1u << slot;
+                return true;
+            };
+            auto load_k = [&](int n, int slot) -> bool { return load_tile(n, slot, &tm.k, &tm.k_small, &tm.sink_k); };
+            auto load_v = [&](int n, int slot) -> bool {
+                if (kLseOnly) return true;
+                if (!load_tile(n, slot, &tm.v, &tm.v_small, &tm.sink_v)) return false;
+                if (kPaged) {
+                    // The rows of a page past the sequence's last key may hold anything (also NaN, and 0 * NaN is
+                    // NaN in the PV product): clear those that the P V product reads before the issuer may use the
+                    // tile.  Only the last band tile of a sequence that does not end on a 16-key boundary is concerned.
+                    const Tile t(w, n);
+                    const int r0 = t.bad0(len_k), r1 = t.bad1();
+                    if (r0 < r1) {
+                        if (!warp_wait(bar(BAR_F + slot), ((phases >> slot) & 1u) ^ 1u, abort_flag)) return false;
+                        const uint32_t dV = sSlots + (uint32_t)(slot * L::kTileBytes);
+                        for (int c = lane; c < (r1 - r0) * 8; c += 32)
 #pragma unroll
-                                for (int pn = 0; pn < L::kPanels; ++pn)
-                                    st_shared_v4(dV + pn * L::kPanelBytes + (r0 + (c >> 3)) * 128 + (c & 7) * 16, 0u, 0u, 0u, 0u);
-                            fence_proxy_async_smem();
-                            __syncwarp();
-                            if (el) mbar_arrive(bar(BAR_VC + s));
-                        }
+                            for (int pn = 0; pn < L::kPanels; ++pn)
+                                st_shared_v4(dV + pn * L::kPanelBytes + (r0 + (c >> 3)) * 128 + (c & 7) * 16, 0u, 0u, 0u, 0u);
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (el) mbar_arrive(bar(BAR_VC + slot));
                     }
                 }
-                v_now = false;
-                if (++s == ST) {
-                    s = 0;
-                    ph ^= 1u;
+                return true;
+            };
+            if (!(kDeepRing && packed)) {
+                for (int n = 0; n < nt && ok; ++n) {
+                    ok = load_k(n, L::kSlotK + sk);
+                    sk = sk + 1 == ST ? 0 : sk + 1;
+                    ok = ok && load_v(n, L::kSlotV + sv);
+                    sv = sv + 1 == ST ? 0 : sv + 1;
                 }
+            } else {
+                // One ring over all slots, in the order in which the issuer uses the tiles: K(0) K(1) V(0) K(2) V(1) K(3) ...
+                // A generated token at a long context runs at the pace of memory, and how far the copies run ahead sets it: with
+                // the two K and two V slots of the usual items one token at 32768 keys takes 421 us, 16 of them 499 us, a
+                // serving step of 4 chunks and 24 generated tokens 805 us; with all six slots 363, 430 and 595 us.
+                bool staging = false;  // the output staging is known to be free
+                auto wait_staging = [&]() {  // once per packed item, so that the barrier is never two phases ahead
+                    if (!staging) ok = ok && warp_wait(bar(BAR_SG), packed_items & 1u, abort_flag);
+                    staging = true;
+                };
+                auto next_slot = [&]() -> int {
+                    const int slot = sx;
+                    sx = sx + 1 == NS ? 0 : sx + 1;
+                    if (slot >= L::kSlotStage) wait_staging();
+                    return slot;
+                };
+                for (int n = -2; n < nt && ok; ++n) {
+                    if (n >= 0) {
+                        const int slot = next_slot();
+                        ok = ok && load_v(n, slot);
+                    }
+                    if (ok && n + 2 < nt) {
+                        const int slot = next_slot();
+                        ok = ok && load_k(n + 2, slot);
+                    }
+                }
+                wait_staging();
+                ++packed_items;
             }
+            if (!ok) break;
             release_work(it);
         }
         if (!ok) {
@@ -751,12 +796,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             bool landed = false;
             while (!landed && global_timer_ns() - t0 < kWaitLimitNs) {
                 landed = items == 0 || mbar_try_wait(bar(BAR_QF), (uint32_t)(items - 1) & 1u);
-                for (int n = max(0, g - ST + 1); n < g; ++n) {
-                    landed = landed && mbar_try_wait(bar(BAR_KF + n % ST), (uint32_t)(n / ST) & 1u);
-                    landed = landed && (kLseOnly || mbar_try_wait(bar(BAR_VF + n % ST), (uint32_t)(n / ST) & 1u));
-                }
-                // the tile that was being issued when the wait ran out
-                if (v_now) landed = landed && mbar_try_wait(bar(BAR_VF + s), ph) && mbar_try_wait(bar(BAR_KF + s), ph);
+                for (int slot = 0; slot < NS; ++slot) landed = landed && mbar_try_wait(bar(BAR_F + slot), ((phases >> slot) & 1u) ^ 1u);
             }
         }
         __syncwarp();
@@ -768,13 +808,13 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         // and one shared high word (stride 1024 B, descriptor version, 128-byte swizzle).
         const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0, 0, 1024) >> 32);
         const uint32_t q_lo = (uint32_t)smem_desc_sw128(sQ, 16, 1024);
-        const uint32_t k_lo = (uint32_t)smem_desc_sw128(sK, 16, 1024);
-        const uint32_t v_lo = (uint32_t)smem_desc_sw128(sV, L::kPanelBytes, 1024);
+        const uint32_t k_lo = (uint32_t)smem_desc_sw128(sSlots, 16, 1024);
+        const uint32_t v_lo = (uint32_t)smem_desc_sw128(sSlots, L::kPanelBytes, 1024);
         constexpr uint32_t kStep = (uint32_t)L::kTileBytes >> 4;
         constexpr uint32_t kIdescQK = make_idesc(BM, BN, 0), kIdescPV = make_idesc(BM, D, 1);
         // Q K^T of a side over the first 16 * nk keys of a tile; q_tile: 0, or the side
-        auto issue_qk = [&](int side, int q_tile, int stage, int nk) {
-            const uint32_t qa = q_lo + (uint32_t)q_tile * kStep, kb = k_lo + (uint32_t)stage * kStep;
+        auto issue_qk = [&](int side, int q_tile, int slot, int nk) {
+            const uint32_t qa = q_lo + (uint32_t)q_tile * kStep, kb = k_lo + (uint32_t)slot * kStep;
             const uint32_t idesc = nk == NK ? kIdescQK : (make_idesc(BM, 0, 0) | ((uint32_t)(2 * nk) << 17));
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
@@ -782,8 +822,8 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 mma_ss_lh(tmem_base + 128u * (uint32_t)side, qa + off, kb + off, desc_hi, idesc, kk > 0 ? 1u : 0u);
             }
         };
-        auto issue_pv = [&](int side, int stage, bool acc, int nk) {
-            const uint32_t vb = v_lo + (uint32_t)stage * kStep, a = tmem_base + 128u * (uint32_t)side;
+        auto issue_pv = [&](int side, int slot, bool acc, int nk) {
+            const uint32_t vb = v_lo + (uint32_t)slot * kStep, a = tmem_base + 128u * (uint32_t)side;
             const uint32_t d = tmem_base + 256u + (uint32_t)(D * side);
 #pragma unroll
             for (int kk = 0; kk < NK; ++kk) {
@@ -792,105 +832,129 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     mma_ts_lh(d, a + (uint32_t)kk * 8u, vb + (((uint32_t)kk * 2048u) >> 4), desc_hi, kIdescPV, (acc || kk > 0) ? 1u : 0u);
             }
         };
-        int sk = 0, sv = 0;            // ring stages of the next K and V tile
-        uint32_t pk = 0, pv = 0;       // their phases
+        uint32_t phases = 0;           // bit: parity of the slot's next use
+        int sk = 0, sv = 0, sx = 0;    // next stage of the K and V rings, next slot of a packed item's ring
         int gs[2] = {0, 0};            // tiles processed per side (phase of P ready)
         int items_side[2] = {0, 0};    // items each side took part in (phase of O free)
         int items = 0;
-        uint32_t vc_phase = 0;         // paged only: bit s = phase of the stage's V-tile-cleared barrier
+        uint32_t vc_phase = 0;         // paged only: bit: phase of the slot's V-tile-cleared barrier
         bool ok = true;
-        auto next_k = [&]() {
-            if (++sk == ST) {
-                sk = 0;
-                pk ^= 1u;
-            }
+        auto slot_full = [&](int slot) -> bool {
+            const uint32_t parity = (phases >> slot) & 1u;
+            phases ^= 1u << slot;
+            return warp_wait(bar(BAR_F + slot), parity, abort_flag);
         };
         for (int it = 0; ok; ++it) {
             ok = wait_work(it);
             if (!ok) break;
             const volatile WorkItem& w = work_slots[it & 1];
             if (!uniform(w.valid)) break;
-            const bool packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
+            const bool is_packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
             const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
-            const int len_k = kPaged ? uniform(w.k_off + w.seq_len) : 0;
-            const bool shared = packed && nt > 1;
-            auto steps_of = [&](int n) -> int { return (kCp && n < n_rem) ? NK : Tile(w, n).nk; };
-            const int ahead = packed ? 2 : 1;  // Q K^T runs this many tiles ahead of P V
-            ok = warp_wait(bar(BAR_QF), (uint32_t)items & 1u, abort_flag);
-            // the first scores of each side
-            for (int n = 0; n < min(ahead, nt) && ok; ++n) {
-                const int nk = steps_of(n);
-                ok = warp_wait(bar(BAR_KF + sk), pk, abort_flag);
-                if (!ok) break;
-                tc_fence_after();
-                if (el) {
-                    issue_qk(n, 0, sk, nk);
-                    tc_commit(bar(BAR_SF + n));
-                    if (hasB) {
-                        issue_qk(1, 1, sk, nk);
-                        tc_commit(bar(BAR_SF + 1));
-                    }
-                    tc_commit(bar(BAR_KE + sk));
-                    if (n == nt - 1) tc_commit(bar(BAR_QE));  // Q is no longer needed by this item
-                }
-                next_k();
-            }
-            for (int n = 0; n < nt && ok; ++n) {
+            // Only the last tile can be narrow, and only the last band tile can have rows past the last key: the loop below reads
+            // nothing of the descriptor.
+            const int nk_last = uniform((kCp && n_rem == nt) ? NK : Tile(w, nt - 1).nk);
+            int vc_tile = -1;
+            if (kPaged) {
+                const int n = n_rem + (w.nb16 - 1) / BN;
                 const Tile t(w, n);
-                const int nk = (kCp && n < n_rem) ? NK : t.nk;
-                const bool has_next = n + ahead < nt;
-                const int nk_next = has_next ? steps_of(n + ahead) : 0;
-                // The tiles first (they landed long ago as a rule), then the side's P: what follows the P barrier is on
-                // the side's critical path softmax -> P V -> Q K^T -> softmax.
-                if (!kLseOnly) ok = warp_wait(bar(BAR_VF + sv), pv, abort_flag);
-                if (kPaged && ok && t.bad0(len_k) < t.bad1()) {  // rows past the last key, cleared by the producer
-                    ok = warp_wait(bar(BAR_VC + sv), (vc_phase >> sv) & 1u, abort_flag);
-                    vc_phase ^= 1u << sv;
-                }
-                if (has_next && !packed) ok = ok && warp_wait(bar(BAR_KF + sk), pk, abort_flag);
-                if (!ok) break;
-#pragma unroll
-                for (int side = 0; side < 2; ++side) {
-                    if (packed ? (n & 1) != side : (side == 1 && !hasB)) continue;
-                    const bool first = n < ahead;  // the side's first tile of this item
-                    ok = ok && warp_wait(bar(BAR_PR + side), (uint32_t)gs[side] & 1u, abort_flag);
-                    // the first P V of an item overwrites O: the previous item's epilogue must have read it
-                    if (!kLseOnly && first) ok = ok && warp_wait(bar(BAR_OF + side), ((uint32_t)items_side[side] & 1u) ^ 1u, abort_flag);
+                vc_tile = uniform(t.bad0(w.k_off + w.seq_len) < t.bad1() ? n : -1);
+            }
+            const bool shared = is_packed && nt > 1;
+            ok = warp_wait(bar(BAR_QF), (uint32_t)items & 1u, abort_flag);
+            auto run_item = [&](auto packed_tag) {
+                const bool packed = decltype(packed_tag)::known ? decltype(packed_tag)::value : is_packed;
+                const bool late_k = kDeepRing && packed;
+                auto steps_of = [&](int n) -> int { return n == nt - 1 ? nk_last : NK; };
+                const int ahead = packed ? 2 : 1;  // Q K^T runs this many tiles ahead of P V
+                auto k_slot = [&]() -> int {
+                    int slot;
+                    if (late_k) {
+                        slot = sx;
+                        sx = sx + 1 == NS ? 0 : sx + 1;
+                    } else {
+                        slot = L::kSlotK + sk;
+                        sk = sk + 1 == ST ? 0 : sk + 1;
+                    }
+                    return slot;
+                };
+                auto v_slot = [&]() -> int {
+                    if (late_k) return k_slot();
+                    const int slot = L::kSlotV + sv;
+                    sv = sv + 1 == ST ? 0 : sv + 1;
+                    return slot;
+                };
+                // the first scores of each side
+                for (int n = 0; n < min(ahead, nt) && ok; ++n) {
+                    const int nk = steps_of(n), ks = k_slot();
+                    ok = slot_full(ks);
                     if (!ok) break;
                     tc_fence_after();
-                    if (!kLseOnly && el) issue_pv(side, sv, !first, nk);
-                    if (has_next && packed) {  // packed items run at the pace of memory: ask for their K tile late
-                        ok = warp_wait(bar(BAR_KF + sk), pk, abort_flag);
+                    if (el) {
+                        issue_qk(n, 0, ks, nk);
+                        tc_commit(bar(BAR_SF + n));
+                        if (hasB) {
+                            issue_qk(1, 1, ks, nk);
+                            tc_commit(bar(BAR_SF + 1));
+                        }
+                        tc_commit(bar(BAR_E + ks));
+                        if (n == nt - 1) tc_commit(bar(BAR_QE));  // Q is no longer needed by this item
+                    }
+                }
+                for (int n = 0; n < nt && ok; ++n) {
+                    const int nk = steps_of(n);
+                    const bool has_next = n + ahead < nt;
+                    const int nk_next = has_next ? steps_of(n + ahead) : 0;
+                    const int vs = kLseOnly ? 0 : v_slot(), ks = has_next ? k_slot() : 0;
+                    // The tiles first (they landed long ago as a rule), then the side's P: what follows the P barrier is on
+                    // the side's critical path softmax -> P V -> Q K^T -> softmax.
+                    if (!kLseOnly) ok = slot_full(vs);
+                    if (kPaged && ok && n == vc_tile) {  // rows past the last key, cleared by the producer
+                        ok = warp_wait(bar(BAR_VC + vs), (vc_phase >> vs) & 1u, abort_flag);
+                        vc_phase ^= 1u << vs;
+                    }
+                    if (has_next && !late_k) ok = ok && slot_full(ks);
+                    if (!ok) break;
+#pragma unroll
+                    for (int side = 0; side < 2; ++side) {
+                        if (packed ? (n & 1) != side : (side == 1 && !hasB)) continue;
+                        const bool first = n < ahead;  // the side's first tile of this item
+                        ok = ok && warp_wait(bar(BAR_PR + side), (uint32_t)gs[side] & 1u, abort_flag);
+                        // the first P V of an item overwrites O: the previous item's epilogue must have read it
+                        if (!kLseOnly && first) ok = ok && warp_wait(bar(BAR_OF + side), ((uint32_t)items_side[side] & 1u) ^ 1u, abort_flag);
                         if (!ok) break;
                         tc_fence_after();
+                        if (!kLseOnly && el) issue_pv(side, vs, !first, nk);
+                        if (has_next && late_k) {  // packed items run at the pace of memory: free the V tile early, ask for K late
+                            if (el) tc_commit(bar(BAR_E + vs));
+                            ok = slot_full(ks);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        if (el) {
+                            // O done is only waited for by the item's epilogue: between tiles S full of the side's next tile
+                            // already implies the P V before it (a commit covers every product issued before it)
+                            if (!kLseOnly && !has_next) tc_commit(bar(BAR_OD + side));
+                            if (has_next) {
+                                issue_qk(side, packed ? 0 : side, ks, nk_next);
+                                tc_commit(bar(BAR_SF + side));
+                            }
+                        }
+                        ++gs[side];
                     }
+                    if (!ok) break;
                     if (el) {
-                        // O done is only waited for by the item's epilogue: between tiles S full of the side's next tile
-                        // already implies the P V before it (a commit covers every product issued before it)
-                        if (!kLseOnly && !has_next) tc_commit(bar(BAR_OD + side));
+                        if (!kLseOnly && !(has_next && late_k)) tc_commit(bar(BAR_E + vs));
                         if (has_next) {
-                            issue_qk(side, packed ? 0 : side, sk, nk_next);
-                            tc_commit(bar(BAR_SF + side));
+                            tc_commit(bar(BAR_E + ks));
+                            if (n + ahead == nt - 1) tc_commit(bar(BAR_QE));
                         }
                     }
-                    ++gs[side];
                 }
-                if (!ok) break;
-                if (!kLseOnly) {
-                    if (el) tc_commit(bar(BAR_VE + sv));
-                    if (++sv == ST) {
-                        sv = 0;
-                        pv ^= 1u;
-                    }
-                }
-                if (has_next) {
-                    if (el) {
-                        tc_commit(bar(BAR_KE + sk));
-                        if (n + ahead == nt - 1) tc_commit(bar(BAR_QE));
-                    }
-                    next_k();
-                }
-            }
+            };
+            if (!kDeepRing) run_item(RuntimeFlag{});
+            else if (is_packed) run_item(ConstFlag<true>{});
+            else run_item(ConstFlag<false>{});
             ++items;
             ++items_side[0];
             if (hasB || shared) ++items_side[1];
@@ -910,9 +974,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const uint32_t tS = tmem_base + lane_base + (uint32_t)side * 128u;
         const uint32_t tO = tmem_base + lane_base + 256u + (uint32_t)side * (uint32_t)D;
-        // phases (bits) of: S full, O done, hand-over of packed items
+        // phases (bits) of: S full, O done (side A also keeps side B's), hand-over of packed items
         uint32_t phases = 0;
-        constexpr uint32_t kPhS = 1u, kPhO = 2u, kPhM = 4u;
+        constexpr uint32_t kPhS = 1u, kPhO = 2u, kPhOB = 4u, kPhM = 8u;
         bool ok = true;
         auto arrive_warp = [&](int b) {
             __syncwarp();
@@ -927,6 +991,10 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             if (!uniform(w.valid)) break;
             const bool packed = !kLseOnly && uniform(w.packed) != 0;
             const bool shared = packed && uniform(w.shared) != 0;
+            if (kDeepRing && packed && lane == 0) {  // the item's ring takes the staging area: earlier output stores have read it
+                tma_store_wait_read();
+                mbar_arrive(bar(BAR_SG));
+            }
             if (side == 1 && !shared && !uniform(w.hasB)) {
                 release_work(it);
                 continue;
@@ -1087,6 +1155,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             const int q_row = packed ? row / p.G : w.q0 + row;  // this thread's query, counted inside the sequence
             const int token = w.seq_start + q_row, tok0 = w.seq_start + w.q0;
             const int h = packed ? w.hA + row - q_row * p.G : w.hA + side;
+            const bool sideB = shared || uniform(w.hasB) != 0;
             release_work(it);
             __nv_bfloat16* orow = p.out + ((size_t)token * p.Hq + h) * D;
             // eight channels of this thread's row
@@ -1100,71 +1169,54 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 tc_fence_before();
                 arrive_warp(BAR_OF + side);
             };
+            const uint32_t od_b = (phases & kPhOB) != 0 ? 1u : 0u;  // side A: parity of side B's O done in this item
+            if (sideB) phases ^= kPhOB;
             if (idle) {
-                if (!kLseOnly) o_free();
+                if (!kLseOnly && !(shared && side == 1)) {
+                    o_free();
+                    if (shared && lane == 0) mbar_arrive(bar(BAR_OF + 1));
+                }
                 continue;
             }
             if (shared) {
-                // Side B hands its rows' (max, sum, O) to the warp of side A with the same rows, through the staging areas
-                // of the two warps: 32 rows x 64 channels of fp32 at a time, 16-byte chunks swizzled by row.
-                const uint32_t mine = sStage + (uint32_t)wq * 4096u +
-                                      (lane < 16 ? (uint32_t)lane * 256u : 16384u + (uint32_t)(lane - 16) * 256u);
-                if (lane == 0) tma_store_wait_read();  // earlier output stores have read the staging areas
-                if (side == 1) s_merge[row] = make_float2(m_used, l_sum);
-                float wa = 1.f, wb = 0.f, inv = 0.f;
-                auto pair_sync = [&]() -> bool {  // the two warps of these rows
+                if (side == 1) {
+                    // Side A's warp of the same rows reads both accumulators; it only lacks (max, sum).  (O done above implies
+                    // that the previous hand-over has been read.)
+                    s_merge[row] = make_float2(m_used, l_sum);
                     arrive_warp(BAR_MG + wq);
-                    phases ^= kPhM;
-                    return warp_wait(bar(BAR_MG + wq), (phases & kPhM) != 0 ? 0u : 1u, abort_flag);
-                };
-#pragma unroll
-                for (int half = 0; half < D / 64 && ok; ++half) {
-                    uint32_t o[64];
-                    tmem_ld32(tO + (uint32_t)(half * 64), o);
-                    tmem_ld32(tO + (uint32_t)(half * 64 + 32), o + 32);
-                    tc_wait_ld();
-                    if (half == D / 64 - 1) o_free();
-                    ok = pair_sync();  // the area is free
-                    if (ok && side == 1) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            st_shared_v4(mine + (uint32_t)((j ^ (lane & 15)) * 16), o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-                    }
-                    ok = ok && pair_sync();  // the area is filled
-                    if (ok && side == 0) {
-                        if (half == 0) {
-                            const float2 other = s_merge[row];
-                            const float M = fmaxf(m_used, other.x);
-                            wa = m_used == -INFINITY ? 0.f : ex2f((m_used - M) * p.sl2);
-                            wb = other.x == -INFINITY ? 0.f : ex2f((other.x - M) * p.sl2);
-                            l_sum = wa * l_sum + wb * other.y;
-                            m_used = M;
-                            inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            uint32_t b4[4];
-                            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                         : "=r"(b4[0]), "=r"(b4[1]), "=r"(b4[2]), "=r"(b4[3])
-                                         : "r"(mine + (uint32_t)((j ^ (lane & 15)) * 16))
-                                         : "memory");
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                // a side without any visible key of the row has no usable O
-                                const float x = wa > 0.f ? __uint_as_float(o[4 * j + e]) * wa : 0.f;
-                                const float y = wb > 0.f ? __uint_as_float(b4[e]) * wb : 0.f;
-                                o[4 * j + e] = __float_as_uint(x + y);
-                            }
-                        }
-                        if (row_ok)
-#pragma unroll
-                            for (int v = 0; v < 8; ++v) *reinterpret_cast<uint4*>(orow + half * 64 + v * 8) = pack8(o + v * 8, inv);
-                    }
+                    continue;
                 }
-                // side A has read the last half before side B's next output uses the area
-                ok = ok && pair_sync();
+                ok = warp_wait(bar(BAR_OD + 1), od_b, abort_flag) &&
+                     warp_wait(bar(BAR_MG + wq), (phases & kPhM) != 0 ? 1u : 0u, abort_flag);
                 if (!ok) break;
-                if (side == 1) continue;
+                phases ^= kPhM;
+                tc_fence_after();
+                const float2 other = s_merge[row];
+                const float M = fmaxf(m_used, other.x);
+                const float wa = m_used == -INFINITY ? 0.f : ex2f((m_used - M) * p.sl2);
+                const float wb = other.x == -INFINITY ? 0.f : ex2f((other.x - M) * p.sl2);
+                l_sum = wa * l_sum + wb * other.y;
+                m_used = M;
+                const float inv = l_sum > 0.f ? 1.f / l_sum : 0.f;
+#pragma unroll 1
+                for (int cc = 0; cc < D / 32; ++cc) {
+                    uint32_t o[32], ob[32];
+                    tmem_ld32(tO + (uint32_t)(cc * 32), o);
+                    tmem_ld32(tO + (uint32_t)(D + cc * 32), ob);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        // a side without any visible key of the row has no usable O
+                        const float x = wa > 0.f ? __uint_as_float(o[e]) * wa : 0.f;
+                        const float y = wb > 0.f ? __uint_as_float(ob[e]) * wb : 0.f;
+                        o[e] = __float_as_uint(x + y);
+                    }
+                    if (row_ok)
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) *reinterpret_cast<uint4*>(orow + cc * 32 + v * 8) = pack8(o + v * 8, inv);
+                }
+                o_free();
+                if (lane == 0) mbar_arrive(bar(BAR_OF + 1));
             } else if (!kLseOnly) {
                 uint32_t orr[D];
 #pragma unroll
