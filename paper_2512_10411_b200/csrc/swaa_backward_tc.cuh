@@ -16,18 +16,23 @@
 // whole block; dQ goes through shared memory (as [rows][D], in the ring stage of the step's Q and dO
 // tiles, which are dead by then) and is added to an fp32 accumulator in global memory by bulk reduce-add copies
 // (per-lane atomics saturate the L2 atomic units and stall the block's
-// other shared-memory traffic behind them).  Two groups of four warps take alternate steps, each with its own S^T/dP^T columns, so the
-// element-wise work of one step overlaps the products of the other.
+// other shared-memory traffic behind them).  Groups of four warps take the steps in turn, each with its own S^T/dP^T
+// columns, so the element-wise work of one step overlaps the products of the others: two groups at D = 128, three at
+// D = 64, where dV and dK leave the columns for a third.
 //
-// Tensor memory (512 columns).  D = 128: dV [0,128) | dK [128,256) | X_0 [256,384) | X_1 [384,512).
-// D = 64: dV [0,64) | dK [64,128) | X_0 [128,256) | X_1 [256,384) | dQ_0 [384,448) | dQ_1 [448,512).  X_g holds
-// S^T [0,64) and dP^T [64,128) of the group's step, then P^T (bf16 pairs, [0,32)) and dS^T ([64,96)); at D = 128
-// then dQ^T [0,64).  The tensor core runs the products of one issuing thread in order, which is what
-// makes these overlays safe.  At D = 64 dQ has columns of its own (64 rows = 16 lanes of every quadrant), so the products
-// that feed a group's next step are issued before it and never wait for its read-out.
+// Tensor memory (512 columns): dV [0,D) | dK [D,2D) | X_0 | X_1 (| X_2), 128 columns each; X_g holds
+// S^T [0,64) and dP^T [64,128) of the group's step, then P^T (bf16 pairs, [0,32)) and dS^T ([64,96)),
+// then dQ^T, or dQ (64 rows = 16 lanes of every quadrant), [0,64).  The tensor core runs the products of one issuing
+// thread in order, which is what makes these overlays safe.
 //
-// Warps 0-7: the two element-wise groups; warp 8: TMA producer (K, V once; Q, dO and the row terms per
-// step through a ring of four stages); warp 9: MMA issuer.  Every wait is bounded.
+// What bounds it.  A group's step is a chain S^T, dP^T -> element-wise part -> dV, dK, dQ -> read-out -> S^T of its next
+// step, several times as long as the products of a step: the more steps in flight, the better.  Packed batch of
+// 16k tokens, Hq = 16, Hkv = 4, D = 64, window 1024, forward + backward: 540 us with two groups, 462 with three (1417 on
+// warp-level MMAs).  At D = 128 tensor memory holds no third group, and a long sample runs against the power cap (1.65 GHz):
+// 16k tokens, Hq = 32, Hkv = 8, window 2048: 2370 us.
+//
+// Warps: 4 per group; then the TMA producer (K, V once; Q, dO and the row terms per
+// step through a ring of stages); then the MMA issuer.  Every wait is bounded.
 #pragma once
 
 #include <type_traits>
@@ -39,12 +44,13 @@ namespace swaa {
 
 constexpr int kBwdTcKeys = 128;    // keys per block
 constexpr int kBwdTcRows = 64;     // query rows per step
-constexpr int kBwdTcThreads = 320;
-constexpr int kBwdTcStages = 4;    // ring of (Q, dO, row terms); a stage also stages the step's dQ on its way out
 
 template <int D>
 struct BackwardTcSmem {
     static constexpr int kPanels = D / 64;
+    static constexpr int kGroups = D == 128 ? 2 : 3;  // of four warps, each with a step of its own in flight
+    static constexpr int kThreads = (4 * kGroups + 2) * 32;
+    static constexpr int kStages = 2 * kGroups;       // ring of (Q, dO, row terms); a stage also stages the step's dQ on its way out
     static constexpr int kKVTileBytes = kBwdTcKeys * D * 2;    // panels of [128][64 ch]
     static constexpr int kKVPanelBytes = kBwdTcKeys * 128;
     static constexpr int kQTileBytes = kBwdTcRows * D * 2;     // panels of [64][64 ch]
@@ -53,10 +59,10 @@ struct BackwardTcSmem {
     static constexpr int kDSBytes = kBwdTcKeys * 128;          // dS^T [128 keys][64 rows] bf16
     static constexpr int kOffK = 0, kOffV = kKVTileBytes;
     static constexpr int kOffRing = 2 * kKVTileBytes;
-    static constexpr int kOffDS = kOffRing + kBwdTcStages * kStageBytes;  // two buffers (one per group)
-    static constexpr int kOffRows = kOffDS + 2 * kDSBytes;     // per stage: lse2[64], delta[64] (fp32)
-    static constexpr int kOffBar = kOffRows + kBwdTcStages * 128 * 4;
-    static constexpr int kNumBars = 1 + 2 * kBwdTcStages + 4 * 2 + 1;
+    static constexpr int kOffDS = kOffRing + kStages * kStageBytes;  // one buffer per group
+    static constexpr int kOffRows = kOffDS + kGroups * kDSBytes;     // per stage: lse2[64], delta[64] (fp32)
+    static constexpr int kOffBar = kOffRows + kStages * 128 * 4;
+    static constexpr int kNumBars = 1 + 2 * kStages + 4 * kGroups + 1;
     static constexpr int kOffMisc = kOffBar + kNumBars * 8;
     static constexpr int kBytes = kOffMisc + 32;
     static constexpr int kDynamicBytes = kBytes;  // the kernel declares the array 1024-byte aligned and checks it
@@ -80,12 +86,12 @@ __device__ __forceinline__ bool group_all(bool pred, int id) {
 }
 
 template <int D>
-__global__ void __launch_bounds__(kBwdTcThreads, 1)
+__global__ void __launch_bounds__(BackwardTcSmem<D>::kThreads, 1)
 backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do,
                    const __grid_constant__ CUtensorMap tm_dq, const BackwardParams p) {
     using L = BackwardTcSmem<D>;
-    constexpr int BK = kBwdTcKeys, BR = kBwdTcRows, NQ = kBwdTcStages;
+    constexpr int BK = kBwdTcKeys, BR = kBwdTcRows, NQ = L::kStages, NG = L::kGroups;
     constexpr uint32_t kIdS = make_idesc(BK, BR, 0);      // S^T, dP^T
     constexpr uint32_t kIdKV = make_idesc(BK, D, 1);      // dV, dK (A from tensor memory)
     constexpr bool kWide = D == 128;
@@ -103,8 +109,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     float* s_rows = reinterpret_cast<float*>(smem_gen + L::kOffRows);
     const uint32_t bars = smem_base + L::kOffBar;
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
-    constexpr int BAR_KV = 0, BAR_QF = 1, BAR_QE = BAR_QF + NQ, BAR_SF = BAR_QE + NQ, BAR_PR = BAR_SF + 2;
-    constexpr int BAR_DQ = BAR_PR + 2, BAR_DR = BAR_DQ + 2, BAR_FIN = BAR_DR + 2;
+    constexpr int BAR_KV = 0, BAR_QF = 1, BAR_QE = BAR_QF + NQ, BAR_SF = BAR_QE + NQ, BAR_PR = BAR_SF + NG;
+    constexpr int BAR_DQ = BAR_PR + NG, BAR_DR = BAR_DQ + NG, BAR_FIN = BAR_DR + NG;
     static_assert(BAR_FIN + 1 == L::kNumBars, "barrier count");
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -147,12 +153,12 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         for (int i = 0; i < L::kNumBars; ++i) {
             uint32_t count = 1u;
             if (i >= BAR_QF && i < BAR_QF + NQ) count = 33u;  // the TMA transaction + the 32 lanes that write the row terms
-            if ((i >= BAR_PR && i < BAR_PR + 2) || (i >= BAR_DR && i < BAR_DR + 2)) count = 128u;
+            if ((i >= BAR_PR && i < BAR_PR + NG) || (i >= BAR_DR && i < BAR_DR + NG)) count = 128u;
             mbar_init(bar(i), count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 9) {
+    if (warp == 4 * NG + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(512u)
                      : "memory");
@@ -164,10 +170,10 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const uint32_t tDV = tmem_base, tDK = tmem_base + (uint32_t)D;
     constexpr uint32_t kX = 2u * (uint32_t)D;          // first column of X_0
-    constexpr uint32_t kDQ = kX + 256u;                // first column of dQ_0 (D = 64)
+    static_assert(2 * D + 128 * NG <= 512, "tensor memory columns");
     const float sl2 = p.scale * 1.4426950408889634f;
 
-    if (warp == 8) {
+    if (warp == 4 * NG) {
         // ================================================================================= producer
         bool ok = true;
         if (lane == 0) {
@@ -214,7 +220,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             }
         }
         __syncwarp();
-    } else if (warp == 9) {
+    } else if (warp == 4 * NG + 1) {
         // =================================================================================== issuer
         // The warp runs the loop as a whole, one elected lane issues: see elect_one.
         const bool el = elect_one();
@@ -227,9 +233,9 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const uint32_t ds_t0 = (uint32_t)smem_desc_sw128(sDS, 16, 1024);                 // dS^T of group 0, MN-major (B, or A at D = 64)
         constexpr uint32_t kStageStep = (uint32_t)L::kStageBytes >> 4, kDoStep = (uint32_t)L::kQTileBytes >> 4;
         constexpr uint32_t kDsStep = (uint32_t)L::kDSBytes >> 4;
-        // S^T = K Q^T (columns [0,64) of X_{s & 1}) and dP^T = V dO^T (columns [64,128)) of step s
-        auto issue_st = [&](int s) {
-            const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
+        // S^T = K Q^T (columns [0,64) of X_g) and dP^T = V dO^T (columns [64,128)) of the step in ring stage st
+        auto issue_st = [&](int g, int st) {
+            const uint32_t qb = q_b0 + (uint32_t)st * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)g;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
@@ -237,8 +243,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 mma_ss_lh(tX, k_a + oa, qb + ob, hi, kIdS, kk > 0 ? 1u : 0u);
             }
         };
-        auto issue_dp = [&](int s) {
-            const uint32_t qb = q_b0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
+        auto issue_dp = [&](int g, int st) {
+            const uint32_t qb = q_b0 + (uint32_t)st * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)g;
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t oa = ((uint32_t)(kk >> 2) * L::kKVPanelBytes + (uint32_t)(kk & 3) * 32u) >> 4;
@@ -246,20 +252,19 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 mma_ss_lh(tX + 64u, v_a + oa, qb + kDoStep + ob, hi, kIdS, kk > 0 ? 1u : 0u);
             }
         };
-        // dV += P^T dO, dK += dS^T Q of step s
-        auto issue_dkv = [&](int s) {
-            const uint32_t qt = q_t0 + (uint32_t)(s % NQ) * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)(s & 1);
+        // dV += P^T dO, dK += dS^T Q
+        auto issue_dkv = [&](int g, int st, bool acc) {
+            const uint32_t qt = q_t0 + (uint32_t)st * kStageStep, tX = tmem_base + kX + 128u * (uint32_t)g;
 #pragma unroll
             for (int kk = 0; kk < BR / 16; ++kk) {  // 16 rows: 8 columns of bf16 pairs, 16 rows of 128 bytes
                 const uint32_t ob = ((uint32_t)kk * 2048u) >> 4;
-                mma_ts_lh(tDV, tX + (uint32_t)kk * 8u, qt + kDoStep + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
-                mma_ts_lh(tDK, tX + 64u + (uint32_t)kk * 8u, qt + ob, hi, kIdKV, (s > 0 || kk > 0) ? 1u : 0u);
+                mma_ts_lh(tDV, tX + (uint32_t)kk * 8u, qt + kDoStep + ob, hi, kIdKV, (acc || kk > 0) ? 1u : 0u);
+                mma_ts_lh(tDK, tX + 64u + (uint32_t)kk * 8u, qt + ob, hi, kIdKV, (acc || kk > 0) ? 1u : 0u);
             }
         };
-        // dQ^T = K^T dS^T (D = 128, over S^T) or dQ = dS K (D = 64) of step s
-        auto issue_dq = [&](int s) {
-            const uint32_t g = (uint32_t)(s & 1), ds = ds_t0 + g * kDsStep;
-            const uint32_t d = tmem_base + (kWide ? kX + 128u * g : kDQ + 64u * g);
+        // dQ^T = K^T dS^T (D = 128) or dQ = dS K (D = 64), over S^T
+        auto issue_dq = [&](int g) {
+            const uint32_t ds = ds_t0 + (uint32_t)g * kDsStep, d = tmem_base + kX + 128u * (uint32_t)g;
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {  // 16 keys: 16 rows of 128 bytes in both operands
                 const uint32_t o = ((uint32_t)kk * 2048u) >> 4;
@@ -267,60 +272,51 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             }
         };
         bool ok = warp_wait(bar(BAR_KV), 0u, abort_flag);
-        for (int s = 0; s < 2 && s < n_steps && ok; ++s) {
-            ok = warp_wait(bar(BAR_QF + s % NQ), 0u, abort_flag);
+        for (int s = 0; s < NG && s < n_steps && ok; ++s) {
+            ok = warp_wait(bar(BAR_QF + s), 0u, abort_flag);
             if (!ok) break;
             tc_fence_after();
             if (el) {
-                issue_dp(s);
-                issue_st(s);
+                issue_dp(s, s);
+                issue_st(s, s);
                 tc_commit(bar(BAR_SF + s));
             }
         }
-        // Steady state: the gradients of step s as soon as the group has written P^T, dS^T; then (D = 64: before dQ) the
-        // products that feed the same group's step s + 2.  dP^T(s+2) only needs columns [64,128), free once dK(s) has run
-        // (products run in issue order); at D = 128 it fills the time until the group has taken dQ^T(s) out of the
-        // columns that S^T(s+2) overwrites.  (At D = 64 the columns of dQ(s - 2) were read out before the group's arrival
-        // with P^T of step s.)
+        // Steady state: the gradients of step s as soon as the group has written P^T, dS^T; then the products that feed the same
+        // group's next step, s + NG.  Its dP^T only needs columns [64,128), free once dK(s) has run
+        // (products run in issue order); it fills the time until the group has taken dQ(s) out of the columns that S^T
+        // overwrites.
+        int g = 0, st = 0, st2 = NG;           // group and ring stage of step s, ring stage of step s + NG
+        uint32_t ph = 0, ph2 = 0;              // phases of the group's barriers, and of stage st2
         for (int s = 0; s < n_steps && ok; ++s) {
-            const int g = s & 1;
-            const uint32_t ph = (uint32_t)(s >> 1) & 1u;
-            const bool more = s + 2 < n_steps;
             ok = warp_wait(bar(BAR_PR + g), ph, abort_flag);
             if (!ok) break;
             tc_fence_after();
-            if (el) issue_dkv(s);
-            if (kWide) {
+            if (el) {
+                issue_dkv(g, st, s > 0);
+                issue_dq(g);
+                tc_commit(bar(BAR_DQ + g));
+            }
+            if (s + NG < n_steps) {
+                ok = warp_wait(bar(BAR_QF + st2), ph2, abort_flag);
+                if (!ok) break;
+                if (el) issue_dp(g, st2);
+                ok = warp_wait(bar(BAR_DR + g), ph, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
                 if (el) {
-                    issue_dq(s);
-                    tc_commit(bar(BAR_DQ + g));
+                    issue_st(g, st2);
+                    tc_commit(bar(BAR_SF + g));
                 }
-                if (more) {
-                    ok = warp_wait(bar(BAR_QF + (s + 2) % NQ), (uint32_t)((s + 2) / NQ) & 1u, abort_flag);
-                    if (!ok) break;
-                    if (el) issue_dp(s + 2);
-                    ok = warp_wait(bar(BAR_DR + g), ph, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after();
-                    if (el) {
-                        issue_st(s + 2);
-                        tc_commit(bar(BAR_SF + g));
-                    }
-                }
-            } else {
-                if (more) {
-                    ok = warp_wait(bar(BAR_QF + (s + 2) % NQ), (uint32_t)((s + 2) / NQ) & 1u, abort_flag);
-                    if (!ok) break;
-                    if (el) {
-                        issue_st(s + 2);
-                        issue_dp(s + 2);
-                        tc_commit(bar(BAR_SF + g));
-                    }
-                }
-                if (el) {
-                    issue_dq(s);
-                    tc_commit(bar(BAR_DQ + g));
-                }
+            }
+            if (++g == NG) {
+                g = 0;
+                ph ^= 1u;
+            }
+            st = st + 1 == NQ ? 0 : st + 1;
+            if (++st2 == NQ) {
+                st2 = 0;
+                ph2 ^= 1u;
             }
         }
         // all products issued by this warp must have retired before the tensor memory is read or freed
@@ -392,18 +388,18 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                              dk[4 * q + 3]);
             }
         };
-        for (int s = grp; s < n_steps && ok; s += 2) {
-            const int st = s % NQ;
-            const uint32_t ph = (uint32_t)(s >> 1) & 1u;
+        int st = grp;                    // ring stage of step s and its phase; phase of the group's barriers
+        uint32_t st_ph = 0, ph = 0;
+        for (int s = grp; s < n_steps && ok; s += NG) {
             const int h = hk * p.G + s / nm, i0 = (m_lo + s % nm) * BR;
             const int i1 = min(i0 + BR, Lseq) - 1;
-            ok = group_all(mbar_wait(bar(BAR_QF + st), (uint32_t)(s / NQ) & 1u, abort_flag) &&
+            ok = group_all(mbar_wait(bar(BAR_QF + st), st_ph, abort_flag) &&
                                mbar_wait(bar(BAR_SF + grp), ph, abort_flag),
                            1 + grp);
             if (!ok) break;
             tc_fence_after();
             if (kl == 0 && pending_stage >= 0) {
-                // the reduce-add of this group's previous step has read its staging (issued two steps ago): hand
+                // the reduce-add of this group's previous step has read its staging (issued NG steps ago): hand
                 // the ring stage back to the producer
                 tma_store_wait_read();
                 mbar_arrive(bar(BAR_QE + pending_stage));
@@ -431,35 +427,28 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             if (!ok) break;
             tc_fence_after();
             const uint32_t stage = sRing + (uint32_t)st * L::kStageBytes;
+            uint32_t v0[32], v1[32];
+            tmem_ld32(tX, v0);
+            tmem_ld32(tX + 32u, v1);
+            tc_wait_ld();
+            // the group's columns may take the next S^T as soon as dQ is in registers
+            tc_fence_before();
+            mbar_arrive(bar(BAR_DR + grp));
             if (kWide) {  // dQ^T: lane = channel, column = row
                 const uint32_t stg = stage + (uint32_t)kl * 4u;
-                uint32_t v0[32], v1[32];
-                tmem_ld32(tX, v0);
-                tmem_ld32(tX + 32u, v1);
-                tc_wait_ld();
-                // the group's columns may take the next S^T as soon as dQ^T is in registers
-                tc_fence_before();
-                mbar_arrive(bar(BAR_DR + grp));
 #pragma unroll
                 for (int e = 0; e < 32; ++e) {
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + (uint32_t)(e * 512)), "r"(v0[e]) : "memory");
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + (uint32_t)((32 + e) * 512)), "r"(v1[e]) : "memory");
                 }
-            } else {  // dQ: row 16 * quad + lane in lanes 0..15 of the quadrant, column = channel; panels of 32 channels, swizzled
-                const uint32_t tQ = tmem_base + lane_bits + kDQ + 64u * (uint32_t)grp;
-                const int r = 16 * quad + (lane & 15);
+            } else if (lane < 16) {  // dQ: row 16 * quad + lane in lanes 0..15, column = channel; panels of 32 channels, swizzled
+                const int r = 16 * quad + lane;
 #pragma unroll
-                for (int pn = 0; pn < 2; ++pn) {
-                    uint32_t v[32];
-                    tmem_ld32(tQ + 32u * (uint32_t)pn, v);
-                    tc_wait_ld();
-                    if (lane < 16)
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            st_shared_v4(stage + (uint32_t)(pn * 8192 + r * 128 + ((j ^ (r & 7)) << 4)), v[4 * j], v[4 * j + 1],
-                                         v[4 * j + 2], v[4 * j + 3]);
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t a = stage + (uint32_t)(r * 128 + ((j ^ (r & 7)) << 4));
+                    st_shared_v4(a, v0[4 * j], v0[4 * j + 1], v0[4 * j + 2], v0[4 * j + 3]);
+                    st_shared_v4(a + 8192u, v1[4 * j], v1[4 * j + 1], v1[4 * j + 2], v1[4 * j + 3]);
                 }
-                tc_fence_before();
             }
             fence_proxy_async_smem();
             asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
@@ -469,11 +458,17 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 tma_store_commit();
                 pending_stage = st;
             }
+            ph ^= 1u;
+            st += NG;
+            if (st >= NQ) {
+                st -= NQ;
+                st_ph ^= 1u;
+            }
         }
         if (kl == 0) tma_store_wait_all();  // this group's reductions into dq have been performed
         // ---- dV (group 0) and dK (group 1) rows of this thread's key
         if (ok) ok = mbar_wait(bar(BAR_FIN), 0u, abort_flag);
-        if (ok) {
+        if (ok && grp < 2) {
             tc_fence_after();
             const uint32_t tAcc = tmem_base + lane_bits + (uint32_t)(D * grp);
             if (split) {
@@ -519,7 +514,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // ---- teardown: every thread arrives here (also after a failed wait); free the tensor memory
     tc_fence_before();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == 4 * NG + 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
     }

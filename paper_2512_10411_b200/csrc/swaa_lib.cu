@@ -737,7 +737,7 @@ static int launch_backward(const void* q, const void* k, const void* v, const vo
     using L = BackwardTcSmem<D>;
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(backward_tc_kernel<D>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
-    rc = launch_overlapped(backward_tc_kernel<D>, grid, kBwdTcThreads, L::kDynamicBytes, st, tq, tk, tv, tdo, tacc, p);
+    rc = launch_overlapped(backward_tc_kernel<D>, grid, L::kThreads, L::kDynamicBytes, st, tq, tk, tv, tdo, tacc, p);
     if (rc != SWAA_OK) return rc;
     rc = launch_overlapped(backward_convert_dq_kernel, dim3((unsigned)((n_acc / 4 + 255) / 256 + 1)), 256, 0, st, p.dq_accum,
                            static_cast<__nv_bfloat16*>(dq), n_acc);
