@@ -7,10 +7,12 @@
 // Work decomposition.  An item is one (sequence, key/value head, chunk of up to 8*NH query heads of
 // that head's group); all query heads of a chunk are processed together so each K/V byte is fetched
 // once.  The visible cache entries of an item are cut into tiles of 64 keys (sink tiles, then window
-// tiles starting at the first window key).  All tiles of all items form one list in (sequence, item,
-// tile) order, and block c of a persistent grid (at most one block per SM; the host prefers a block count that puts
-// the cuts on item boundaries, see plan_decode) owns the contiguous run
-// [c * tpc, (c+1) * tpc) of it, so every SM streams the same number of bytes whatever the batch
+// tiles starting at the first window key).  The rows of a cache interleave its kv heads (a 64-key tile of one head is 64
+// pieces of 2*D bytes, Hkv*2*D bytes apart), so HBM is used best when the heads of a sequence are streamed at the same rows at
+// the same time (64 ragged sequences of 512 to 32768 entries in pages, Hkv = 8, Hq = 64: 309 us with the heads one after
+// another, 270 in step).  So `hs` blocks in a row form a group that walks the same positions, each for a head of its own: the tiles
+// of (sequence, set of hs items, tile) form one list in that order, group c of a persistent grid (at most one block per SM)
+// owns the contiguous run [c * tpc, (c+1) * tpc) of it, so every SM streams the same number of bytes whatever the batch
 // shape.  A block therefore holds at most two incomplete items (the first and the last of its run);
 // it writes complete items straight to `out` and incomplete ones as (max, sum, unnormalised O)
 // partials, which the last block to finish an item merges (atomic ticket, same launch).  A ticket
@@ -42,6 +44,8 @@ struct DecodeParams {
     int B, Lmax, Hq, Hkv, G;
     int HG;        // head chunks per kv head (each chunk holds up to 8*NH query heads)
     int IPB;       // items per sequence = Hkv * HG
+    int hs, sets;  // items streamed in step by a group of hs blocks; sets of hs items per sequence = IPB / hs
+    int groups_equal;  // groups that a batch whose sequences have the same number of tiles is cut over
     int window, n_sink, is_full;
     float sl2;     // softmax scale * log2(e)
     unsigned long long* tickets;  // [gridDim.x]; (call stamp << 16 | arrivals), needs no initialisation
@@ -143,7 +147,7 @@ __host__ __device__ inline SeqGeom decode_shard_geom(int len, int rows, int pos0
 // Position in the global tile list; every role of a block walks the same positions.
 template <bool kPaged, bool kShard>
 struct DecodeWalker {
-    int b, hv, ti;
+    int b, set, ti;
     SeqGeom s;
     static __device__ __forceinline__ SeqGeom geom(const DecodeParams& p, int b) {
         if (kShard) return decode_shard_geom(__ldg(p.seqlens + b), p.Lmax, p.pos0, p.window, p.n_sink, p.is_full);
@@ -152,14 +156,14 @@ struct DecodeWalker {
     __device__ __forceinline__ void seek(const DecodeParams& p, int b0, long long off) {
         b = b0;
         s = geom(p, b);
-        hv = (int)(off / s.nt);
-        ti = (int)(off - (long long)hv * s.nt);
+        set = (int)(off / s.nt);
+        ti = (int)(off - (long long)set * s.nt);
     }
     __device__ __forceinline__ void next(const DecodeParams& p) {
         if (++ti < s.nt) return;
         ti = 0;
-        if (++hv < p.IPB) return;
-        hv = 0;
+        if (++set < p.sets) return;
+        set = 0;
         while (++b < p.B) {
             s = geom(p, b);
             if (s.nt > 0) return;
@@ -224,6 +228,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int ncta = (int)gridDim.x, cta = (int)blockIdx.x;
+    const int group = cta / p.hs, member = cta - group * p.hs;
+    int ngroups = ncta / p.hs;
 
     if (tid == 0) {
         *abort_flag = 0;
@@ -244,8 +250,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
 
     grid_wait();  // nothing above touches global memory
 
-    // ---- where does this block's run of the global tile list start?  (scan of tiles per sequence)
-    auto tiles_of = [&](int b) -> long long { return (long long)DecodeWalker<kPaged, kShard>::geom(p, b).nt * p.IPB; };
+    // ---- where does this group's run of the global tile list start?  (scan of tiles per sequence)
+    auto tiles_of = [&](int b) -> long long { return (long long)DecodeWalker<kPaged, kShard>::geom(p, b).nt * p.sets; };
     // A sequence without tiles.  Dense / paged cache: its length is out of range; report it and zero its output
     // rows.  Shard: also what a shard that holds none of the sequence's visible keys looks like; its rows get the
     // empty partial (-inf, 0, 0...), and only a length < 1 is an error.  One block does the stores.
@@ -266,20 +272,24 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     if (p.B <= kDecodeWarpScanMaxB) {
         // small batch: every warp scans all sequences by itself with shuffles, no block-level exchange
         total = 0;
+        const long long nb_first = tiles_of(0);
+        bool equal = true;
         for (int base = 0; base < p.B; base += 32) {
             const int b = base + lane;
             long long nb = 0;
             if (b < p.B) {
                 nb = tiles_of(b);
+                equal = equal && nb == nb_first;
                 if (nb == 0 && warp == 0) zero_fill_bad(b);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) nb += __shfl_xor_sync(0xffffffffu, nb, o);
             total += nb;
         }
-        tpc = (total + ncta - 1) / ncta;
+        if (__all_sync(0xffffffffu, equal)) ngroups = p.groups_equal;
+        tpc = (total + ngroups - 1) / ngroups;
         if (tpc < kDecodeMinTilesPerBlock) tpc = kDecodeMinTilesPerBlock;
-        t0 = (long long)cta * tpc;
+        t0 = (long long)group * tpc;
         t1 = total < t0 + tpc ? total : t0 + tpc;
         if (t0 < t1) {
             long long run = 0;
@@ -322,9 +332,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             __syncthreads();
         }
         total = sc_scan[kDecodeThreads - 1];
-        tpc = (total + ncta - 1) / ncta;
+        tpc = (total + ngroups - 1) / ngroups;
         if (tpc < kDecodeMinTilesPerBlock) tpc = kDecodeMinTilesPerBlock;
-        t0 = (long long)cta * tpc;
+        t0 = (long long)group * tpc;
         t1 = total < t0 + tpc ? total : t0 + tpc;
         if (t0 < t1 && sc_scan[tid] - mine <= t0 && t0 < sc_scan[tid]) {
             long long acc = sc_scan[tid] - mine;
@@ -356,7 +366,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             for (; n < cnt; ++n, w.next(p)) {
                 ok = mbar_wait(bar_e(s), ph ^ 1u, abort_flag);
                 if (!ok) break;
-                const int key0 = w.key0(), hk = w.hv / p.HG;
+                const int key0 = w.key0(), hk = (w.set * p.hs + member) / p.HG;
                 int c2 = key0, c3 = w.b;  // TMA coordinates: (entry, sequence) or (row in page, page)
                 if (kPaged) {
                     const int tile = key0 / kDecodeTileKeys;
@@ -418,7 +428,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     uint32_t ph = 0;
     while (n < cnt) {
         // ---- one segment: the tiles of the current item that belong to this block
-        const int b = w.b, hv = w.hv, ti_begin = w.ti, nt = w.s.nt;
+        const int b = w.b, hv = w.set * p.hs + member, ti_begin = w.ti, nt = w.s.nt;
         const int seg_tiles = min(cnt - n, nt - ti_begin);
         const long long seg_t0 = t0 + n;
         const int hk = hv / p.HG, ch = hv - hk * p.HG;
@@ -606,14 +616,14 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
         if (!complete) {
             // ---- the last block of this item to arrive merges the item's partials
             const long long T0 = seg_t0 - ti_begin, T1 = T0 + nt;
-            const int c_first = (int)(T0 / tpc), c_last = (int)((T1 - 1) / tpc);
+            const int c_first = (int)(T0 / tpc), c_last = (int)((T1 - 1) / tpc);  // groups
             const int n_parts = c_last - c_first + 1;
             __threadfence();  // this block's partial is visible before its ticket
             consumer_sync();
             if (tid == 0) {
                 // A ticket whose stamp is not this call's is left over from an earlier call (or was never
                 // written): the first block to arrive restarts it, so the workspace needs no clearing.
-                unsigned long long* t = p.tickets + c_first;
+                unsigned long long* t = p.tickets + c_first * p.hs + member;
                 if (n_parts == 2) {
                     // two blocks share the item (the common case): one exchange tells who came second
                     const unsigned long long mine = (p.stamp << 16) | 1ull;
@@ -633,7 +643,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             if (*sm_last && ok) {
                 __threadfence();
                 const bool first_is_slot1 = (long long)c_first * tpc != T0;
-                auto slot_of = [&](int cc) { return 2 * cc + ((cc == c_first && first_is_slot1) ? 1 : 0); };
+                auto slot_of = [&](int cc) { return 2 * (cc * p.hs + member) + ((cc == c_first && first_is_slot1) ? 1 : 0); };
                 for (int idx = tid; idx < gc * D; idx += kDecodeConsumerThreads) {
                     const int hh = idx / D, d = idx - hh * D;
                     float M = -INFINITY, den = 0.f, num = 0.f;

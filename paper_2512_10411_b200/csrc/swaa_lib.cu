@@ -51,7 +51,9 @@ static int current_device_info(DeviceInfo* out) {
 struct DecodePlan {
     int NH;      // 8-head blocks per chunk (1 or 2)
     int HG;      // chunks per kv head
-    int blocks;  // persistent grid size
+    int hs;      // items of a sequence that a group of hs blocks streams in step
+    int blocks;  // persistent grid size, a multiple of hs
+    int groups_equal;  // groups of hs blocks that a batch of equal lengths is cut over
     bool too_large;
     size_t off_part, bytes;
 };
@@ -69,29 +71,42 @@ static DecodePlan plan_decode(int B, int Hq, int Hkv, int D, int Lmax, int windo
     // upper bound on the tiles of one item: a shorter sequence may have one more (ragged) sink tile; a shard of a
     // longer sequence at most its rows in tiles plus a ragged sink and a ragged window tile
     const long long per_item = shard ? ((long long)Lmax + kDecodeTileKeys - 1) / kDecodeTileKeys + 2 : (long long)longest.nt + 1;
-    const long long tiles_ub = (long long)B * Hkv * pl.HG * per_item;
-    long long blocks = (tiles_ub + kDecodeMinTilesPerBlock - 1) / kDecodeMinTilesPerBlock;
     const long long sms = sm_count > 0 ? sm_count : 148;
-    if (blocks > sms) blocks = sms;
-    if (blocks < 1) blocks = 1;
-    // Cuts on item boundaries.  The cache rows of one sequence interleave its kv heads (a 64-key tile of one head is
-    // 64 pieces of 2*D bytes, Hkv*2*D bytes apart), so HBM is used best when the heads of a sequence are streamed
-    // at the same rows at the same time.  That is what happens when every block owns whole items, or every item is
-    // cut into the same number of blocks: consecutive blocks then walk consecutive heads in step (equal lengths
-    // assumed; ragged batches lose the alignment, not the correctness).  Measured on workload 4 with 128 items:
-    // 128 blocks against 148: FA decode 597 us against 652 us, SWA decode 47 us against 54 us (there is also no
-    // partial-result merge left); 120 or 132 blocks are no better than 148.  Below three quarters of the SMs the
-    // loss of parallel streams outweighs the gain (111 blocks: 660 us).
-    const long long items = (long long)B * Hkv * pl.HG;
-    if (blocks == sms) {
-        for (long long b = sms; b * 4 >= sms * 3; --b)
-            if (items % b == 0 || b % items == 0) {
-                blocks = b;
+    // As many of a sequence's items in step as divide them evenly and leave at most a tenth of the SMs without a block, and
+    // no more blocks than there are runs of kDecodeMinTilesPerBlock tiles.
+    const int items = Hkv * pl.HG;
+    const long long runs = ((long long)B * items * per_item + kDecodeMinTilesPerBlock - 1) / kDecodeMinTilesPerBlock;
+    pl.hs = 1;
+    for (int h = items; h > 1; --h)
+        if (items % h == 0 && h <= runs && sms / h >= 1 && sms / h * h * 10 >= sms * 9) {
+            pl.hs = h;
+            break;
+        }
+    const long long units = (long long)B * (items / pl.hs);  // runs of tiles that a group could own whole
+    const long long tiles_ub = units * per_item;             // per member of a group
+    long long groups = (tiles_ub + kDecodeMinTilesPerBlock - 1) / kDecodeMinTilesPerBlock;
+    const long long most = sms / pl.hs;
+    if (groups > most) groups = most;
+    if (groups < 1) groups = 1;
+    // A batch of equal lengths (or of equal windows) is cut over a group count that lets every group own whole items, or
+    // cuts every item into the same number of parts: no partial results to merge, and the groups end together.  Batch of 16,
+    // Hkv = 8, D = 128, 16 groups against 18: 43.3 us against 49.8 at 4100 visible entries each, 84.2 against 91.4 at 8196,
+    // 624 against 673 at 65536 (on another GPU 662 against 629).  Ragged batches use every group: 64 sequences of 512 to
+    // 32768 entries 270 us with 18 groups, 281 with 16.  The lengths are known on the device only: it chooses, except where a
+    // run has at most 3/2 * D tiles.  There the grid itself is cut to the smaller count (43.3 us as above; 47.4 where blocks
+    // come in only to find that they have no work), ragged or not.
+    pl.groups_equal = (int)groups;
+    if (groups == most) {
+        for (long long g = most; g * 4 >= most * 3; --g)
+            if (units % g == 0 || g % units == 0) {
+                pl.groups_equal = (int)g;
                 break;
             }
     }
+    if (2 * tiles_ub <= 3 * D * groups) groups = pl.groups_equal;
+    const long long blocks = groups * pl.hs;
     pl.blocks = (int)blocks;
-    pl.too_large = tiles_ub / blocks > 0x3fffffffLL;  // the kernel counts a block's tiles in an int
+    pl.too_large = tiles_ub / pl.groups_equal > 0x3fffffffLL;  // the kernel counts a block's tiles in an int
     pl.off_part = ((size_t)pl.blocks * sizeof(unsigned long long) + 255) / 256 * 256;
     pl.bytes = pl.off_part + (size_t)2 * pl.blocks * HC * (D + 2) * sizeof(float);
     return pl;
@@ -309,6 +324,9 @@ static int decode_impl(const void* q, const void* kcache, const void* vcache, vo
     p.G = Hq / Hkv;
     p.HG = pl.HG;
     p.IPB = Hkv * pl.HG;
+    p.hs = pl.hs;
+    p.sets = p.IPB / pl.hs;
+    p.groups_equal = pl.groups_equal;
     p.window = window;
     p.n_sink = n_sink;
     p.is_full = is_full ? 1 : 0;
