@@ -32,6 +32,8 @@
 // their loops without computing or storing, and the producer waits (bounded) for its copies in flight.
 #pragma once
 
+#include <type_traits>
+
 #include "swaa_internal.cuh"
 #include "swaa_ptx.cuh"
 
@@ -629,13 +631,17 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                     const unsigned long long mine = (p.stamp << 16) | 1ull;
                     *sm_last = atomicExch(t, mine) == mine ? 1 : 0;
                 } else {
-                    unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(t), want;
-                    for (;;) {
-                        want = (seen >> 16) == p.stamp ? seen + 1ull : ((p.stamp << 16) | 1ull);
-                        const unsigned long long prev = atomicCAS(t, seen, want);
-                        if (prev == seen) break;
+                    // with this call's stamp in place a plain add counts (no retries among the item's blocks)
+                    unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(t), want = 0;
+                    while ((seen >> 16) != p.stamp) {
+                        const unsigned long long prev = atomicCAS(t, seen, (p.stamp << 16) | 1ull);
+                        if (prev == seen) {
+                            want = (p.stamp << 16) | 1ull;
+                            break;
+                        }
                         seen = prev;
                     }
+                    if (want == 0) want = atomicAdd(t, 1ull) + 1ull;
                     *sm_last = ((int)(want & 0xffffull) == n_parts) ? 1 : 0;
                 }
             }
@@ -644,72 +650,59 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                 __threadfence();
                 const bool first_is_slot1 = (long long)c_first * tpc != T0;
                 auto slot_of = [&](int cc) { return 2 * (cc * p.hs + member) + ((cc == c_first && first_is_slot1) ? 1 : 0); };
-                for (int idx = tid; idx < gc * D; idx += kDecodeConsumerThreads) {
-                    const int hh = idx / D, d = idx - hh * D;
-                    float M = -INFINITY, den = 0.f, num = 0.f;
-                    if (n_parts <= 4) {
-                        // few parts: every load is issued before the first is needed (one round trip to L2)
-                        float ms[4], ls[4], os[4];
+                // Two channels per thread; the partials are taken kBatch at a time into a running (max, sum, O), all loads of a
+                // batch issued before the first is needed (one round trip to L2 each): an item of one long sequence has 18.  One
+                // sequence of 65536 entries 57.6 -> 51.0 us, one of 2052 visible entries 11.9 -> 10.6 us against one channel per
+                // thread and eight partials at a time.
+                auto merge = [&](auto batch_tag) {
+                    constexpr int kBatch = decltype(batch_tag)::value;
+                    for (int idx = tid; idx < gc * D / 2; idx += kDecodeConsumerThreads) {
+                        const int hh = idx / (D / 2), d = 2 * (idx - hh * (D / 2));
+                        float M = -INFINITY, den = 0.f, num0 = 0.f, num1 = 0.f;
+                        for (int c0 = c_first; c0 <= c_last; c0 += kBatch) {
+                            float2 ml[kBatch], os[kBatch];
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            ms[i] = -INFINITY;
-                            ls[i] = os[i] = 0.f;
-                            if (i < n_parts) {
-                                const float* pp = p.part + ((size_t)slot_of(c_first + i) * HC + hh) * (D + 2);
-                                ms[i] = __ldcg(pp);
-                                ls[i] = __ldcg(pp + 1);
-                                os[i] = __ldcg(pp + 2 + d);
-                            }
-                        }
-                        M = fmaxf(fmaxf(ms[0], ms[1]), fmaxf(ms[2], ms[3]));
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float wgt = ms[i] == -INFINITY ? 0.f : ex2f((ms[i] - M) * p.sl2);
-                            den += wgt * ls[i];
-                            num += wgt * os[i];
-                        }
-                    } else {
-                        // many parts (a long item of a small batch): eight partials per round trip to L2, merged
-                        // into a running (max, sum, O) -- loads one by one would cost a round trip each
-                        for (int c0 = c_first; c0 <= c_last; c0 += 8) {
-                            float ms[8], ls[8], os[8];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                ms[i] = -INFINITY;
-                                ls[i] = os[i] = 0.f;
+                            for (int i = 0; i < kBatch; ++i) {
+                                ml[i] = make_float2(-INFINITY, 0.f);
+                                os[i] = make_float2(0.f, 0.f);
                                 if (c0 + i <= c_last) {
                                     const float* pp = p.part + ((size_t)slot_of(c0 + i) * HC + hh) * (D + 2);
-                                    ms[i] = __ldcg(pp);
-                                    ls[i] = __ldcg(pp + 1);
-                                    os[i] = __ldcg(pp + 2 + d);
+                                    ml[i] = __ldcg(reinterpret_cast<const float2*>(pp));
+                                    os[i] = __ldcg(reinterpret_cast<const float2*>(pp + 2 + d));
                                 }
                             }
                             float Mn = M;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) Mn = fmaxf(Mn, ms[i]);
+                            for (int i = 0; i < kBatch; ++i) Mn = fmaxf(Mn, ml[i].x);
                             const float keep = M == -INFINITY ? 0.f : ex2f((M - Mn) * p.sl2);
                             den *= keep;
-                            num *= keep;
+                            num0 *= keep;
+                            num1 *= keep;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float wgt = ms[i] == -INFINITY ? 0.f : ex2f((ms[i] - Mn) * p.sl2);
-                                den += wgt * ls[i];
-                                num += wgt * os[i];
+                            for (int i = 0; i < kBatch; ++i) {
+                                const float wgt = ml[i].x == -INFINITY ? 0.f : ex2f((ml[i].x - Mn) * p.sl2);
+                                den += wgt * ml[i].y;
+                                num0 += wgt * os[i].x;
+                                num1 += wgt * os[i].y;
                             }
                             M = Mn;
                         }
-                    }
-                    if (kShard) {
-                        float* po = p.part_out + ((size_t)b * p.Hq + h0 + hh) * (D + 2);
-                        po[2 + d] = num;
-                        if (d == 0) {
-                            po[0] = M * p.scale;
-                            po[1] = den;
+                        if (kShard) {
+                            float* po = p.part_out + ((size_t)b * p.Hq + h0 + hh) * (D + 2);
+                            po[2 + d] = num0;
+                            po[3 + d] = num1;
+                            if (d == 0) {
+                                po[0] = M * p.scale;
+                                po[1] = den;
+                            }
+                        } else {
+                            const float inv = den > 0.f ? 1.f / den : 0.f;
+                            *reinterpret_cast<uint32_t*>(p.out + ((size_t)b * p.Hq + h0 + hh) * D + d) = pack_bf16x2(num0 * inv, num1 * inv);
                         }
-                    } else {
-                        p.out[((size_t)b * p.Hq + h0 + hh) * D + d] = __float2bfloat16_rn(den > 0.f ? num / den : 0.f);
                     }
-                }
+                };
+                if (n_parts <= 4) merge(std::integral_constant<int, 4>{});
+                else merge(std::integral_constant<int, 18>{});
             }
         }
         consumer_sync();  // the merge buffers are free for the next segment
