@@ -266,6 +266,14 @@ __device__ __forceinline__ void pin64(uint32_t* r) {
     for (int i = 0; i < 64; ++i) asm volatile("" : "+r"(r[i]));
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : SWAA_R8(r, 0), SWAA_R8(r, 8)
+        : "r"(taddr)
+        : "memory");
+}
+
 // Shared-memory matrix descriptors for tiles stored as 128-byte rows with the 128-byte swizzle (what
 // TMA writes for a [rows][64 bf16] box).  14-bit fields hold byte values >> 4.
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -500,7 +508,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         // short ones fill the end: sequences by the keys that an item of theirs visits (32 sequences at a time, the last
         // ones of the batch first), last tile of a sequence first.  Lane l looks after sequence base_b - l.
         // Serving step of 4 chunks and 24 generated tokens at 1k to 32k keys in pages: 582 us in batch order, 493 this way.
-        if (lane == 0 && (p.cu_seqlens[0] != 0 || p.cu_seqlens[p.B] != p.T)) record_device_error(SWAA_ERR_BAD_SEQLENS);
         int base_b = p.B - 1;       // sequence of lane 0
         int base_w = 0;             // index of the first item of this group of 32 sequences
         int f_s = 0, f_len = 0, f_ks = 0, f_off = 0, f_full = full_all ? 1 : 0, f_sink = p.n_sink, f_srem = 0;
@@ -629,6 +636,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             nb_phase ^= 1u;
             w = uniform(next_block_answer(s_answer));
         }
+        if (lane == 0 && (p.cu_seqlens[0] != 0 || p.cu_seqlens[p.B] != p.T)) record_device_error(SWAA_ERR_BAD_SEQLENS);
         // the last items have to be done before the end is published, lest one is to be run again
         while (ok) {
             ok = free_slot();
@@ -1023,6 +1031,55 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 phases ^= kPhS;
                 tc_fence_after();
                 if (idle) {
+                    arrive_warp(BAR_PR + side);
+                    continue;
+                }
+                if (!kChunked && !kLseOnly && t.cb == 0 && t.left <= 32) {
+                    // A few sink keys in a tile of their own, which every row sees: 32 columns instead of 128.  A block's last
+                    // step before its output, so it counts in full where a block has few tiles: 1024 tokens, 4 heads of 64,
+                    // window 128: 11.8 -> 10.6 us; 63 sequences at head size 64, forward and backward: 459 -> 455.  In the
+                    // instances with a key list of its own the step's items are long and it measured nothing (506, 509).
+                    uint32_t sn[32];
+                    tmem_ld32(tS, sn);
+                    tc_wait_ld();
+                    float mx = -INFINITY;
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        sn[c] = c < t.left ? sn[c] : 0xff800000u;  // -inf
+                        mx = fmaxf(mx, __uint_as_float(sn[c]));
+                    }
+                    const float m_new = fmaxf(m_used, mx);
+                    const bool need = (m_used != -INFINITY) && ((m_new - m_used) * p.sl2 > kRescaleThreshold);
+                    if (__any_sync(0xffffffffu, row_ok && need)) {
+                        const float alpha = (m_used == -INFINITY) ? 1.f : ex2f((m_used - m_new) * p.sl2);
+#pragma unroll 1
+                        for (int cc = 0; cc < D / 16; ++cc) {
+                            uint32_t orr[16];
+                            tmem_ld16(tO + (uint32_t)(cc * 16), orr);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) orr[c] = __float_as_uint(__uint_as_float(orr[c]) * alpha);
+                            tmem_st16(tO + (uint32_t)(cc * 16), orr);
+                        }
+                        tc_wait_st();
+                        l_sum *= alpha;
+                        m_used = m_new;
+                    } else if (m_used == -INFINITY) {
+                        m_used = m_new;
+                    }
+                    fresh = __any_sync(0xffffffffu, row_ok && m_used == -INFINITY);
+                    const float off = m_used == -INFINITY ? 0.f : m_used * p.sl2;
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        const float p0 = ex2f(fmaf(__uint_as_float(sn[2 * c]), p.sl2, -off));
+                        const float p1 = ex2f(fmaf(__uint_as_float(sn[2 * c + 1]), p.sl2, -off));
+                        l_sum += p0 + p1;
+                        pk[c] = pack_bf16x2(p0, p1);
+                    }
+                    tmem_st16(tS, pk);
+                    tc_wait_st();
+                    tc_fence_before();
                     arrive_warp(BAR_PR + side);
                     continue;
                 }

@@ -1,13 +1,16 @@
 """GPU parity of the prefill kernel's work items where they can go wrong: sequences around the size that is packed into
 one item per kv head, batches of more sequences than one look of the scheduler covers, tiles that join band and sink
-keys, and scores that outgrow the exponent range of the reference within one tile (the item is then run again)."""
+keys, a few sink keys in a tile of their own, and scores that outgrow the exponent range of the reference within one tile
+(the item is then run again)."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2512_10411_b200 import inputs
 from helpers import check_against_oracle
 from test_prefill_chunked_gpu import make, run_chunked
+from test_prefill_gpu import run_prefill
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +39,22 @@ def test_more_sequences_than_one_look_of_the_scheduler():
     lq = tuple(int(x) for x in rng.integers(1, 200, 70))
     lk = tuple(a + int(x) for a, x in zip(lq, rng.integers(0, 200, 70)))
     _check(lq, lk, 4, 2, 128, 100, 4, False, seed=60)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("S", [1, 16, 31, 32, 33, 160])
+def test_few_sink_keys_in_a_tile_of_their_own(D, S):
+    # window 128: the band fills its two tiles exactly, so the sink keys start one; 160 leaves 32 for the second.  The
+    # large scale makes them outgrow the reference of the band keys.
+    lens = (300, 129, 517, 40)
+    q, k, v = make(lens, lens, 3, 1, D, 90 + S)
+    cu = np.concatenate([[0], np.cumsum(lens)])
+    for W, scale in ((128, 0.0), (128, 4.0), (112, 0.0)):
+        out, lse, status = run_prefill(q, k, v, torch.tensor(cu, dtype=torch.int32, device="cuda"), max(lens), W, S, False, scale)
+        assert status == 0
+        ref = oracle.prefill(*(inputs.to_f32_numpy(t) for t in (q, k, v)), cu, W, S, False, scale=scale if scale > 0 else None)
+        check_against_oracle(out, ref["out"], f"D={D} W={W} S={S} scale={scale}")
+        np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
 
 
 @pytest.mark.parametrize("D", [64, 128])
