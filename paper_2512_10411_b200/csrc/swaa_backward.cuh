@@ -25,6 +25,7 @@ struct BackwardParams {
     float* dkv_accum;        // [2][B][sink_rows][Hkv][D] fp32, zeroed: dk, dv of the sink tiles, which are split over blocks
     int sink_tiles;          // key tiles that hold sink keys (their query range is cut into chunks), 0 for full attention
     int chunks;              // blocks per sink tile
+    int key_tiles;           // key tiles of a sequence of max_seqlen
     float* dq_accum;         // [T, Hq, D] fp32, zeroed before the launch
     __nv_bfloat16* dk;       // [T, Hkv, D]
     __nv_bfloat16* dv;

@@ -28,8 +28,8 @@
 // What bounds it.  A group's step is a chain S^T, dP^T -> element-wise part -> dV, dK, dQ -> read-out -> S^T of its next
 // step, several times as long as the products of a step: the more steps in flight, the better.  Packed batch of
 // 16k tokens, Hq = 16, Hkv = 4, D = 64, window 1024, forward + backward: 540 us with two groups, 462 with three (1417 on
-// warp-level MMAs).  At D = 128 tensor memory holds no third group, and a long sample runs against the power cap (1.65 GHz):
-// 16k tokens, Hq = 32, Hkv = 8, window 2048: 2370 us.
+// warp-level MMAs), 390 with the blocks in order of their length.  At D = 128 tensor memory holds no third group, and a long sample runs against the power cap (1.65 GHz):
+// 16k tokens, Hq = 32, Hkv = 8, window 2048: 2360 us.
 //
 // Warps: 4 per group; then the TMA producer (K, V once; Q, dO and the row terms per
 // step through a ring of stages); then the MMA issuer.  Every wait is bounded.
@@ -117,18 +117,25 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
     grid_wait();
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const int hk = blockIdx.y, b = blockIdx.z;
-    // blockIdx.x -> (key tile, chunk of its query range): the tiles that hold sink keys meet every later query
-    // tile, so their range is cut into chunks of kBwdChunkTiles query tiles handled by separate blocks
-    int n_tile, chunk = -1;
-    if ((int)blockIdx.x < p.sink_tiles * p.chunks) {
-        n_tile = (int)blockIdx.x / p.chunks;
-        chunk = (int)blockIdx.x - n_tile * p.chunks;
-    } else {
-        n_tile = p.sink_tiles + ((int)blockIdx.x - p.sink_tiles * p.chunks);
-    }
+    const int b = (int)blockIdx.x / p.Hkv, hk = (int)blockIdx.x - b * p.Hkv;
     const int seq_start = p.cu_seqlens[b], Lseq = p.cu_seqlens[b + 1] - seq_start;
-    const int j0 = n_tile * BK;
+    // Blocks start in the order of their index, x first, so the second index orders the work of all sequences and heads from
+    // the longest to the shortest: first the tiles that hold sink keys, which meet every later query tile and whose query
+    // range is cut into chunks of kBwdChunkTiles query tiles handled by separate blocks, then the other key tiles by their
+    // distance from the end of the sequence, the furthest first.  In the order
+    // (head, sequence, key tile) the last blocks to start were as long as any: forward + backward of the packed batch above
+    // 455 us, 390 this way; one sequence of 4096 tokens, 32 heads of 128, 8 key heads, window 1024: 436 and 366, full
+    // attention 706 and 597; 16k tokens of one sequence, window 2048, at the power cap: 2370 and 2357.
+    int slot = (int)(blockIdx.z * gridDim.y + blockIdx.y), n_tile, chunk = -1;
+    if (slot < p.sink_tiles * p.chunks) {
+        n_tile = slot / p.chunks;
+        chunk = slot - n_tile * p.chunks;
+    } else {
+        slot -= p.sink_tiles * p.chunks;
+        n_tile = (Lseq + BK - 1) / BK - p.key_tiles + slot;
+        if (n_tile < p.sink_tiles || slot >= p.key_tiles) n_tile = Lseq;  // none
+    }
+    const int j0 = n_tile >= Lseq ? Lseq : n_tile * BK;
     if (Lseq <= 0 || Lseq > p.max_seqlen || j0 >= Lseq || seq_start < 0 ||
         seq_start + Lseq > p.T) {  // uniform: before any barrier or allocation
         if (threadIdx.x == 0 && (Lseq < 0 || Lseq > p.max_seqlen || seq_start < 0 || seq_start + Lseq > p.T))

@@ -733,7 +733,7 @@ static BackwardWorkspace backward_workspace(int B, int T, int Hq, int Hkv, int D
 
 template <int D>
 static int launch_backward(const void* q, const void* k, const void* v, const void* out, const void* dout,
-                           const BackwardParams& p, void* dq, int max_seqlen, size_t dkv_zero_bytes, cudaStream_t st) {
+                           const BackwardParams& p, void* dq, size_t dkv_zero_bytes, cudaStream_t st) {
     constexpr int kKeyTile = kBwdTcKeys;
     CUtensorMap tq, tk, tv, tdo, tacc;
     int rc;
@@ -750,8 +750,8 @@ static int launch_backward(const void* q, const void* k, const void* v, const vo
                            static_cast<const __nv_bfloat16*>(out), static_cast<const __nv_bfloat16*>(dout), p.lse,
                            const_cast<float*>(p.delta), const_cast<float*>(p.lse2), p.dq_accum, p.T, p.Hq);
     if (rc != SWAA_OK) return rc;
-    const int ntiles = (max_seqlen + kKeyTile - 1) / kKeyTile;
-    const dim3 grid((unsigned)(p.sink_tiles * p.chunks + (ntiles - p.sink_tiles)), (unsigned)p.Hkv, (unsigned)p.B);
+    const unsigned slots = (unsigned)(p.sink_tiles * p.chunks + p.key_tiles), rows = slots < 32768u ? slots : 32768u;
+    const dim3 grid((unsigned)p.B * (unsigned)p.Hkv, rows, (slots + rows - 1) / rows);
     using L = BackwardTcSmem<D>;
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(backward_tc_kernel<D>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
@@ -825,11 +825,12 @@ extern "C" int swaa_prefill_backward(const void* q, const void* k, const void* v
         if (p.sink_tiles * key_tile > w.sink_rows) p.sink_tiles = w.sink_rows / key_tile;
     }
     if (p.sink_tiles == 0) p.chunks = 1;
-    if ((long long)p.sink_tiles * p.chunks + (ntiles - p.sink_tiles) > 0x7fffffffLL) return SWAA_ERR_UNSUPPORTED;
+    p.key_tiles = ntiles;
+    if ((long long)p.sink_tiles * p.chunks + ntiles > 0x7fffffffLL || (long long)B * Hkv > 0x7fffffffLL) return SWAA_ERR_UNSUPPORTED;
     const size_t dkv_zero_bytes = 2 * (size_t)B * p.sink_tiles * key_tile * Hkv * D * sizeof(float);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    return D == 128 ? launch_backward<128>(q, k, v, out, dout, p, dq, max_seqlen, dkv_zero_bytes, st)
-                    : launch_backward<64>(q, k, v, out, dout, p, dq, max_seqlen, dkv_zero_bytes, st);
+    return D == 128 ? launch_backward<128>(q, k, v, out, dout, p, dq, dkv_zero_bytes, st)
+                    : launch_backward<64>(q, k, v, out, dout, p, dq, dkv_zero_bytes, st);
 }
 
 // ------------------------------------------------------------------------------------ lazy ratio
