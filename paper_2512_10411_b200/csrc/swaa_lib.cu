@@ -480,7 +480,7 @@ static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStr
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(prefill_kernel<D, kMode, kLseOnly>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
     // one block per item (an upper bound); the blocks that run take over the indices of those that wait
-    const unsigned blocks = (unsigned)p.n_pairs * (unsigned)p.tiles_ub;
+    const unsigned blocks = (unsigned)p.n_units * (unsigned)p.tiles_ub;
     return launch_overlapped(prefill_kernel<D, kMode, kLseOnly>, dim3(blocks), kPrefillThreads, L::kDynamicBytes, st, tm, p);
 }
 
@@ -582,12 +582,18 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.Hkv = Hkv;
     p.G = G;
     p.pack_tokens = pack_tokens;
-    p.pairs_per_kv = (p.G + 1) / 2;
-    p.n_pairs = Hkv * p.pairs_per_kv;
     const long long ub_a = (long long)Tq / kPrefillBM + B;
     const long long ub_b = (long long)B * ((max_seqlen_q + kPrefillBM - 1) / kPrefillBM);
     const long long ub = ub_a < ub_b ? ub_a : ub_b;
-    if (ub > 2147483647LL / p.n_pairs) return SWAA_ERR_UNSUPPORTED;
+    // Two heads per item read K and V once for both, but each side walks all key tiles.  Where all items of one head each
+    // start at once on an SM of their own, an item takes one head and its two sides alternate key tiles.  1024 tokens, 4 heads
+    // of 64, window 128: 10.9 us with two heads, 9.1 with one; 2048 tokens, 8 heads of 128: 17.7 and 15.3 (window 512), 34.2
+    // and 31.0 (full); 500 tokens behind 31000 in pages, 32 heads: 68.0 and 51.7.  Past that point items of one head take a
+    // second turn on the SMs, which is the same work again.
+    p.heads = ub <= info.sm_count / Hq ? 1 : 2;
+    p.units_per_kv = (p.G + p.heads - 1) / p.heads;
+    p.n_units = Hkv * p.units_per_kv;
+    if (ub > 2147483647LL / p.n_units) return SWAA_ERR_UNSUPPORTED;
     p.tiles_ub = (int)ub;
     if (p.tiles_ub == 0) return SWAA_OK;  // max_seqlen == 0: nothing can be valid
     // a window that covers the longest key sequence is full causal attention for every row; clamping keeps the

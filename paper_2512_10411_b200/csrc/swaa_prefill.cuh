@@ -60,8 +60,9 @@ struct PrefillParams {
     // block_table[b * max_blocks + j / page_size] at row j % page_size
     const int32_t* block_table;
     int max_blocks, page_size, num_pages;
-    int pairs_per_kv;       // ceil(G / 2)
-    int n_pairs;            // Hkv * pairs_per_kv
+    int heads;              // query heads per unpacked item: two, one per side, or one
+    int units_per_kv;       // ceil(G / heads)
+    int n_units;            // Hkv * units_per_kv
     int tiles_ub;           // upper bound on the number of query tiles over all sequences
     int pack_tokens;        // 128 / G: a sequence of at most this many queries is one item per kv head (see WorkItem)
     int window, n_sink, is_full;
@@ -319,7 +320,8 @@ struct PrefillSmem {
     static_assert(kDynamicBytes <= 232448, "shared memory per block");
 };
 
-// One unit of work.  Usual form: a 128-row query tile of one sequence for one pair of query heads (one per side).
+// One unit of work.  Usual form: a 128-row query tile of one sequence for one pair of query heads (one per side), or for a
+// single query head, both sides on its rows, when the call has too few tiles for the SMs (see the launch).
 // Packed form, for sequences whose queries times the group size fit in 128 rows (generated tokens, very short
 // prompts): the rows are (query, head of the group) for ALL heads of one kv head, so K and V are read once per kv head
 // and no row is padding that another head could use; the two sides then take alternate key tiles and merge at the end.
@@ -333,9 +335,9 @@ struct WorkItem {
     int valid, seq_start, seq_len;
     int q0;       // first query of the tile, counted inside the sequence's queries
     int hk, hA;   // kv head, (side A's, first) query head
-    int packed;
+    int packed;   // both sides work on one tile of rows; heads of a row group: rows = (query, head of the group), 1: queries of one head
     int hasB;     // side B has a query head of its own (unpacked items)
-    int shared;   // packed item of several tiles: both sides work on the same rows, alternate key tiles
+    int shared;   // packed item of several tiles: the sides take alternate key tiles and merge
     int full;     // this item runs full causal attention (per sequence in a mixed batch)
     int k_start;  // first packed key token of the sequence (= seq_start for self attention; sequence index when paged)
     int k_off;    // index of the sequence's first query among its (local) keys: len_k - len_q (0 for self attention)
@@ -348,8 +350,8 @@ struct WorkItem {
     int n_rows;   // rows in use
     int careful;  // second run of an item whose scores left the exponent range of the first (see the softmax role)
 
-    // fills the rest from seq_len, q0, packed, full, k_off, n_sink, s_rem and the unit: head pair, or kv head when packed
-    template <int BN, bool kPaged, bool kCp>
+    // fills the rest from seq_len, q0, packed, full, k_off, n_sink, s_rem and the unit: head pair (or head), or kv head when packed
+    template <int BN, bool kPaged, bool kCp, bool kLseOnly>
     __device__ __forceinline__ void complete(const PrefillParams& p, int unit) {
         if (packed) {
             hk = unit;
@@ -358,10 +360,12 @@ struct WorkItem {
             n_rows = seq_len * p.G;
             i0 = k_off;
             i1 = k_off + seq_len - 1;
+            packed = p.G;
         } else {
-            hk = unit / p.pairs_per_kv;
-            hA = hk * p.G + 2 * (unit - hk * p.pairs_per_kv);
-            hasB = (hA + 1) < (hk + 1) * p.G ? 1 : 0;
+            hk = unit / p.units_per_kv;
+            hA = hk * p.G + p.heads * (unit - hk * p.units_per_kv);
+            hasB = p.heads == 2 && (hA + 1) < (hk + 1) * p.G ? 1 : 0;
+            if (!kLseOnly && p.heads == 1) packed = 1;  // one tile of rows, both sides on it as in a packed item
             n_rows = min(kPrefillBM, seq_len - q0);
             i0 = q0 + k_off;
             i1 = i0 + n_rows - 1;
@@ -548,7 +552,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 f_s = s0;
                 f_len = len;
                 f_packed = !kLseOnly && len <= p.pack_tokens ? 1 : 0;
-                f_items = len == 0 ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_pairs);
+                f_items = len == 0 ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_units);
             }
             group_items = __reduce_add_sync(0xffffffffu, f_items);
             f_before = 0;
@@ -607,7 +611,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     d.valid = 1;
                     d.seq_start = f_s;
                     d.seq_len = f_len;
-                    d.q0 = f_packed ? 0 : ((f_len + BM - 1) / BM - 1 - local / p.n_pairs) * BM;
+                    d.q0 = f_packed ? 0 : ((f_len + BM - 1) / BM - 1 - local / p.n_units) * BM;
                     d.packed = f_packed;
                     d.full = f_full;
                     d.k_start = f_ks;
@@ -616,7 +620,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     d.s_rem = f_srem;
                     d.b = base_b - lane;
                     d.careful = 0;
-                    d.complete<BN, kPaged, kCp>(p, f_packed ? local : local % p.n_pairs);
+                    d.complete<BN, kPaged, kCp, kLseOnly>(p, f_packed ? local : local % p.n_units);
                     volatile int* to = slot_words(it & 1);
                     const int* from = reinterpret_cast<const int*>(&d);
 #pragma unroll
@@ -676,7 +680,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             if (!ok) break;
             if (el) {
                 const int hA = w.hA, tq = w.seq_start + w.q0;
-                if (packed) {  // rows = (query, head of the group)
+                if (packed && w.packed > 1) {  // rows = (query, head of the group)
                     mbar_arrive_expect_tx(bar(BAR_QF), (uint32_t)(p.pack_tokens * p.G * 128 * L::kPanels));
 #pragma unroll
                     for (int pn = 0; pn < L::kPanels; ++pn)
@@ -1105,7 +1109,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                         // of the sink keys that follow the band (cb <= c < left), which every row sees.
                         const bool full = w.full != 0;
                         // index of this thread's query among the (local) keys; rows past the end take the last one's
-                        const int i = min(w.i0 + (packed ? row / p.G : row), w.i1);
+                        const int i = min(w.i0 + (packed && w.packed > 1 ? row / p.G : row), w.i1);
                         const int dc = remote ? -1 : min(i - t.jb, t.cb - 1);
                         const int wl = full ? 0 : i - t.jb - p.window + 1;
                         const int sk = full ? 0 : w.n_sink - t.jb;
@@ -1214,9 +1218,10 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 phases ^= kPhO;
                 tc_fence_after();
             }
-            const int q_row = packed ? row / p.G : w.q0 + row;  // this thread's query, counted inside the sequence
+            const int q_off = packed && w.packed > 1 ? row / p.G : row;
+            const int q_row = w.q0 + q_off;  // this thread's query, counted inside the sequence
             const int token = w.seq_start + q_row, tok0 = w.seq_start + w.q0;
-            const int h = packed ? w.hA + row - q_row * p.G : w.hA + side;
+            const int h = w.hA + (packed ? (w.packed > 1 ? row - q_off * p.G : 0) : side);
             const bool sideB = shared || uniform(w.hasB) != 0;
             release_work(it);
             __nv_bfloat16* orow = p.out + ((size_t)token * p.Hq + h) * D;

@@ -57,6 +57,15 @@ def test_few_sink_keys_in_a_tile_of_their_own(D, S):
         np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
 
 
+@pytest.mark.parametrize("Hq,Hkv", [(24, 8), (32, 8), (12, 12), (9, 3)])  # with 13 tiles at most: two heads per item but for 9
+@pytest.mark.parametrize("D", [64, 128])
+def test_one_and_two_heads_per_item(Hq, Hkv, D):
+    lq, lk = (300, 1, 129, 128, 517), (300, 70, 400, 128, 600)
+    for W, S, full in ((1, 0, True), (128, 4, False), (200, 130, False)):
+        _check(lq, lq, Hq, Hkv, D, W, S, full, seed=120 + Hq)
+        _check(lq, lk, Hq, Hkv, D, W, S, full, seed=121 + Hq)
+
+
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("scale", [4.0, 30.0])
 def test_scores_that_leave_the_exponent_range_of_the_reference(D, scale):
