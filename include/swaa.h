@@ -67,7 +67,7 @@ typedef enum {
  *   scale       softmax scale; <= 0 selects 1/sqrt(D).
  *   lse         device, float32 [Hq, T], natural-log sum of exp(scale * q.k) over the visible keys of
  *               each row; may be NULL.
- * Only the key tiles that hold a visible key are visited: the sink tiles and the diagonal band.
+ * Only keys near a visible one are visited: the diagonal band and the sinks.
  */
 int swaa_prefill(const void* q, const void* k, const void* v, void* out, const int32_t* cu_seqlens, int B, int T,
                  int max_seqlen, int Hq, int Hkv, int D, int window, int n_sink, int is_full, float scale,
@@ -214,7 +214,7 @@ int swaa_lazy_ratio(const void* q, const void* k, const void* v, const int32_t* 
  *   workspace       device scratch of at least swaa_decode_workspace_size(...) bytes for the same
  *                   shape arguments, 256-byte aligned; contents need not be initialised and are
  *                   overwritten.  Two calls that overlap on the GPU must not share a workspace.
- * The visible cache entries of all sequences and heads form one list of 64-entry tiles that is cut
+ * The visible cache entries of all sequences form one list of 64-entry tiles, the heads of a sequence in step, that is cut
  * evenly over a persistent grid (split-K across blocks wherever a cut falls inside a sequence);
  * partial results are merged by a log-sum-exp combine inside the same launch.  Cache entries past
  * seqlens[b] are never used, whatever they hold.
@@ -347,11 +347,11 @@ int swaa_schedule_select_fa_layers(const float* ratio, int n_layers, int n_heads
                                    uint8_t* fa_mask_out);
 
 /*
- * Key-tile enumeration of the prefill kernel, exposed for host-side verification (App. A: only
- * O(N*W) work).  For the query tile of rows [m*BM, min(L, (m+1)*BM)) of a sequence of length L, the
- * kernel visits key tiles (of BN keys) 0 .. *n_sink_tiles-1 and *n_lo .. *n_hi.  Returns SWAA_OK or
+ * Key tiles, on a grid of whole tiles, that hold a key visible to a query tile, for host-side verification (App. A: only
+ * O(N*W) work; the kernel itself cuts the same keys from the first one on, sinks behind the band).  For the query tile of
+ * rows [m*BM, min(L, (m+1)*BM)) of a sequence of length L, the tiles (of BN keys) are 0 .. *n_sink_tiles-1 and *n_lo .. *n_hi.  Returns SWAA_OK or
  * SWAA_ERR_INVALID_ARG.  swaa_prefill_tile_needs_mask returns 1 when some (row, key) pair of the
- * tile is not visible (the kernel then applies the element predicate), 0 when every pair is visible.
+ * tile is not visible (the element predicate is then needed), 0 when every pair is visible.
  */
 int swaa_prefill_tile_range(int L, int m, int BM, int BN, int window, int n_sink, int is_full, int* n_sink_tiles,
                             int* n_lo, int* n_hi);
