@@ -16,7 +16,8 @@
 // shape.  A block therefore holds at most two incomplete items (the first and the last of its run);
 // it writes complete items straight to `out` and incomplete ones as (max, sum, unnormalised O)
 // partials, which the last block to finish an item merges (atomic ticket, same launch).  A ticket
-// carries a per-call stamp, so stale workspace contents are recognised and nothing has to be cleared.
+// carries a per-call stamp, so stale workspace contents are recognised and nothing has to be cleared before the call; the
+// last block of an item sets its ticket back to 0, because a call replayed by a CUDA graph comes with the same stamp again.
 //
 // Data path.  One producer thread keeps a ring of shared-memory stages full with TMA tile copies
 // (K and V boxes of [64 keys][64 channels], 128-byte swizzle; a 16-key box for tiles with at most 16
@@ -644,6 +645,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                     if (want == 0) want = atomicAdd(t, 1ull) + 1ull;
                     *sm_last = ((int)(want & 0xffffull) == n_parts) ? 1 : 0;
                 }
+                if (*sm_last) *reinterpret_cast<volatile unsigned long long*>(t) = 0ull;
             }
             consumer_sync();
             if (*sm_last && ok) {

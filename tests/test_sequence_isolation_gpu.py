@@ -1,0 +1,85 @@
+"""What a sequence must not see does not reach its results: keys and values of its neighbours in a packed batch that hold NaN,
+forward and backward; and values near the top of bf16's range next to scores that grow from tile to tile."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2512_10411_b200 as swaa
+from paper_2512_10411_b200 import inputs
+from helpers import check_against_oracle
+from test_prefill_chunked_gpu import make, run_chunked
+from test_prefill_gpu import run_prefill
+
+pytestmark = pytest.mark.gpu
+
+
+def _cu(lens):
+    return torch.tensor(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), device="cuda")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("W,S,full", [(64, 4, False), (100, 0, False), (100, 20, False), (1, 0, True)])
+def test_forward_next_to_a_sequence_of_nan_keys_and_values(D, W, S, full):
+    # key lengths that end on a tile: no key tile on the grid of whole tiles holds keys of two sequences
+    for lq, lk in (((256, 128), (256, 128)), ((256, 128, 77), (640, 256, 77)), ((3, 256, 40), (256, 384, 40))):
+        q, k, v = make(lq, lk, 4, 2, D, 50 + W)
+        want, want_lse, _ = run_chunked(q, k, v, lq, lk, W, S, full)
+        n_q, n_k = sum(lq[:-1]), sum(lk[:-1])
+        k[n_k:] = float("nan")
+        v[n_k:] = float("nan")
+        outs = [run_chunked(q, k, v, lq, lk, W, S, full)]
+        if lq == lk:
+            outs.append(run_prefill(q, k, v, _cu(lq), max(lq), W, S, full))
+        for out, lse, status in outs:
+            assert status == 0
+            assert torch.equal(out[:n_q], want[:n_q]) and torch.equal(lse[:, :n_q], want_lse[:, :n_q]), (lq, lk)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("L0", [64, 100, 192, 256])
+def test_backward_next_to_a_sequence_of_nan_keys(D, L0):
+    lens, Hq, Hkv, W, S = (L0, 200), 4, 2, 100, 4
+    q, k, v = make(lens, lens, Hq, Hkv, D, 60 + L0)
+    out, lse, _ = run_prefill(q, k, v, _cu(lens), max(lens), W, S, False)
+    dout = make(lens, lens, Hq, Hkv, D, 61 + L0)[0]
+    ws = torch.empty(swaa.prefill_backward_workspace_size(2, sum(lens), Hq, Hkv, D, S), dtype=torch.uint8, device="cuda")
+
+    def grads(kk):
+        g = [torch.full_like(t, float("nan")) for t in (q, k, v)]
+        swaa.swaa_prefill_backward(q, kk, v, out, dout, lse, _cu(lens), max(lens), W, S, False, *g, ws)
+        assert swaa.last_device_status() == 0
+        return g
+
+    want = grads(k)
+    for bad, kept in ((slice(L0, None), slice(0, L0)), (slice(0, L0), slice(L0, None))):
+        kk = k.clone()
+        kk[bad] = float("nan")
+        for got, w, name in zip(grads(kk), want, ("dq", "dk", "dv")):
+            err = (got[kept].double() - w[kept].double()).norm() / w[kept].double().norm()
+            assert err.item() <= 1e-3, (name, bad)  # the order of the fp32 sums into dq varies: bf16 roundings that flip
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("lq,lk,Hq,Hkv", [((1024,), (1024,), 2, 1), ((640, 30, 1), (1024, 900, 700), 4, 1), ((2560,), (2560,), 16, 2)])
+def test_large_values_where_scores_grow_from_tile_to_tile(D, lq, lk, Hq, Hkv):
+    """Values around 2^95 and a key in an unmasked tile whose score lies 2^40 above all before it: the products stay below
+    2^127 only against a reference that follows the scores."""
+    q, k, v = (t.float() for t in make(lq, lk, Hq, Hkv, D, 70))
+    u = torch.randn(D, device="cuda")
+    u = u / u.norm()
+    q = 0.2 * q + 16.0 * u
+    k = 0.2 * k
+    for a in np.concatenate([[0], np.cumsum(lk)[:-1]]):
+        k[a + 300] += u * (40 * 0.6931 * D ** 0.5 / 16.0)
+    q, k = q.to(torch.bfloat16), k.to(torch.bfloat16)
+    v = (v * 2.0 ** 95).to(torch.bfloat16)
+    out, lse, status = run_chunked(q, k, v, lq, lk, 1, 0, True)
+    assert status == 0
+    rows = np.unique(np.linspace(0, sum(lq) - 1, 400).astype(np.int64))
+    rh = (rows % Hq).astype(np.int32)
+    cu_q, cu_k = _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy()
+    ref = oracle.prefill_chunked(*(inputs.to_f32_numpy(t) for t in (q, k, v * 2.0 ** -95)), cu_q, cu_k, 1, 0, True, rows=(rows, rh))
+    got = out[torch.as_tensor(rows, device="cuda"), torch.as_tensor(rh.astype(np.int64), device="cuda")] * 2.0 ** -95
+    check_against_oracle(got, ref["out"], f"{lq} {lk} D={D}")
+    np.testing.assert_allclose(lse.cpu().numpy()[rh, rows], ref["lse"], rtol=0, atol=2e-3)
