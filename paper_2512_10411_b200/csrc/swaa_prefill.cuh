@@ -328,8 +328,10 @@ struct PrefillSmem {
 //
 // Key columns of an item: the keys are enumerated as one list [band keys lo .. i1, rounded up
 // to 16 | the sink keys before them] and cut into tiles of BN columns: a few sink keys share the last band tile or make
-// a narrow tile of their own, and a tile that is not full runs fewer MMA steps.  In pages lo is rounded down to a tile,
-// so that a tile of band keys lies in one page.  A context-parallel item has n_rem whole tiles from the sink buffer in front.
+// a narrow tile of their own, and a tile that is not full runs fewer MMA steps.  lo is the first key of the window rounded
+// down to 16 keys, so that the columns are whole groups of 16 keys counted from the start of the sequence: a sequence
+// whose length is a multiple of 16 reads no key of the next one (a column that is not visible still counts as 0 * V in the
+// P V product, and V may hold NaN there).  In pages lo is rounded down to a tile, so that a tile of band keys lies in one page.  A context-parallel item has n_rem whole tiles from the sink buffer in front.
 // The scheduler writes the descriptor to shared memory; the other roles read the fields from there as they need them.
 struct WorkItem {
     int valid, seq_start, seq_len;
@@ -371,8 +373,8 @@ struct WorkItem {
             i1 = i0 + n_rows - 1;
         }
         const int first = i0 - p.window + 1;
-        lo = (full || first <= 0) ? 0 : (kPaged ? first / BN * BN : first);
-        nb16 = (i1 + 1 - lo + 15) & ~15;
+        lo = (full || first <= 0) ? 0 : (kPaged ? first / BN * BN : first / 16 * 16);
+        nb16 = (i1 + 1 - lo + 15) / 16 * 16;
         const int ns = full ? 0 : min(n_sink, lo);
         nv = ns > 0 ? nb16 + ns : i1 + 1 - lo;
         n_rem = kCp ? (s_rem + BN - 1) / BN : 0;

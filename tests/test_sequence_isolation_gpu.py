@@ -1,0 +1,32 @@
+"""What a sequence must not see does not reach its results: keys and values of its neighbours in a packed batch that hold
+NaN."""
+import numpy as np
+import pytest
+import torch
+
+from test_prefill_chunked_gpu import make, run_chunked
+from test_prefill_gpu import run_prefill
+
+pytestmark = pytest.mark.gpu
+
+
+def _cu(lens):
+    return torch.tensor(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), device="cuda")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("W,S,full", [(64, 4, False), (100, 0, False), (100, 20, False), (1, 0, True)])
+def test_forward_next_to_a_sequence_of_nan_keys_and_values(D, W, S, full):
+    # key lengths that end on a tile: no key tile on the grid of whole tiles holds keys of two sequences
+    for lq, lk in (((256, 128), (256, 128)), ((256, 128, 77), (640, 256, 77)), ((3, 256, 40), (256, 384, 40))):
+        q, k, v = make(lq, lk, 4, 2, D, 50 + W)
+        want, want_lse, _ = run_chunked(q, k, v, lq, lk, W, S, full)
+        n_q, n_k = sum(lq[:-1]), sum(lk[:-1])
+        k[n_k:] = float("nan")
+        v[n_k:] = float("nan")
+        outs = [run_chunked(q, k, v, lq, lk, W, S, full)]
+        if lq == lk:
+            outs.append(run_prefill(q, k, v, _cu(lq), max(lq), W, S, full))
+        for out, lse, status in outs:
+            assert status == 0
+            assert torch.equal(out[:n_q], want[:n_q]) and torch.equal(lse[:, :n_q], want_lse[:, :n_q]), (lq, lk)
