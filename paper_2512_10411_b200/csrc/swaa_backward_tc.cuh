@@ -279,6 +279,16 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             }
         };
         bool ok = warp_wait(bar(BAR_KV), 0u, abort_flag);
+        if (ok && Lseq - j0 < BK) {
+            // The last key tile of a sequence also holds keys of the next one.  Their dS is 0, but 0 * K is NaN in the dQ
+            // product where such a key is not finite: clear those rows.  (S, dP, dK and dV of a key stay in that key's lane.)
+            for (int c = (Lseq - j0) * 8 + lane; c < BK * 8; c += 32)
+#pragma unroll
+                for (int pn = 0; pn < L::kPanels; ++pn)
+                    st_shared_v4(sK + (uint32_t)(pn * L::kKVPanelBytes + c * 16), 0u, 0u, 0u, 0u);
+            fence_proxy_async_smem();
+            __syncwarp();
+        }
         for (int s = 0; s < NG && s < n_steps && ok; ++s) {
             ok = warp_wait(bar(BAR_QF + s), 0u, abort_flag);
             if (!ok) break;
@@ -428,8 +438,8 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
             // ---- dQ of this step -> [64 rows][D] fp32 in the step's
             // ring stage (Q and dO are no longer needed once dQ is complete) -> bulk reduce-add
-            // into the fp32 accumulator.  Rows past the end of the sequence receive exact zeros (their
-            // dS^T columns are zero); rows past T are clipped by the copy.
+            // into the fp32 accumulator.  Rows past the end of the sequence belong to the next one and receive exact
+            // zeros, whatever this sequence's keys hold; rows past T are clipped by the copy.
             ok = group_all(mbar_wait(bar(BAR_DQ + grp), ph, abort_flag), 1 + grp);
             if (!ok) break;
             tc_fence_after();
@@ -438,6 +448,15 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             tmem_ld32(tX, v0);
             tmem_ld32(tX + 32u, v1);
             tc_wait_ld();
+            if (i0 + BR > Lseq) {
+                // rows of the tile in the sequence: column e of D = 128's dQ^T is row e, lane r of D = 64's quadrant row 16 quad + r
+                const int n = Lseq - i0 - (kWide ? 0 : 16 * quad + lane);
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    v0[e] = (kWide ? e : 0) < n ? v0[e] : 0u;
+                    v1[e] = (kWide ? 32 + e : 0) < n ? v1[e] : 0u;
+                }
+            }
             // the group's columns may take the next S^T as soon as dQ is in registers
             tc_fence_before();
             mbar_arrive(bar(BAR_DR + grp));
