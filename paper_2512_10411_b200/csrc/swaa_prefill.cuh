@@ -1023,6 +1023,10 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             const bool idle = wq * 32 >= n_rows;  // none of this warp's rows exists: it only keeps the barriers going
             float m_used = -INFINITY, l_sum = 0.f;
             const bool careful = uniform(w.careful) != 0;
+            if (careful) {  // the first run of this item stored the same rows: its copies have to be performed before the next ones start
+                if (lane == 0) tma_store_wait_all();
+                __syncwarp();
+            }
             bool fresh = true;   // some row of this warp has no reference yet, or one that is far behind
             for (int n = shared ? side : 0; n < nt; n += shared ? 2 : 1) {
                 // a tile from the sink buffer holds positions before every local key: all rows see exactly its keys

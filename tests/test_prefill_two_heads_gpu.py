@@ -1,0 +1,95 @@
+"""GPU parity of prefill items that take two query heads, one per side: the form of every call with more query tiles than
+SMs / query heads (on 148 SMs at 32 heads: more than 4), for each layout of the keys, at both head sizes.  Small calls take
+one head per item, and so do most shapes of the other prefill tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2512_10411_b200 as swaa
+from paper_2512_10411_b200 import inputs
+from helpers import check_against_oracle
+from test_prefill_chunked_gpu import _cu, make, run_chunked
+from test_prefill_context_parallel_gpu import split
+from test_prefill_gpu import run_prefill
+
+pytestmark = pytest.mark.gpu
+
+HEADS = [(32, 8), (28, 4)]  # an even group, and an odd one, whose last item has a single head
+
+
+def _two_heads(lq, Hq):
+    return min(sum(lq) // 128 + len(lq), len(lq) * -(-max(lq) // 128)) > torch.cuda.get_device_properties(0).multi_processor_count // Hq
+
+
+def _pages(k, v, lk, page, seed):
+    """The same keys in pages of a pool in random order; rows that hold no key are NaN."""
+    blocks = [-(-n // page) for n in lk]
+    perm = torch.as_tensor(np.random.default_rng(seed).permutation(sum(blocks)), device="cuda")
+    table = torch.full((len(lk), max(blocks)), -1, dtype=torch.int32, device="cuda")
+    pools = [torch.full((sum(blocks) * page, *k.shape[1:]), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    start = used = 0
+    for b, n in enumerate(lk):
+        table[b, :blocks[b]] = perm[used:used + blocks[b]].int()
+        rows = (perm[used:used + blocks[b], None] * page + torch.arange(page, device="cuda")).reshape(-1)[:n]
+        for pool, t in zip(pools, (k, v)):
+            pool[rows] = t[start:start + n]
+        start += n
+        used += blocks[b]
+    return [pool.view(-1, page, *k.shape[1:]) for pool in pools], table
+
+
+def _check(layout, lq, lk, Hq, Hkv, D, W, S, full, seed, scale=0.0):
+    assert _two_heads(lq, Hq)
+    q, k, v = make(lq, lk, Hq, Hkv, D, seed)
+    sc = scale if scale > 0 else None
+    what = f"{layout} {lq[:3]} Hq={Hq} D={D} W={W} S={S} full={full} scale={scale}"
+    host = [inputs.to_f32_numpy(t) for t in (q, k, v)]
+    cu_q, cu_k = (np.concatenate([[0], np.cumsum(n)]) for n in (lq, lk))
+    out, lse = torch.full_like(q, float("nan")), torch.full((Hq, sum(lq)), float("nan"), device="cuda")
+    flags = [int(full or b % 2 == 1) for b in range(len(lq))]  # of a batch with a policy per sequence
+    if layout == "self":
+        out, lse, status = run_prefill(q, k, v, _cu(lq), max(lq), W, S, full, scale)
+        assert status == 0
+    elif layout == "chunked":
+        out, lse, status = run_chunked(q, k, v, lq, lk, W, S, full, scale)
+        assert status == 0
+    else:
+        (kp, vp), table = _pages(k, v, lk, 128, seed)
+        fs = torch.tensor(flags, dtype=torch.uint8, device="cuda") if layout == "paged mixed" else None
+        swaa.swaa_prefill_paged(q, kp, vp, out, _cu(lq), torch.tensor(lk, dtype=torch.int32, device="cuda"), table, max(lq), W, S, full,
+                                scale=scale, lse=lse, is_full_seq=fs)
+        assert swaa.last_device_status() == 0
+    ref = oracle.prefill_chunked(*host, cu_q, cu_k, W, S, full, scale=sc, is_full_seq=flags if layout == "paged mixed" else None)
+    check_against_oracle(out, ref["out"], what)
+    np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3, err_msg=what)
+
+
+def _check_context_parallel(lens, Hq, Hkv, D, W, S, seed, P=2, scale=0.0):
+    q, k, v = make(lens, lens, Hq, Hkv, D, seed)
+    for r in range(P):
+        qr, kl, vl, sk, sv, lq, lk, p0, _ = split(q, k, v, lens, r, P, W, S)
+        assert _two_heads(lq, Hq)
+        out, lse = torch.full_like(qr, float("nan")), torch.full((Hq, sum(lq)), float("nan"), device="cuda")
+        swaa.swaa_prefill_context_parallel(qr, kl, vl, sk, sv, out, _cu(lq), _cu(lk), torch.tensor(p0, dtype=torch.int32, device="cuda"),
+                                           max(lq), max(lk), W, S, scale=scale, lse=lse)
+        assert swaa.last_device_status() == 0
+        ref = oracle.prefill_cp(*(inputs.to_f32_numpy(t) for t in (qr, kl, vl, sk, sv)), _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(),
+                                p0, W, S, False, scale=scale if scale > 0 else None)
+        check_against_oracle(out, ref["out"], f"context-parallel rank {r} Hq={Hq} D={D} W={W} S={S} scale={scale}")
+        np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("layout", ["self", "chunked", "paged", "paged mixed", "context-parallel"])
+def test_items_that_are_run_again(layout, D):
+    """|scaled scores| reach 1350: rows grow by far more than 60 in log2 units from one tile to the next, and items of full
+    128-row tiles, whose rows leave by tensor copies, are run again and store the same rows twice."""
+    lq = (300, 129, 517, 128)
+    lk = lq if layout == "self" else (300, 400, 600, 900)
+    for W, S, full in ((1, 0, True), (300, 4, False)):
+        for _ in range(3):
+            if layout != "context-parallel":
+                _check(layout, lq, lk, 32, 8, D, W, S, full, 300 + D, scale=30.0)
+            elif not full:
+                _check_context_parallel((900, 300, 601), 32, 8, D, W, S, 310 + D, scale=30.0)
