@@ -312,8 +312,8 @@ struct PrefillSmem {
     static constexpr int kOffBar = kOffMerge + 128 * 8;
     // barriers: Q full/empty; full/empty/V-tile-cleared (paged keys only) per slot; per side S full / P ready / O done /
     // O free; work descriptor full/empty per slot, next-block answer, hand-over of packed items per row quadrant,
-    // staging free, final
-    static constexpr int kNumBars = 2 + 3 * kSlots + 2 * 4 + 5 + 4 + 2;
+    // staging free per work slot, final
+    static constexpr int kNumBars = 2 + 3 * kSlots + 2 * 4 + 5 + 4 + 3;
     static constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) / 16 * 16;  // next-block answer, tmem slot, flags, work descriptors
     static constexpr int kBytes = kOffMisc + 32 + 2 * kWorkInts * 4;
     static constexpr int kDynamicBytes = kBytes + 1024;          // room to align the base to 1024 B
@@ -451,9 +451,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     // per side: S full; P ready; O done, O free
     constexpr int BAR_SF = BAR_VC + NS, BAR_PR = BAR_SF + 2, BAR_OD = BAR_PR + 2, BAR_OF = BAR_OD + 2;
     // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), staging free
-    // for the ring of a packed item, final
+    // for the ring of a packed item (per work slot), final
     constexpr int BAR_WF = BAR_OF + 2, BAR_WE = BAR_WF + 2, BAR_NB = BAR_WE + 2, BAR_MG = BAR_NB + 1, BAR_SG = BAR_MG + 4;
-    constexpr int BAR_FIN = BAR_SG + 1;
+    constexpr int BAR_FIN = BAR_SG + 2;
     static_assert(BAR_FIN + 1 == L::kNumBars, "barrier count");
     const uint32_t s_answer = smem_base + L::kOffMisc;  // 16 bytes
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc + 16);
@@ -472,7 +472,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             uint32_t count = 1u;
             if ((i >= BAR_PR && i < BAR_OD) || i == BAR_OF || i == BAR_OF + 1) count = 4u;  // a lane of each softmax warp of the side
             if (i == BAR_WE || i == BAR_WE + 1) count = 10u;   // producer, issuer, eight softmax warps
-            if (i == BAR_SG) count = 8u;                       // a lane of each softmax warp
+            if (i == BAR_SG || i == BAR_SG + 1) count = 8u;    // a lane of each softmax warp
             mbar_init(bar(i), count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -665,7 +665,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         const bool el = elect_one();
         uint32_t phases = 0;             // bit: parity of the slot's next use
         int sk = 0, sv = 0, sx = 0;      // next stage of the K and V rings, next slot of a packed item's ring
-        uint32_t packed_items = 0;
+        uint32_t sg_phase = 0;           // bit: parity of the work slot's next packed item
         bool ok = true;
         int items = 0;
         for (int it = 0; ok; ++it) {
@@ -782,9 +782,12 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 // A generated token at a long context runs at the pace of memory, and how far the copies run ahead sets it: with
                 // the two K and two V slots of the usual items one token at 32768 keys takes 421 us, 16 of them 499 us, a
                 // serving step of 4 chunks and 24 generated tokens 805 us; with all six slots 363, 430 and 595 us.
+                // Every softmax warp says once per packed item that it has no store from the staging under way.  The warps of a
+                // side without work run ahead into the next item, so the barrier goes with the work slot: a slot takes another
+                // item only when all roles have released this one, that is after all of its eight arrivals and this wait.
                 bool staging = false;  // the output staging is known to be free
-                auto wait_staging = [&]() {  // once per packed item, so that the barrier is never two phases ahead
-                    if (!staging) ok = ok && warp_wait(bar(BAR_SG), packed_items & 1u, abort_flag);
+                auto wait_staging = [&]() {
+                    if (!staging) ok = ok && warp_wait(bar(BAR_SG + (it & 1)), (sg_phase >> (it & 1)) & 1u, abort_flag);
                     staging = true;
                 };
                 auto next_slot = [&]() -> int {
@@ -804,7 +807,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     }
                 }
                 wait_staging();
-                ++packed_items;
+                sg_phase ^= 1u << (it & 1);
             }
             if (!ok) break;
             release_work(it);
@@ -1012,7 +1015,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             const bool shared = packed && uniform(w.shared) != 0;
             if (kDeepRing && packed && lane == 0) {  // the item's ring takes the staging area: earlier output stores have read it
                 tma_store_wait_read();
-                mbar_arrive(bar(BAR_SG));
+                mbar_arrive(bar(BAR_SG + (it & 1)));
             }
             if (side == 1 && !shared && !uniform(w.hasB)) {
                 release_work(it);

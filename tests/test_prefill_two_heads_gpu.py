@@ -93,3 +93,16 @@ def test_items_that_are_run_again(layout, D):
                 _check(layout, lq, lk, 32, 8, D, W, S, full, 300 + D, scale=30.0)
             elif not full:
                 _check_context_parallel((900, 300, 601), 32, 8, D, W, S, 310 + D, scale=30.0)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("layout", ["chunked", "paged mixed"])
+def test_tokens_of_short_context_behind_items_of_one_head(layout, D):
+    """Seven heads per kv head: every fourth item of a prompt has one head, and side B goes ahead to the tokens behind it, whose
+    keys fit in one tile and which leave side B without work too; their key ring takes the area from which side A may still
+    be storing."""
+    rng = np.random.default_rng(8)
+    lq = (900, 517, 300) + (1,) * 150
+    lk = (900, 700, 300) + tuple(int(x) for x in rng.integers(1, 129, 150))
+    for _ in range(4):
+        _check(layout, lq, lk, 28, 4, D, 128, 4, False, 400 + D)
