@@ -422,6 +422,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 mbar_arrive(bar(BAR_QE + pending_stage));
                 pending_stage = -1;
             }
+            __syncwarp();  // the tensor-memory loads below need all lanes together
             const float* rows = s_rows + st * 128;
             const bool need_mask = i0 + BR > Lseq || tile_needs_mask(i0, i1, j0, j1, p.window, p.n_sink, full);
             if (need_mask) {

@@ -235,7 +235,8 @@ constexpr uint32_t kPolyPairMask = 0x8420u;
 #define SWAA_I8(r, o) "r"(r[o + 0]), "r"(r[o + 1]), "r"(r[o + 2]), "r"(r[o + 3]), "r"(r[o + 4]), "r"(r[o + 5]), "r"(r[o + 6]), "r"(r[o + 7])
 
 // 32 lanes x 32 consecutive columns: thread `lane` of the warp receives columns c .. c+31 of TMEM
-// lane (quadrant base + lane).
+// lane (quadrant base + lane).  These and the waits for them are .aligned: all lanes have to arrive together, so a branch that
+// only some lanes take (a lane that arrives on a barrier, rows that do not exist) is closed with a __syncwarp first.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -501,6 +502,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     auto release_work = [&](int it) {
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(BAR_WE + (it & 1)));
+        __syncwarp();
     };
     auto uniform = [](int x) -> int { return __shfl_sync(0xffffffffu, x, 0); };
 
@@ -1017,6 +1019,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 tma_store_wait_read();
                 mbar_arrive(bar(BAR_SG + (it & 1)));
             }
+            __syncwarp();
             if (side == 1 && !shared && !uniform(w.hasB)) {
                 release_work(it);
                 continue;
@@ -1213,7 +1216,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     // largest argument.  Far out of range (also: not a number) the whole item is run again, forming every
                     // tile's maximum.
                     fresh = true;
-                    if (__any_sync(0xffffffffu, row_ok && !(sum <= kSumLimit && hi <= 60.f)) && lane == 0) s_again[it & 1] = 1;
+                    if (__any_sync(0xffffffffu, row_ok && !(sum <= kSumLimit && hi <= 60.f))) s_again[it & 1] = 1;  // all lanes the same
                 }
                 if (!kLseOnly) tc_wait_st();
                 tc_fence_before();
@@ -1277,6 +1280,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
 #pragma unroll 1
                 for (int cc = 0; cc < D / 32; ++cc) {
                     uint32_t o[32], ob[32];
+                    __syncwarp();  // behind the stores of rows that exist
                     tmem_ld32(tO + (uint32_t)(cc * 32), o);
                     tmem_ld32(tO + (uint32_t)(D + cc * 32), ob);
                     tc_wait_ld();
