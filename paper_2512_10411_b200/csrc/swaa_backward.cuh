@@ -42,9 +42,9 @@ constexpr int kBwdChunkTiles = 32;  // query tiles (64 rows) per block of a sink
 // input per lane, which also clear the row of the fp32 dq accumulator.  Bound by memory: 2 * 2 D bytes read and 4 D bytes
 // written per row.
 template <int D>
-__global__ void backward_delta_kernel(const __nv_bfloat16* __restrict__ out, const __nv_bfloat16* __restrict__ dout,
-                                      const float* __restrict__ lse, float* __restrict__ delta,
-                                      float* __restrict__ lse2, float* __restrict__ dq_accum, int T, int Hq) {
+__global__ void backward_delta_kernel(const __nv_bfloat16* out, const __nv_bfloat16* dout,
+                                      const float* lse, float* delta,
+                                      float* lse2, float* dq_accum, int T, int Hq) {
     grid_wait();
     constexpr int kLanes = D / 8;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -53,8 +53,8 @@ __global__ void backward_delta_kernel(const __nv_bfloat16* __restrict__ out, con
     const bool in = row < (long long)T * Hq;  // whole groups of kLanes lanes
     float acc = 0.f;
     if (in) {
-        const uint4 a = __ldg(reinterpret_cast<const uint4*>(out + row * D) + l);
-        const uint4 b = __ldg(reinterpret_cast<const uint4*>(dout + row * D) + l);
+        const uint4 a = reinterpret_cast<const uint4*>(out + row * D)[l];
+        const uint4 b = reinterpret_cast<const uint4*>(dout + row * D)[l];
         const uint32_t av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
         float4* acc_row = reinterpret_cast<float4*>(dq_accum + row * D);
         acc_row[l] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -76,7 +76,7 @@ __global__ void backward_delta_kernel(const __nv_bfloat16* __restrict__ out, con
 }
 
 // dq = bf16(dq_accum)
-__global__ void backward_convert_dq_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dq, size_t n) {
+__global__ void backward_convert_dq_kernel(const float* acc, __nv_bfloat16* dq, size_t n) {
     grid_wait();
     const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (i + 3 < n) {
@@ -88,8 +88,8 @@ __global__ void backward_convert_dq_kernel(const float* __restrict__ acc, __nv_b
 }
 
 // dk, dv rows of the split key tiles = bf16(dkv_accum); one thread per four channels of one (b, row, kv head).
-__global__ void backward_convert_dkv_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dk,
-                                            __nv_bfloat16* __restrict__ dv, const int32_t* __restrict__ cu_seqlens, int B,
+__global__ void backward_convert_dkv_kernel(const float* acc, __nv_bfloat16* dk,
+                                            __nv_bfloat16* dv, const int32_t* cu_seqlens, int B,
                                             int T, int max_seqlen, int sink_rows, int Hkv, int D) {
     grid_wait();
     const size_t plane = (size_t)B * sink_rows * Hkv * D;

@@ -153,8 +153,8 @@ struct DecodeWalker {
     int b, set, ti;
     SeqGeom s;
     static __device__ __forceinline__ SeqGeom geom(const DecodeParams& p, int b) {
-        if (kShard) return decode_shard_geom(__ldg(p.seqlens + b), p.Lmax, p.pos0, p.window, p.n_sink, p.is_full);
-        return decode_seq_geom(__ldg(p.seqlens + b), p.Lmax, p.window, p.n_sink, p.is_full, kPaged);
+        if (kShard) return decode_shard_geom(p.seqlens[b], p.Lmax, p.pos0, p.window, p.n_sink, p.is_full);
+        return decode_seq_geom(p.seqlens[b], p.Lmax, p.window, p.n_sink, p.is_full, kPaged);
     }
     __device__ __forceinline__ void seek(const DecodeParams& p, int b0, long long off) {
         b = b0;
@@ -259,7 +259,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
     // rows.  Shard: also what a shard that holds none of the sequence's visible keys looks like; its rows get the
     // empty partial (-inf, 0, 0...), and only a length < 1 is an error.  One block does the stores.
     auto zero_fill_bad = [&](int b) {
-        if (!kShard || __ldg(p.seqlens + b) < 1) record_device_error(SWAA_ERR_BAD_SEQLENS);
+        if (!kShard || p.seqlens[b] < 1) record_device_error(SWAA_ERR_BAD_SEQLENS);
         if (b % ncta == cta) {
             if (kShard) {
                 float* o = p.part_out + (size_t)b * p.Hq * (D + 2);
@@ -373,7 +373,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
                 int c2 = key0, c3 = w.b;  // TMA coordinates: (entry, sequence) or (row in page, page)
                 if (kPaged) {
                     const int tile = key0 / kDecodeTileKeys;
-                    c3 = __ldg(p.block_table + (size_t)w.b * p.max_blocks + tile / p.page_tiles);
+                    c3 = p.block_table[(size_t)w.b * p.max_blocks + tile / p.page_tiles];
                     c2 = (tile % p.page_tiles) * kDecodeTileKeys;
                     if (c3 < 0 || c3 >= p.num_pages) {
                         record_device_error(SWAA_ERR_BAD_SEQLENS);
@@ -446,8 +446,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
             const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + ((size_t)b * p.Hq + h0 + (hh < gc ? hh : 0)) * D);
 #pragma unroll
             for (int kk = 0; kk < NKK; ++kk) {
-                qf[nh][kk][0] = hh < gc ? __ldg(qrow + kk * 8 + c) : 0u;
-                qf[nh][kk][1] = hh < gc ? __ldg(qrow + kk * 8 + c + 4) : 0u;
+                qf[nh][kk][0] = hh < gc ? qrow[kk * 8 + c] : 0u;
+                qf[nh][kk][1] = hh < gc ? qrow[kk * 8 + c + 4] : 0u;
             }
         }
         float m_run[NH][2], l_run[NH][2], oacc[NH][NKK][4];
@@ -716,7 +716,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ 
 // part [P][rows][D + 2] = (max in natural-log units, sum, unnormalised O); empty partials (sum == 0) are skipped; a
 // row without any non-empty partial gives zeros.
 template <int D>
-__global__ void decode_combine_kernel(const float* __restrict__ part, int P, int rows, __nv_bfloat16* __restrict__ out) {
+__global__ void decode_combine_kernel(const float* part, int P, int rows, __nv_bfloat16* out) {
     grid_wait();
     const int row = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (row >= rows) return;

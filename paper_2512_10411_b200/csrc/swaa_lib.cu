@@ -843,8 +843,8 @@ extern "C" int swaa_prefill_backward(const void* q, const void* k, const void* v
 namespace swaa {
 
 // ratio[h] = mean over t of exp(lse_recent[h, t] - lse_full[h, t]); one block per head.
-__global__ void lazy_ratio_reduce_kernel(const float* __restrict__ lse_recent, const float* __restrict__ lse_full,
-                                         int Tq, float* __restrict__ ratio) {
+__global__ void lazy_ratio_reduce_kernel(const float* lse_recent, const float* lse_full,
+                                         int Tq, float* ratio) {
     __shared__ float warp_sums[8];
     grid_wait();
     const int h = blockIdx.x;

@@ -702,7 +702,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             ++items;
             // page of a key, out of range (the copy delivers zeros) when the table is wrong
             auto page_of = [&](int key) -> int {
-                const int page = __ldg(p.block_table + (size_t)k_start * p.max_blocks + key / p.page_size);
+                const int page = p.block_table[(size_t)k_start * p.max_blocks + key / p.page_size];
                 if (page >= 0 && page < p.num_pages) return page;
                 record_device_error(SWAA_ERR_BAD_SEQLENS);
                 return p.num_pages;

@@ -11,6 +11,8 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 
 // Waits until the kernel before this one on the stream has ended and its writes are visible.  Every thread of every kernel
 // calls it before it touches global memory (see launch_overlapped), so the order of the stream's work is unchanged.
+// Nothing is read through __ldg or const __restrict__ pointers: those promise that the data does not change while the kernel
+// is resident, which the kernel before it may still be writing, and let the compiler move a load above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

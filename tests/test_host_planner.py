@@ -193,3 +193,13 @@ def test_backward_workspace_size_covers_its_parts(_lib):
         want = base + 2 * B * rows * Hkv * D * 4
         assert want <= size(B, T, Hq, Hkv, D, n_sink) <= want + 3 * 256, n_sink
     assert size(0, T, Hq, Hkv, D, 4) == 256 and size(B, T, Hq, Hkv, D, -1) == 256  # invalid shapes: the minimum
+
+
+def test_kernels_promise_no_read_only_data():
+    """Every kernel may be resident while the one before it on the stream still writes what it reads: no load may go through
+    the read-only path or be moved ahead of the wait for that kernel."""
+    csrc = os.path.join(ROOT, "paper_2512_10411_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        with open(os.path.join(csrc, name)) as f:
+            code = re.sub(r"//[^\n]*", "", f.read())
+        assert "__ldg" not in code and "__restrict__" not in code and "ld.global.nc" not in code, name
