@@ -540,7 +540,7 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
 
     const int G = Hq / Hkv;
     const int pack_tokens = ex.lse_only ? 0 : kPrefillBM / G;
-    PrefillMaps tm;
+    PrefillMaps tm = {};  // maps that the call has no use for stay zero
     if ((rc = make_token_major_map(&tm.q, q, Tq, Hq, D)) != SWAA_OK) return rc;
     if (pack_tokens > 0 && (rc = make_token_major_map(&tm.q_packed, q, Tq, Hq, D, pack_tokens, G)) != SWAA_OK) return rc;
     if (is_paged) {  // (D, Hkv, page_size, num_pages), boxes of rows of one page

@@ -480,7 +480,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     }
     if (warp == 8 && elect_one()) {
         prefetch_map(&tm.q);
-        prefetch_map(&tm.q_packed);
+        if (p.pack_tokens > 0) prefetch_map(&tm.q_packed);
         prefetch_map(&tm.k);
         prefetch_map(&tm.v);
     }
