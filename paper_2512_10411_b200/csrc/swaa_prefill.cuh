@@ -47,6 +47,7 @@ constexpr int kPrefillThreads = 384;  // 8 softmax warps + 4 auxiliary warps (pr
 constexpr int kPrefillSmallBox = 16;                        // rows of the small TMA boxes over K and V
 constexpr int kWorkInts = 24;                               // words of a work descriptor
 constexpr float kRescaleThreshold = 8.0f;                   // log2 units
+constexpr float kGrowLimit = 32768.f;                       // 2^15: row sum of a tile above which the reference is looked at
 constexpr float kSumLimit = 1.152921504606847e18f;          // 2^60: row sum of a tile above which the item is run again
 
 struct PrefillParams {
@@ -998,9 +999,10 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
         const uint32_t tS = tmem_base + lane_base + (uint32_t)side * 128u;
         const uint32_t tO = tmem_base + lane_base + 256u + (uint32_t)side * (uint32_t)D;
-        // phases (bits) of: S full, O done (side A also keeps side B's), hand-over of packed items
+        // phases (bits) of: S full, O done (side A also keeps side B's), hand-over of packed items; and of the item:
+        // some tile's scores outgrew the reference of a row of this warp by far
         uint32_t phases = 0;
-        constexpr uint32_t kPhS = 1u, kPhO = 2u, kPhOB = 4u, kPhM = 8u;
+        constexpr uint32_t kPhS = 1u, kPhO = 2u, kPhOB = 4u, kPhM = 8u, kGrown = 16u;
         bool ok = true;
         auto arrive_warp = [&](int b) {
             __syncwarp();
@@ -1109,8 +1111,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 // Usual tile: the exponentials are taken against the reference as it stands, without forming the tile's maximum
                 // first (64 of some 600 instructions per row and tile; 3.5 % of the kernel's time at 32k tokens).  That loses
                 // no precision as long as nothing leaves the exponent range: bf16 P and the fp32 sums do not mind a common
-                // factor.  Masked tiles, and the tile after one whose scores outgrew the reference by 2^16, do form the
-                // maximum, and raise the reference where it is more than 2^8 behind.
+                // factor.  Masked tiles, and the tile after one whose row sum came out above 2^15 (the most that 128 scores
+                // within 2^8 of the reference give), do form the maximum, and raise the reference where it is more than 2^8
+                // behind.
                 const bool exact = need_mask || fresh || careful;
                 if (exact) {
                     tc_wait_ld();
@@ -1211,11 +1214,13 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     sum = a0 + a1;
                 }
                 l_sum += sum;
-                if (!exact && __any_sync(0xffffffffu, row_ok && !(sum <= 65536.f && hi <= 16.f))) {
+                if (!exact && __any_sync(0xffffffffu, row_ok && !(sum <= kGrowLimit && hi <= 15.f))) {
                     // Growth shows in the row sum, except in the columns of the polynomial path: those are bounded by their
                     // largest argument.  Far out of range (also: not a number) the whole item is run again, forming every
-                    // tile's maximum.
+                    // tile's maximum.  Up to there P and its sums are as precise as ever, and whether O stayed finite, which
+                    // depends on the values too, is looked at when the item is done.
                     fresh = true;
+                    phases |= kGrown;
                     if (__any_sync(0xffffffffu, row_ok && !(sum <= kSumLimit && hi <= 60.f))) s_again[it & 1] = 1;  // all lanes the same
                 }
                 if (!kLseOnly) tc_wait_st();
@@ -1229,6 +1234,24 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 if (!ok) break;
                 phases ^= kPhO;
                 tc_fence_after();
+                if ((phases & kGrown) != 0) {  // an accumulator that left the range of fp32: the item is run again
+                    phases &= ~kGrown;
+                    uint32_t top = 0;  // largest magnitude (bits) of the row; no branch in which lanes could differ
+#pragma unroll 1
+                    for (int cc = 0; cc < D / 32; ++cc) {
+                        uint32_t o[32];
+                        __syncwarp();
+                        tmem_ld32(tO + (uint32_t)(cc * 32), o);
+                        tc_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 32; ++e) {
+                            asm volatile("" : "+r"(o[e]));  // behind the wait
+                            top = max(top, o[e] & 0x7fffffffu);
+                        }
+                    }
+                    if (__any_sync(0xffffffffu, row_ok && top >= 0x7f800000u)) s_again[it & 1] = 1;
+                    __syncwarp();
+                }
             }
             const int q_off = packed && w.packed > 1 ? row / p.G : row;
             const int q_row = w.q0 + q_off;  // this thread's query, counted inside the sequence
