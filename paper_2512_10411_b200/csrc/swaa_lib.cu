@@ -89,12 +89,14 @@ static DecodePlan plan_decode(int B, int Hq, int Hkv, int D, int Lmax, int windo
     if (groups > most) groups = most;
     if (groups < 1) groups = 1;
     // A batch of equal lengths (or of equal windows) is cut over a group count that lets every group own whole items, or
-    // cuts every item into the same number of parts: no partial results to merge, and the groups end together.  Batch of 16,
-    // Hkv = 8, D = 128, 16 groups against 18: 43.3 us against 49.8 at 4100 visible entries each, 84.2 against 91.4 at 8196,
-    // 624 against 673 at 65536 (on another GPU 662 against 629).  Ragged batches use every group: 64 sequences of 512 to
-    // 32768 entries 270 us with 18 groups, 281 with 16.  The lengths are known on the device only: it chooses, except where a
-    // run has at most 3/2 * D tiles.  There the grid itself is cut to the smaller count (43.3 us as above; 47.4 where blocks
-    // come in only to find that they have no work), ragged or not.
+    // cuts every item into the same number of parts: no partial results to merge, and the groups end together.  Ragged batches
+    // want every group.  The lengths are known on the device only: it chooses.  Blocks that come in only to find that they
+    // have no work still cost the others at D = 128, so there the grid itself is cut to the smaller count, ragged or not,
+    // where a run has at most 192 tiles.  Hkv = 8, us with the grid cut and with the choice on the device:
+    //   D = 128, equal:  16 sequences of 4100 visible entries 44 and 47-49, 2048 25 and 28, 8192 81 and 88; 16384 (past the
+    //                    line) 167 and 167-172; 14, 15 and 17 sequences of 4100 within 3 %.
+    //   D = 128, ragged: 14 to 17 sequences under a window of 4096 44, 43, 39, 48 and 39, 42, 40, 44; 16384 92-95 and 92.
+    //   D = 64,  equal:  within 1 % throughout.  Ragged: the same four 32, 29, 34, 35 and 27, 28, 33, 33; 16384 69-82 and 54-73.
     pl.groups_equal = (int)groups;
     if (groups == most) {
         for (long long g = most; g * 4 >= most * 3; --g)
@@ -103,7 +105,7 @@ static DecodePlan plan_decode(int B, int Hq, int Hkv, int D, int Lmax, int windo
                 break;
             }
     }
-    if (2 * tiles_ub <= 3 * D * groups) groups = pl.groups_equal;
+    if (D == 128 && tiles_ub <= 192 * groups) groups = pl.groups_equal;
     const long long blocks = groups * pl.hs;
     pl.blocks = (int)blocks;
     pl.too_large = tiles_ub / pl.groups_equal > 0x3fffffffLL;  // the kernel counts a block's tiles in an int

@@ -163,6 +163,15 @@ def test_decode_split_plan_is_consistent():
     assert swaa.decode_num_blocks(1, 4, 2, 64, 100, 8, 0, 0) == 1
 
 
+def test_decode_grid_is_cut_to_whole_items_for_short_runs_at_head_size_128_only():
+    # 8 heads in step, 18 groups at most on 148 SMs; 14 sequences own whole items over 14 groups
+    assert swaa.decode_num_blocks(14, 32, 8, 128, 16384, 4096, 4, 0) == 14 * 8
+    assert swaa.decode_num_blocks(14, 32, 8, 128, 12200, 1, 0, 1) == 14 * 8   # 14 * 192 tiles over 14 of 18 groups
+    assert swaa.decode_num_blocks(14, 32, 8, 128, 65536, 1, 0, 1) == 18 * 8
+    assert swaa.decode_num_blocks(14, 32, 8, 64, 16384, 4096, 4, 0) == 18 * 8
+    assert swaa.decode_num_blocks(14, 32, 8, 64, 65536, 1, 0, 1) == 18 * 8
+
+
 def test_trimmed_cache_holds_exactly_the_visible_keys():
     """Appending tokens 0 .. len-1 into the trimmed cache leaves, in its occupied slots, exactly the positions
     the oracle's SWA predicate shows to the decode query at position len-1 (App. A)."""
