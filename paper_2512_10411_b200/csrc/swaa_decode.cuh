@@ -46,8 +46,7 @@ struct DecodeParams {
     const int32_t* seqlens;
     int B, Lmax, Hq, Hkv, G;
     int HG;        // head chunks per kv head (each chunk holds up to 8*NH query heads)
-    int IPB;       // items per sequence = Hkv * HG
-    int hs, sets;  // items streamed in step by a group of hs blocks; sets of hs items per sequence = IPB / hs
+    int hs, sets;  // items streamed in step by a group of hs blocks; sets of hs items per sequence = Hkv * HG / hs
     int groups_equal;  // groups that a batch whose sequences have the same number of tiles is cut over
     int window, n_sink, is_full;
     float sl2;     // softmax scale * log2(e)

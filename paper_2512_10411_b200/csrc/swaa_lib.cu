@@ -325,9 +325,8 @@ static int decode_impl(const void* q, const void* kcache, const void* vcache, vo
     p.Hkv = Hkv;
     p.G = Hq / Hkv;
     p.HG = pl.HG;
-    p.IPB = Hkv * pl.HG;
     p.hs = pl.hs;
-    p.sets = p.IPB / pl.hs;
+    p.sets = Hkv * pl.HG / pl.hs;
     p.groups_equal = pl.groups_equal;
     p.window = window;
     p.n_sink = n_sink;
