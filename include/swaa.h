@@ -347,9 +347,21 @@ int swaa_schedule_select_fa_layers(const float* ratio, int n_layers, int n_heads
                                    uint8_t* fa_mask_out);
 
 /*
- * Key tiles, on a grid of whole tiles, that hold a key visible to a query tile, for host-side verification (App. A: only
- * O(N*W) work; the kernel itself cuts the same keys from the first one on, sinks behind the band).  For the query tile of
- * rows [m*BM, min(L, (m+1)*BM)) of a sequence of length L, the tiles (of BN keys) are 0 .. *n_sink_tiles-1 and *n_lo .. *n_hi.  Returns SWAA_OK or
+ * Key columns of one prefill work item, as the kernel enumerates and masks them, for host-side verification (App. A: only
+ * O(N*W) work).  The item holds the n_rows (at most swaa_prefill_block_m) queries at indices i0 .. i0+n_rows-1 among the
+ * len_k keys of its sequence; paged != 0: keys in pages; s_rem > 0 (context-parallel): sink keys that come from the sink
+ * buffer, with n_sink further ones at the start of the local keys.  Writes, tile after tile of swaa_prefill_block_n columns,
+ *   keys[c]  index of the column's key (-s_rem .. -1: from the sink buffer), INT32_MAX where the column holds none
+ *   seen[c]  1 where query i0 + row takes the column
+ * and returns the number of columns, SWAA_ERR_INVALID_ARG, or SWAA_ERR_WORKSPACE when that is above max_columns.
+ */
+int swaa_prefill_item_keys(int len_k, int i0, int n_rows, int window, int n_sink, int is_full, int paged, int s_rem, int row,
+                           int max_columns, int32_t* keys, uint8_t* seen);
+
+/*
+ * Key tiles of a grid of whole tiles that hold a key visible to a query tile (host only; the prefill kernel's own columns
+ * are those of swaa_prefill_item_keys).  For the query tile of rows [m*BM, min(L, (m+1)*BM)) of a sequence of length L, the
+ * tiles (of BN keys) are 0 .. *n_sink_tiles-1 and *n_lo .. *n_hi.  Returns SWAA_OK or
  * SWAA_ERR_INVALID_ARG.  swaa_prefill_tile_needs_mask returns 1 when some (row, key) pair of the
  * tile is not visible (the element predicate is then needed), 0 when every pair is visible.
  */

@@ -12,6 +12,7 @@ from .binding import (  # noqa: F401
     decode_workspace_size,
     kernel_launch_count,
     prefill_block_shape,
+    prefill_item_keys,
     prefill_tile_needs_mask,
     prefill_tile_range,
     lib_path,

@@ -117,6 +117,8 @@ def load_library():
     lib.swaa_schedule_select_fa_layers.restype = ci
     lib.swaa_prefill_tile_range.argtypes = [ci] * 7 + [ctypes.POINTER(ci)] * 3
     lib.swaa_prefill_tile_range.restype = ci
+    lib.swaa_prefill_item_keys.argtypes = [ci] * 10 + [vp, vp]
+    lib.swaa_prefill_item_keys.restype = ci
     lib.swaa_prefill_tile_needs_mask.argtypes = [ci] * 8
     lib.swaa_prefill_tile_needs_mask.restype = ci
     lib.swaa_prefill_block_m.restype = ci
@@ -514,6 +516,17 @@ def prefill_tile_needs_mask(L, m, n, BM, BN, window, n_sink, is_full) -> bool:
     if rc < 0:
         raise SwaaError(rc, "swaa_prefill_tile_needs_mask")
     return bool(rc)
+
+
+def prefill_item_keys(len_k, i0, n_rows, window, n_sink, is_full, row, paged=False, s_rem=0):
+    """Forwards to C swaa_prefill_item_keys: (keys, seen) of the item's columns, two lists."""
+    cap = 128 * (len_k // 128 + s_rem // 128 + n_sink // 128 + 5)
+    keys, seen = (ctypes.c_int32 * cap)(), (ctypes.c_uint8 * cap)()
+    n = load_library().swaa_prefill_item_keys(len_k, i0, n_rows, int(window), int(n_sink), int(bool(is_full)), int(bool(paged)),
+                                              s_rem, row, cap, ctypes.addressof(keys), ctypes.addressof(seen))
+    if n < 0:
+        raise SwaaError(n, "swaa_prefill_item_keys")
+    return keys[:n], seen[:n]
 
 
 def prefill_block_shape():

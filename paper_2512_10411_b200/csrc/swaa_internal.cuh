@@ -25,16 +25,14 @@ inline std::atomic<uint64_t>& launch_counter() {
 }
 
 // ---------------------------------------------------------------- tile arithmetic (host + device)
-// Key tiles visited by the query tile of rows [i0, i1] (positions inside one sequence), App. A: only
-// the tiles holding a visible key are enumerated, which makes prefill work linear in L at fixed W.
+// Key tiles of a grid of whole tiles that hold a key visible to the query tile of rows [i0, i1] (positions inside one
+// sequence), App. A: their number is linear in L at fixed W.  Host only; the prefill kernel's columns are WorkItem's.
 struct TileRange {
     int n_sink_tiles;  // tiles 0 .. n_sink_tiles-1 hold sink keys that lie before the band
     int n_lo, n_hi;    // band (or, for full attention, whole causal prefix): tiles n_lo .. n_hi
-    __host__ __device__ int count() const { return n_sink_tiles + (n_hi - n_lo + 1); }
-    __host__ __device__ int tile(int t) const { return t < n_sink_tiles ? t : n_lo + (t - n_sink_tiles); }
 };
 
-__host__ __device__ inline TileRange tile_range(int i0, int i1, int BN, int W, int S, bool is_full) {
+inline TileRange tile_range(int i0, int i1, int BN, int W, int S, bool is_full) {
     TileRange r;
     r.n_hi = i1 / BN;
     if (is_full) {

@@ -988,7 +988,7 @@ extern "C" long long swaa_trimmed_cache_len(long long len, int window, int n_sin
     return len < cap ? len : cap;
 }
 
-// ------------------------------------------------------------------------------- tile enumeration
+// ------------------------------------------------------------------------ key enumeration on the host
 extern "C" int swaa_prefill_block_m(void) { return kPrefillBM; }
 extern "C" int swaa_prefill_block_n(void) { return kPrefillBN; }
 
@@ -1014,6 +1014,40 @@ extern "C" int swaa_prefill_tile_needs_mask(int L, int m, int n, int BM, int BN,
     const int i0 = m * BM;
     const int i1 = (L < i0 + BM ? L : i0 + BM) - 1;
     return tile_needs_mask(i0, i1, n * BN, n * BN + BN - 1, window, n_sink, is_full != 0) ? 1 : 0;
+}
+
+extern "C" int swaa_prefill_item_keys(int len_k, int i0, int n_rows, int window, int n_sink, int is_full, int paged, int s_rem,
+                                      int row, int max_columns, int32_t* keys, uint8_t* seen) {
+    constexpr int BN = kPrefillBN;
+    if (i0 < 0 || n_rows < 1 || n_rows > kPrefillBM || len_k < i0 + n_rows || n_sink < 0 || s_rem < 0 || row < 0 || row >= n_rows ||
+        (!is_full && window < 1) || (paged && s_rem > 0) || !keys || !seen)
+        return SWAA_ERR_INVALID_ARG;
+    PrefillParams p = {};
+    p.heads = p.units_per_kv = p.G = 1;
+    p.window = is_full ? 1 : window;
+    WorkItem w = {};
+    w.seq_len = n_rows;
+    w.k_off = i0;
+    w.full = is_full ? 1 : 0;
+    w.n_sink = n_sink;
+    w.s_rem = s_rem;
+    if (paged) w.complete<BN, true, false, false>(p, 0);
+    else if (s_rem > 0) w.complete<BN, false, true, false>(p, 0);
+    else w.complete<BN, false, false, false>(p, 0);
+    if ((long long)w.nt * BN > max_columns) return SWAA_ERR_WORKSPACE;
+    for (int t = 0; t < w.nt; ++t) {
+        const bool remote = t < w.n_rem;
+        const TileGeom<BN> g(w, t);
+        const auto v = g.seen(w, t, remote, w.i0 + row, p.window);
+        const bool mask = g.needs_mask(w, t, remote, p.window);
+        for (int c = 0; c < BN; ++c) {
+            const bool run = remote || c < 16 * g.nk;
+            const int key = !remote ? g.key(c) : (t * BN + c < s_rem ? t * BN + c - s_rem : INT32_MAX);
+            keys[t * BN + c] = run ? key : INT32_MAX;
+            seen[t * BN + c] = run && (!mask || (c <= v.dc && (c >= v.wl || c < v.sk)) || (c >= v.s0 && c < v.s1)) ? 1 : 0;
+        }
+    }
+    return w.nt * BN;
 }
 
 // ------------------------------------------------------------------------------------------ status

@@ -338,7 +338,7 @@ struct WorkItem {
 
     // fills the rest from seq_len, q0, packed, full, k_off, n_sink, s_rem and the unit: head pair (or head), or kv head when packed
     template <int BN, bool kPaged, bool kCp, bool kLseOnly>
-    __device__ __forceinline__ void complete(const PrefillParams& p, int unit) {
+    __host__ __device__ __forceinline__ void complete(const PrefillParams& p, int unit) {
         if (packed) {
             hk = unit;
             hA = unit * p.G;
@@ -372,7 +372,7 @@ static_assert(sizeof(WorkItem) == kWorkInts * 4, "words of a work descriptor");
 template <int BN>
 struct TileGeom {
     int cb, jb, js, left, nk;  // left: columns of the list from this tile on
-    __device__ __forceinline__ TileGeom(const volatile WorkItem& g, int t) {
+    __host__ __device__ __forceinline__ TileGeom(const volatile WorkItem& g, int t) {
         const int v0 = (t - g.n_rem) * BN, nb16 = g.nb16;
         cb = max(0, min(BN, nb16 - v0));
         jb = g.lo + v0;
@@ -380,8 +380,29 @@ struct TileGeom {
         left = g.nv - v0;
         nk = min(BN / 16, (left + 15) / 16);
     }
-    __device__ __forceinline__ int key(int c) const { return c < cb ? jb + c : js + c; }
+    __host__ __device__ __forceinline__ int key(int c) const { return c < cb ? jb + c : js + c; }
     __device__ __forceinline__ bool joins_sinks() const { return cb < 16 * nk; }
+    // Columns of the tile that the query at index i (among the local keys) sees: band keys (c < cb) not after it (c <= dc) that
+    // lie in its window (c >= wl) or among the sinks (c < sk), and the sink keys that follow the band (s0 <= c < s1), which
+    // every query sees.  A remote tile (from the sink buffer) holds positions before every local key: its keys below s_rem.
+    struct Seen {
+        int dc, wl, sk, s0, s1;
+    };
+    __host__ __device__ __forceinline__ Seen seen(const volatile WorkItem& g, int t, bool remote, int i, int window) const {
+        const bool full = g.full != 0;
+        Seen s;
+        s.dc = remote ? -1 : min(i - jb, cb - 1);
+        s.wl = full ? 0 : i - jb - window + 1;
+        s.sk = full ? 0 : g.n_sink - jb;
+        s.s0 = remote ? 0 : cb;
+        s.s1 = remote ? g.s_rem - t * BN : left;
+        return s;
+    }
+    // whether some query of the item does not see some column
+    __host__ __device__ __forceinline__ bool needs_mask(const volatile WorkItem& g, int t, bool remote, int window) const {
+        return remote ? g.s_rem - t * BN < BN
+                      : (cb < BN ? (cb > 0 || left < BN) : (jb + BN - 1 > g.i0 || (!g.full && jb <= g.i1 - window)));
+    }
     // rows [bad0, bad1) of the tile lie past the last of len_k keys (none: bad0 >= bad1)
     __device__ __forceinline__ int bad0(int len_k) const { return cb > 0 ? len_k - jb : BN; }
     __device__ __forceinline__ int bad1() const { return min(cb, 16 * nk); }
@@ -1019,13 +1040,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
             }
             bool fresh = true;   // some row of this warp has no reference yet, or one that is far behind
             for (int n = shared ? side : 0; n < nt; n += shared ? 2 : 1) {
-                // a tile from the sink buffer holds positions before every local key: all rows see exactly its keys
-                // below s_rem; no window or causal edge runs through it
                 const bool remote = kCp && n < w.n_rem;
                 const Tile t(w, n);
-                const bool need_mask = remote ? w.s_rem - n * BN < BN
-                                              : (t.cb < BN ? (t.cb > 0 || t.left < BN)
-                                                           : (t.jb + BN - 1 > w.i0 || (!w.full && t.jb <= w.i1 - p.window)));
+                const bool need_mask = t.needs_mask(w, n, remote, p.window);
                 ok = warp_wait(bar(BAR_SF + side), (phases & kPhS) != 0 ? 1u : 0u, abort_flag);
                 if (!ok) break;
                 phases ^= kPhS;
@@ -1101,23 +1118,17 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     tc_wait_ld();
                     pin64(sr + 64);
                     if (need_mask) {
-                        // Bit b of vis <=> column c = 32*cc + b of this tile is visible to this row: a band key (c < cb)
-                        // not after the row (c <= dc) that lies in its window (c >= wl) or among the sinks (c < sk), or one
-                        // of the sink keys that follow the band (cb <= c < left), which every row sees.
-                        const bool full = w.full != 0;
+                        // Bit b of vis <=> column 32*cc + b of this tile is visible to this row (see Seen).
                         // index of this thread's query among the (local) keys; rows past the end take the last one's
                         const int i = min(w.i0 + (packed && w.packed > 1 ? row / p.G : row), w.i1);
-                        const int dc = remote ? -1 : min(i - t.jb, t.cb - 1);
-                        const int wl = full ? 0 : i - t.jb - p.window + 1;
-                        const int sk = full ? 0 : w.n_sink - t.jb;
-                        const int s0 = remote ? 0 : t.cb, s1 = remote ? w.s_rem - n * BN : t.left;
+                        const typename Tile::Seen v = t.seen(w, n, remote, i, p.window);
 #pragma unroll
                         for (int cc = 0; cc < 4; ++cc) {
                             auto below = [&](int x) -> uint32_t {  // bits below x of this 32-column chunk
                                 const int d = x - 32 * cc;
                                 return d <= 0 ? 0u : (d >= 32 ? 0xffffffffu : (1u << d) - 1u);
                             };
-                            const uint32_t vis = (below(dc + 1) & (~below(wl) | below(sk))) | (below(s1) & ~below(s0));
+                            const uint32_t vis = (below(v.dc + 1) & (~below(v.wl) | below(v.sk))) | (below(v.s1) & ~below(v.s0));
 #pragma unroll
                             for (int b = 0; b < 32; ++b)
                                 sr[cc * 32 + b] = ((vis >> b) & 1u) ? sr[cc * 32 + b] : 0xff800000u;  // -inf

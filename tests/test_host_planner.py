@@ -1,8 +1,9 @@
-"""CPU tests of the host-side logic of the library: tile enumeration, layer schedule, symbol table.
+"""CPU tests of the host-side logic of the library: key columns of the prefill kernel's items, tile enumeration, layer
+schedule, symbol table.
 
-The tile enumeration is the part of the prefill kernel that makes work linear in L (App. A); expanded to
-(query, key) pairs on the CPU it must cover the oracle's visible set exactly, and tiles reported as
-needing no mask must be entirely visible.
+The key columns are what makes the prefill kernel's work linear in L (App. A); the masked set of every row must be the
+oracle's visible set exactly.  The enumeration on a grid of whole tiles must cover it, and tiles reported as needing no mask
+must be entirely visible.
 """
 import os
 import re
@@ -62,8 +63,47 @@ def test_tile_enumeration_covers_exactly_the_visible_set(BM, BN):
         assert not (vis & ~covered).any(), f"visible pair outside the enumerated tiles: {(L, W, S, full)}"
 
 
+ITEMS = [(i0, n) for i0 in (0, 1, 5, 128, 200, 383, 640, 1000) for n in (1, 2, 31, 127, 128)]
+ITEM_POLICIES = [(1, 0, True), (1, 0, False), (16, 0, False), (100, 4, False), (128, 4, False), (128, 16, False), (129, 130, False),
+                 (300, 33, False), (640, 200, False), (4096, 4, False)]
+
+
+@pytest.mark.parametrize("paged", [False, True])
+def test_columns_of_a_prefill_item_are_exactly_the_visible_keys(paged):
+    BN = swaa.prefill_block_shape()[1]
+    for i0, n in ITEMS:
+        i1 = i0 + n - 1
+        for len_k in (i1 + 1, i1 + 50):
+            for W, S, full in ITEM_POLICIES:
+                first = 0 if full else max(0, i0 - W + 1)
+                for row in sorted({0, n // 2, n - 1}):
+                    keys, seen = (np.array(x) for x in swaa.prefill_item_keys(len_k, i0, n, W, S, full, row, paged))
+                    what = (i0, n, len_k, W, S, full, row)
+                    got = keys[seen == 1]
+                    want = [j for j in range(i0 + row + 1) if oracle.visible(i0 + row, j, W, S, full)]
+                    assert sorted(got.tolist()) == want, what
+                    # what is computed at all: groups of 16 keys from the start of the sequence (in pages: whole tiles before the
+                    # window), so that a sequence that ends on 16 keys takes none of the next one's, and the sinks
+                    run = keys[keys < 2 ** 31 - 1]
+                    lo = first // (BN if paged else 16) * (BN if paged else 16)
+                    sinks = 0 if full else -(-min(S, lo) // 16) * 16
+                    assert (((run >= lo) & (run < -(-(i1 + 1) // 16) * 16)) | (run < sinks)).all(), what
+                    assert len(keys) <= BN * -(-(i1 + 16 - lo + sinks) // BN), what
+
+
+def test_columns_of_a_context_parallel_prefill_item():
+    for i0, n in ((0, 128), (130, 70), (299, 1)):
+        for s_rem in (1, 16, 128, 130):       # sinks from the sink buffer; the others are the first local keys
+            for W, n_local in ((1, 0), (100, 5), (129, 0)):
+                for row in (0, n - 1):
+                    keys, seen = (np.array(x) for x in swaa.prefill_item_keys(i0 + n, i0, n, W, n_local, False, row, s_rem=s_rem))
+                    i = i0 + row
+                    want = list(range(-s_rem, 0)) + [j for j in range(i + 1) if oracle.visible(i, j, W, n_local, False)]
+                    assert sorted(keys[seen == 1].tolist()) == want, (i0, n, s_rem, W, n_local, row)
+
+
 def test_tile_counts_of_the_benchmark_workloads():
-    """Tiles visited per head at the kernel's own tile shape: linear in L for SWA, quadratic for full."""
+    """Whole tiles of the kernel's tile shape that hold a visible key, per head: linear in L for SWA, quadratic for full."""
     BM, BN = swaa.prefill_block_shape()
     assert (BM, BN) == (128, 128)
 
