@@ -41,12 +41,12 @@ def test_prefill_tiny_workload_every_row():
     print(f"cfg1: max abs err {r[0]:.3e}, max rel err {r[1]:.3e}")
 
 
-SMALL = [
+SMALL = [  # calls of few tiles: one query head per item (pairs of heads: test_prefill_two_heads_gpu.py)
     # seqlens, Hq, Hkv, D
     ((300, 1, 129, 128, 517), 4, 2, 128),
     ((1000,), 2, 1, 64),
-    ((257, 640), 3, 1, 128),      # odd group size: the last pair has one head only
-    ((200, 333), 2, 2, 64),       # no grouping: every block runs a single side
+    ((257, 640), 3, 1, 128),      # odd group size
+    ((200, 333), 2, 2, 64),       # no grouping
     ((127,), 8, 2, 128),
     ((1,), 2, 1, 64),
 ]

@@ -41,6 +41,7 @@ def _pages(k, v, lk, page, seed):
 
 def _check(layout, lq, lk, Hq, Hkv, D, W, S, full, seed, scale=0.0):
     assert _two_heads(lq, Hq)
+    lk = lk or lq
     q, k, v = make(lq, lk, Hq, Hkv, D, seed)
     sc = scale if scale > 0 else None
     what = f"{layout} {lq[:3]} Hq={Hq} D={D} W={W} S={S} full={full} scale={scale}"
@@ -78,6 +79,69 @@ def _check_context_parallel(lens, Hq, Hkv, D, W, S, seed, P=2, scale=0.0):
                                 p0, W, S, False, scale=scale if scale > 0 else None)
         check_against_oracle(out, ref["out"], f"context-parallel rank {r} Hq={Hq} D={D} W={W} S={S} scale={scale}")
         np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("Hq,Hkv", HEADS)
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("layout", ["self", "chunked", "paged", "paged mixed", "context-parallel"])
+def test_ragged_sequences(layout, D, Hq, Hkv):
+    lq = (200, 129, 1, 128, 257, 5)
+    lk = lq if layout == "self" else (200, 300, 70, 500, 400, 900)
+    for W, S, full in ((1, 0, True), (128, 4, False), (100, 20, False), (129, 130, False), (1, 0, False)):
+        if layout != "context-parallel":
+            _check(layout, lq, lk, Hq, Hkv, D, W, S, full, 320 + D)
+        elif not full:
+            _check_context_parallel((517, 300, 129, 200, 256, 3), Hq, Hkv, D, W, S, 330 + D)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("S", [1, 16, 32, 33, 160])
+def test_few_sink_keys_in_a_tile_of_their_own(D, S):
+    # window 128: the band fills its two tiles exactly; the large scale makes the sinks outgrow the reference of the band keys
+    for W, scale in ((128, 0.0), (128, 4.0), (112, 0.0)):
+        _check("self", (300, 129, 517, 40), None, 32, 8, D, W, S, False, 340 + S, scale)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_visible_set_is_bit_exact(D):
+    """Q = 0 and one-hot V: out[c] > 0 exactly where key t*D+c is visible to the row, exactly 0 elsewhere, in both heads of a pair."""
+    lens, Hq, Hkv = (640, 300), 32, 8
+    assert _two_heads(lens, Hq)
+    T = sum(lens)
+    q = torch.zeros((T, Hq, D), dtype=torch.bfloat16, device="cuda")
+    k = make(lens, lens, Hq, Hkv, D, 350)[1]
+    pos = torch.cat([torch.arange(n, device="cuda") for n in lens])
+    for W, S, full in ((128, 4, False), (1, 0, False), (100, 130, False), (257, 1, False), (1, 0, True)):
+        seen = np.zeros((T, 640 // D * D + D), dtype=bool)
+        for t in range(-(-640 // D)):
+            v = torch.zeros((T, Hkv, D), dtype=torch.bfloat16, device="cuda")
+            rows = torch.nonzero(pos // D == t)[:, 0]
+            v[rows, :, pos[rows] - t * D] = 1.0
+            out, lse, status = run_prefill(q, k, v, _cu(lens), 640, W, S, full)
+            assert status == 0
+            o = out.float().cpu().numpy()
+            assert (o >= 0).all() and all(np.array_equal(o[:, h] > 0, o[:, 0] > 0) for h in range(1, Hq))
+            seen[:, t * D:(t + 1) * D] = o[:, 0] > 0
+        counts = np.rint(np.exp(lse.cpu().numpy().astype(np.float64)))
+        start = 0
+        for n in lens:
+            want = np.array([[j < n and oracle.visible(i, j, W, S, full) for j in range(seen.shape[1])] for i in range(n)])
+            assert np.array_equal(seen[start:start + n], want), (W, S, full)
+            assert np.array_equal(counts[:, start:start + n], np.tile(want.sum(1), (Hq, 1)))
+            start += n
+
+
+def test_log_sum_exp_of_the_lazy_ratio_probe():
+    lq, lk, Hq, Hkv, D = (300, 400), (900, 1500), 32, 8, 128
+    assert _two_heads(lq, Hq)
+    q, k, _ = make(lq, lk, Hq, Hkv, D, 360)
+    ratio, scratch = torch.empty(Hq, device="cuda"), torch.full((2, Hq, sum(lq)), float("nan"), device="cuda")
+    swaa.swaa_lazy_ratio(q, k, None, _cu(lq), _cu(lk), max(lq), max(lk), 256, 4, ratio, None, scratch)
+    assert swaa.last_device_status() == 0
+    host = [inputs.to_f32_numpy(t) for t in (q, k, k)]
+    for n, (W, S, full) in enumerate(((256, 4, False), (1, 0, True))):
+        ref = oracle.prefill_chunked(*host, _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(), W, S, full)["lse"]
+        np.testing.assert_allclose(scratch[n].cpu().numpy().T, ref, rtol=0, atol=2e-3)
 
 
 @pytest.mark.parametrize("D", [64, 128])
