@@ -77,24 +77,26 @@ def test_scores_that_leave_the_exponent_range_of_the_reference(D, scale):
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("bits,v_exp", [(40, 95), (100, 0), (100, 95), (118, 0)])
 @pytest.mark.parametrize("lq,lk,Hq,Hkv", [((1024,), (1024,), 2, 1), ((640, 30, 1), (1024, 900, 700), 4, 1), ((2560,), (2560,), 16, 2)])
-def test_large_values_where_scores_grow_from_tile_to_tile(D, lq, lk, Hq, Hkv):
-    """Values around 2^95 and a key in an unmasked tile whose score lies 2^40 above all before it: the products stay below
-    2^127 only against a reference that follows the scores."""
+def test_scores_that_grow_within_one_tile(D, lq, lk, Hq, Hkv, bits, v_exp):
+    """A key in an unmasked tile whose score lies 2^bits above all before it: taken as it comes with the reference raised behind
+    it (40, 100), past what is taken that way (118), and with values around 2^95, whose products stay below 2^127 only
+    against a reference that follows the scores."""
     q, k, v = (t.float() for t in make(lq, lk, Hq, Hkv, D, 70))
     u = q[0, 0] / q[0, 0].norm()
     q = 0.2 * q + 16.0 * u
     k = 0.2 * k
     for a in np.concatenate([[0], np.cumsum(lk)[:-1]]):
-        k[a + 300] += u * (40 * 0.6931 * D ** 0.5 / 16.0)
+        k[a + 300] += u * (bits * 0.6931 * D ** 0.5 / 16.0)
     q, k = q.to(torch.bfloat16), k.to(torch.bfloat16)
-    v = (v * 2.0 ** 95).to(torch.bfloat16)
+    v = (v * 2.0 ** v_exp).to(torch.bfloat16)
     out, lse, status = run_chunked(q, k, v, lq, lk, 1, 0, True)
     assert status == 0
     rows = np.unique(np.linspace(0, sum(lq) - 1, 400).astype(np.int64))
     rh = (rows % Hq).astype(np.int32)
     cu_q, cu_k = (np.concatenate([[0], np.cumsum(n)]) for n in (lq, lk))
-    ref = oracle.prefill_chunked(*(inputs.to_f32_numpy(t) for t in (q, k, v * 2.0 ** -95)), cu_q, cu_k, 1, 0, True, rows=(rows, rh))
-    got = out[torch.as_tensor(rows, device="cuda"), torch.as_tensor(rh.astype(np.int64), device="cuda")] * 2.0 ** -95
+    ref = oracle.prefill_chunked(*(inputs.to_f32_numpy(t) for t in (q, k, v * 2.0 ** -v_exp)), cu_q, cu_k, 1, 0, True, rows=(rows, rh))
+    got = out[torch.as_tensor(rows, device="cuda"), torch.as_tensor(rh.astype(np.int64), device="cuda")] * 2.0 ** -v_exp
     check_against_oracle(got, ref["out"], f"{lq} {lk} D={D}")
     np.testing.assert_allclose(lse.cpu().numpy()[rh, rows], ref["lse"], rtol=0, atol=2e-3)

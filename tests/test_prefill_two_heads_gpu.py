@@ -15,6 +15,11 @@ from test_prefill_gpu import run_prefill
 
 pytestmark = pytest.mark.gpu
 
+# An output element is rounded to bf16 (relative 2^-8 at most), and so is every probability: |err| <= 2^-8 (|out| + sum p |v|), at
+# most 2^-7 max |v| where a steep softmax leaves one key.  Normal values reach 5.3 among so many; 7/16 of them keep the bound
+# below the common absolute tolerance of 2e-2.
+V_STEEP = 0.4375
+
 HEADS = [(32, 8), (28, 4)]  # an even group, and an odd one, whose last item has a single head
 
 
@@ -43,6 +48,8 @@ def _check(layout, lq, lk, Hq, Hkv, D, W, S, full, seed, scale=0.0):
     assert _two_heads(lq, Hq)
     lk = lk or lq
     q, k, v = make(lq, lk, Hq, Hkv, D, seed)
+    if scale > 0:
+        v = (v.float() * V_STEEP).to(torch.bfloat16)
     sc = scale if scale > 0 else None
     what = f"{layout} {lq[:3]} Hq={Hq} D={D} W={W} S={S} full={full} scale={scale}"
     host = [inputs.to_f32_numpy(t) for t in (q, k, v)]
@@ -68,6 +75,8 @@ def _check(layout, lq, lk, Hq, Hkv, D, W, S, full, seed, scale=0.0):
 
 def _check_context_parallel(lens, Hq, Hkv, D, W, S, seed, P=2, scale=0.0):
     q, k, v = make(lens, lens, Hq, Hkv, D, seed)
+    if scale > 0:
+        v = (v.float() * V_STEEP).to(torch.bfloat16)
     for r in range(P):
         qr, kl, vl, sk, sv, lq, lk, p0, _ = split(q, k, v, lens, r, P, W, S)
         assert _two_heads(lq, Hq)
