@@ -1039,7 +1039,7 @@ extern "C" int swaa_prefill_item_keys(int len_k, int i0, int n_rows, int window,
         const bool remote = t < w.n_rem;
         const TileGeom<BN> g(w, t);
         const auto v = g.seen(w, t, remote, w.i0 + row, p.window);
-        const bool mask = g.needs_mask(w, t, remote, p.window);
+        const bool mask = SWAA_TILE_NEEDS_MASK(g, w, t, remote, p.window, BN);
         for (int c = 0; c < BN; ++c) {
             const bool run = remote || c < 16 * g.nk;
             const int key = !remote ? g.key(c) : (t * BN + c < s_rem ? t * BN + c - s_rem : INT32_MAX);
