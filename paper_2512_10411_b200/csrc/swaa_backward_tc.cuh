@@ -28,8 +28,8 @@
 // What bounds it.  A group's step is a chain S^T, dP^T -> element-wise part -> dV, dK, dQ -> read-out -> S^T of its next
 // step, several times as long as the products of a step: the more steps in flight, the better.  Packed batch of
 // 16k tokens, Hq = 16, Hkv = 4, D = 64, window 1024, forward + backward: 540 us with two groups, 462 with three (1417 on
-// warp-level MMAs), 390 with the blocks in order of their length.  At D = 128 tensor memory holds no third group, and a long sample runs against the power cap (1.65 GHz):
-// 16k tokens, Hq = 32, Hkv = 8, window 2048: 2360 us.
+// warp-level MMAs), 390 with the blocks in order of their length.  At D = 128 tensor memory holds no third group and the tensor
+// pipe is active 49 % of a block's cycles: 16k tokens, Hq = 32, Hkv = 8, window 2048: 2330 us.
 //
 // Warps: 4 per group; then the TMA producer (K, V once; Q, dO and the row terms per
 // step through a ring of stages); then the MMA issuer.  Every wait is bounded.
@@ -125,7 +125,7 @@ backward_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // distance from the end of the sequence, the furthest first.  In the order
     // (head, sequence, key tile) the last blocks to start were as long as any: forward + backward of the packed batch above
     // 455 us, 390 this way; one sequence of 4096 tokens, 32 heads of 128, 8 key heads, window 1024: 436 and 366, full
-    // attention 706 and 597; 16k tokens of one sequence, window 2048, at the power cap: 2370 and 2357.
+    // attention 706 and 597; 16k tokens of one sequence, window 2048: 2370 and 2357.
     int slot = (int)(blockIdx.z * gridDim.y + blockIdx.y), n_tile, chunk = -1;
     if (slot < p.sink_tiles * p.chunks) {
         n_tile = slot / p.chunks;

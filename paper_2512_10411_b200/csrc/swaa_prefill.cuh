@@ -22,13 +22,12 @@
 // (and O rescaled) only when a tile's scores outgrow it by far; the final division by the row sum makes the result
 // independent of that choice.
 //
-// What bounds it (32k tokens, Hq = 32, Hkv = 8, D = 128, full causal): the power cap.  At 1000 W the SM clock settles at
-// 1.52 GHz (1.60 before), so fewer cycles per tile buy about half their share in time.  Per 128 x 128 tile of both sides
-// 3260 cycles (3710 before) against 2050 of products and 1970 of softmax: a side is a chain softmax -> P V -> Q K^T.
-// Against the kernel that had one issuing lane, a maximum pass on every tile, sink tiles of their own and a fixed
-// assignment of items: 8280 -> 7640 us; the same prompt with a 2048-key window 1178 -> 1101 us; eight ragged prompts of
-// 146k tokens, Hq = 64, window 4096: 17550 -> 16230 us; a serving step of 4 prompt chunks and 24 generated tokens in
-// pages: 1136 -> 493 us.
+// What bounds it.  A side is a chain softmax -> P V -> Q K^T, and two sides are in flight: per 128 x 128 tile of both 3260 cycles
+// against 2050 of products and 1970 of softmax (32k tokens, Hq = 32, Hkv = 8, D = 128, full causal); with a window of 2048 the
+// tensor pipe is active 59 % of the cycles.  Against the kernel that had one issuing lane, a maximum pass on every tile, sink
+// tiles of their own and a fixed assignment of items (3710 cycles): 8320 -> 7580 us; the same prompt with the window 1187 -> 1087;
+// eight ragged prompts of 146k tokens, Hq = 64, window 4096: 17600 -> 16090 us; a serving step of 4 prompt chunks and 24 generated
+// tokens in pages: 1134 -> 504 us.
 //
 // Every wait is bounded: a wait that runs out records SWAA_ERR_TIMEOUT, all roles leave their loops,
 // the block waits (bounded) for its outstanding copies, frees its tensor memory and returns.
