@@ -153,6 +153,29 @@ int swaa_prefill_paged_mixed(const void* q, const void* kpages, const void* vpag
                              void* stream);
 
 /*
+ * swaa_prefill_chunked(_mixed) and swaa_prefill_paged(_mixed) with a workspace, which lets the key lists of sequences with few
+ * queries (up to 32 rows of queries times group size: generated tokens) be cut into parts that several SMs walk; the last part
+ * to end merges them.  is_full_seq (device, uint8 [B]) may be NULL: all sequences then follow is_full.
+ *
+ *   workspace     device, 256-byte aligned, at least swaa_prefill_split_workspace_size(...) bytes; contents need not be
+ *                 initialised.  Calls that may overlap need one each.
+ *   any_full      whether any sequence of the call runs full attention (a mixed call: 1)
+ * swaa_prefill_split_workspace_size returns 0 when no sequence of the call can be long enough to be cut, and while `stream` is
+ * being captured (the workspace would have to live as long as the graph): call the form without a workspace then.
+ */
+size_t swaa_prefill_split_workspace_size(int B, int max_seqlen_k, int Hq, int Hkv, int D, int window, int n_sink, int any_full,
+                                         void* stream);
+int swaa_prefill_chunked_split(const void* q, const void* k, const void* v, void* out, const int32_t* cu_seqlens_q,
+                               const int32_t* cu_seqlens_k, const uint8_t* is_full_seq, int B, int Tq, int Tk, int max_seqlen_q,
+                               int max_seqlen_k, int Hq, int Hkv, int D, int window, int n_sink, int is_full, float scale,
+                               float* lse, void* workspace, size_t workspace_bytes, void* stream);
+int swaa_prefill_paged_split(const void* q, const void* kpages, const void* vpages, void* out, const int32_t* cu_seqlens_q,
+                             const int32_t* seqlens_k, const int32_t* block_table, const uint8_t* is_full_seq, int B, int Tq,
+                             int max_seqlen_q, int max_blocks, int num_pages, int page_size, int Hq, int Hkv, int D, int window,
+                             int n_sink, int is_full, float scale, float* lse, void* workspace, size_t workspace_bytes,
+                             void* stream);
+
+/*
  * Context-parallel SWA prefill: the compute step of one participant that owns a contiguous stretch of every
  * sequence (App. A: SWA prefill costs O(N * W) because a token only looks at the window before it; Sec. 3.2.1: and
  * at the first k tokens).  Before the call the participant has, in its own memory,

@@ -79,6 +79,12 @@ def load_library():
     lib.swaa_prefill_paged_mixed.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, ci, ci, ci, ci, ci, ci, ci, ci, ci, ci, ci, cf,
                                              vp, vp]
     lib.swaa_prefill_paged_mixed.restype = ci
+    lib.swaa_prefill_split_workspace_size.argtypes = [ci] * 8 + [vp]
+    lib.swaa_prefill_split_workspace_size.restype = ctypes.c_size_t
+    lib.swaa_prefill_chunked_split.argtypes = [vp] * 7 + [ci] * 11 + [cf, vp, vp, ctypes.c_size_t, vp]
+    lib.swaa_prefill_chunked_split.restype = ci
+    lib.swaa_prefill_paged_split.argtypes = [vp] * 8 + [ci] * 12 + [cf, vp, vp, ctypes.c_size_t, vp]
+    lib.swaa_prefill_paged_split.restype = ci
     lib.swaa_prefill_context_parallel.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, vp, ci, ci, ci, ci, ci, ci, ci, ci, ci,
                                                   ci, ci, cf, vp, vp]
     lib.swaa_prefill_context_parallel.restype = ci
@@ -162,6 +168,18 @@ def _stream_ptr(stream):
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _split_workspace(lib, device, stream, st: int, B, max_seqlen_k, Hq, Hkv, D, window, n_sink, any_full):
+    """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator
+    (None: nothing to cut)."""
+    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, Hq, Hkv, D, window, n_sink, any_full, st)
+    if nbytes == 0:
+        return None
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    if stream is not None:  # allocated on the current stream, used on this one
+        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st, device=device))
+    return ws
+
+
 def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink: int, is_full: bool,
                  scale: float = 0.0, lse=None, stream=None) -> None:
     """Forwards to C swaa_prefill.  q, out [T,Hq,D]; k, v [T,Hkv,D] bf16; cu_seqlens int32 [B+1]; lse f32 [Hq,T]."""
@@ -198,9 +216,23 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
     if lse is not None and lse.shape != (Hq, Tq):
         raise ValueError("swaa_prefill_chunked: lse must be [Hq, Tq]")
     bf = torch.bfloat16
+    if is_full_seq is not None and is_full_seq.numel() != B:
+        raise ValueError("swaa_prefill_chunked: is_full_seq must have one entry per sequence")
+    st = _stream_ptr(stream)
+    ws = _split_workspace(lib, q.device, stream, st, B, int(max_seqlen_k), Hq, Hkv, D, int(window), int(n_sink),
+                          int(is_full_seq is not None or bool(is_full))) if q.is_cuda else None
+    if ws is not None:
+        rc = lib.swaa_prefill_chunked_split(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"),
+                                            _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
+                                            _dev_ptr(cu_seqlens_k, torch.int32, "cu_seqlens_k"),
+                                            _dev_ptr(is_full_seq, torch.uint8, "is_full_seq"), B, Tq, Tk,
+                                            int(max_seqlen_q), int(max_seqlen_k), Hq, Hkv, D, int(window), int(n_sink),
+                                            int(bool(is_full)), float(scale), _dev_ptr(lse, torch.float32, "lse"),
+                                            ws.data_ptr(), ws.numel(), st)
+        if rc != SWAA_OK:
+            raise SwaaError(rc, "swaa_prefill_chunked_split")
+        return
     if is_full_seq is not None:
-        if is_full_seq.numel() != B:
-            raise ValueError("swaa_prefill_chunked: is_full_seq must have one entry per sequence")
         rc = lib.swaa_prefill_chunked_mixed(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"),
                                             _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
                                             _dev_ptr(cu_seqlens_k, torch.int32, "cu_seqlens_k"),
@@ -262,9 +294,24 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
     if lse is not None and lse.shape != (Hq, Tq):
         raise ValueError("swaa_prefill_paged: lse must be [Hq, Tq]")
     bf = torch.bfloat16
+    if is_full_seq is not None and is_full_seq.numel() != B:
+        raise ValueError("swaa_prefill_paged: is_full_seq must have one entry per sequence")
+    st = _stream_ptr(stream)
+    ws = _split_workspace(lib, q.device, stream, st, B, min(block_table.shape[1] * page_size, 2147483647), Hq, Hkv, D, int(window), int(n_sink),
+                          int(is_full_seq is not None or bool(is_full))) if q.is_cuda else None
+    if ws is not None:
+        rc = lib.swaa_prefill_paged_split(_dev_ptr(q, bf, "q"), _dev_ptr(kpages, bf, "kpages"), _dev_ptr(vpages, bf, "vpages"),
+                                          _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
+                                          _dev_ptr(seqlens_k, torch.int32, "seqlens_k"),
+                                          _dev_ptr(block_table, torch.int32, "block_table"),
+                                          _dev_ptr(is_full_seq, torch.uint8, "is_full_seq"), B, Tq, int(max_seqlen_q),
+                                          block_table.shape[1], num_pages, page_size, Hq, Hkv, D, int(window), int(n_sink),
+                                          int(bool(is_full)), float(scale), _dev_ptr(lse, torch.float32, "lse"),
+                                          ws.data_ptr(), ws.numel(), st)
+        if rc != SWAA_OK:
+            raise SwaaError(rc, "swaa_prefill_paged_split")
+        return
     if is_full_seq is not None:
-        if is_full_seq.numel() != B:
-            raise ValueError("swaa_prefill_paged: is_full_seq must have one entry per sequence")
         rc = lib.swaa_prefill_paged_mixed(_dev_ptr(q, bf, "q"), _dev_ptr(kpages, bf, "kpages"),
                                           _dev_ptr(vpages, bf, "vpages"), _dev_ptr(out, bf, "out"),
                                           _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),

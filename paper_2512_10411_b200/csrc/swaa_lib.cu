@@ -476,12 +476,12 @@ static int make_accum_map(CUtensorMap* map, const float* base, int T, int H, int
 }
 
 template <int D, int kMode, bool kLseOnly = false>
-static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStream_t st) {
+static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStream_t st, unsigned more_blocks = 0) {
     using L = PrefillSmem<D>;
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(prefill_kernel<D, kMode, kLseOnly>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
     // one block per item (an upper bound); the blocks that run take over the indices of those that wait
-    const unsigned blocks = (unsigned)p.n_units * (unsigned)p.tiles_ub;
+    const unsigned blocks = (unsigned)p.n_units * (unsigned)p.tiles_ub + more_blocks;
     return launch_overlapped(prefill_kernel<D, kMode, kLseOnly>, dim3(blocks), kPrefillThreads, L::kDynamicBytes, st, tm, p);
 }
 
@@ -505,7 +505,30 @@ struct PrefillExtras {
     const void* sink_k = nullptr;
     const void* sink_v = nullptr;
     int sink_rows = 0;
+    void* workspace = nullptr;  // chunked / paged: lets long items of generated tokens be split
+    size_t workspace_bytes = 0;
 };
+
+// Workspace of split items, [tickets | (max, sum) | O] of the slots, and the blocks that the parts add to the launch.  The
+// scheduler cuts the key tiles of all items that may be split into at most four parts per SM, which is as many parts as there are
+// items more at most, in twice as many slots (see load_group).
+struct SplitPlan {
+    int slots, blocks;  // none: no item can be long enough
+    size_t off_ml, off_o, bytes;
+};
+static SplitPlan split_plan(int B, int max_seqlen_k, int G, int Hkv, int D, int window, int n_sink, bool any_full, int sms) {
+    SplitPlan s;
+    long long keys = max_seqlen_k;  // of one item, in whole tiles at both ends of the window
+    if (!any_full) keys = std::min(keys, (long long)window + n_sink + 3 * kPrefillBN);
+    const long long tiles = (keys + kPrefillBN - 1) / kPrefillBN;
+    const long long parts = G > kTokenRows ? 0 : std::min((long long)B * Hkv * (tiles / kSplitMinTiles), 4ll * sms);
+    s.blocks = tiles > kSplitMinTiles ? (int)parts : 0;
+    s.slots = 2 * s.blocks;
+    s.off_ml = ((size_t)s.slots * kTokenRows * sizeof(unsigned long long) + 255) / 256 * 256;
+    s.off_o = s.off_ml + (size_t)s.slots * kTokenRows * sizeof(float2);
+    s.bytes = s.off_o + (size_t)s.slots * kTokenRows * D * sizeof(float);
+    return s;
+}
 
 static int prefill_impl(const void* q, const void* k, const void* v, void* out, const int32_t* cu_seqlens_q,
                         const int32_t* cu_seqlens_k, int B, int Tq, int Tk, int max_seqlen_q, int max_seqlen_k, int Hq,
@@ -566,6 +589,7 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
         if ((rc = make_cache_map(&tm.sink_v, ex.sink_v, B, ex.sink_rows, Hkv, D, kPrefillBN)) != SWAA_OK) return rc;
     }
     PrefillParams p;
+    p.q = static_cast<const __nv_bfloat16*>(q);
     p.out = static_cast<__nv_bfloat16*>(out);
     p.lse = lse;
     p.cu_seqlens = cu_seqlens_q;
@@ -594,7 +618,8 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.heads = ub <= info.sm_count / Hq ? 1 : 2;
     p.units_per_kv = (p.G + p.heads - 1) / p.heads;
     p.n_units = Hkv * p.units_per_kv;
-    if (ub > 2147483647LL / p.n_units) return SWAA_ERR_UNSUPPORTED;
+    const SplitPlan split = split_plan(B, max_seqlen_k, G, Hkv, D, window, n_sink, is_full || ex.is_full_seq != nullptr, info.sm_count);
+    if (ub > (2147483647LL - split.blocks) / p.n_units) return SWAA_ERR_UNSUPPORTED;
     p.tiles_ub = (int)ub;
     if (p.tiles_ub == 0) return SWAA_OK;  // max_seqlen == 0: nothing can be valid
     // a window that covers the longest key sequence is full causal attention for every row; clamping keeps the
@@ -618,15 +643,27 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     if (ex.context_parallel)
         return D == 128 ? launch_prefill<128, 3>(tm, p, st)
                         : launch_prefill<64, 3>(tm, p, st);
+    unsigned more_blocks = 0;
+    p.split_tickets = nullptr;
+    if (ex.workspace != nullptr && split.blocks > 0) {
+        if ((reinterpret_cast<uintptr_t>(ex.workspace) & 255u) != 0 || ex.workspace_bytes < split.bytes) return SWAA_ERR_WORKSPACE;
+        char* ws = static_cast<char*>(ex.workspace);
+        p.split_tickets = reinterpret_cast<unsigned long long*>(ws);
+        p.split_ml = reinterpret_cast<float2*>(ws + split.off_ml);
+        p.split_o = reinterpret_cast<float*>(ws + split.off_o);
+        p.stamp = next_call_stamp();
+        p.sms = info.sm_count;
+        more_blocks = (unsigned)split.blocks;
+    }
     if (is_paged)
-        return D == 128 ? launch_prefill<128, 2>(tm, p, st)
-                        : launch_prefill<64, 2>(tm, p, st);
+        return D == 128 ? launch_prefill<128, 2>(tm, p, st, more_blocks)
+                        : launch_prefill<64, 2>(tm, p, st, more_blocks);
     if (ex.lse_only)
         return D == 128 ? launch_prefill<128, 1, true>(tm, p, st)
                         : launch_prefill<64, 1, true>(tm, p, st);
     if (cu_seqlens_k != nullptr)
-        return D == 128 ? launch_prefill<128, 1>(tm, p, st)
-                        : launch_prefill<64, 1>(tm, p, st);
+        return D == 128 ? launch_prefill<128, 1>(tm, p, st, more_blocks)
+                        : launch_prefill<64, 1>(tm, p, st, more_blocks);
     return D == 128 ? launch_prefill<128, 0>(tm, p, st)
                     : launch_prefill<64, 0>(tm, p, st);
 }
@@ -649,10 +686,11 @@ extern "C" int swaa_prefill_chunked(const void* q, const void* k, const void* v,
                         window, n_sink, is_full, scale, lse, stream);
 }
 
-extern "C" int swaa_prefill_paged(const void* q, const void* kpages, const void* vpages, void* out,
-                                  const int32_t* cu_seqlens_q, const int32_t* seqlens_k, const int32_t* block_table, int B,
-                                  int Tq, int max_seqlen_q, int max_blocks, int num_pages, int page_size, int Hq, int Hkv,
-                                  int D, int window, int n_sink, int is_full, float scale, float* lse, void* stream) {
+// Keys and values in pages, with or without a mask policy per sequence.
+static int prefill_paged(const void* q, const void* kpages, const void* vpages, void* out, const int32_t* cu_seqlens_q,
+                         const int32_t* seqlens_k, const int32_t* block_table, int B, int Tq, int max_seqlen_q, int max_blocks,
+                         int num_pages, int page_size, int Hq, int Hkv, int D, int window, int n_sink, int is_full, float scale,
+                         float* lse, void* stream, const PrefillExtras& ex = PrefillExtras()) {
     if (!seqlens_k || !block_table) return SWAA_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(block_table) & 3u) != 0) return SWAA_ERR_INVALID_ARG;
     if (max_blocks < 1 || num_pages < 1 || page_size < 1) return SWAA_ERR_INVALID_ARG;
@@ -663,7 +701,15 @@ extern "C" int swaa_prefill_paged(const void* q, const void* kpages, const void*
     pg.num_pages = num_pages;
     pg.page_size = page_size;
     return prefill_impl(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, B, Tq, 0, max_seqlen_q, max_blocks * page_size, Hq,
-                        Hkv, D, window, n_sink, is_full, scale, lse, stream, pg);
+                        Hkv, D, window, n_sink, is_full, scale, lse, stream, pg, ex);
+}
+
+extern "C" int swaa_prefill_paged(const void* q, const void* kpages, const void* vpages, void* out,
+                                  const int32_t* cu_seqlens_q, const int32_t* seqlens_k, const int32_t* block_table, int B,
+                                  int Tq, int max_seqlen_q, int max_blocks, int num_pages, int page_size, int Hq, int Hkv,
+                                  int D, int window, int n_sink, int is_full, float scale, float* lse, void* stream) {
+    return prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_table, B, Tq, max_seqlen_q, max_blocks, num_pages, page_size,
+                         Hq, Hkv, D, window, n_sink, is_full, scale, lse, stream);
 }
 
 extern "C" int swaa_prefill_chunked_mixed(const void* q, const void* k, const void* v, void* out,
@@ -683,19 +729,55 @@ extern "C" int swaa_prefill_paged_mixed(const void* q, const void* kpages, const
                                         const int32_t* block_table, const uint8_t* is_full_seq, int B, int Tq,
                                         int max_seqlen_q, int max_blocks, int num_pages, int page_size, int Hq, int Hkv,
                                         int D, int window, int n_sink, float scale, float* lse, void* stream) {
-    if (!seqlens_k || !block_table || !is_full_seq) return SWAA_ERR_INVALID_ARG;
-    if ((reinterpret_cast<uintptr_t>(block_table) & 3u) != 0) return SWAA_ERR_INVALID_ARG;
-    if (max_blocks < 1 || num_pages < 1 || page_size < 1) return SWAA_ERR_INVALID_ARG;
-    if (page_size % kPrefillBN != 0 || (long long)max_blocks * page_size > 2147483647LL) return SWAA_ERR_UNSUPPORTED;
-    PagedKV pg;
-    pg.block_table = block_table;
-    pg.max_blocks = max_blocks;
-    pg.num_pages = num_pages;
-    pg.page_size = page_size;
+    if (!is_full_seq) return SWAA_ERR_INVALID_ARG;
     PrefillExtras ex;
     ex.is_full_seq = is_full_seq;
-    return prefill_impl(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, B, Tq, 0, max_seqlen_q, max_blocks * page_size, Hq,
-                        Hkv, D, window, n_sink, 0, scale, lse, stream, pg, ex);
+    return prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_table, B, Tq, max_seqlen_q, max_blocks, num_pages, page_size,
+                         Hq, Hkv, D, window, n_sink, 0, scale, lse, stream, ex);
+}
+
+extern "C" size_t swaa_prefill_split_workspace_size(int B, int max_seqlen_k, int Hq, int Hkv, int D, int window, int n_sink, int any_full,
+                                                    void* stream) {
+    if (B < 1 || max_seqlen_k < 1 || Hq < 1 || Hkv < 1 || Hq % Hkv != 0 || (D != 64 && D != 128) || n_sink < 0) return 0;
+    DeviceInfo info;
+    if (current_device_info(&info) != SWAA_OK) info.sm_count = 148;
+    const SplitPlan s = split_plan(B, max_seqlen_k, Hq / Hkv, Hkv, D, window, n_sink, any_full != 0, info.sm_count);
+    if (s.blocks == 0) return 0;
+    // A captured call would need the workspace for as long as the graph lives.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(reinterpret_cast<cudaStream_t>(stream), &capture) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    return capture == cudaStreamCaptureStatusNone ? s.bytes : 0;
+}
+
+extern "C" int swaa_prefill_chunked_split(const void* q, const void* k, const void* v, void* out, const int32_t* cu_seqlens_q,
+                                          const int32_t* cu_seqlens_k, const uint8_t* is_full_seq, int B, int Tq, int Tk,
+                                          int max_seqlen_q, int max_seqlen_k, int Hq, int Hkv, int D, int window, int n_sink,
+                                          int is_full, float scale, float* lse, void* workspace, size_t workspace_bytes,
+                                          void* stream) {
+    if (!cu_seqlens_k || !workspace) return SWAA_ERR_INVALID_ARG;
+    PrefillExtras ex;
+    ex.is_full_seq = is_full_seq;
+    ex.workspace = workspace;
+    ex.workspace_bytes = workspace_bytes;
+    return prefill_impl(q, k, v, out, cu_seqlens_q, cu_seqlens_k, B, Tq, Tk, max_seqlen_q, max_seqlen_k, Hq, Hkv, D, window, n_sink,
+                        is_full_seq != nullptr ? 0 : is_full, scale, lse, stream, PagedKV(), ex);
+}
+
+extern "C" int swaa_prefill_paged_split(const void* q, const void* kpages, const void* vpages, void* out,
+                                        const int32_t* cu_seqlens_q, const int32_t* seqlens_k, const int32_t* block_table,
+                                        const uint8_t* is_full_seq, int B, int Tq, int max_seqlen_q, int max_blocks, int num_pages,
+                                        int page_size, int Hq, int Hkv, int D, int window, int n_sink, int is_full, float scale,
+                                        float* lse, void* workspace, size_t workspace_bytes, void* stream) {
+    if (!workspace) return SWAA_ERR_INVALID_ARG;
+    PrefillExtras ex;
+    ex.is_full_seq = is_full_seq;
+    ex.workspace = workspace;
+    ex.workspace_bytes = workspace_bytes;
+    return prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_table, B, Tq, max_seqlen_q, max_blocks, num_pages, page_size,
+                         Hq, Hkv, D, window, n_sink, is_full_seq != nullptr ? 0 : is_full, scale, lse, stream, ex);
 }
 
 extern "C" int swaa_prefill_context_parallel(const void* q, const void* k_local, const void* v_local,

@@ -1,0 +1,90 @@
+"""Long key lists of generated tokens cut into parts (chunked and paged prefill with a workspace) against the float64 oracle:
+key counts around the smallest part, up to the most parts of an item, rows that end inside a warp, and the sequences that are
+not cut next to them."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2512_10411_b200 as swaa
+from paper_2512_10411_b200 import binding, inputs
+from helpers import check_against_oracle
+from test_prefill_chunked_gpu import _cu, make
+
+pytestmark = pytest.mark.gpu
+
+BATCHES = [
+    # new tokens, context lengths
+    ((1,), (1025,)),                                 # one tile more than a part: two parts
+    ((1, 1), (1024, 9000)),                          # not cut, and many parts
+    ((3, 200, 1, 2), (5000, 700, 4481, 2049)),       # several rows per token group next to a chunk
+    (tuple([1] * 40), tuple(range(300, 300 + 40 * 150, 150))),  # more than 32 sequences: two groups of the scheduler
+]
+
+
+def _run(paged, q, k, v, lq, lk, W, S, full, full_seq, **kw):
+    out = torch.full_like(q, float("nan"))
+    lse = torch.full((q.shape[1], q.shape[0]), float("nan"), device="cuda")
+    fs = None if full_seq is None else torch.tensor(full_seq, dtype=torch.uint8, device="cuda")
+    if not paged:
+        swaa.swaa_prefill_chunked(q, k, v, out, _cu(lq), _cu(lk), max(lq), max(lk), W, S, full, lse=lse, is_full_seq=fs, **kw)
+    else:
+        page, Hkv, D = 128, k.shape[1], k.shape[2]
+        used = [-(-n // page) for n in lk]
+        order = torch.randperm(sum(used), generator=torch.Generator().manual_seed(3))
+        kp = torch.full((sum(used), page, Hkv, D), float("nan"), dtype=torch.bfloat16, device="cuda")
+        vp, table, n, pos = kp.clone(), torch.zeros(len(lk), max(used), dtype=torch.int32), 0, 0
+        for b, L in enumerate(lk):
+            for i in range(used[b]):
+                m = min(page, L - i * page)
+                kp[order[n], :m], vp[order[n], :m] = k[pos + i * page:pos + i * page + m], v[pos + i * page:pos + i * page + m]
+                table[b, i] = order[n]
+                n += 1
+            pos += L
+        swaa.swaa_prefill_paged(q, kp, vp, out, _cu(lq), torch.tensor(lk, dtype=torch.int32, device="cuda"), table.cuda(), max(lq), W, S,
+                                full, lse=lse, is_full_seq=fs, **kw)
+    assert swaa.last_device_status() == 0
+    return out, lse
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("heads,D", [((4, 1), 128), ((16, 2), 64), ((6, 6), 128)])
+@pytest.mark.parametrize("batch", range(len(BATCHES)))
+def test_split_items_against_the_oracle(batch, heads, D, paged):
+    lq, lk = BATCHES[batch]
+    Hq, Hkv = heads
+    q, k, v = make(lq, lk, Hq, Hkv, D, 900 + batch)
+    k[::97] *= 6  # scores that outgrow the reference in the middle of a part
+    qh, kh, vh = (inputs.to_f32_numpy(t) for t in (q, k, v))
+    for W, S, full, full_seq in ((1, 0, True, None), (2500, 4, False, None), (100, 20, False, [b % 2 for b in range(len(lq))])):
+        out, lse = _run(paged, q, k, v, lq, lk, W, S, full, full_seq)
+        kw = {} if full_seq is None else {"is_full_seq": np.array(full_seq, dtype=np.uint8)}
+        ref = oracle.prefill_chunked(qh, kh, vh, _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(), W, S, full, **kw)
+        check_against_oracle(out, ref["out"], f"split {batch} {heads} D={D} paged={paged} W={W} S={S} full={full}")
+        np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
+def test_split_calls_on_other_streams_and_in_a_graph():
+    """A stream of its own (object and address), and a capture, where the call goes without a workspace."""
+    lq, lk, W, S = (1, 1, 70), (6000, 1300, 900), 64, 4
+    q, k, v = make(lq, lk, 8, 2, 128, 77)
+    want, _ = _run(False, q, k, v, lq, lk, W, S, True, None)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    for stream in (side, side.cuda_stream):
+        got, _ = _run(False, q, k, v, lq, lk, W, S, True, None, stream=stream)
+        side.synchronize()
+        assert torch.equal(got, want)
+    lib = binding.load_library()
+    assert lib.swaa_prefill_split_workspace_size(3, 6000, 8, 2, 128, W, S, 1, None) > 0
+    assert lib.swaa_prefill_split_workspace_size(3, 1024, 8, 2, 128, W, S, 1, None) == 0
+    assert lib.swaa_prefill_split_workspace_size(3, 6000, 8, 2, 128, W, S, 0, None) == 0  # windows of 64 keys
+    cu_q, cu_k, out = _cu(lq), _cu(lk), torch.full_like(q, float("nan"))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        assert lib.swaa_prefill_split_workspace_size(3, 6000, 8, 2, 128, W, S, 1, torch.cuda.current_stream().cuda_stream) == 0
+        swaa.swaa_prefill_chunked(q, k, v, out, cu_q, cu_k, max(lq), max(lk), W, S, True)
+    g.replay()
+    torch.cuda.synchronize()
+    assert (out.float() - want.float()).norm() / want.float().norm() < 1e-2  # two correct splits: bf16 outputs differ by 2e-3
