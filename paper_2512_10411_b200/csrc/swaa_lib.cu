@@ -14,6 +14,7 @@
 #include "swaa_internal.cuh"
 #include "swaa_decode.cuh"
 #include "swaa_prefill.cuh"
+#include "swaa_prefill_token.cuh"
 #include "swaa_backward.cuh"
 #include "swaa_backward_tc.cuh"
 
@@ -476,13 +477,21 @@ static int make_accum_map(CUtensorMap* map, const float* base, int T, int H, int
 }
 
 template <int D, int kMode, bool kLseOnly = false>
-static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStream_t st, unsigned more_blocks = 0) {
+static int launch_prefill(const PrefillMaps& tm, const PrefillParams& p, cudaStream_t st) {
     using L = PrefillSmem<D>;
     static std::atomic<bool> attr_done[64];
     if (ensure_dynamic_smem(prefill_kernel<D, kMode, kLseOnly>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
     // one block per item (an upper bound); the blocks that run take over the indices of those that wait
-    const unsigned blocks = (unsigned)p.n_units * (unsigned)p.tiles_ub + more_blocks;
+    const unsigned blocks = (unsigned)p.n_units * (unsigned)p.tiles_ub;
     return launch_overlapped(prefill_kernel<D, kMode, kLseOnly>, dim3(blocks), kPrefillThreads, L::kDynamicBytes, st, tm, p);
+}
+
+template <int D, bool kPaged>
+static int launch_tokens(const PrefillMaps& tm, const PrefillParams& p, unsigned blocks, cudaStream_t st) {
+    using L = TokenSmem<D>;
+    static std::atomic<bool> attr_done[64];
+    if (ensure_dynamic_smem(token_kernel<D, kPaged>, L::kDynamicBytes, attr_done) != SWAA_OK) return SWAA_ERR_CUDA;
+    return launch_overlapped(token_kernel<D, kPaged>, dim3(blocks), kTokenThreads, L::kDynamicBytes, st, tm.k, tm.v, tm.k_small, tm.v_small, p);
 }
 
 }  // namespace swaa
@@ -509,9 +518,9 @@ struct PrefillExtras {
     size_t workspace_bytes = 0;
 };
 
-// Workspace of split items, [tickets | (max, sum) | O] of the slots, and the blocks that the parts add to the launch.  The
-// scheduler cuts the key tiles of all items that may be split into at most four parts per SM, which is as many parts as there are
-// items more at most, in twice as many slots (see load_group).
+// Workspace of split token items, [tickets | (max, sum) | O] of the slots, and the blocks that the parts add to the launch: the
+// key tiles of all items are cut into at most four parts per SM, which is as many parts as there are items more at most, in
+// twice as many slots (see token_kernel).
 struct SplitPlan {
     int slots, blocks;  // none: no item can be long enough
     size_t off_ml, off_o, bytes;
@@ -592,6 +601,7 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.q = static_cast<const __nv_bfloat16*>(q);
     p.out = static_cast<__nv_bfloat16*>(out);
     p.lse = lse;
+    p.token_len = -1;
     p.cu_seqlens = cu_seqlens_q;
     p.cu_seqlens_k = cu_seqlens_k;
     p.B = B;
@@ -619,7 +629,7 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.units_per_kv = (p.G + p.heads - 1) / p.heads;
     p.n_units = Hkv * p.units_per_kv;
     const SplitPlan split = split_plan(B, max_seqlen_k, G, Hkv, D, window, n_sink, is_full || ex.is_full_seq != nullptr, info.sm_count);
-    if (ub > (2147483647LL - split.blocks) / p.n_units) return SWAA_ERR_UNSUPPORTED;
+    if (ub > 2147483647LL / p.n_units) return SWAA_ERR_UNSUPPORTED;
     p.tiles_ub = (int)ub;
     if (p.tiles_ub == 0) return SWAA_OK;  // max_seqlen == 0: nothing can be valid
     // a window that covers the longest key sequence is full causal attention for every row; clamping keeps the
@@ -643,7 +653,14 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     if (ex.context_parallel)
         return D == 128 ? launch_prefill<128, 3>(tm, p, st)
                         : launch_prefill<64, 3>(tm, p, st);
-    unsigned more_blocks = 0;
+    // Sequences of so few queries that their rows (query, head of the group) fit the token kernel are left to it.  A batch of
+    // nothing else goes there alone; one that cannot hold any, because the queries do not add up otherwise, does without.
+    int token_len = -1;
+    if (!ex.lse_only && cu_seqlens_k != nullptr && G <= kTokenRows) {
+        token_len = kTokenRows / G;
+        if (Tq > (long long)(B - 1) * max_seqlen_q + token_len || (long long)B * Hkv > 2147483647LL - split.blocks) token_len = -1;
+    }
+    const bool only_tokens = max_seqlen_q <= token_len;
     p.split_tickets = nullptr;
     if (ex.workspace != nullptr && split.blocks > 0) {
         if ((reinterpret_cast<uintptr_t>(ex.workspace) & 255u) != 0 || ex.workspace_bytes < split.bytes) return SWAA_ERR_WORKSPACE;
@@ -653,17 +670,22 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
         p.split_o = reinterpret_cast<float*>(ws + split.off_o);
         p.stamp = next_call_stamp();
         p.sms = info.sm_count;
-        more_blocks = (unsigned)split.blocks;
     }
-    if (is_paged)
-        return D == 128 ? launch_prefill<128, 2>(tm, p, st, more_blocks)
-                        : launch_prefill<64, 2>(tm, p, st, more_blocks);
+    p.token_len = only_tokens ? -1 : token_len;
+    if (cu_seqlens_k != nullptr && !ex.lse_only) {
+        rc = SWAA_OK;
+        if (!only_tokens) {
+            if (is_paged) rc = D == 128 ? launch_prefill<128, 2>(tm, p, st) : launch_prefill<64, 2>(tm, p, st);
+            else rc = D == 128 ? launch_prefill<128, 1>(tm, p, st) : launch_prefill<64, 1>(tm, p, st);
+        }
+        if (rc != SWAA_OK || token_len < 0) return rc;
+        const unsigned blocks = (unsigned)(B * Hkv) + (p.split_tickets != nullptr ? (unsigned)split.blocks : 0u);
+        if (is_paged) return D == 128 ? launch_tokens<128, true>(tm, p, blocks, st) : launch_tokens<64, true>(tm, p, blocks, st);
+        return D == 128 ? launch_tokens<128, false>(tm, p, blocks, st) : launch_tokens<64, false>(tm, p, blocks, st);
+    }
     if (ex.lse_only)
         return D == 128 ? launch_prefill<128, 1, true>(tm, p, st)
                         : launch_prefill<64, 1, true>(tm, p, st);
-    if (cu_seqlens_k != nullptr)
-        return D == 128 ? launch_prefill<128, 1>(tm, p, st, more_blocks)
-                        : launch_prefill<64, 1>(tm, p, st, more_blocks);
     return D == 128 ? launch_prefill<128, 0>(tm, p, st)
                     : launch_prefill<64, 0>(tm, p, st);
 }

@@ -35,8 +35,6 @@
 
 #include <cuda.h>
 
-#include <type_traits>
-
 #include "swaa_internal.cuh"
 #include "swaa_ptx.cuh"
 
@@ -46,10 +44,7 @@ constexpr int kPrefillBM = 128;
 constexpr int kPrefillBN = 128;
 constexpr int kPrefillThreads = 384;  // 8 softmax warps + 4 auxiliary warps (producer, issuer, scheduler, 1 idle)
 constexpr int kPrefillSmallBox = 16;                        // rows of the small TMA boxes over K and V
-constexpr int kWorkInts = 28;                               // words of a work descriptor
-constexpr int kTokenRows = 8;                               // rows of a token item (see WorkItem)
-constexpr int kSplitMinTiles = 8;                           // key tiles of a part of a token item, at least
-constexpr int kSplitMaxParts = 32;                          // parts of an item (one lane each when they are merged)
+constexpr int kWorkInts = 24;                               // words of a work descriptor
 constexpr float kRescaleThreshold = 8.0f;                   // log2 units
 constexpr float kGrowLimit = 32768.f;                       // 2^15: row sum of a tile above which the reference is looked at
 constexpr float kLeadLimit = 1073741824.f;                  // 2^30: row sum so far that the reference is raised by
@@ -57,7 +52,7 @@ constexpr float kArgLimit = 110.f;                          // argument of an ex
 constexpr float kSumLimit = 1.298074214633707e33f;          // above which the item is run again
 
 struct PrefillParams {
-    const __nv_bfloat16* q;  // token items only
+    const __nv_bfloat16* q;  // token_kernel only
     __nv_bfloat16* out;
     float* lse;             // nullable, [Hq, T]
     const int32_t* cu_seqlens;    // queries (and keys, when cu_seqlens_k is null)
@@ -81,33 +76,16 @@ struct PrefillParams {
     int sink_rows;
     float sl2;              // softmax scale * log2(e)
     float scale;
-    // Split token items (kMode 1, 2; null: none are split).  A part leaves (max, sum) and the unnormalised O of its rows in a
-    // slot, [kTokenRows] and [kTokenRows][D] floats; the last part of an item to arrive at a row merges it.
-    unsigned long long* split_tickets;  // [slots][kTokenRows], see split_arrive
+    // Chunked / paged: sequences of at most this many queries are left to token_kernel, which is launched behind this kernel
+    // and may start as soon as all blocks of this one have (-1: there are none).
+    int token_len;
+    // token_kernel: tickets, (max, sum) and unnormalised O of the rows of split items (null: none are split), see there
+    unsigned long long* split_tickets;
     float2* split_ml;
     float* split_o;
-    unsigned long long stamp;           // 48-bit number unique to this call (never 0)
+    unsigned long long stamp;     // 48-bit number unique to this call (never 0)
     int sms;
 };
-
-// Counts the parts of an item's row that are done; true for the last one.  The word holds (stamp of the call << 16 | arrivals): one
-// whose stamp is not this call's is left over and starts again, so nothing has to be cleared before a call, and the last
-// arrival clears it, because a call that a CUDA graph replays comes with the same stamp again.
-__device__ __forceinline__ bool split_arrive(unsigned long long* t, unsigned long long stamp, int parts) {
-    unsigned long long seen = *reinterpret_cast<volatile unsigned long long*>(t), now = 0;
-    while ((seen >> 16) != stamp) {
-        const unsigned long long prev = atomicCAS(t, seen, (stamp << 16) | 1ull);
-        if (prev == seen) {
-            now = (stamp << 16) | 1ull;
-            break;
-        }
-        seen = prev;
-    }
-    if (now == 0) now = atomicAdd(t, 1ull) + 1ull;
-    const bool last = (int)(now & 0xffffull) == parts;
-    if (last) *reinterpret_cast<volatile unsigned long long*>(t) = 0ull;
-    return last;
-}
 
 // Tensor maps of one call; an instance reads those that it needs.
 struct PrefillMaps {
@@ -118,51 +96,6 @@ struct PrefillMaps {
     CUtensorMap out;               // [32 rows] x 1 head
     CUtensorMap sink_k, sink_v;    // context-parallel
 };
-
-// Merges the parts of a row (at stride kTokenRows): lane = part for (max, sum), then lane = D / 32 channels, sixteen parts in
-// flight.  (Loads past the last part are repeated and not used: conditional loads into an array cost 44 registers, which spilled.)
-template <int D>
-struct RowResult {
-    float m, l, o[D / 32];
-};
-template <int D>
-__device__ __forceinline__ RowResult<D> merge_parts(const float2* part_ml, const float* part_o, int parts, float sl2) {
-    constexpr int kCh = D / 32, kBatch = 16;
-    using Vec = typename std::conditional<kCh == 4, float4, float2>::type;
-    const int lane = threadIdx.x & 31;
-    RowResult<D> r;
-    float2 ml = __ldcg(part_ml + min(lane, parts - 1) * kTokenRows);
-    if (lane >= parts) ml = make_float2(-INFINITY, 0.f);
-    float wgt = 0.f;
-#pragma unroll
-    for (int e = 0; e < kCh; ++e) r.o[e] = 0.f;
-#pragma unroll 1
-    for (int j = 0; j < parts; j += kBatch) {
-        Vec u[kBatch];
-#pragma unroll
-        for (int i = 0; i < kBatch; ++i)
-            u[i] = __ldcg(reinterpret_cast<const Vec*>(part_o + (size_t)min(j + i, parts - 1) * kTokenRows * D) + lane);
-        if (j == 0) {
-            r.m = ml.x;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) r.m = fmaxf(r.m, __shfl_xor_sync(0xffffffffu, r.m, o));
-            wgt = ml.x == -INFINITY ? 0.f : ex2f((ml.x - r.m) * sl2);
-            r.l = wgt * ml.y;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) r.l += __shfl_xor_sync(0xffffffffu, r.l, o);
-        }
-#pragma unroll
-        for (int i = 0; i < kBatch; ++i) {
-            const float wi = __shfl_sync(0xffffffffu, wgt, (j + i) & 31);
-            if (j + i < parts) {
-                const float* y = reinterpret_cast<const float*>(&u[i]);
-#pragma unroll
-                for (int e = 0; e < kCh; ++e) r.o[e] = fmaf(wi, y[e], r.o[e]);
-            }
-        }
-    }
-    return r;
-}
 
 // ------------------------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -375,25 +308,18 @@ struct PrefillSmem {
     // barriers: Q full/empty; full/empty/V-tile-cleared (paged keys only) per slot; per side S full / P ready / O done /
     // O free; work descriptor full/empty per slot, next-block answer, hand-over of packed items per row quadrant,
     // staging free per work slot, final
-    // full/empty per slot for token items, their partial results written/read, their start
-    static constexpr int kNumBars = 2 + 3 * kSlots + 2 * 4 + 5 + 4 + 3 + 2 * kSlots + 3;
+    static constexpr int kNumBars = 2 + 3 * kSlots + 2 * 4 + 5 + 4 + 3;
     static constexpr int kOffMisc = (kOffBar + kNumBars * 8 + 15) / 16 * 16;  // next-block answer, tmem slot, flags, work descriptors
-    static constexpr int kOffToken = kOffMisc + 32 + 2 * kWorkInts * 4;  // token items: ring state per softmax warp and of the producer
-    static constexpr int kBytes = kOffToken + 9 * 4;
+    static constexpr int kBytes = kOffMisc + 32 + 2 * kWorkInts * 4;
     static constexpr int kDynamicBytes = kBytes + 1024;          // room to align the base to 1024 B
     static_assert(kDynamicBytes <= 232448, "shared memory per block");
 };
 
 // One unit of work.  Usual form: a 128-row query tile of one sequence for one pair of query heads (one per side), or for a
 // single query head, both sides on its rows, when the call has too few tiles for the SMs (see the launch).
-// Packed form, for sequences whose queries times the group size fit in 128 rows (generated tokens, very short
-// prompts): the rows are (query, head of the group) for ALL heads of one kv head, so K and V are read once per kv head
+// Packed form, for sequences whose queries times the group size fit in 128 rows (very short prompts; generated tokens where
+// token_kernel does not take them): the rows are (query, head of the group) for ALL heads of one kv head, so K and V are read once per kv head
 // and no row is padding that another head could use; the two sides then take alternate key tiles and merge at the end.
-// Token form (chunked and paged keys), for those of at most kTokenRows rows: the softmax warps do all of it on warp-level MMAs
-// (token_item).  On tcgen05 a tile of such an item costs as much as one of 128 rows, 2300 cycles with the waits of one issuing
-// warp, against 1100 this way and 790 for its copies.  Its key list is cut into parts for several SMs where the call brings a
-// workspace.  24 generated tokens at 1k to 32k keys in pages: 312 us as packed items, 160 in parts; one at 32k 297 and 37; a
-// serving step of these with 4 prompt chunks 486 and 435.
 //
 // Key columns of an item: the keys are enumerated as one list [band keys lo .. i1, rounded up
 // to 16 | the sink keys before them] and cut into tiles of BN columns: a few sink keys share the last band tile or make
@@ -420,15 +346,10 @@ struct WorkItem {
     int b;        // context-parallel: sequence index (row of the sink buffer)
     int n_rows;   // rows in use
     int careful;  // second run of an item whose scores left the exponent range of the first (see the softmax role)
-    int parts;    // token item: parts of its key list (1: not split), else 0
-    int t0;       // first tile of the item's part of the key list (nt: tiles of the part)
-    int slot, first_slot;  // slots of this part and of the item's first one
 
     // fills the rest from seq_len, q0, packed, full, k_off, n_sink, s_rem and the unit: head pair (or head), or kv head when packed
     template <int BN, bool kPaged, bool kCp, bool kLseOnly>
     __host__ __device__ __forceinline__ void complete(const PrefillParams& p, int unit) {
-        parts = t0 = 0;
-        slot = first_slot = 0;
         if (packed) {
             hk = unit;
             hA = unit * p.G;
@@ -454,16 +375,6 @@ struct WorkItem {
         n_rem = kCp ? (s_rem + BN - 1) / BN : 0;
         nt = n_rem + (nv + BN - 1) / BN;
         shared = packed && nt > 1 ? 1 : 0;
-    }
-    // token item: keeps part i of n of the key list, even parts
-    __device__ __forceinline__ void keep_part(int i, int n, int slot_base) {
-        const int end = (int)((long long)nt * (i + 1) / n);
-        t0 = (int)((long long)nt * i / n);
-        nt = end - t0;
-        parts = n;
-        first_slot = slot_base;
-        slot = slot_base + i;
-        shared = 0;
     }
 };
 static_assert(sizeof(WorkItem) == kWorkInts * 4, "words of a work descriptor");
@@ -520,359 +431,6 @@ struct RuntimeFlag {
     static constexpr bool known = false, value = false;
 };
 
-// Barrier numbers; NS: tile slots.
-template <int NS>
-struct PrefillBars {
-    static constexpr int QF = 0, QE = 1, F = 2, E = F + NS;  // Q full, Q empty; slot full, slot empty
-    // paged only, one per slot: the rows of the V tile in that slot past the last key have been cleared.
-    // Completed once per cleared tile; the issuer keeps the slot's phase bit.  The producer cannot
-    // clear a slot twice before the issuer has waited for the first clear: reusing the slot needs the
-    // issuer's empty commit, which follows that wait.
-    static constexpr int VC = E + NS;
-    static constexpr int SF = VC + NS, PR = SF + 2, OD = PR + 2, OF = OD + 2;  // per side: S full; P ready; O done, O free
-    // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), staging free
-    // for the ring of a packed item (per work slot), final
-    static constexpr int WF = OF + 2, WE = WF + 2, NB = WE + 2, MG = NB + 1, SG = MG + 4, FIN = SG + 2;
-    // token items (their tiles are used by the softmax warps): slot full, slot empty; partial results of the warps written, read;
-    // every warp is done with the item before (so the Q tile and the hand-over area are free)
-    static constexpr int TF = FIN + 1, TE = TF + NS, TW = TE + NS, TR = TW + 1, TI = TR + 1;
-};
-
-// The copies of a token item: K(0) V(0) K(1) V(1) ..., tiles to the two sides in turn, each side's in its half of the slots.
-// staging: parity of the barrier of the output staging, which the last slots overlay.  (Not inlined: see token_item.)
-template <int D, bool kPaged>
-__device__ __noinline__ bool token_loads(const PrefillMaps& tm, const PrefillParams& p, uint32_t smem_base, int work_slot, uint32_t staging) {
-    using L = PrefillSmem<D>;
-    constexpr int BN = kPrefillBN, NS = L::kSlots, kHalf = NS / 2;
-    using B = PrefillBars<NS>;
-    using Tile = TileGeom<BN>;
-    uint8_t* smem_gen = reinterpret_cast<uint8_t*>(__cvta_shared_to_generic(smem_base));
-    auto bar = [&](int i) -> uint32_t { return smem_base + (uint32_t)L::kOffBar + 8u * (uint32_t)i; };
-    auto uniform = [](int x) -> int { return __shfl_sync(0xffffffffu, x, 0); };
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + L::kOffMisc + 20);
-    volatile uint32_t* state = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kOffToken) + 8;
-    const volatile WorkItem& w = reinterpret_cast<volatile WorkItem*>(smem_gen + L::kOffMisc + 32)[work_slot];
-    const int lane = threadIdx.x & 31;
-    const bool el = elect_one();
-    // next slot of each half (four bits each) and, from bit 8, the parity of every slot's next use
-    int next[2] = {(int)(*state & 15u), (int)((*state >> 4) & 15u)};
-    uint32_t phases = *state >> 8;
-    const int t0 = uniform(w.t0), nt = uniform(w.nt), lo = uniform(w.lo), hk = uniform(w.hk), k_start = uniform(w.k_start);
-    const int nb16 = uniform(w.nb16);
-    bool ok = true, staged = false;
-    // page of a key, out of range (the copy delivers zeros) when the table is wrong
-    auto page_of = [&](int key) -> int {
-        const int page = p.block_table[(size_t)k_start * p.max_blocks + key / p.page_size];
-        if (page >= 0 && page < p.num_pages) return page;
-        record_device_error(SWAA_ERR_BAD_SEQLENS);
-        return p.num_pages;
-    };
-    if (lane == 0) mbar_arrive(bar(B::TI));  // what the item before had in shared memory is no longer used
-    __syncwarp();
-    int pages = 0;  // lane l: page of tile l of 32
-    for (int n = 0; n < nt && ok; ++n) {
-        const int side = n & 1, key = lo + (t0 + n) * BN;
-        if (kPaged && (n & 31) == 0) {
-            __syncwarp();
-            if (key - lo + lane * BN < nb16 && n + lane < nt) pages = page_of(key + lane * BN);
-            __syncwarp();
-        }
-        const int page = kPaged ? __shfl_sync(0xffffffffu, pages, n & 31) : 0;
-        const int row = kPaged ? key % p.page_size : k_start + key;
-        const bool whole = key - lo + BN <= nb16 || !Tile(w, t0 + n).joins_sinks();  // one box per panel
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            const int slot = side * kHalf + next[side];
-            next[side] = next[side] + 1 == kHalf ? 0 : next[side] + 1;
-            if (slot >= L::kSlotStage && !staged) {
-                ok = ok && warp_wait(bar(B::SG + work_slot), staging, abort_flag);
-                staged = true;
-            }
-            ok = ok && warp_wait(bar(B::TE + slot), ((phases >> slot) & 1u) ^ 1u, abort_flag);
-            if (!ok) break;
-            if (el) {
-                const uint32_t full_bar = bar(B::TF + slot), dst = smem_base + L::kOffSlots + (uint32_t)(slot * L::kTileBytes);
-                if (whole) {
-                    const CUtensorMap* map = v ? &tm.v : &tm.k;
-                    mbar_arrive_expect_tx(full_bar, (uint32_t)L::kTileBytes);
-#pragma unroll
-                    for (int pn = 0; pn < L::kPanels; ++pn) {
-                        if (kPaged) tma_load_4d(dst + pn * L::kPanelBytes, map, pn * 64, hk, row, page, full_bar);
-                        else tma_load_3d(dst + pn * L::kPanelBytes, map, pn * 64, hk, row, full_bar);
-                    }
-                } else {  // joins sink keys: pieces of 16 keys
-                    const CUtensorMap* map = v ? &tm.v_small : &tm.k_small;
-                    const Tile t(w, t0 + n);
-                    mbar_arrive_expect_tx(full_bar, (uint32_t)(t.nk * 16 * 128 * L::kPanels));
-                    for (int x = 0; x < t.nk; ++x) {
-                        const int k16 = t.key(16 * x), pg = kPaged ? page_of(k16) : 0;
-#pragma unroll
-                        for (int pn = 0; pn < L::kPanels; ++pn) {
-                            const uint32_t d = dst + (uint32_t)(pn * L::kPanelBytes + x * 2048);
-                            if (kPaged) tma_load_4d(d, map, pn * 64, hk, k16 % p.page_size, pg, full_bar);
-                            else tma_load_3d(d, map, pn * 64, hk, k_start + k16, full_bar);
-                        }
-                    }
-                }
-            }
-            phases ^= 1u << slot;
-        }
-    }
-    if (ok && !staged) ok = warp_wait(bar(B::SG + work_slot), staging, abort_flag);
-    __syncwarp();
-    if (lane == 0) *state = (uint32_t)next[0] | ((uint32_t)next[1] << 4) | (phases << 8);
-    __syncwarp();
-    return ok;
-}
-
-// A token item (see WorkItem), on warp-level MMAs with the rows in N, as the decode kernel does.  The two sides' warps take
-// tiles in turn, a warp 32 keys of a tile: what a warp does with a tile is a chain of latencies (look at a barrier, ldmatrix,
-// MMA, maximum across lanes, exponential, MMA).
-// A function of its own, not inlined: with its code in the softmax role the tile loop of the other items comes out slower (prompt
-// chunks of a serving step 315 us, 308 this way).
-template <int D>
-__device__ __noinline__ bool token_item(const PrefillParams& p, uint32_t smem_base, int work_slot) {
-    using L = PrefillSmem<D>;
-    constexpr int BN = kPrefillBN, NS = L::kSlots;
-    using B = PrefillBars<NS>;
-    using Tile = TileGeom<BN>;
-    uint8_t* smem_gen = reinterpret_cast<uint8_t*>(__cvta_shared_to_generic(smem_base));
-    const uint32_t sSlots = smem_base + L::kOffSlots;
-    auto bar = [&](int i) -> uint32_t { return smem_base + (uint32_t)L::kOffBar + 8u * (uint32_t)i; };
-    auto uniform = [](int x) -> int { return __shfl_sync(0xffffffffu, x, 0); };
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_gen + L::kOffMisc + 20);
-    const volatile WorkItem& wv = reinterpret_cast<volatile WorkItem*>(smem_gen + L::kOffMisc + 32)[work_slot];
-    float2* s_merge = reinterpret_cast<float2*>(smem_gen + L::kOffMerge);
-    const int lane = threadIdx.x & 31, warp = uniform((int)(threadIdx.x >> 5)), side = warp >> 2, wq = warp & 3;
-    constexpr int NKK = D / 16, kCh = D / 32;
-    using Vec = typename std::conditional<kCh == 4, float4, float2>::type;
-    volatile uint32_t* t_state = reinterpret_cast<volatile uint32_t*>(smem_gen + L::kOffToken) + warp;
-    int t_slot = (int)(*t_state & 0xffu), t_items = (int)(*t_state >> 31);  // next slot, parity of the items so far
-    uint32_t t_phases = (*t_state >> 8) & 0x7fffffu;                        // bit: parity of the slot's next use
-    auto arrive = [&](int b) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(b));
-    };
-    arrive(B::TI);
-    WorkItem w;  // in registers
-    w.full = uniform(wv.full);
-    w.i0 = uniform(wv.i0);
-    w.i1 = uniform(wv.i1);
-    w.lo = uniform(wv.lo);
-    w.nb16 = uniform(wv.nb16);
-    w.nv = uniform(wv.nv);
-    w.n_sink = uniform(wv.n_sink);
-    w.n_rem = w.s_rem = 0;
-    const int n_rows = uniform(wv.n_rows), G = uniform(wv.packed), t0 = uniform(wv.t0), t1 = t0 + uniform(wv.nt);
-    const int tok = uniform(wv.seq_start), hA = uniform(wv.hA);
-    const int g = lane >> 2, c = lane & 3;
-    const int key0 = 32 * wq;  // first of the warp's keys in a tile
-    const int krow = key0 + (lane & 15), kchk = lane >> 4;                              // ldmatrix rows: see decode_kernel
-    const int vrow = key0 + (lane & 7) + 8 * (lane >> 4), vchk = (lane >> 3) & 1;
-    // Q^T fragments: lane (g, c) holds channels 16kk + 2c, +1 and 16kk + 2c + 8, +9 of row g
-    uint32_t qf[NKK][2];
-    const uint32_t* qrow = reinterpret_cast<const uint32_t*>(p.q + ((size_t)(tok + (g < n_rows ? g / G : 0)) * p.Hq + hA + (g < n_rows ? g % G : 0)) * D);
-#pragma unroll
-    for (int kk = 0; kk < NKK; ++kk) {
-        qf[kk][0] = g < n_rows ? qrow[kk * 8 + c] : 0u;
-        qf[kk][1] = g < n_rows ? qrow[kk * 8 + c + 4] : 0u;
-    }
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f}, oacc[NKK][4];
-#pragma unroll
-    for (int qb = 0; qb < NKK; ++qb) oacc[qb][0] = oacc[qb][1] = oacc[qb][2] = oacc[qb][3] = 0.f;
-    // A half of the slots is this side's ring.  (Sides that shared a ring would wait for a use of a slot without having seen
-    // the other side's use before it, and take that for this one's while it has not landed.)
-    auto pass_slot = [&]() {
-        t_phases ^= 1u << t_slot;
-        t_slot = t_slot + 1 == (side + 1) * (NS / 2) ? side * (NS / 2) : t_slot + 1;
-    };
-    auto landed = [&]() -> bool { return warp_wait(bar(B::TF + t_slot), (t_phases >> t_slot) & 1u, abort_flag); };
-    for (int n = t0 + side; n < t1; n += 2) {
-        const Tile t(w, n);
-        const bool need_mask = SWAA_TILE_NEEDS_MASK(t, w, n, false, p.window, BN);
-        // what the first and the last row of the item see
-        const typename Tile::Seen first = t.seen(w, n, false, w.i0, p.window), last = t.seen(w, n, false, w.i1, p.window);
-        auto seen_by_any = [&](int col) -> bool {
-            return !need_mask || (col <= last.dc && (col >= first.wl || col < last.sk)) || (col >= last.s0 && col < last.s1);
-        };
-        const bool mine = !need_mask || __any_sync(0xffffffffu, seen_by_any(key0 + lane)) != 0;
-        if (!landed()) return false;
-        uint32_t tile = sSlots + (uint32_t)(t_slot * L::kTileBytes);
-        uint32_t pb[2][2];
-        if (mine) {
-            // ---- S^T = K Q^T: rows = keys (g, g + 8) of two groups of 16, columns = rows of the item (2c, 2c + 1)
-            float sa[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-            for (int kk = 0; kk < NKK; ++kk) {
-                const int chunk = 2 * kk + kchk;
-                const uint32_t at = tile + (uint32_t)((chunk >> 3) * L::kPanelBytes + krow * 128 + (((chunk & 7) ^ (krow & 7)) << 4));
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4(at + (uint32_t)(h * 2048), a0, a1, a2, a3);
-                    mma_bf16_16816(sa[h], a0, a1, a2, a3, qf[kk][0], qf[kk][1]);
-                }
-            }
-            arrive(B::TE + t_slot);
-            __syncwarp();
-            float alpha[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                if (need_mask) {
-                    const typename Tile::Seen v = t.seen(w, n, false, min(w.i0 + (2 * c + e) / G, w.i1), p.window);
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) {
-                        const int col = key0 + g + 8 * x;
-                        const bool seen = (col <= v.dc && (col >= v.wl || col < v.sk)) || (col >= v.s0 && col < v.s1);
-                        float& s = sa[x >> 1][2 * (x & 1) + e];
-                        s = seen ? s : -INFINITY;
-                    }
-                }
-                float bm = fmaxf(fmaxf(sa[0][e], sa[0][2 + e]), fmaxf(sa[1][e], sa[1][2 + e]));
-                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
-                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 8));
-                bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 16));
-                const float m_new = fmaxf(m_run[e], bm);
-                alpha[e] = m_run[e] == m_new ? 1.f : ex2f((m_run[e] - m_new) * p.sl2);
-                m_run[e] = m_new;
-                const float off = m_new == -INFINITY ? 0.f : m_new * p.sl2;  // a row that none of the warp's keys reaches yet
-                float sum = 0.f;
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    float& s = sa[x >> 1][2 * (x & 1) + e];
-                    s = ex2f(fmaf(s, p.sl2, -off));
-                    sum += s;
-                }
-                l_run[e] = l_run[e] * alpha[e] + sum;
-            }
-            if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f)) {
-#pragma unroll
-                for (int qb = 0; qb < NKK; ++qb) {
-                    oacc[qb][0] *= alpha[0];
-                    oacc[qb][1] *= alpha[1];
-                    oacc[qb][2] *= alpha[0];
-                    oacc[qb][3] *= alpha[1];
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                pb[h][0] = movmatrix_trans(pack_bf16x2(sa[h][0], sa[h][1]));
-                pb[h][1] = movmatrix_trans(pack_bf16x2(sa[h][2], sa[h][3]));
-            }
-        } else {
-            arrive(B::TE + t_slot);
-            __syncwarp();
-        }
-        pass_slot();
-        if (!landed()) return false;
-        if (mine) {
-            // ---- O^T += V^T P^T: rows = channels (16qb + g, + 8), columns = rows of the item.  Rows of V that no row of the
-            // item sees may hold anything (also NaN), or were not fetched: they are cleared.
-            tile = sSlots + (uint32_t)(t_slot * L::kTileBytes);
-            uint32_t mask[2][2] = {{0xffffffffu, 0xffffffffu}, {0xffffffffu, 0xffffffffu}};
-            if (need_mask)
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int col = key0 + 2 * c + 8 * x;
-                    mask[x >> 1][x & 1] = (seen_by_any(col) ? 0x0000ffffu : 0u) | (seen_by_any(col + 1) ? 0xffff0000u : 0u);
-                }
-#pragma unroll
-            for (int qb = 0; qb < NKK; ++qb) {
-                const int chunk = 2 * qb + vchk;
-                const uint32_t at = tile + (uint32_t)((chunk >> 3) * L::kPanelBytes + vrow * 128 + (((chunk & 7) ^ (vrow & 7)) << 4));
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t a0, a1, a2, a3;
-                    ldmatrix_x4_trans(at + (uint32_t)(h * 2048), a0, a1, a2, a3);
-                    mma_bf16_16816(oacc[qb], a0 & mask[h][0], a1 & mask[h][0], a2 & mask[h][1], a3 & mask[h][1], pb[h][0], pb[h][1]);
-                }
-            }
-        }
-        arrive(B::TE + t_slot);
-        __syncwarp();
-        pass_slot();
-    }
-    // ---- the warps' partial results meet in shared memory, in the Q tile: row r of warp i at (8 i + r) D, channels
-    // rotated by 8 per pair of rows (no bank conflicts); warp r then takes row r
-    // (a side without a tile gets here at once)
-    if (!warp_wait(bar(B::TR), (uint32_t)t_items ^ 1u, abort_flag)) return false;  // of the item before have been read
-    if (!warp_wait(bar(B::TI), (uint32_t)t_items, abort_flag)) return false;
-    float* part_o = reinterpret_cast<float*>(smem_gen + L::kOffQ);
-    float2* part_ml = s_merge;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        float l = l_run[e];
-        l += __shfl_xor_sync(0xffffffffu, l, 4);
-        l += __shfl_xor_sync(0xffffffffu, l, 8);
-        l += __shfl_xor_sync(0xffffffffu, l, 16);
-        const int r = 2 * c + e;
-        if (g == 0) part_ml[8 * warp + r] = make_float2(m_run[e], l);
-        float* row_o = part_o + (8 * warp + r) * D;
-#pragma unroll
-        for (int qb = 0; qb < NKK; ++qb) {
-            row_o[(16 * qb + g + 8 * c) & (D - 1)] = oacc[qb][e];
-            row_o[(16 * qb + g + 8 + 8 * c) & (D - 1)] = oacc[qb][2 + e];
-        }
-    }
-    arrive(B::TW);
-    if (!warp_wait(bar(B::TW), (uint32_t)t_items, abort_flag)) return false;
-    __syncwarp();
-    if (lane == 0) *t_state = (uint32_t)t_slot | (t_phases << 8) | ((uint32_t)(t_items ^ 1) << 31);
-    __syncwarp();
-    const int r = warp;
-    float M = -INFINITY, den = 0.f, acc[kCh];
-#pragma unroll
-    for (int e = 0; e < kCh; ++e) acc[e] = 0.f;
-    if (r < n_rows) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) M = fmaxf(M, part_ml[8 * i + r].x);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const float2 ml = part_ml[8 * i + r];
-            const float wgt = ml.x == -INFINITY ? 0.f : ex2f((ml.x - M) * p.sl2);
-            den = fmaf(wgt, ml.y, den);
-            const Vec v = *reinterpret_cast<const Vec*>(part_o + (8 * i + r) * D + ((lane * kCh + 8 * (r >> 1)) & (D - 1)));
-            const float* x = reinterpret_cast<const float*>(&v);
-#pragma unroll
-            for (int e = 0; e < kCh; ++e) acc[e] = fmaf(wgt, x[e], acc[e]);
-        }
-    }
-    fence_proxy_async_smem();  // the next Q tile is written here by a copy
-    arrive(B::TR);
-    __syncwarp();
-    if (r >= n_rows) return true;
-    const int parts = uniform(wv.parts);
-    if (parts > 1) {
-        // this part's row to its slot; the last part to arrive merges the row
-        const size_t at = (size_t)wv.slot * kTokenRows + r, at0 = (size_t)wv.first_slot * kTokenRows + r;
-        Vec v;
-        float* x = reinterpret_cast<float*>(&v);
-#pragma unroll
-        for (int e = 0; e < kCh; ++e) x[e] = acc[e];
-        reinterpret_cast<Vec*>(p.split_o + at * D)[lane] = v;
-        if (lane == 0) p.split_ml[at] = make_float2(M, den);
-        __threadfence();
-        __syncwarp();
-        int done = 0;
-        if (lane == 0) done = split_arrive(p.split_tickets + at0, p.stamp, parts) ? 1 : 0;
-        if (!uniform(done)) return true;
-        __threadfence();
-        const RowResult<D> row = merge_parts<D>(p.split_ml + at0, p.split_o + at0 * D, parts, p.sl2);
-        M = row.m;
-        den = row.l;
-#pragma unroll
-        for (int e = 0; e < kCh; ++e) acc[e] = row.o[e];
-    }
-    const float inv = den > 0.f ? 1.f / den : 0.f;
-    const int t = tok + r / G, h = hA + r % G;
-    uint32_t* to = reinterpret_cast<uint32_t*>(p.out + ((size_t)t * p.Hq + h) * D + lane * kCh);
-#pragma unroll
-    for (int e = 0; e < kCh; e += 2) to[e / 2] = pack_bf16x2(acc[e] * inv, acc[e + 1] * inv);
-    if (p.lse != nullptr && lane == 0)
-        p.lse[(size_t)h * p.T + t] = M == -INFINITY ? -INFINITY : (M * p.sl2 + log2f(den)) * 0.6931471805599453f;
-    return true;
-}
-
 // kMode 0: self attention.  1: chunked prefill, the queries are the last len_q tokens of a longer key sequence
 // (separate packing of the keys).  2: the same with keys and values in pages addressed through a block table.
 // 3: context-parallel prefill, mode 1 with the local keys starting at position key_pos0[b] of their sequence and the
@@ -883,7 +441,7 @@ __device__ __noinline__ bool token_item(const PrefillParams& p, uint32_t smem_ba
 // meaning "S has been read"; items are never packed.
 template <int D, int kMode, bool kLseOnly = false>
 __global__ void __launch_bounds__(kPrefillThreads, 1)
-prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ PrefillParams p) {
+prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
     using L = PrefillSmem<D>;
     constexpr bool kChunked = kMode >= 1, kPaged = kMode == 2, kCp = kMode == 3;
     constexpr int BM = kPrefillBM, BN = kPrefillBN;
@@ -892,7 +450,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
     // A packed item's ring spans all slots where the keys of a short sequence can be many (generated tokens).  In the
     // self-attention instance they cannot, and the loops are shorter without the second order of slots.
     constexpr bool kDeepRing = kChunked && !kLseOnly;
-    constexpr bool kToken = kDeepRing && !kCp;
     using Tile = TileGeom<BN>;
 
     extern __shared__ uint8_t smem_raw[];
@@ -904,11 +461,19 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
     auto bar = [&](int i) -> uint32_t { return bars + 8u * (uint32_t)i; };
     // barrier indices
     constexpr int NS = L::kSlots;
-    using B = PrefillBars<NS>;
-    constexpr int BAR_QF = B::QF, BAR_QE = B::QE, BAR_F = B::F, BAR_E = B::E, BAR_VC = B::VC, BAR_SF = B::SF, BAR_PR = B::PR, BAR_OD = B::OD;
-    constexpr int BAR_OF = B::OF, BAR_WF = B::WF, BAR_WE = B::WE, BAR_NB = B::NB, BAR_MG = B::MG, BAR_SG = B::SG, BAR_FIN = B::FIN;
-    constexpr int BAR_TF = B::TF, BAR_TE = B::TE, BAR_TW = B::TW;
-    static_assert(B::TI + 1 == L::kNumBars, "barrier count");
+    constexpr int BAR_QF = 0, BAR_QE = 1, BAR_F = 2, BAR_E = BAR_F + NS;  // slot full, slot empty
+    // paged only, one per slot: the rows of the V tile in that slot past the last key have been cleared.
+    // Completed once per cleared tile; the issuer keeps the slot's phase bit.  The producer cannot
+    // clear a slot twice before the issuer has waited for the first clear: reusing the slot needs the
+    // issuer's empty commit, which follows that wait.
+    constexpr int BAR_VC = BAR_E + NS;
+    // per side: S full; P ready; O done, O free
+    constexpr int BAR_SF = BAR_VC + NS, BAR_PR = BAR_SF + 2, BAR_OD = BAR_PR + 2, BAR_OF = BAR_OD + 2;
+    // work descriptor full / empty per slot, next-block answer, hand-over of packed items (per row quadrant), staging free
+    // for the ring of a packed item (per work slot), final
+    constexpr int BAR_WF = BAR_OF + 2, BAR_WE = BAR_WF + 2, BAR_NB = BAR_WE + 2, BAR_MG = BAR_NB + 1, BAR_SG = BAR_MG + 4;
+    constexpr int BAR_FIN = BAR_SG + 2;
+    static_assert(BAR_FIN + 1 == L::kNumBars, "barrier count");
     const uint32_t s_answer = smem_base + L::kOffMisc;  // 16 bytes
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_gen + L::kOffMisc + 16);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -926,9 +491,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
             uint32_t count = 1u;
             if ((i >= BAR_PR && i < BAR_OD) || i == BAR_OF || i == BAR_OF + 1) count = 4u;  // a lane of each softmax warp of the side
             if (i == BAR_WE || i == BAR_WE + 1) count = 10u;   // producer, issuer, eight softmax warps
-            if (i == BAR_SG || i == BAR_SG + 1 || i >= BAR_TW) count = 8u;  // a lane of each softmax warp
-            if (i >= BAR_TE && i < BAR_TW) count = 4u;                      // of the four warps that share a tile
-            if (i == B::TI) count = 9u;                                     // of each softmax warp, and the producer
+            if (i == BAR_SG || i == BAR_SG + 1) count = 8u;    // a lane of each softmax warp
             mbar_init(bar(i), count);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -950,6 +513,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     grid_wait();  // nothing above touches global memory
+    if ((kMode == 1 || kMode == 2) && p.token_len >= 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // Consumers of the work descriptors: item `it` is in slot it & 1; they read it in place and release it at their end of
     // the item.
@@ -969,36 +533,16 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
         // The grid has one block per item (an upper bound); as many as fit start, and each takes over the indices of
         // blocks that have not started, so items go to whichever SM is free.  Items are ordered heavy-first, so that the
         // short ones fill the end: sequences by the keys that an item of theirs visits (32 sequences at a time, the last
-        // ones of the batch first), last tile of a sequence first.  Lane l looks after sequence base_b - l.  Token items come
-        // behind the others: an SM that changes between the two kinds waits until its ring is empty, and the parts, the shortest
-        // items, fill the end.  (Serving step of 4 chunks and 24 generated tokens: 426 us; token items spread evenly among the
-        // others 543, spread over their first half or three quarters 468 and 486, in order of their keys 434.)
-        // Serving step of 4 chunks and 24 generated tokens at 1k to 32k keys in pages: 582 us in batch order, 493 this way.
+        // ones of the batch first), last tile of a sequence first.  Lane l looks after sequence base_b - l.
+        // Serving step of 4 chunks and 24 generated tokens at 1k to 32k keys in pages, all as items of this kernel: 582 us in batch
+        // order, 493 this way.
         int base_b = p.B - 1;       // sequence of lane 0
         int base_w = 0;             // index of the first item of this group of 32 sequences
         int f_s = 0, f_len = 0, f_ks = 0, f_off = 0, f_full = full_all ? 1 : 0, f_sink = p.n_sink, f_srem = 0;
         int f_packed = 0, f_items = 0, f_before = 0, group_items = 0;  // items of the lane's sequence, those ahead of them, and all of the group
-        int f_parts = 1, f_slot = 0, group_slots = 0, base_slot = 0;   // parts of an item, slots as items
-        int part_tiles = 0;  // key tiles of a part, 0: no item is split
-        int group_tokens = 0;  // token items of the group
-        // key tiles of a token item of the lane's sequence, 0 where it has none
-        auto token_tiles = [&]() -> int {
-            if (f_items == 0 || f_len * p.G > kTokenRows) return 0;
-            WorkItem d;
-            d.seq_len = f_len;
-            d.packed = 1;
-            d.full = f_full;
-            d.k_off = f_off;
-            d.n_sink = f_sink;
-            d.s_rem = 0;
-            d.complete<BN, kPaged, kCp, kLseOnly>(p, 0);
-            return d.nt;
-        };
         auto load_group = [&]() {
             const int b = base_b - lane;
             f_items = 0;
-            f_parts = 1;
-            int slots = 0;
             if (b >= 0) {
                 const int s0 = p.cu_seqlens[b], e0 = p.cu_seqlens[b + 1];
                 int len = e0 - s0;
@@ -1032,50 +576,19 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
                 f_s = s0;
                 f_len = len;
                 f_packed = !kLseOnly && len <= p.pack_tokens ? 1 : 0;
-                f_items = len == 0 ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_units);
-                if (kToken && part_tiles > 0 && f_items > 0) {
-                    const int tiles = token_tiles();
-                    f_parts = min(kSplitMaxParts, max(1, (tiles + part_tiles - 1) / part_tiles));
-                    f_items *= f_parts;
-                    if (f_parts > 1) slots = f_items;
-                }
-            }
-            if (kToken && part_tiles > 0) {
-                f_slot = 0;
-                for (int j = 0; j < 32; ++j) {
-                    const int sj = __shfl_sync(0xffffffffu, slots, j);
-                    if (j < lane) f_slot += sj;
-                }
-                group_slots = __reduce_add_sync(0xffffffffu, slots);
+                f_items = len == 0 || (kChunked && !kCp && len <= p.token_len) ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_units);
             }
             group_items = __reduce_add_sync(0xffffffffu, f_items);
             f_before = 0;
             if (p.B > 1) {
                 const int len_k = f_off + f_len;
-                int weight = f_items == 0 ? 0 : (f_full ? len_k : (int)min((long long)len_k, (long long)p.window + p.n_sink + BM));
-                if (kToken && f_parts > 1) weight = min(weight, part_tiles * BN);
-                const bool tok = kToken && f_len * p.G <= kTokenRows;
+                const int weight = f_items == 0 ? 0 : (f_full ? len_k : (int)min((long long)len_k, (long long)p.window + p.n_sink + BM));
                 for (int j = 0; j < min(32, p.B); ++j) {
                     const int wj = __shfl_sync(0xffffffffu, weight, j), ij = __shfl_sync(0xffffffffu, f_items, j);
-                    const bool tj = kToken && __shfl_sync(0xffffffffu, tok ? 1 : 0, j) != 0;
-                    if (tj == tok && (wj > weight || (wj == weight && j < lane))) f_before += ij;
+                    if (wj > weight || (wj == weight && j < lane)) f_before += ij;
                 }
-                if (kToken) group_tokens = __reduce_add_sync(0xffffffffu, tok ? f_items : 0);
             }
         };
-        if (kToken && p.split_tickets != nullptr) {
-            // The key tiles of the token items of all sequences are cut into one to four parts per SM of at least
-            // kSplitMinTiles tiles.  (The launch allows for four parts per SM more than there are items, and twice as many slots.)
-            long long total = 0;
-            for (base_b = p.B - 1; base_b >= 0; base_b -= 32) {
-                load_group();
-                total += (long long)__reduce_add_sync(0xffffffffu, min(token_tiles(), 1 << 24)) * p.Hkv;
-            }
-            const long long waves = min(4ll, max(1ll, total / ((long long)kSplitMinTiles * p.sms)));
-            const long long tiles = max((long long)kSplitMinTiles, (total + waves * p.sms - 1) / (waves * p.sms));
-            part_tiles = (int)min(tiles, 1ll << 30);
-            base_b = p.B - 1;
-        }
         load_group();
         int w = (int)blockIdx.x, it = 0;
         auto slot_words = [&](int slot) -> volatile int* { return reinterpret_cast<volatile int*>(work_slots + slot); };
@@ -1103,7 +616,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
             if (w < base_w) {  // an index before this group of sequences: start over
                 base_b = p.B - 1;
                 base_w = 0;
-                base_slot = 0;
                 load_group();
             }
             bool valid;  // an index past the last item is passed over (the grid is an upper bound)
@@ -1111,22 +623,14 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
                 valid = w < base_w + group_items;
                 if (valid || base_b < 32) break;
                 base_w += group_items;
-                base_slot += group_slots;
                 base_b -= 32;
                 load_group();
             }
             if (valid) {
-                int local = w - base_w;
-                bool of_kind = true;
-                if (kToken && p.B > 1) {  // token items behind the others
-                    const bool tok = local >= group_items - group_tokens;
-                    of_kind = tok == (f_len * p.G <= kTokenRows);
-                    if (tok) local -= group_items - group_tokens;
-                }
-                local -= f_before;
+                const int local = w - base_w - f_before;
                 ok = free_slot();
                 if (!ok) break;
-                if (of_kind && local >= 0 && local < f_items) {  // one lane
+                if (local >= 0 && local < f_items) {  // one lane
                     WorkItem d;
                     d.valid = 1;
                     d.seq_start = f_s;
@@ -1140,10 +644,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
                     d.s_rem = f_srem;
                     d.b = base_b - lane;
                     d.careful = 0;
-                    // parts of a sequence: the same keys of all heads one after another
-                    const int unit = f_packed ? (kToken ? local % p.Hkv : local) : local % p.n_units;
-                    d.complete<BN, kPaged, kCp, kLseOnly>(p, unit);
-                    if (kToken && f_len * p.G <= kTokenRows) d.keep_part(local / p.Hkv, f_parts, base_slot + f_slot + unit * f_parts);
+                    d.complete<BN, kPaged, kCp, kLseOnly>(p, f_packed ? local : local % p.n_units);
                     volatile int* to = slot_words(it & 1);
                     const int* from = reinterpret_cast<const int*>(&d);
 #pragma unroll
@@ -1187,39 +688,14 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
         uint32_t phases = 0;             // bit: parity of the slot's next use
         int sk = 0, sv = 0, sx = 0;      // next stage of the K and V rings, next slot of a packed item's ring
         uint32_t sg_phase = 0;           // bit: parity of the work slot's next packed item
-        bool after_token = false;        // the item before this one was a token item
-        if (kToken) {
-            if (lane == 0) reinterpret_cast<uint32_t*>(smem_gen + L::kOffToken)[8] = 0;
-            __syncwarp();
-        }
         bool ok = true;
-        int items = 0;                   // items with a Q tile
+        int items = 0;
         for (int it = 0; ok; ++it) {
             ok = wait_work(it);
             if (!ok) break;
             const volatile WorkItem& w = work_slots[it & 1];
             if (!uniform(w.valid)) break;
             const bool packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
-            // Token items and the others have barriers of their own for the same slots (and the token items keep their partial
-            // results where the others keep Q): between the two kinds the producer waits until the kind before is done.
-            if (kToken && uniform(w.parts) > 0) {
-                if (!after_token) {
-                    ok = warp_wait(bar(BAR_QE), ((uint32_t)items & 1u) ^ 1u, abort_flag);
-                    for (int slot = 0; slot < NS; ++slot)
-                        ok = ok && warp_wait(bar(BAR_E + slot), ((phases >> slot) & 1u) ^ 1u, abort_flag);
-                }
-                after_token = true;
-                ok = ok && token_loads<D, kPaged>(tm, p, smem_base, it & 1, (sg_phase >> (it & 1)) & 1u);
-                if (!ok) break;
-                sg_phase ^= 1u << (it & 1);
-                release_work(it);
-                continue;
-            }
-            if (kToken && after_token) {
-                ok = warp_wait(bar(BAR_WE + ((it - 1) & 1)), (uint32_t)((it - 1) >> 1) & 1u, abort_flag);
-                if (!ok) break;
-                after_token = false;
-            }
             const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
             const int len_k = uniform(w.k_off + w.seq_len), hk = uniform(w.hk), k_start = uniform(w.k_start);
             // Q tiles of both sides (the previous item's last Q K^T must have retired); packed: one tile serves both
@@ -1364,10 +840,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
             bool landed = false;
             while (!landed && global_timer_ns() - t0 < kWaitLimitNs) {
                 landed = items == 0 || mbar_try_wait(bar(BAR_QF), (uint32_t)(items - 1) & 1u);
-                const uint32_t t_phases = kToken ? reinterpret_cast<volatile uint32_t*>(smem_gen + L::kOffToken)[8] >> 8 : 0u;
-                for (int slot = 0; slot < NS; ++slot)
-                    landed = landed && mbar_try_wait(bar(BAR_F + slot), ((phases >> slot) & 1u) ^ 1u) &&
-                             mbar_try_wait(bar(BAR_TF + slot), ((t_phases >> slot) & 1u) ^ 1u);
+                for (int slot = 0; slot < NS; ++slot) landed = landed && mbar_try_wait(bar(BAR_F + slot), ((phases >> slot) & 1u) ^ 1u);
             }
         }
         __syncwarp();
@@ -1420,10 +893,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
             if (!ok) break;
             const volatile WorkItem& w = work_slots[it & 1];
             if (!uniform(w.valid)) break;
-            if (kToken && uniform(w.parts) > 0) {  // no product of it runs here
-                release_work(it);
-                continue;
-            }
             const bool is_packed = !kLseOnly && uniform(w.packed) != 0, hasB = uniform(w.hasB) != 0;
             const int nt = uniform(w.nt), n_rem = kCp ? uniform(w.n_rem) : 0;
             // Only the last tile can be narrow, and only the last band tile can have rows past the last key: the loop below reads
@@ -1558,10 +1027,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(b));
         };
-        if (kToken) {
-            if (lane == 0) reinterpret_cast<uint32_t*>(smem_gen + L::kOffToken)[warp] = (uint32_t)(side * (NS / 2));
-            __syncwarp();
-        }
         for (int it = 0; ok; ++it) {
             // every decision taken after a bounded wait is made for the whole warp: the warp-wide tensor-memory
             // instructions and votes below need all 32 lanes
@@ -1576,12 +1041,6 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const __grid_constant__ P
                 mbar_arrive(bar(BAR_SG + (it & 1)));
             }
             __syncwarp();
-            if (kToken && uniform(w.parts) > 0) {
-                ok = token_item<D>(p, smem_base, it & 1);
-                if (!ok) break;
-                release_work(it);
-                continue;
-            }
             if (side == 1 && !shared && !uniform(w.hasB)) {
                 release_work(it);
                 continue;
