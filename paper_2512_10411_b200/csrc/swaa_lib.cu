@@ -602,6 +602,7 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
     p.out = static_cast<__nv_bfloat16*>(out);
     p.lse = lse;
     p.token_len = -1;
+    p.sms = info.sm_count;
     p.cu_seqlens = cu_seqlens_q;
     p.cu_seqlens_k = cu_seqlens_k;
     p.B = B;
@@ -669,7 +670,6 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
         p.split_ml = reinterpret_cast<float2*>(ws + split.off_ml);
         p.split_o = reinterpret_cast<float*>(ws + split.off_o);
         p.stamp = next_call_stamp();
-        p.sms = info.sm_count;
     }
     p.token_len = only_tokens ? -1 : token_len;
     if (cu_seqlens_k != nullptr && !ex.lse_only) {

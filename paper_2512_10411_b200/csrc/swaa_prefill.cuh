@@ -79,12 +79,12 @@ struct PrefillParams {
     // Chunked / paged: sequences of at most this many queries are left to token_kernel, which is launched behind this kernel
     // and may start as soon as all blocks of this one have (-1: there are none).
     int token_len;
+    int sms;
     // token_kernel: tickets, (max, sum) and unnormalised O of the rows of split items (null: none are split), see there
     unsigned long long* split_tickets;
     float2* split_ml;
     float* split_o;
     unsigned long long stamp;     // 48-bit number unique to this call (never 0)
-    int sms;
 };
 
 // Tensor maps of one call; an instance reads those that it needs.
@@ -532,17 +532,19 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         // ====================================================================== work scheduler
         // The grid has one block per item (an upper bound); as many as fit start, and each takes over the indices of
         // blocks that have not started, so items go to whichever SM is free.  Items are ordered heavy-first, so that the
-        // short ones fill the end: sequences by the keys that an item of theirs visits (32 sequences at a time, the last
-        // ones of the batch first), last tile of a sequence first.  Lane l looks after sequence base_b - l.
-        // Serving step of 4 chunks and 24 generated tokens at 1k to 32k keys in pages, all as items of this kernel: 582 us in batch
-        // order, 493 this way.
+        // short ones fill the end: by the key tiles that they visit, over 32 sequences at a time (the last ones of the batch
+        // first), and last tile of a sequence first.  Lane l looks after sequence base_b - l.  Sequences one after another, the heaviest
+        // first, had left SMs with long items of the last sequence when the others were done: 3366 and 3292 tokens, full attention,
+        // 28 heads of 128: 200 -> 186 us; five of 149 to 3766, 16 heads: 172 -> 155; eight of 641 to 3009: 159 -> 148.  The look for
+        // an item costs 0.3 us where a block waits for its first one.
         int base_b = p.B - 1;       // sequence of lane 0
         int base_w = 0;             // index of the first item of this group of 32 sequences
         int f_s = 0, f_len = 0, f_ks = 0, f_off = 0, f_full = full_all ? 1 : 0, f_sink = p.n_sink, f_srem = 0;
-        int f_packed = 0, f_items = 0, f_before = 0, group_items = 0;  // items of the lane's sequence, those ahead of them, and all of the group
+        int f_packed = 0, f_tiles = 0, f_units = 0, f_top = 0;  // of the lane's sequence: query tiles, items per tile, most key tiles of an item
+        int group_items = 0, group_top = 0;                     // of the 32 sequences: items, most key tiles of an item
         auto load_group = [&]() {
             const int b = base_b - lane;
-            f_items = 0;
+            f_tiles = f_units = f_top = 0;
             if (b >= 0) {
                 const int s0 = p.cu_seqlens[b], e0 = p.cu_seqlens[b + 1];
                 int len = e0 - s0;
@@ -576,20 +578,24 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 f_s = s0;
                 f_len = len;
                 f_packed = !kLseOnly && len <= p.pack_tokens ? 1 : 0;
-                f_items = len == 0 || (kChunked && !kCp && len <= p.token_len) ? 0 : (f_packed ? p.Hkv : (len + BM - 1) / BM * p.n_units);
-            }
-            group_items = __reduce_add_sync(0xffffffffu, f_items);
-            f_before = 0;
-            if (p.B > 1) {
-                const int len_k = f_off + f_len;
-                const int weight = f_items == 0 ? 0 : (f_full ? len_k : (int)min((long long)len_k, (long long)p.window + p.n_sink + BM));
-                for (int j = 0; j < min(32, p.B); ++j) {
-                    const int wj = __shfl_sync(0xffffffffu, weight, j), ij = __shfl_sync(0xffffffffu, f_items, j);
-                    if (wj > weight || (wj == weight && j < lane)) f_before += ij;
+                if (len > 0 && !(kChunked && !kCp && len <= p.token_len)) {
+                    f_tiles = f_packed ? 1 : (len + BM - 1) / BM;
+                    f_units = f_packed ? p.Hkv : p.n_units;
+                    f_top = (f_off + len + BM - 1) / BM;
+                    if (!f_full) f_top = (int)min((long long)f_top, ((long long)p.window + p.n_sink + BM) / BM + 1);
                 }
             }
+            group_items = __reduce_add_sync(0xffffffffu, f_tiles * f_units);
+            group_top = __reduce_max_sync(0xffffffffu, f_top);
+        };
+        // query tiles of the lane's sequence (the last ones) whose items visit at least `level` key tiles, nearly: an order, no more
+        auto tiles_from = [&](int level) -> int {
+            if (level > f_top) return 0;
+            const int x = (level - 1) * BM - f_off;
+            return x <= 0 ? f_tiles : max(0, f_tiles - x / BM);
         };
         load_group();
+        const bool at_once = p.B <= 32 && group_items <= p.sms;  // every item starts at once: any order will do
         int w = (int)blockIdx.x, it = 0;
         auto slot_words = [&](int slot) -> volatile int* { return reinterpret_cast<volatile int*>(work_slots + slot); };
         // publishes the descriptor that lies in slot it & 1 as a second run of the item of slot o
@@ -627,15 +633,39 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 load_group();
             }
             if (valid) {
-                const int local = w - base_w - f_before;
+                int local = w - base_w, last = f_tiles - 1;  // among the items of a lane's tiles up to the last one
+                bool mine = lane == 0;
+                if (p.B > 1) {
+                    int lo = 1, hi = group_top + 1;  // the item's level: items from lo on are more than `local`, from hi on they are not
+                    int above = 0;                   // items from hi on
+                    while (hi - lo > 1 && !at_once) {
+                        const int mid = (lo + hi) / 2, n = __reduce_add_sync(0xffffffffu, f_units * tiles_from(mid));
+                        if (n > local) {
+                            lo = mid;
+                        } else {
+                            hi = mid;
+                            above = n;
+                        }
+                    }
+                    last -= tiles_from(hi);
+                    const int own = f_units * (last + 1 - (f_tiles - tiles_from(lo)));
+                    int before = own;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int x = __shfl_up_sync(0xffffffffu, before, o);
+                        if (lane >= o) before += x;
+                    }
+                    local -= above + before - own;
+                    mine = local >= 0 && local < own;
+                }
                 ok = free_slot();
                 if (!ok) break;
-                if (local >= 0 && local < f_items) {  // one lane
+                if (mine) {  // one lane
                     WorkItem d;
                     d.valid = 1;
                     d.seq_start = f_s;
                     d.seq_len = f_len;
-                    d.q0 = f_packed ? 0 : ((f_len + BM - 1) / BM - 1 - local / p.n_units) * BM;
+                    d.q0 = f_packed ? 0 : (last - local / f_units) * BM;
                     d.packed = f_packed;
                     d.full = f_full;
                     d.k_start = f_ks;
@@ -644,7 +674,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     d.s_rem = f_srem;
                     d.b = base_b - lane;
                     d.careful = 0;
-                    d.complete<BN, kPaged, kCp, kLseOnly>(p, f_packed ? local : local % p.n_units);
+                    d.complete<BN, kPaged, kCp, kLseOnly>(p, local % f_units);
                     volatile int* to = slot_words(it & 1);
                     const int* from = reinterpret_cast<const int*>(&d);
 #pragma unroll
