@@ -154,7 +154,7 @@ int swaa_prefill_paged_mixed(const void* q, const void* kpages, const void* vpag
 
 /*
  * swaa_prefill_chunked(_mixed) and swaa_prefill_paged(_mixed) with a workspace, which lets the key lists of sequences with few
- * queries (up to 32 rows of queries times group size: generated tokens) be cut into parts that several SMs walk; the last part
+ * queries (queries times group size at most 8: generated tokens) be cut into parts that several SMs walk; the last part
  * to end merges them.  is_full_seq (device, uint8 [B]) may be NULL: all sequences then follow is_full.
  *
  *   workspace     device, 256-byte aligned, at least swaa_prefill_split_workspace_size(...) bytes; contents need not be

@@ -168,15 +168,21 @@ def _stream_ptr(stream):
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-def _split_workspace(lib, device, stream, st: int, B, max_seqlen_k, Hq, Hkv, D, window, n_sink, any_full):
-    """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator
-    (None: nothing to cut)."""
-    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, Hq, Hkv, D, window, n_sink, any_full, st)
+def _split_workspace(lib, q, stream, B, max_seqlen_k, Hkv, window, n_sink, any_full):
+    """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator.
+    None where there is nothing to cut, or no memory left: the call goes without."""
+    if not isinstance(q, torch.Tensor) or not q.is_cuda:  # refused with the other arguments
+        return None
+    st = _stream_ptr(stream)
+    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, q.shape[1], Hkv, q.shape[2], window, n_sink, any_full, st)
     if nbytes == 0:
         return None
-    ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+    try:
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
+    except torch.OutOfMemoryError:
+        return None
     if stream is not None:  # allocated on the current stream, used on this one
-        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st, device=device))
+        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st, device=q.device))
     return ws
 
 
@@ -218,9 +224,7 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
     bf = torch.bfloat16
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_chunked: is_full_seq must have one entry per sequence")
-    st = _stream_ptr(stream)
-    ws = _split_workspace(lib, q.device, stream, st, B, int(max_seqlen_k), Hq, Hkv, D, int(window), int(n_sink),
-                          int(is_full_seq is not None or bool(is_full))) if q.is_cuda else None
+    ws = _split_workspace(lib, q, stream, B, int(max_seqlen_k), Hkv, int(window), int(n_sink), int(is_full_seq is not None or bool(is_full)))
     if ws is not None:
         rc = lib.swaa_prefill_chunked_split(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"),
                                             _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
@@ -228,7 +232,7 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
                                             _dev_ptr(is_full_seq, torch.uint8, "is_full_seq"), B, Tq, Tk,
                                             int(max_seqlen_q), int(max_seqlen_k), Hq, Hkv, D, int(window), int(n_sink),
                                             int(bool(is_full)), float(scale), _dev_ptr(lse, torch.float32, "lse"),
-                                            ws.data_ptr(), ws.numel(), st)
+                                            ws.data_ptr(), ws.numel(), _stream_ptr(stream))
         if rc != SWAA_OK:
             raise SwaaError(rc, "swaa_prefill_chunked_split")
         return
@@ -296,9 +300,8 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
     bf = torch.bfloat16
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_paged: is_full_seq must have one entry per sequence")
-    st = _stream_ptr(stream)
-    ws = _split_workspace(lib, q.device, stream, st, B, min(block_table.shape[1] * page_size, 2147483647), Hq, Hkv, D, int(window), int(n_sink),
-                          int(is_full_seq is not None or bool(is_full))) if q.is_cuda else None
+    ws = _split_workspace(lib, q, stream, B, min(block_table.shape[1] * page_size, 2147483647), Hkv, int(window), int(n_sink),
+                          int(is_full_seq is not None or bool(is_full)))
     if ws is not None:
         rc = lib.swaa_prefill_paged_split(_dev_ptr(q, bf, "q"), _dev_ptr(kpages, bf, "kpages"), _dev_ptr(vpages, bf, "vpages"),
                                           _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
@@ -307,7 +310,7 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
                                           _dev_ptr(is_full_seq, torch.uint8, "is_full_seq"), B, Tq, int(max_seqlen_q),
                                           block_table.shape[1], num_pages, page_size, Hq, Hkv, D, int(window), int(n_sink),
                                           int(bool(is_full)), float(scale), _dev_ptr(lse, torch.float32, "lse"),
-                                          ws.data_ptr(), ws.numel(), st)
+                                          ws.data_ptr(), ws.numel(), _stream_ptr(stream))
         if rc != SWAA_OK:
             raise SwaaError(rc, "swaa_prefill_paged_split")
         return
