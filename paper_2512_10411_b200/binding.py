@@ -168,22 +168,29 @@ def _stream_ptr(stream):
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
+def _scratch(nbytes: int, device, stream):
+    """Scratch of a call on `stream` (None: the current one), taken from torch's allocator in the order of that stream: a block that
+    another stream has freed may still be in use there.  None when no memory is left."""
+    try:
+        if stream is None:
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        if not isinstance(stream, torch.cuda.Stream):
+            st = _stream_ptr(stream)  # (a stream object made from address 0 would not be the default stream)
+            stream = torch.cuda.ExternalStream(st, device=device) if st else torch.cuda.default_stream(device)
+        with torch.cuda.stream(stream):
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        return None
+
+
 def _split_workspace(lib, q, stream, B, max_seqlen_k, Hkv, window, n_sink, any_full):
     """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator.
     None where there is nothing to cut, or no memory left: the call goes without."""
     if not isinstance(q, torch.Tensor) or not q.is_cuda:  # refused with the other arguments
         return None
-    st = _stream_ptr(stream)
-    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, q.shape[1], Hkv, q.shape[2], window, n_sink, any_full, st)
-    if nbytes == 0:
-        return None
-    try:
-        ws = torch.empty(nbytes, dtype=torch.uint8, device=q.device)
-    except torch.OutOfMemoryError:
-        return None
-    if stream is not None:  # allocated on the current stream, used on this one
-        ws.record_stream(stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(st, device=q.device))
-    return ws
+    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, q.shape[1], Hkv, q.shape[2], window, n_sink, any_full,
+                                                   _stream_ptr(stream))
+    return _scratch(nbytes, q.device, stream) if nbytes else None
 
 
 def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink: int, is_full: bool,

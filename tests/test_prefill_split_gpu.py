@@ -22,12 +22,14 @@ BATCHES = [
 ]
 
 
-def _run(paged, q, k, v, lq, lk, W, S, full, full_seq, **kw):
+def _run(paged, q, k, v, lq, lk, W, S, full, full_seq, stream=None):
+    """The call, on `stream` (a torch stream, or the address of one) behind all that the current one has been given."""
     out = torch.full_like(q, float("nan"))
     lse = torch.full((q.shape[1], q.shape[0]), float("nan"), device="cuda")
     fs = None if full_seq is None else torch.tensor(full_seq, dtype=torch.uint8, device="cuda")
     if not paged:
-        swaa.swaa_prefill_chunked(q, k, v, out, _cu(lq), _cu(lk), max(lq), max(lk), W, S, full, lse=lse, is_full_seq=fs, **kw)
+        cu_q, cu_k = _cu(lq), _cu(lk)
+        call = lambda: swaa.swaa_prefill_chunked(q, k, v, out, cu_q, cu_k, max(lq), max(lk), W, S, full, lse=lse, is_full_seq=fs, stream=stream)
     else:
         page, Hkv, D = 128, k.shape[1], k.shape[2]
         used = [-(-n // page) for n in lk]
@@ -41,10 +43,21 @@ def _run(paged, q, k, v, lq, lk, W, S, full, full_seq, **kw):
                 table[b, i] = order[n]
                 n += 1
             pos += L
-        swaa.swaa_prefill_paged(q, kp, vp, out, _cu(lq), torch.tensor(lk, dtype=torch.int32, device="cuda"), table.cuda(), max(lq), W, S,
-                                full, lse=lse, is_full_seq=fs, **kw)
-    assert swaa.last_device_status() == 0
+        cu_q, len_k, table = _cu(lq), torch.tensor(lk, dtype=torch.int32, device="cuda"), table.cuda()
+        call = lambda: swaa.swaa_prefill_paged(q, kp, vp, out, cu_q, len_k, table, max(lq), W, S, full, lse=lse, is_full_seq=fs, stream=stream)
+    torch_stream = _torch_stream(stream)
+    torch_stream.wait_stream(torch.cuda.current_stream())
+    call()
+    assert swaa.last_device_status(stream) == 0  # waits for the call
     return out, lse
+
+
+def _torch_stream(stream):
+    if stream is None:
+        return torch.cuda.current_stream()
+    if isinstance(stream, int):
+        return torch.cuda.ExternalStream(stream) if stream else torch.cuda.default_stream()
+    return stream
 
 
 @pytest.mark.parametrize("paged", [False, True])
@@ -70,10 +83,8 @@ def test_split_calls_on_other_streams_and_in_a_graph():
     q, k, v = make(lq, lk, 8, 2, 128, 77)
     want, _ = _run(False, q, k, v, lq, lk, W, S, True, None)
     side = torch.cuda.Stream()
-    side.wait_stream(torch.cuda.current_stream())
-    for stream in (side, side.cuda_stream):
+    for stream in (side, side.cuda_stream, 0):
         got, _ = _run(False, q, k, v, lq, lk, W, S, True, None, stream=stream)
-        side.synchronize()
         assert torch.equal(got, want)
     lib = binding.load_library()
     assert lib.swaa_prefill_split_workspace_size(3, 6000, 8, 2, 128, W, S, 1, None) > 0
@@ -88,3 +99,31 @@ def test_split_calls_on_other_streams_and_in_a_graph():
     g.replay()
     torch.cuda.synchronize()
     assert (out.float() - want.float()).norm() / want.float().norm() < 1e-2  # two correct splits: bf16 outputs differ by 2e-3
+
+
+@pytest.mark.parametrize("by", ["stream", "address", "zero"])
+def test_scratch_is_not_a_block_that_another_stream_still_uses(by):
+    """A block of the scratch's size, freed on the current stream with its reader still queued behind slow work, stays what it is
+    while a call on another stream runs, and the call's result is the usual one."""
+    lq, lk, W, S = (1, 1, 70), (6000, 1300, 900), 64, 4
+    q, k, v = make(lq, lk, 8, 2, 128, 77)
+    want, _ = _run(False, q, k, v, lq, lk, W, S, True, None)
+    side = torch.cuda.Stream()
+    stream = {"stream": side, "address": side.cuda_stream, "zero": 0}[by]
+    nbytes = binding.load_library().swaa_prefill_split_workspace_size(3, 6000, 8, 2, 128, W, S, 1, None)
+    work, kept, out = torch.zeros(1 << 28, device="cuda"), torch.zeros(nbytes, dtype=torch.uint8, device="cuda"), torch.zeros_like(q)
+    cu_q, cu_k = _cu(lq), _cu(lk)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):  # the current stream of the caller
+        for _ in range(2):
+            block = torch.full((nbytes,), 7, dtype=torch.uint8, device="cuda")
+            for _ in range(40):  # 2 GiB each: over 10 ms
+                work.add_(1.0)
+            kept.copy_(block)
+            del block
+            swaa.swaa_prefill_chunked(q, k, v, out, cu_q, cu_k, max(lq), max(lk), W, S, True, stream=stream)
+            torch.cuda.synchronize()
+            assert torch.equal(out, want) and bool((kept == 7).all())
+            kept.zero_()
+            out.zero_()
+            torch.cuda.synchronize()
