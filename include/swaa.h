@@ -161,7 +161,9 @@ int swaa_prefill_paged_mixed(const void* q, const void* kpages, const void* vpag
  *                 initialised.  Calls that may overlap need one each.
  *   any_full      whether any sequence of the call runs full attention (a mixed call: 1)
  * swaa_prefill_split_workspace_size returns 0 when no sequence of the call can be long enough to be cut, and while `stream` is
- * being captured (the workspace would have to live as long as the graph): call the form without a workspace then.
+ * being captured: what is allocated for this call alone would have to live as long as the graph.  Call the form without a
+ * workspace then (one SM walks a list as a whole; sums in another order, so the last bits differ), or ask before the capture and
+ * pass a workspace that lives as long as the graph.
  */
 size_t swaa_prefill_split_workspace_size(int B, int max_seqlen_k, int Hq, int Hkv, int D, int window, int n_sink, int any_full,
                                          void* stream);

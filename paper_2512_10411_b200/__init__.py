@@ -13,6 +13,7 @@ from .binding import (  # noqa: F401
     kernel_launch_count,
     prefill_block_shape,
     prefill_item_keys,
+    prefill_split_workspace_size,
     prefill_tile_needs_mask,
     prefill_tile_range,
     lib_path,

@@ -183,9 +183,19 @@ def _scratch(nbytes: int, device, stream):
         return None
 
 
-def _split_workspace(lib, q, stream, B, max_seqlen_k, Hkv, window, n_sink, any_full):
-    """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator.
-    None where there is nothing to cut, or no memory left: the call goes without."""
+def prefill_split_workspace_size(B, max_seqlen_k, Hq, Hkv, D, window, n_sink, any_full) -> int:
+    """Forwards to C swaa_prefill_split_workspace_size (bytes) for the current stream: ask outside a capture.  max_seqlen_k of a paged
+    call: max_blocks * page_size.  any_full: whether a sequence of the call may run full attention (is_full, or is_full_seq given)."""
+    return int(load_library().swaa_prefill_split_workspace_size(int(B), int(max_seqlen_k), int(Hq), int(Hkv), int(D), int(window),
+                                                                int(n_sink), int(bool(any_full)), _stream_ptr(None)))
+
+
+def _split_workspace(lib, q, stream, B, max_seqlen_k, Hkv, window, n_sink, any_full, workspace):
+    """Scratch of a call that may cut long key lists of generated tokens into parts: the caller's workspace, or from torch's
+    stream-ordered allocator.  None where there is nothing to cut, or no memory left: the call goes without."""
+    if workspace is not None:
+        _dev_ptr(workspace, torch.uint8, "workspace")
+        return workspace if workspace.numel() else None
     if not isinstance(q, torch.Tensor) or not q.is_cuda:  # refused with the other arguments
         return None
     nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, q.shape[1], Hkv, q.shape[2], window, n_sink, any_full,
@@ -214,10 +224,16 @@ def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink:
 
 
 def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q: int, max_seqlen_k: int, window: int,
-                         n_sink: int, is_full: bool, scale: float = 0.0, lse=None, stream=None, is_full_seq=None) -> None:
+                         n_sink: int, is_full: bool, scale: float = 0.0, lse=None, stream=None, is_full_seq=None,
+                         workspace=None) -> None:
     """Forwards to C swaa_prefill_chunked, or, when is_full_seq (uint8 [B], a mask policy per sequence) is given, to
-    C swaa_prefill_chunked_mixed.  q, out [Tq,Hq,D]; k, v [Tk,Hkv,D] bf16; cu_seqlens_* int32 [B+1];
-    lse f32 [Hq,Tq].  The queries of each sequence are the last len_q tokens of its len_k-token context."""
+    C swaa_prefill_chunked_mixed; to C swaa_prefill_chunked_split where key lists of generated tokens may be cut over several SMs.
+    q, out [Tq,Hq,D]; k, v [Tk,Hkv,D] bf16; cu_seqlens_* int32 [B+1];
+    lse f32 [Hq,Tq].  The queries of each sequence are the last len_q tokens of its len_k-token context.
+    workspace: scratch for the cut lists, uint8 of prefill_split_workspace_size(...) bytes, for this call alone until it has ended; an
+    empty tensor: no list is cut.  None: taken from torch's allocator, except while the stream is captured (no list is cut then: its
+    scratch would have to live as long as the graph).  A captured call that is to cut its lists, and to have the bits of the plain
+    call, is given a workspace that outlives the graph."""
     lib = load_library()
     Tq, Hq, D = q.shape
     Tk, Hkv = k.shape[0], k.shape[1]
@@ -231,7 +247,8 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
     bf = torch.bfloat16
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_chunked: is_full_seq must have one entry per sequence")
-    ws = _split_workspace(lib, q, stream, B, int(max_seqlen_k), Hkv, int(window), int(n_sink), int(is_full_seq is not None or bool(is_full)))
+    ws = _split_workspace(lib, q, stream, B, int(max_seqlen_k), Hkv, int(window), int(n_sink), int(is_full_seq is not None or bool(is_full)),
+                          workspace)
     if ws is not None:
         rc = lib.swaa_prefill_chunked_split(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"),
                                             _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
@@ -291,9 +308,12 @@ def swaa_prefill_backward(q, k, v, out, dout, lse, cu_seqlens, max_seqlen: int, 
 
 
 def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_table, max_seqlen_q: int, window: int,
-                       n_sink: int, is_full: bool, scale: float = 0.0, lse=None, stream=None, is_full_seq=None) -> None:
-    """Forwards to C swaa_prefill_paged (to C swaa_prefill_paged_mixed when is_full_seq, uint8 [B], is given).  q, out [Tq,Hq,D]; kpages, vpages [num_pages,page_size,Hkv,D] bf16;
-    cu_seqlens_q int32 [B+1]; seqlens_k int32 [B]; block_table int32 [B,max_blocks]; lse f32 [Hq,Tq]."""
+                       n_sink: int, is_full: bool, scale: float = 0.0, lse=None, stream=None, is_full_seq=None,
+                       workspace=None) -> None:
+    """Forwards to C swaa_prefill_paged (to C swaa_prefill_paged_mixed when is_full_seq, uint8 [B], is given; to C
+    swaa_prefill_paged_split where key lists may be cut).  q, out [Tq,Hq,D]; kpages, vpages [num_pages,page_size,Hkv,D] bf16;
+    cu_seqlens_q int32 [B+1]; seqlens_k int32 [B]; block_table int32 [B,max_blocks]; lse f32 [Hq,Tq].  workspace: as in
+    swaa_prefill_chunked, with max_seqlen_k = max_blocks * page_size."""
     lib = load_library()
     Tq, Hq, D = q.shape
     num_pages, page_size, Hkv, _ = kpages.shape
@@ -308,7 +328,7 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_paged: is_full_seq must have one entry per sequence")
     ws = _split_workspace(lib, q, stream, B, min(block_table.shape[1] * page_size, 2147483647), Hkv, int(window), int(n_sink),
-                          int(is_full_seq is not None or bool(is_full)))
+                          int(is_full_seq is not None or bool(is_full)), workspace)
     if ws is not None:
         rc = lib.swaa_prefill_paged_split(_dev_ptr(q, bf, "q"), _dev_ptr(kpages, bf, "kpages"), _dev_ptr(vpages, bf, "vpages"),
                                           _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),

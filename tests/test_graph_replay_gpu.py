@@ -1,6 +1,7 @@
 """Calls captured in a CUDA graph and replayed with other inputs in the same buffers give what a plain call gives for those
 inputs: decode with items cut into two and into many parts (the workspace then holds what the replay before left there),
-and a training step."""
+a serving step of prompt chunks and generated tokens, and a training step."""
+import numpy as np
 import pytest
 import torch
 
@@ -71,6 +72,75 @@ def test_decode(form, lens, Hq, Hkv, D):
         sl.copy_(torch.tensor([max(n - 37 * step, 1) for n in lens], dtype=torch.int32))
 
     _replay_and_compare(call, _capture(call), out, refill)
+
+
+@pytest.mark.parametrize("workspace", [False, True])
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("Hq,Hkv,D", [(8, 2, 128), (16, 2, 64)])
+@pytest.mark.parametrize("tokens_only", [False, True])
+def test_serving_step(tokens_only, Hq, Hkv, D, paged, workspace):
+    """Generated tokens whose key lists a plain call cuts over several SMs.  Captured with a workspace the call has the bits of the
+    plain one (whatever the replay before left there); captured without, those of a call that cuts no list."""
+    lq = (1, 1, 1, 1) if tokens_only else (70, 1, 1, 1)
+    caps, W, S, page = (1500, 9000, 41000, 1100), 200, 4, 128  # the third list: the most parts, 32
+    B, Tq, nb = len(lq), sum(lq), -(-max(caps) // page)
+    q = torch.empty((Tq, Hq, D), dtype=torch.bfloat16, device="cuda")
+    out, lse = torch.empty_like(q), torch.empty((Hq, Tq), device="cuda")
+    n_pages = sum(-(-n // page) for n in caps)
+    kv = [torch.empty((n_pages * page if paged else sum(caps), Hkv, D), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    pages = [t.view(n_pages, page, Hkv, D) if paged else None for t in kv]
+    cu_q = torch.tensor(np.concatenate([[0], np.cumsum(lq)]).astype(np.int32), device="cuda")
+    cu_k, lens = torch.zeros(B + 1, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    full_seq = torch.tensor([0, 1, 1, 0], dtype=torch.uint8, device="cuda")
+    table, n = torch.zeros((B, nb), dtype=torch.int32), 0
+    for b, c in enumerate(caps):
+        table[b, :-(-c // page)] = torch.arange(n, n + -(-c // page), dtype=torch.int32).flip(0)
+        n += -(-c // page)
+    table = table.cuda()
+
+    def call(ws=None):
+        if paged:
+            swaa.swaa_prefill_paged(q, *pages, out, cu_q, lens, table, max(lq), W, S, False, lse=lse, is_full_seq=full_seq, workspace=ws)
+        else:
+            swaa.swaa_prefill_chunked(q, *kv, out, cu_q, cu_k, max(lq), max(caps), W, S, False, lse=lse, is_full_seq=full_seq, workspace=ws)
+
+    nbytes = swaa.prefill_split_workspace_size(B, nb * page if paged else max(caps), Hq, Hkv, D, W, S, True)
+    assert nbytes > 0
+    own = torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda") if workspace else None
+
+    def refill(step):
+        g = torch.Generator(device="cuda").manual_seed(700 + step)
+        for t in (q, *kv):
+            t.copy_(torch.randn(t.shape, generator=g, device="cuda"))
+        lens.copy_(torch.tensor([c - 300 * step for c in caps], dtype=torch.int32))
+        cu_k[1:] = lens.cumsum(0)
+
+    refill(0)
+    graph, want = _capture(lambda: call(own)), []
+    for step in range(3):
+        refill(step)
+        call(None if workspace else q.new_empty(0, dtype=torch.uint8))
+        want.append((out.clone(), lse.clone()))
+    for rep in range(2):
+        for step in range(3):
+            refill(step)
+            out.fill_(float("nan"))
+            lse.fill_(float("nan"))
+            graph.replay()
+            assert swaa.last_device_status() == 0
+            assert torch.equal(out, want[step][0]) and torch.equal(lse, want[step][1]), f"replay {rep}, inputs {step}"
+
+
+def test_a_workspace_that_is_too_small_is_refused():
+    q, kv = torch.zeros((2, 8, 128), dtype=torch.bfloat16, device="cuda"), torch.zeros((6000, 2, 128), dtype=torch.bfloat16, device="cuda")
+    cu_q, cu_k = (torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([0, 1, 2], [0, 3000, 6000]))
+    nbytes = swaa.prefill_split_workspace_size(2, 3000, 8, 2, 128, 1, 0, True)
+    with pytest.raises(swaa.SwaaError, match="SWAA_ERR_WORKSPACE"):
+        swaa.swaa_prefill_chunked(q, kv, kv, torch.empty_like(q), cu_q, cu_k, 1, 3000, 1, 0, True,
+                                  workspace=torch.empty(nbytes - 1, dtype=torch.uint8, device="cuda"))
+    with pytest.raises(TypeError, match="workspace"):
+        swaa.swaa_prefill_chunked(q, kv, kv, torch.empty_like(q), cu_q, cu_k, 1, 3000, 1, 0, True,
+                                  workspace=torch.empty(nbytes, dtype=torch.float32, device="cuda"))
 
 
 @pytest.mark.parametrize("D", [64, 128])
