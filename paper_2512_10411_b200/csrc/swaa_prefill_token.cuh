@@ -77,6 +77,7 @@ __device__ __forceinline__ bool split_arrive(unsigned long long* t, unsigned lon
 
 // Merges the parts of a row (at stride kTokenRows): lane = part for (max, sum), then lane = D / 32 channels, sixteen parts in
 // flight.  (Loads past the last part are repeated and not used: conditional loads into an array cost 44 registers, which spilled.)
+// A part in which the row sees no key is left out: its O is 0 times values of keys that other rows see, which may not be numbers.
 template <int D>
 struct RowResult {
     float m, l, o[D / 32];
@@ -110,7 +111,7 @@ __device__ __forceinline__ RowResult<D> merge_parts(const float2* part_ml, const
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             const float wi = __shfl_sync(0xffffffffu, wgt, (j + i) & 31);
-            if (j + i < parts) {
+            if (j + i < parts && wi != 0.f) {
                 const float* y = reinterpret_cast<const float*>(&u[i]);
 #pragma unroll
                 for (int e = 0; e < kCh; ++e) r.o[e] = fmaf(wi, y[e], r.o[e]);
@@ -545,7 +546,7 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
                     const Vec v = *reinterpret_cast<const Vec*>(part_o + (8 * i + r) * D + ((lane * kCh + 8 * (r >> 1)) & (D - 1)));
                     const float* x = reinterpret_cast<const float*>(&v);
 #pragma unroll
-                    for (int e = 0; e < kCh; ++e) acc[e] = fmaf(wgt, x[e], acc[e]);
+                    for (int e = 0; e < kCh; ++e) acc[e] = wgt != 0.f ? fmaf(wgt, x[e], acc[e]) : acc[e];  // (see merge_parts)
                 }
             }
             arrive(L::kBarR);

@@ -1,5 +1,5 @@
 """What a sequence must not see does not reach its results: keys and values of its neighbours in a packed batch that hold
-NaN."""
+NaN, and those of later tokens in a key tile that earlier ones do not reach."""
 import numpy as np
 import pytest
 import torch
@@ -55,3 +55,19 @@ def test_backward_next_to_a_sequence_of_nan_keys(D, L0):
         for got, w, name in zip(grads(kk), want, ("dq", "dk", "dv")):
             err = (got[kept].double() - w[kept].double()).norm() / w[kept].double().norm()
             assert err.item() <= 1e-3, (name, bad)  # the order of the fp32 sums into dq varies: bf16 roundings that flip
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("len_q,first_bad", [(2, 128), (8, 128), (8, 133)])
+def test_values_of_later_tokens_in_a_tile_of_their_own(D, bad, len_q, first_bad):
+    # one query head per kv head, so that several tokens are rows of one item; the keys from 128 on are its second tile
+    len_k = 129 if len_q == 2 else 134
+    q, k, v = make((len_q, 40), (len_k, 300), 4, 4, D, 70)
+    want, want_lse, _ = run_chunked(q, k, v, (len_q, 40), (len_k, 300), 1, 0, True)
+    k[first_bad:len_k], v[first_bad:len_k] = float("nan"), bad
+    out, lse, status = run_chunked(q, k, v, (len_q, 40), (len_k, 300), 1, 0, True)
+    n = 128 - (len_k - len_q)  # queries that see the first tile only
+    assert status == 0 and n > 0
+    assert torch.equal(out[:n], want[:n]) and torch.equal(lse[:, :n], want_lse[:, :n])
+    assert torch.equal(out[len_q:], want[len_q:])
