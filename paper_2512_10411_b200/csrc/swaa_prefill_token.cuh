@@ -234,6 +234,7 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
         int next[2] = {0, 0};   // next slot of each half of the ring
         uint32_t phases = 0;    // bit: parity of the slot's next use
         uint32_t nb_phase = 0;
+        bool asked = false;     // for the next index, and the answer has not been seen
         int w = (int)blockIdx.x, it = 0;
         bool ok = true;
         // page of a key, out of range (the copy delivers zeros) when the table is wrong
@@ -252,6 +253,7 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
                 next_block_request(s_answer, bar(L::kBarNB));
             }
             __syncwarp();
+            asked = true;
             if (w < base_w) {  // an index before this group of sequences: start over
                 base_b = p.B - 1;
                 base_w = base_slot = 0;
@@ -339,6 +341,7 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
             }
             ok = warp_wait(bar(L::kBarNB), nb_phase, abort_flag);
             if (!ok) break;
+            asked = false;
             nb_phase ^= 1u;
             w = uniform(next_block_answer(s_answer));
         }
@@ -349,11 +352,11 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
             mbar_arrive(bar(L::kBarWF + (it & 1)));
         }
         if (!ok) {
-            // give outstanding copies a bounded chance to land before the block's memory is released
+            // give outstanding copies, and the answer to the last request, a bounded chance to land before the block's memory is released
             const uint64_t start = global_timer_ns();
             bool done = false;
             while (!done && global_timer_ns() - start < kWaitLimitNs) {
-                done = true;
+                done = !asked || mbar_try_wait(bar(L::kBarNB), nb_phase);
                 for (int slot = 0; slot < L::kSlots; ++slot) done = done && mbar_try_wait(bar(L::kBarF + slot), ((phases >> slot) & 1u) ^ 1u);
             }
         }
