@@ -190,17 +190,29 @@ def prefill_split_workspace_size(B, max_seqlen_k, Hq, Hkv, D, window, n_sink, an
                                                                 int(n_sink), int(bool(any_full)), _stream_ptr(None)))
 
 
-def _split_workspace(lib, q, stream, B, max_seqlen_k, Hkv, window, n_sink, any_full, workspace):
-    """Scratch of a call that may cut long key lists of generated tokens into parts: the caller's workspace, or from torch's
-    stream-ordered allocator.  None where there is nothing to cut, or no memory left: the call goes without."""
-    if workspace is not None:
-        _dev_ptr(workspace, torch.uint8, "workspace")
-        return workspace if workspace.numel() else None
-    if not isinstance(q, torch.Tensor) or not q.is_cuda:  # refused with the other arguments
+_UNCUT_KEYS = 1024  # lists of up to so many keys are not cut
+
+
+def _split_workspace(lib, q, stream, B, max_seqlen_q, max_seqlen_k, Hkv, window, n_sink, any_full):
+    """Scratch of a call that may cut long key lists of generated tokens into parts, from torch's stream-ordered allocator.  None
+    where there is nothing to cut, or no memory left: the call goes without.  (What can be told without the library is looked at
+    first: asking it takes 3 us of a host call of 9.)"""
+    if not isinstance(q, torch.Tensor) or not q.is_cuda or Hkv < 1:  # refused with the other arguments
         return None
-    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, q.shape[1], Hkv, q.shape[2], window, n_sink, any_full,
-                                                   _stream_ptr(stream))
+    if not any_full and window + n_sink + 3 * 128 <= _UNCUT_KEYS:  # whole tiles at both ends of the window
+        return None
+    Tq, Hq, D = q.shape
+    tokens = 8 // (Hq // Hkv or 8)  # queries of a sequence whose rows (query, head of the group) are at most 8
+    if tokens == 0 or Tq > (B - 1) * max_seqlen_q + tokens:  # the others cannot have so many queries: every sequence has more
+        return None
+    nbytes = lib.swaa_prefill_split_workspace_size(B, max_seqlen_k, Hq, Hkv, D, window, n_sink, int(any_full), _stream_ptr(stream))
     return _scratch(nbytes, q.device, stream) if nbytes else None
+
+
+def _own_workspace(workspace):
+    """The caller's workspace; None for an empty one, which asks for no list to be cut."""
+    _dev_ptr(workspace, torch.uint8, "workspace")
+    return workspace if workspace.numel() else None
 
 
 def swaa_prefill(q, k, v, out, cu_seqlens, max_seqlen: int, window: int, n_sink: int, is_full: bool,
@@ -247,8 +259,13 @@ def swaa_prefill_chunked(q, k, v, out, cu_seqlens_q, cu_seqlens_k, max_seqlen_q:
     bf = torch.bfloat16
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_chunked: is_full_seq must have one entry per sequence")
-    ws = _split_workspace(lib, q, stream, B, int(max_seqlen_k), Hkv, int(window), int(n_sink), int(is_full_seq is not None or bool(is_full)),
-                          workspace)
+    if workspace is not None:
+        ws = _own_workspace(workspace)
+    elif max_seqlen_k > _UNCUT_KEYS:
+        ws = _split_workspace(lib, q, stream, B, int(max_seqlen_q), int(max_seqlen_k), Hkv, int(window), int(n_sink),
+                              is_full_seq is not None or bool(is_full))
+    else:
+        ws = None
     if ws is not None:
         rc = lib.swaa_prefill_chunked_split(_dev_ptr(q, bf, "q"), _dev_ptr(k, bf, "k"), _dev_ptr(v, bf, "v"),
                                             _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),
@@ -327,8 +344,14 @@ def swaa_prefill_paged(q, kpages, vpages, out, cu_seqlens_q, seqlens_k, block_ta
     bf = torch.bfloat16
     if is_full_seq is not None and is_full_seq.numel() != B:
         raise ValueError("swaa_prefill_paged: is_full_seq must have one entry per sequence")
-    ws = _split_workspace(lib, q, stream, B, min(block_table.shape[1] * page_size, 2147483647), Hkv, int(window), int(n_sink),
-                          int(is_full_seq is not None or bool(is_full)), workspace)
+    max_seqlen_k = block_table.shape[1] * page_size
+    if workspace is not None:
+        ws = _own_workspace(workspace)
+    elif max_seqlen_k > _UNCUT_KEYS:
+        ws = _split_workspace(lib, q, stream, B, int(max_seqlen_q), min(max_seqlen_k, 2147483647), Hkv, int(window), int(n_sink),
+                              is_full_seq is not None or bool(is_full))
+    else:
+        ws = None
     if ws is not None:
         rc = lib.swaa_prefill_paged_split(_dev_ptr(q, bf, "q"), _dev_ptr(kpages, bf, "kpages"), _dev_ptr(vpages, bf, "vpages"),
                                           _dev_ptr(out, bf, "out"), _dev_ptr(cu_seqlens_q, torch.int32, "cu_seqlens_q"),

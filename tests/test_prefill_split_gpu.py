@@ -77,6 +77,21 @@ def test_split_items_against_the_oracle(batch, heads, D, paged):
         np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
 
 
+def test_calls_that_the_library_would_cut_ask_it():
+    """What the binding tells without the library, over random calls: none that the library has a workspace size for goes without."""
+    rng, lib, cut = np.random.default_rng(0), binding.load_library(), 0
+    for _ in range(2000):
+        G, Hkv, B = (int(x) for x in (rng.choice([1, 2, 3, 4, 7, 8, 16]), rng.choice([1, 2, 8]), rng.integers(1, 40)))
+        max_k, window = (int(np.exp(rng.uniform(np.log(lo), np.log(5000)))) for lo in (100, 1))
+        n_sink, full = int(rng.choice([0, 4, 200])), bool(rng.integers(2))
+        q = torch.empty((B, G * Hkv, 64), dtype=torch.bfloat16, device="cuda")  # a token each
+        nbytes = lib.swaa_prefill_split_workspace_size(B, max_k, G * Hkv, Hkv, 64, window, n_sink, int(full), None)
+        ws = binding._split_workspace(lib, q, None, B, 1, max_k, Hkv, window, n_sink, full) if max_k > binding._UNCUT_KEYS else None
+        assert (0 if ws is None else ws.numel()) == nbytes
+        cut += nbytes > 0
+    assert 200 < cut < 1800
+
+
 def test_split_calls_on_other_streams_and_in_a_graph():
     """A stream of its own (object and address), and a capture, where the call goes without a workspace."""
     lq, lk, W, S = (1, 1, 70), (6000, 1300, 900), 64, 4

@@ -34,9 +34,10 @@ class _Library:
     """Stand-in for libswaa: notes the scratch and the stream of each launch, and asks for `nbytes` of scratch."""
 
     def __init__(self, nbytes):
-        self.nbytes, self.launches = nbytes, []
+        self.nbytes, self.launches, self.asked = nbytes, [], 0
 
     def swaa_prefill_split_workspace_size(self, *args):
+        self.asked += 1
         return self.nbytes
 
     def _split(self, *args):
@@ -120,3 +121,18 @@ def test_without_memory_the_call_goes_without_scratch(monkeypatch, allocator, st
     current, taken, _ = allocator
     assert _call(monkeypatch, allocator, 1 << 31, paged, stream) == [(None, launched_on)]
     assert taken == [] and current == [CALLERS]
+
+
+@pytest.mark.parametrize("Tq,B,max_q,Hq,Hkv,asked", [
+    (512, 1, 512, 8, 2, 0), (5, 1, 5, 8, 2, 0), (2, 1, 2, 8, 2, 1),    # one prompt; two tokens are eight rows
+    (1024, 2, 512, 8, 2, 0), (515, 2, 512, 8, 2, 0), (514, 2, 512, 8, 2, 1),
+    (520, 2, 512, 4, 4, 1), (521, 2, 512, 4, 4, 0), (100, 4, 50, 32, 2, 0), (100, 4, 50, 28, 4, 1),
+])
+def test_calls_without_room_for_a_generated_token_do_not_ask_for_scratch(monkeypatch, allocator, Tq, B, max_q, Hq, Hkv, asked):
+    lib = _Library(4096)
+    q, kv, cu = _cuda(Tq, Hq, 64), _cuda(3000, Hkv, 64), _cuda(B + 1, dtype=torch.int32)
+    with monkeypatch.context() as m:
+        m.setattr(binding, "load_library", lambda: lib)
+        m.setattr(torch, "empty", allocator[2])
+        binding.swaa_prefill_chunked(q, kv, kv, q, cu, cu, max_q, 3000, 64, 4, True)
+    assert lib.asked == asked and lib.launches == [(0xb10c if asked else None, CALLERS)]
