@@ -522,6 +522,7 @@ struct PrefillExtras {
 // key tiles of all items are cut into at most four parts per SM, which is as many parts as there are items more at most, in
 // twice as many slots (see token_kernel).
 struct SplitPlan {
+    long long tiles;    // of the longest item
     int slots, blocks;  // none: no item can be long enough
     size_t off_ml, off_o, bytes;
 };
@@ -529,9 +530,9 @@ static SplitPlan split_plan(int B, int max_seqlen_k, int G, int Hkv, int D, int 
     SplitPlan s;
     long long keys = max_seqlen_k;  // of one item, in whole tiles at both ends of the window
     if (!any_full) keys = std::min(keys, (long long)window + n_sink + 3 * kPrefillBN);
-    const long long tiles = (keys + kPrefillBN - 1) / kPrefillBN;
-    const long long parts = G > kTokenRows ? 0 : std::min((long long)B * Hkv * (tiles / kSplitMinTiles), 4ll * sms);
-    s.blocks = tiles > kSplitMinTiles ? (int)parts : 0;
+    s.tiles = (keys + kPrefillBN - 1) / kPrefillBN;
+    const long long parts = G > kTokenRows ? 0 : std::min((long long)B * Hkv * (s.tiles / kSplitMinTiles), 4ll * sms);
+    s.blocks = s.tiles > kSplitMinTiles ? (int)parts : 0;
     s.slots = 2 * s.blocks;
     s.off_ml = ((size_t)s.slots * kTokenRows * sizeof(unsigned long long) + 255) / 256 * 256;
     s.off_o = s.off_ml + (size_t)s.slots * kTokenRows * sizeof(float2);
@@ -662,6 +663,16 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
         if (Tq > (long long)(B - 1) * max_seqlen_q + token_len || (long long)B * Hkv > 2147483647LL - split.blocks) token_len = -1;
     }
     const bool only_tokens = max_seqlen_q <= token_len;
+    long long tokens = B;  // sequences that can be among them: more would leave the others with more than max_seqlen_q queries each
+    if (token_len >= 0 && !only_tokens) {
+        tokens = std::min(tokens, ((long long)B * max_seqlen_q - Tq) / (max_seqlen_q - token_len));
+        // Next to prompts, a few short lists stay packed items of the prefill kernel: a second kernel costs 3 to 5 us behind it,
+        // also one that finds nothing to do.  Packed (us, left) and in the token kernel, 250 mixed steps of 1 to 4 chunks
+        // and 0 to 64 tokens: lists of up to 10 tiles, at most two tiles per SM in all, 9.4 and 14.2 (four tokens, 28 heads), 10.4
+        // and 14.0 (64 tokens, 4 heads), 16.8 and 18.8, 14.9 and 13.9 at worst; longer lists 23.0 and 17.7 (13 tiles), 45.5 and
+        // 17.5 (34 tiles); more of them 24.4 and 17.5 (32 of 4 tiles, 8 kv heads), 26.9 and 19.6 (64 of 2).
+        if (split.tiles <= kTokenPackedTiles && tokens * Hkv * split.tiles <= 2ll * info.sm_count) token_len = -1;
+    }
     p.split_tickets = nullptr;
     if (ex.workspace != nullptr && split.blocks > 0) {
         if ((reinterpret_cast<uintptr_t>(ex.workspace) & 255u) != 0 || ex.workspace_bytes < split.bytes) return SWAA_ERR_WORKSPACE;
@@ -679,7 +690,8 @@ static int prefill_impl(const void* q, const void* k, const void* v, void* out, 
             else rc = D == 128 ? launch_prefill<128, 1>(tm, p, st) : launch_prefill<64, 1>(tm, p, st);
         }
         if (rc != SWAA_OK || token_len < 0) return rc;
-        const unsigned blocks = (unsigned)(B * Hkv) + (p.split_tickets != nullptr ? (unsigned)split.blocks : 0u);
+        const long long parts = p.split_tickets != nullptr ? std::min((long long)split.blocks, tokens * Hkv * (split.tiles / kSplitMinTiles)) : 0;
+        const unsigned blocks = (unsigned)(tokens * Hkv + parts);
         if (is_paged) return D == 128 ? launch_tokens<128, true>(tm, p, blocks, st) : launch_tokens<64, true>(tm, p, blocks, st);
         return D == 128 ? launch_tokens<128, false>(tm, p, blocks, st) : launch_tokens<64, false>(tm, p, blocks, st);
     }

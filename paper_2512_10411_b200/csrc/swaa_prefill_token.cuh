@@ -25,6 +25,7 @@ namespace swaa {
 
 constexpr int kTokenThreads = 288;
 constexpr int kTokenRows = 8;
+constexpr int kTokenPackedTiles = 10;  // a few lists of up to this many key tiles stay with the prefill kernel (see the launch)
 constexpr int kSplitMinTiles = 8;   // key tiles of a part, at least
 constexpr int kSplitMaxParts = 32;  // parts of an item (one lane each when they are merged)
 

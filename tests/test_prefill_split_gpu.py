@@ -92,6 +92,30 @@ def test_calls_that_the_library_would_cut_ask_it():
     assert 200 < cut < 1800
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("lq,lk,heads,kernels", [
+    ((1, 2, 1), (1281, 70, 9), (8, 2), 1),                           # tokens alone: the token kernel
+    ((100, 1, 1), (1280, 1280, 700), (8, 2), 1),                     # lists of ten tiles stay with the prompts
+    ((100, 1, 1), (1281, 1280, 700), (8, 2), 2),                     # of eleven do not
+    ((20,) + (1,) * 36, (90,) + (100,) * 36, (8, 8), 1),             # two tiles per SM in all (37 lists of one, eight heads)
+    ((20,) + (1,) * 37, (90,) + (100,) * 37, (8, 8), 2),             # one more
+    ((60, 70), (2000, 1500), (8, 2), 1),                             # no room for a token
+    ((70, 2, 0), (2000, 1500, 0), (6, 2), 2),
+    ((70, 3), (2000, 1500), (32, 2), 1),                             # sixteen heads to a group
+])
+def test_which_kernels_take_the_tokens(lq, lk, heads, kernels, paged):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the lines are those of 148 SMs")
+    q, k, v = make(lq, lk, *heads, 64, 950)
+    qh, kh, vh = (inputs.to_f32_numpy(t) for t in (q, k, v))
+    before = swaa.kernel_launch_count()
+    out, lse = _run(paged, q, k, v, lq, lk, 1, 0, True, None)
+    assert swaa.kernel_launch_count() - before == kernels
+    ref = oracle.prefill_chunked(qh, kh, vh, _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(), 1, 0, True)
+    check_against_oracle(out, ref["out"], f"{lq} {lk} {heads} paged={paged}")
+    np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
 def test_split_calls_on_other_streams_and_in_a_graph():
     """A stream of its own (object and address), and a capture, where the call goes without a workspace."""
     lq, lk, W, S = (1, 1, 70), (6000, 1300, 900), 64, 4

@@ -60,14 +60,15 @@ def test_backward_next_to_a_sequence_of_nan_keys(D, L0):
 @pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 @pytest.mark.parametrize("len_q,first_bad", [(2, 128), (8, 128), (8, 133)])
-def test_values_of_later_tokens_in_a_tile_of_their_own(D, bad, len_q, first_bad):
+@pytest.mark.parametrize("other", [(3, 300), (40, 3000), (40, 300)])  # tokens alone; behind a prompt; with the prompt, packed
+def test_values_of_later_tokens_in_a_tile_of_their_own(D, bad, len_q, first_bad, other):
     # one query head per kv head, so that several tokens are rows of one item; the keys from 128 on are its second tile
-    len_k = 129 if len_q == 2 else 134
-    q, k, v = make((len_q, 40), (len_k, 300), 4, 4, D, 70)
-    want, want_lse, _ = run_chunked(q, k, v, (len_q, 40), (len_k, 300), 1, 0, True)
-    k[first_bad:len_k], v[first_bad:len_k] = float("nan"), bad
-    out, lse, status = run_chunked(q, k, v, (len_q, 40), (len_k, 300), 1, 0, True)
-    n = 128 - (len_k - len_q)  # queries that see the first tile only
+    lq, lk = (len_q, other[0]), (129 if len_q == 2 else 134, other[1])
+    q, k, v = make(lq, lk, 4, 4, D, 70)
+    want, want_lse, _ = run_chunked(q, k, v, lq, lk, 1, 0, True)
+    k[first_bad:lk[0]], v[first_bad:lk[0]] = float("nan"), bad
+    out, lse, status = run_chunked(q, k, v, lq, lk, 1, 0, True)
+    n = 128 - (lk[0] - len_q)  # queries that see the first tile only
     assert status == 0 and n > 0
     assert torch.equal(out[:n], want[:n]) and torch.equal(lse[:, :n], want_lse[:, :n])
     assert torch.equal(out[len_q:], want[len_q:])
