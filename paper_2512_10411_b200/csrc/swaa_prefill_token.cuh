@@ -78,7 +78,6 @@ __device__ __forceinline__ bool split_arrive(unsigned long long* t, unsigned lon
 
 // Merges the parts of a row (at stride kTokenRows): lane = part for (max, sum), then lane = D / 32 channels, sixteen parts in
 // flight.  (Loads past the last part are repeated and not used: conditional loads into an array cost 44 registers, which spilled.)
-// A part in which the row sees no key is left out: its O is 0 times values of keys that other rows see, which may not be numbers.
 template <int D>
 struct RowResult {
     float m, l, o[D / 32];
@@ -112,7 +111,7 @@ __device__ __forceinline__ RowResult<D> merge_parts(const float2* part_ml, const
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             const float wi = __shfl_sync(0xffffffffu, wgt, (j + i) & 31);
-            if (j + i < parts && wi != 0.f) {
+            if (j + i < parts) {
                 const float* y = reinterpret_cast<const float*>(&u[i]);
 #pragma unroll
                 for (int e = 0; e < kCh; ++e) r.o[e] = fmaf(wi, y[e], r.o[e]);
@@ -515,6 +514,13 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
             }
             // ---- the warps' partial results meet in shared memory: row r of warp i at (8 i + r) D, channels rotated by 8 per pair of
             // rows (no bank conflicts); warp r then takes row r
+            if (__any_sync(0xffffffffu, m_run[0] == -INFINITY || m_run[1] == -INFINITY)) {
+                // A row that sees none of the warp's keys: 0 times the values of keys that other rows see, which may not be numbers.
+#pragma unroll
+                for (int qb = 0; qb < NKK; ++qb)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) oacc[qb][e] = m_run[e & 1] == -INFINITY ? 0.f : oacc[qb][e];
+            }
             if (!warp_wait(bar(L::kBarR), t_items ^ 1u, abort_flag)) return false;  // of the item before have been read
             float* part_o = reinterpret_cast<float*>(smem_gen + L::kOffPart);
             float2* part_ml = reinterpret_cast<float2*>(smem_gen + L::kOffMl);
@@ -550,7 +556,7 @@ token_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ C
                     const Vec v = *reinterpret_cast<const Vec*>(part_o + (8 * i + r) * D + ((lane * kCh + 8 * (r >> 1)) & (D - 1)));
                     const float* x = reinterpret_cast<const float*>(&v);
 #pragma unroll
-                    for (int e = 0; e < kCh; ++e) acc[e] = wgt != 0.f ? fmaf(wgt, x[e], acc[e]) : acc[e];  // (see merge_parts)
+                    for (int e = 0; e < kCh; ++e) acc[e] = fmaf(wgt, x[e], acc[e]);
                 }
             }
             arrive(L::kBarR);
