@@ -535,8 +535,9 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
         // short ones fill the end: by the key tiles that they visit, over 32 sequences at a time (the last ones of the batch
         // first), and last tile of a sequence first.  Lane l looks after sequence base_b - l.  Sequences one after another, the heaviest
         // first, had left SMs with long items of the last sequence when the others were done: 3366 and 3292 tokens, full attention,
-        // 28 heads of 128: 200 -> 186 us; five of 149 to 3766, 16 heads: 172 -> 155; eight of 641 to 3009: 159 -> 148.  The look for
-        // an item costs 0.3 us where a block waits for its first one.
+        // 28 heads of 128: 200 -> 186 us; five of 149 to 3766, 16 heads: 172 -> 155; eight of 641 to 3009: 159 -> 148.  A block waits
+        // for the look for its first item, mostly for instructions that are not in its cache yet: the loops are not unrolled, and
+        // calls whose items all start at once pass the search over.
         int base_b = p.B - 1;       // sequence of lane 0
         int base_w = 0;             // index of the first item of this group of 32 sequences
         int f_s = 0, f_len = 0, f_ks = 0, f_off = 0, f_full = full_all ? 1 : 0, f_sink = p.n_sink, f_srem = 0;
@@ -636,21 +637,23 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 int local = w - base_w, last = f_tiles - 1;  // among the items of a lane's tiles up to the last one
                 bool mine = lane == 0;
                 if (p.B > 1) {
-                    int lo = 1, hi = group_top + 1;  // the item's level: items from lo on are more than `local`, from hi on they are not
-                    int above = 0;                   // items from hi on
-                    while (hi - lo > 1 && !at_once) {
-                        const int mid = (lo + hi) / 2, n = __reduce_add_sync(0xffffffffu, f_units * tiles_from(mid));
-                        if (n > local) {
-                            lo = mid;
-                        } else {
-                            hi = mid;
-                            above = n;
+                    int own = f_tiles * f_units, above = 0;
+                    if (!at_once) {
+                        int lo = 1, hi = group_top + 1;  // the item's level: items from lo on are more than `local`, from hi on they are not
+                        while (hi - lo > 1) {            // above: items from hi on
+                            const int mid = (lo + hi) / 2, n = __reduce_add_sync(0xffffffffu, f_units * tiles_from(mid));
+                            if (n > local) {
+                                lo = mid;
+                            } else {
+                                hi = mid;
+                                above = n;
+                            }
                         }
+                        last -= tiles_from(hi);
+                        own = f_units * (last + 1 - (f_tiles - tiles_from(lo)));
                     }
-                    last -= tiles_from(hi);
-                    const int own = f_units * (last + 1 - (f_tiles - tiles_from(lo)));
                     int before = own;
-#pragma unroll
+#pragma unroll 1
                     for (int o = 1; o < 32; o <<= 1) {
                         const int x = __shfl_up_sync(0xffffffffu, before, o);
                         if (lane >= o) before += x;
@@ -665,7 +668,8 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     d.valid = 1;
                     d.seq_start = f_s;
                     d.seq_len = f_len;
-                    d.q0 = f_packed ? 0 : (last - local / f_units) * BM;
+                    const int back = (int)((unsigned)local / (unsigned)f_units);
+                    d.q0 = f_packed ? 0 : (last - back) * BM;
                     d.packed = f_packed;
                     d.full = f_full;
                     d.k_start = f_ks;
@@ -674,7 +678,7 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                     d.s_rem = f_srem;
                     d.b = base_b - lane;
                     d.careful = 0;
-                    d.complete<BN, kPaged, kCp, kLseOnly>(p, local % f_units);
+                    d.complete<BN, kPaged, kCp, kLseOnly>(p, local - back * f_units);
                     volatile int* to = slot_words(it & 1);
                     const int* from = reinterpret_cast<const int*>(&d);
 #pragma unroll
