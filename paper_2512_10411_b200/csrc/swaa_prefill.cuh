@@ -694,7 +694,12 @@ prefill_kernel(const __grid_constant__ PrefillMaps tm, const PrefillParams p) {
                 next_block_request(s_answer, bar(BAR_NB));
             }
             ok = warp_wait(bar(BAR_NB), nb_phase, abort_flag);
-            if (!ok) break;
+            if (!ok) {  // another role gave up: the answer has to land before the block's memory is released
+                const uint64_t t0 = global_timer_ns();
+                while (!mbar_try_wait(bar(BAR_NB), nb_phase) && global_timer_ns() - t0 < kWaitLimitNs) {
+                }
+                break;
+            }
             nb_phase ^= 1u;
             w = uniform(next_block_answer(s_answer));
         }
