@@ -1,6 +1,6 @@
 """Long key lists of generated tokens cut into parts (chunked and paged prefill with a workspace) against the float64 oracle:
-key counts around the smallest part, up to the most parts of an item, rows that end inside a warp, and the sequences that are
-not cut next to them."""
+key counts around the smallest part, more parts than one round of the merge takes and the most there are, every group size,
+tokens alone and next to prompts, which kernel takes them, and whose memory the scratch is."""
 import numpy as np
 import pytest
 import torch
@@ -19,6 +19,8 @@ BATCHES = [
     ((1, 1), (1024, 9000)),                          # not cut, and many parts
     ((3, 200, 1, 2), (5000, 700, 4481, 2049)),       # several rows per token group next to a chunk
     (tuple([1] * 40), tuple(range(300, 300 + 40 * 150, 150))),  # more than 32 sequences: two groups of the scheduler
+    ((1, 90, 1), (20500, 130, 4000)),                # 21 parts where there is one kv head: two rounds of the merge
+    ((1,), (41000,)),                                # 321 tiles: 32 parts, the most, of ten and eleven tiles
 ]
 
 
@@ -75,6 +77,29 @@ def test_split_items_against_the_oracle(batch, heads, D, paged):
         ref = oracle.prefill_chunked(qh, kh, vh, _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(), W, S, full, **kw)
         check_against_oracle(out, ref["out"], f"split {batch} {heads} D={D} paged={paged} W={W} S={S} full={full}")
         np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("G", [1, 2, 3, 4, 5, 6, 7, 8])
+def test_group_sizes(G, paged):
+    """As many tokens as fill the rows (8 // G), one, and lists that end inside a tile; the tokens have the same bits alone (one kernel, which
+    waits for what is before it) and next to a prompt (behind the prefill kernel)."""
+    most, Hkv, W, S = 8 // G, 2, 300, 20
+    lq, lk = (most, 1, most), (2500, 1111, 77)
+    q, k, v = make(lq, lk, G * Hkv, Hkv, 64, 920 + G)
+    for full, full_seq in ((True, None), (False, None), (False, [1, 0, 1])):
+        out, lse = _run(paged, q, k, v, lq, lk, W, S, full, full_seq)
+        kw = {} if full_seq is None else {"is_full_seq": np.array(full_seq, dtype=np.uint8)}
+        ref = oracle.prefill_chunked(*(inputs.to_f32_numpy(t) for t in (q, k, v)), _cu(lq).cpu().numpy(), _cu(lk).cpu().numpy(), W, S, full, **kw)
+        check_against_oracle(out, ref["out"], f"G={G} paged={paged} full={full} {full_seq}")
+        np.testing.assert_allclose(lse.cpu().numpy().T, ref["lse"], rtol=0, atol=2e-3)
+        if not full and full_seq is None:
+            continue  # few short lists: next to a prompt they are not the token kernel's
+        # the prompt in front: 150 queries of 2900 keys
+        p, pk, pv = make((150,), (2900,), G * Hkv, Hkv, 64, 930 + G)
+        both, both_lse = _run(paged, torch.cat([p, q]), torch.cat([pk, k]), torch.cat([pv, v]), (150, *lq), (2900, *lk), W, S, full,
+                              None if full_seq is None else [0, *full_seq])
+        assert torch.equal(both[150:], out) and torch.equal(both_lse[:, 150:], lse)
 
 
 def test_calls_that_the_library_would_cut_ask_it():

@@ -34,6 +34,26 @@ def test_forward_next_to_a_sequence_of_nan_keys_and_values(D, W, S, full):
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("W,S,full", [(100, 0, False), (100, 20, False), (1, 0, True)])
+@pytest.mark.parametrize("lq,lk", [((3, 2), (256, 300)), ((1, 4, 3), (2500, 2304, 130)), ((1, 3, 60), (144, 2512, 2600))])
+def test_generated_tokens_next_to_a_sequence_of_nan_keys_and_values(D, W, S, full, lq, lk):
+    q, k, v = make(lq, lk, 4, 2, D, 80 + W)
+    want, want_lse, _ = run_chunked(q, k, v, lq, lk, W, S, full)
+    # lists that end inside a tile; tokens alone also inside a group of 16 keys (next to a prompt a few short lists are the prefill
+    # kernel's, which reads keys in such groups)
+    for bad in range(len(lk)):
+        kk, vv = k.clone(), v.clone()
+        rows = slice(sum(lk[:bad]), sum(lk[:bad + 1]))
+        kk[rows] = vv[rows] = float("nan")
+        out, lse, status = run_chunked(q, kk, vv, lq, lk, W, S, full)
+        assert status == 0
+        for b in range(len(lq)):
+            mine = slice(sum(lq[:b]), sum(lq[:b + 1]))
+            if b != bad and lq[b] <= 4:
+                assert torch.equal(out[mine], want[mine]) and torch.equal(lse[:, mine], want_lse[:, mine]), (bad, b)
+
+
+@pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("L0", [64, 100, 192, 256])
 def test_backward_next_to_a_sequence_of_nan_keys(D, L0):
     lens, Hq, Hkv, W, S = (L0, 200), 4, 2, 100, 4
