@@ -135,7 +135,7 @@ int swaa_prefill_paged(const void* q, const void* kpages, const void* vpages, vo
                        int is_full, float scale, float* lse, void* stream);
 
 /*
- * Mixed batch: swaa_prefill_chunked / swaa_prefill_paged with a mask policy PER SEQUENCE, so that one launch serves
+ * Mixed batch: swaa_prefill_chunked / swaa_prefill_paged with a mask policy PER SEQUENCE, so that one call serves
  * sequences in different phases (Fig. 1a: prompt tokens under the SWA mask next to generated tokens under full
  * attention; App. "Inference Efficiency": a serving engine batches prefill chunks and decode tokens together).
  *   is_full_seq   device, uint8 [B]; sequence b runs full causal attention iff is_full_seq[b] != 0, else the

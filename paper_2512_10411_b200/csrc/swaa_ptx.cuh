@@ -10,7 +10,11 @@ namespace swaa {
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s per wait
 
 // Waits until the kernel before this one on the stream has ended and its writes are visible.  Every thread of every kernel
-// calls it before it touches global memory (see launch_overlapped), so the order of the stream's work is unchanged.
+// calls it before it touches global memory (see launch_overlapped), so the order of the stream's work is unchanged.  The one
+// exception is a kernel whose predecessor lets it in early (griddepcontrol.launch_dependents): token_kernel behind the
+// prefill kernel of the same call.  What makes that sound, and has to hold for any other pair: the predecessor lets it in behind
+// its own grid_wait, so that all earlier work has ended; the kernel touches nothing that the predecessor writes and writes nothing that it
+// reads; and every thread calls grid_wait before it leaves, so that its end stands for the end of both.
 // Nothing is read through __ldg or const __restrict__ pointers: those promise that the data does not change while the kernel
 // is resident, which the kernel before it may still be writing, and let the compiler move a load above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
