@@ -170,10 +170,13 @@ def _stream_ptr(stream):
 
 def _scratch(nbytes: int, device, stream):
     """Scratch of a call on `stream` (None: the current one), taken from torch's allocator in the order of that stream: a block that
-    another stream has freed may still be in use there.  None when no memory is left."""
+    another stream has freed may still be in use there.  None when no memory is left, or when it is the current stream that is being
+    captured: to take memory for another one could end the capture."""
     try:
         if stream is None:
             return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        if torch.cuda.is_current_stream_capturing():
+            return None
         if not isinstance(stream, torch.cuda.Stream):
             st = _stream_ptr(stream)  # (a stream object made from address 0 would not be the default stream)
             stream = torch.cuda.ExternalStream(st, device=device) if st else torch.cuda.default_stream(device)

@@ -131,6 +131,28 @@ def test_serving_step(tokens_only, Hq, Hkv, D, paged, workspace):
             assert torch.equal(out, want[step][0]) and torch.equal(lse, want[step][1]), f"replay {rep}, inputs {step}"
 
 
+def test_plain_call_on_another_stream_during_a_capture():
+    """The call is not part of the graph, and the capture goes on."""
+    q, kv = torch.randn((2, 8, 128), device="cuda").bfloat16(), torch.randn((6000, 2, 128), device="cuda").bfloat16()
+    cu_q, cu_k = (torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([0, 1, 2], [0, 3000, 6000]))
+    want, out, x, side = torch.empty_like(q), torch.empty_like(q), torch.zeros(10, device="cuda"), torch.cuda.Stream()
+    call = lambda o, **kw: swaa.swaa_prefill_chunked(q, kv, kv, o, cu_q, cu_k, 1, 3000, 1, 0, True, **kw)
+    call(want, workspace=q.new_empty(0, dtype=torch.uint8))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        x.add_(1.0)
+        call(out, stream=side)
+        x.add_(1.0)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    out.zero_()
+    x.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool((x == 2).all()) and bool((out == 0).all())
+
+
 def test_a_workspace_that_is_too_small_is_refused():
     q, kv = torch.zeros((2, 8, 128), dtype=torch.bfloat16, device="cuda"), torch.zeros((6000, 2, 128), dtype=torch.bfloat16, device="cuda")
     cu_q, cu_k = (torch.tensor(x, dtype=torch.int32, device="cuda") for x in ([0, 1, 2], [0, 3000, 6000]))

@@ -84,6 +84,7 @@ def allocator(monkeypatch):
     monkeypatch.setattr(torch.cuda, "default_stream", lambda device=None: _Stream(0))
     monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: _Stream(current[-1]))
     monkeypatch.setattr(torch.cuda, "is_initialized", lambda: False)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
     monkeypatch.setattr(torch.cuda, "stream", stream_context)
     return current, taken, empty
 
@@ -121,6 +122,14 @@ def test_without_memory_the_call_goes_without_scratch(monkeypatch, allocator, st
     current, taken, _ = allocator
     assert _call(monkeypatch, allocator, 1 << 31, paged, stream) == [(None, launched_on)]
     assert taken == [] and current == [CALLERS]
+
+
+@pytest.mark.parametrize("stream", [_Stream(0x2200), 0x3300, 0])
+def test_while_the_callers_stream_is_captured_nothing_is_taken_for_another(monkeypatch, allocator, stream):
+    _, taken, _ = allocator
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: True)
+    assert _call(monkeypatch, allocator, 4096, False, stream) == [(None, getattr(stream, "cuda_stream", stream))]
+    assert taken == []
 
 
 @pytest.mark.parametrize("Tq,B,max_q,Hq,Hkv,asked", [
